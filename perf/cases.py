@@ -158,14 +158,15 @@ def _levels(sids, V, depth):
 
 
 def _matcher(kind, rng, sids, V, B, num_nodes, share):
-    """(kind, host words, log2 of the filter's bits, hashes): every request may see its own random `share` of the SIDs."""
+    """Per request the SIDs it may see, its own random `share` of them (None: all), and the matcher that says so:
+    (kind, host words, log2 of the filter's bits, hashes)."""
     if kind == "none":
-        return (api.MATCH_NONE, None, 0, 0)
+        return None, (api.MATCH_NONE, None, 0, 0)
     seen = [rng.random(sids.shape[0]) < share for _ in range(B)]
     if kind == "bitmask":
-        return (api.MATCH_NODE_BITMASK, np.stack([api.grace_node_bitmask_build(sids, V, e, num_nodes) for e in seen]), 0, 0)
+        return seen, (api.MATCH_NODE_BITMASK, np.stack([api.grace_node_bitmask_build(sids, V, e, num_nodes) for e in seen]), 0, 0)
     log2_bits = 22 if sids.shape[0] > 100_000 else 20
-    return (api.MATCH_PREFIX_BLOOM, np.stack([api.grace_bloom_build(sids, V, e, log2_bits, 4) for e in seen]), log2_bits, 4)
+    return seen, (api.MATCH_PREFIX_BLOOM, np.stack([api.grace_bloom_build(sids, V, e, log2_bits, 4) for e in seen]), log2_bits, 4)
 
 
 def _weights(g, model, V, L):
@@ -183,19 +184,35 @@ def _weights(g, model, V, L):
     return dict(embed=lin(V + 1, D), pos=lin(L, D), lnf_g=one, lnf_b=zero, w_out=lin(V, D), layers=layers)
 
 
-def _decoder(c, rng, g):
+def _decoder_inputs(c, rng, g):
+    """What the decoder of a case is made from: catalog, what every request may see, weights."""
     beams = [int(x) for x in c["beams"].split(",")]
     L = len(beams)
+    i = SimpleNamespace(beams=beams, L=L, sids=_catalog(rng, c["n_sids"], c["V"], L))
+    i.bits, i.base, i.level_start = api.grace_trie_build_dense(i.sids, c["V"])
+    i.seen, i.matcher = _matcher(c["matcher"], rng, i.sids, c["V"], c["B"], int(i.level_start[-1]), 0.3)
+    i.weights = _weights(g, c["model"], c["V"], L)
+    return i
+
+
+def _decoder(c, i):
     n_layers, D, H, dh, F = MODELS[c["model"]]
-    sids = _catalog(rng, c["n_sids"], c["V"], L)
-    bits, base, level_start = api.grace_trie_build_dense(sids, c["V"])
-    matcher = _matcher(c["matcher"], rng, sids, c["V"], c["B"], int(level_start[-1]), 0.3)
-    dec = Decoder(n_layers=n_layers, d_model=D, n_heads=H, d_head=dh, d_ffn=F, V=c["V"], L=L, T_ctx=c["T"], B=c["B"],
-                  beam_sizes=beams + [c["K"]], weights=_weights(g, c["model"], c["V"], L), trie_bits=bits, trie_base=base,
-                  num_nodes=int(level_start[-1]), matcher=matcher, device=DEV, residual_bf16=c["bf16_stream"],
-                  level_start=level_start, logits_allowed_only=c["kind"] != "step" and c["bf16_stream"],
-                  masked_from_step=0 if c["kind"] == "step" else None)     # `logp` then keeps the raw logits
-    return dec, sids, level_start, beams
+    return Decoder(n_layers=n_layers, d_model=D, n_heads=H, d_head=dh, d_ffn=F, V=c["V"], L=i.L, T_ctx=c["T"], B=c["B"],
+                   beam_sizes=i.beams + [c["K"]], weights=i.weights, trie_bits=i.bits, trie_base=i.base,
+                   num_nodes=int(i.level_start[-1]), matcher=i.matcher, device=DEV, residual_bf16=c["bf16_stream"],
+                   level_start=i.level_start, logits_allowed_only=c["kind"] != "step" and c["bf16_stream"],
+                   masked_from_step=0 if c["kind"] == "step" else None)     # `logp` then keeps the raw logits
+
+
+def _step_state(c, i, rng, g):
+    """The state before step t: beam, parents of every step up to t, earlier steps' K and V (as QKV projections)."""
+    B, t, (n_layers, D, H, dh, F) = c["B"], c["t"], MODELS[c["model"]]
+    s = SimpleNamespace()
+    s.node, s.key, s.token, s.score = _beam(rng, i.sids, c["V"], B, i.beams[t], t, i.level_start)
+    s.parents = [None] + [torch.randint(0, i.beams[j - 1], (B * i.beams[j],), device=DEV, generator=g, dtype=torch.int32)
+                          for j in range(1, t + 1)]
+    s.qkv = [[_normal(g, B * i.beams[j], 3, H, dh) for j in range(t)] for _ in range(n_layers)]
+    return s
 
 
 def _beam(rng, sids, V, B, M, depth, level_start):
@@ -255,8 +272,9 @@ def prepare(case, seed):
     rng, g = _generators(seed)
     s = SimpleNamespace(c=c, kind=c["kind"])
     if s.kind in ("decode", "serve", "step"):
-        s.dec, sids, level_start, beams = _decoder(c, rng, g)
-        D, B, T = s.dec.d_model, c["B"], c["T"]
+        i = _decoder_inputs(c, rng, g)
+        s.dec = _decoder(c, i)
+        B, T, D = c["B"], c["T"], s.dec.d_model
         if s.kind == "serve":
             n = c["batches"]
             s.enc = [_normal(g, B, T, D).cpu().pin_memory() for _ in range(n)]
@@ -266,18 +284,17 @@ def prepare(case, seed):
         s.enc = _normal(g, B, T, D)
         if s.kind == "step":
             t = c["t"]
+            st = _step_state(c, i, rng, g)
             s.dec.reset()
             s.dec.project_cross_kv(s.enc)
-            R = B * beams[t]
-            node, key, token, score = _beam(rng, sids, c["V"], B, beams[t], t, level_start)
-            s.dec.node[t & 1][:R], s.dec.key[t & 1][:R] = node, key
-            s.dec.token[t & 1][:R], s.dec.score[t & 1][:R] = token, score
+            R = B * i.beams[t]
+            s.dec.node[t & 1][:R], s.dec.key[t & 1][:R] = st.node, st.key
+            s.dec.token[t & 1][:R], s.dec.score[t & 1][:R] = st.token, st.score
             for j in range(1, t + 1):
-                s.dec.parents[j][:B * beams[j]] = torch.randint(0, beams[j - 1], (B * beams[j],), device=DEV, generator=g,
-                                                                dtype=torch.int32)
-            for slabs in s.dec.qkv_slabs:
+                s.dec.parents[j][:B * i.beams[j]] = st.parents[j]
+            for slabs, qkv in zip(s.dec.qkv_slabs, st.qkv):
                 for j in range(t):
-                    slabs[j][:B * beams[j]] = _normal(g, B * beams[j], *slabs.shape[2:])
+                    slabs[j][:B * i.beams[j]] = qkv[j].view(-1, *slabs.shape[2:])
         return s
     if s.kind == "cross":
         B, M, H, d, T = c["B"], c["M"], c["H"], c["d"], c["T"]
@@ -304,7 +321,7 @@ def prepare(case, seed):
     sids = _catalog(rng, c["n_sids"], V, L)
     if s.kind == "select":
         bits, base, level_start = api.grace_trie_build_dense(sids, V)
-        kind, words, log2_bits, hashes = _matcher(c["matcher"], rng, sids, V, B, int(level_start[-1]), 0.2)
+        _, (kind, words, log2_bits, hashes) = _matcher(c["matcher"], rng, sids, V, B, int(level_start[-1]), 0.2)
         up = lambda a: torch.from_numpy(a.view(np.int64)).to(DEV)  # noqa: E731
         s.trie = api.make_trie(up(bits), torch.from_numpy(base).to(DEV), V, L, int(level_start[-1]))
         s.matcher = api.make_matcher(kind, None if words is None else up(words), log2_bits, hashes)
@@ -360,6 +377,233 @@ def run(s):
     update, index = ((api.grace_beam_update, s.trie) if s.kind == "select" else (api.grace_beam_update_csr, s.index))
     update(n["parent"].view(-1), n["token"].view(-1), n["score"].view(-1), s.node, s.key, index, n["node"], n["key"], B, K, M, t)
     return dict(n, cand=s.cand)
+
+
+# ------------------------------------------------------------------------------------------------
+# the same in 64 bits, with none of the library's arithmetic
+# ------------------------------------------------------------------------------------------------
+def _up(a):
+    return torch.from_numpy(np.ascontiguousarray(a)).to(DEV)
+
+
+def _attend(q, k, v, n_keys=None):
+    """q [H, M, d], k and v [H, T, d] -> [M, H, d]; of the keys the first n_keys."""
+    k, v = (k, v) if n_keys is None else (k[:, :n_keys], v[:, :n_keys])
+    p = torch.softmax(q @ k.transpose(1, 2) * q.shape[-1] ** -0.5, dim=-1)
+    return (p @ v).permute(1, 0, 2)
+
+
+def _attend_prefix(q, rows, keys, values):
+    """q [R, H, d]; rows[j] [R] into keys[j] and values[j] -> [R, H, d]."""
+    s = torch.stack([(q * k[r].double()).sum(-1) for k, r in zip(keys, rows)]) * q.shape[-1] ** -0.5
+    p = torch.softmax(s, dim=0)
+    return sum(p[j][..., None] * values[j][rows[j]].double() for j in range(len(rows)))
+
+
+def _ancestors(parents, beams, B, t):
+    """Row of every step 0..t that holds the prefix of each row of step t; parents[j] counts within the request."""
+    rows = [None] * (t + 1)
+    rows[t] = torch.arange(B * beams[t], device=DEV)
+    for j in range(t, 0, -1):
+        rows[j - 1] = torch.div(rows[j], beams[j], rounding_mode="floor") * beams[j - 1] + parents[j][rows[j]].long()
+    return rows
+
+
+def _mix64(key):
+    """The splitmix64 finaliser on int64 tensors (wrapping)."""
+    def shifted(z, n):
+        return (z >> n) & ((1 << (64 - n)) - 1)
+
+    def signed(c):
+        return c - (1 << 64) if c >= 1 << 63 else c
+
+    z = key + signed(0x9E3779B97F4A7C15)
+    z = (z ^ shifted(z, 30)) * signed(0xBF58476D1CE4E5B9)
+    z = (z ^ shifted(z, 27)) * signed(0x94D049BB133111EB)
+    return z ^ shifted(z, 31)
+
+
+class _Constraint:
+    """Which continuations of a prefix a request may see: prefixes of the catalog that its matcher lets through."""
+
+    def __init__(self, sids, V, seen, matcher):
+        self.V, self.matcher = V, matcher
+        depth = sids.shape[1]
+        level = [_levels(sids, V, j) for j in range(depth + 1)]
+        self.codes = [_up(codes) for _, codes in level]
+        self.words = _up(matcher[1].view(np.int64)) if matcher[0] == api.MATCH_PREFIX_BLOOM else None
+        self.marks = None
+        if matcher[0] == api.MATCH_NODE_BITMASK:
+            self.marks = [torch.zeros(len(seen), c.numel(), dtype=torch.bool, device=DEV) for c in self.codes]
+            for j, (index, _) in enumerate(level):
+                index = _up(index)
+                for b, e in enumerate(seen):
+                    self.marks[j][b, index[_up(e)]] = True
+
+    def let_through(self, b, depth):
+        """bool over the distinct prefixes of `depth` tokens."""
+        if self.marks is not None:
+            return self.marks[depth][b]
+        code = self.codes[depth]
+        if self.words is None:
+            return torch.ones_like(code, dtype=torch.bool)
+        key = torch.zeros_like(code)
+        for j in range(depth - 1, -1, -1):
+            key |= (code % self.V + 1) << (16 * j)
+            code = torch.div(code, self.V, rounding_mode="floor")
+        z = _mix64(key)
+        h1, h2 = z & 0xFFFFFFFF, ((z >> 32) & 0xFFFFFFFF) | 1
+        ok = torch.ones_like(key, dtype=torch.bool)
+        for i in range(self.matcher[3]):
+            pos = (h1 + i * h2) & ((1 << self.matcher[2]) - 1)
+            ok &= ((self.words[b][pos >> 6] >> (pos & 63)) & 1).bool()
+        return ok
+
+    def allowed(self, b, depth, prefix, marks=None):
+        """(bool [M, V], number of the continuation among the distinct ones [M, V]) for prefixes given by number."""
+        want = self.codes[depth][prefix][:, None] * self.V + torch.arange(self.V, device=DEV)
+        at = torch.searchsorted(self.codes[depth + 1], want).clamp_(max=self.codes[depth + 1].numel() - 1)
+        return (self.codes[depth + 1][at] == want) & (self.let_through(b, depth + 1) if marks is None else marks)[at], at
+
+
+def _best(cand, K):
+    """The K largest of every request, -inf where there are fewer."""
+    score, flat = cand.topk(min(K, cand.shape[1]), dim=1, sorted=True)
+    return torch.nn.functional.pad(score, (0, K - score.shape[1]), value=-math.inf), flat
+
+
+class _ExactDecoder:
+    def __init__(self, c, i, enc):
+        self.c, self.i, w = c, i, i.weights
+        self.n_layers, self.D, self.H, self.dh, self.F = MODELS[c["model"]]
+        self.w = {k: _up(a).double() for k, a in w.items() if k != "layers"}
+        self.layers = [{k: _up(a) for k, a in lay.items()} for lay in w["layers"]]       # widened where they are used
+        heads = (c["B"], c["T"], self.H, self.dh)
+        x = enc.double().view(-1, self.D)
+        self.k_cross = [(x @ lay["w_kc"].double().T).view(heads) for lay in self.layers]
+        self.v_cross = [(x @ lay["w_vc"].double().T).view(heads) for lay in self.layers]
+
+    def norm(self, x, lay, name):
+        return torch.nn.functional.layer_norm(x, (self.D,), lay[name + "_g"].double(), lay[name + "_b"].double(), 1e-5)
+
+    def logits(self, t, token, rows, keys, values):
+        """Logits of a step's rows [B M, V] and every layer's QKV projection; keys[layer][j] of the steps before."""
+        B, M, H, d = self.c["B"], self.i.beams[t], self.H, self.dh
+        x, projections = self.w["embed"][token.long()] + self.w["pos"][t], []
+        for li, lay in enumerate(self.layers):
+            qkv = (self.norm(x, lay, "ln1") @ lay["w_qkv"].double().T).view(B * M, 3, H, d)
+            projections.append(qkv)
+            a = _attend_prefix(qkv[:, 0], rows, keys[li] + [qkv[:, 1]], values[li] + [qkv[:, 2]])
+            x = x + a.reshape(B * M, -1) @ lay["w_o"].double().T
+            q = (self.norm(x, lay, "ln2") @ lay["w_qc"].double().T).view(B, M, H, d)
+            a = torch.stack([_attend(q[b].transpose(0, 1), self.k_cross[li][b].transpose(0, 1), self.v_cross[li][b].transpose(0, 1))
+                             for b in range(B)])
+            x = x + a.reshape(B * M, -1) @ lay["w_oc"].double().T
+            x = x + torch.relu(self.norm(x, lay, "ln3") @ lay["w_1"].double().T) @ lay["w_2"].double().T
+        return self.norm(x, self.w, "lnf") @ self.w["w_out"].T, projections
+
+    def select(self, constraint, t, logits, score, prefix, K):
+        """Ranked scores [B, K] of a step and what the next one starts from."""
+        B, M, V = self.c["B"], self.i.beams[t], self.c["V"]
+        best, parent, token, number = [], [], [], []
+        for b in range(B):
+            r = slice(b * M, (b + 1) * M)
+            allowed, at = constraint.allowed(b, t, prefix[r])
+            cand = score[r, None] + torch.log_softmax(logits[r], dim=1)
+            s, flat = _best(torch.where(allowed, cand, -math.inf).view(1, -1), K)
+            best.append(s), parent.append(torch.div(flat, V, rounding_mode="floor")), token.append(flat % V)
+            number.append(at.view(-1)[flat])
+        return torch.cat(best), torch.cat(parent).view(-1), torch.cat(token).view(-1), torch.cat(number).view(-1)
+
+    def search(self):
+        c, beams, B = self.c, self.i.beams, self.c["B"]
+        constraint = _Constraint(self.i.sids, c["V"], self.i.seen, self.i.matcher)
+        token = torch.full((B,), c["V"], device=DEV)
+        score, prefix = torch.zeros(B, device=DEV, dtype=torch.float64), torch.zeros(B, device=DEV, dtype=torch.int64)
+        parents = [None] * (len(beams) + 1)
+        keys, values = [[] for _ in self.layers], [[] for _ in self.layers]
+        for t in range(len(beams)):
+            logits, qkv = self.logits(t, token, _ancestors(parents, beams, B, t), keys, values)
+            for li, p in enumerate(qkv):
+                keys[li].append(p[:, 1]), values[li].append(p[:, 2])
+            best, parents[t + 1], token, prefix = self.select(constraint, t, logits, score, prefix, (beams + [c["K"]])[t + 1])
+            score = best.view(-1)
+        return score
+
+
+def exact(case, seed):
+    c = dict(case)
+    kind = c["kind"]
+    if kind in ("decode", "serve", "step"):
+        rng, g = _generators(seed)
+        i = _decoder_inputs(c, rng, g)
+        enc = [_normal(g, c["B"], c["T"], MODELS[c["model"]][1]) for _ in range(c.get("batches", 1))]
+        if kind == "serve":
+            return [_ExactDecoder(c, i, e).search() for e in enc]
+        dec = _ExactDecoder(c, i, enc[0])
+        if kind == "decode":
+            return dict(score=dec.search(), k_cross=dec.k_cross, v_cross=dec.v_cross)
+        t, st = c["t"], _step_state(c, i, rng, g)
+        logits, qkv = dec.logits(t, st.token, _ancestors(st.parents, i.beams, c["B"], t),
+                                 [[p[:, 1] for p in lay] for lay in st.qkv], [[p[:, 2] for p in lay] for lay in st.qkv])
+        best = dec.select(_Constraint(i.sids, c["V"], i.seen, i.matcher), t, logits, st.score.double(),
+                          st.node.long() - int(i.level_start[t]), c["K"])[0]
+        return dict(logits=logits, lse=torch.logsumexp(logits, 1), qkv=qkv, score=best.view(-1))
+    s = prepare(case, seed)
+    if kind == "cross":
+        B, M = c["B"], c["M"]
+        lengths = [None] * B if s.enc_len is None else s.enc_len.tolist()
+        return torch.cat([_attend(s.q[b * M:(b + 1) * M].double().transpose(0, 1), s.k[b].double(), s.v[b].double(), lengths[b])
+                          for b in range(B)])
+    if kind == "self":
+        t, new = c["t"], (s.qkv[:, 1], s.qkv[:, 2])
+        keys, values = ([cache[j] for j in range(t)] + [p] for cache, p in zip((s.k_cache, s.v_cache), new))
+        a = _attend_prefix(s.qkv[:, 0].double(), _ancestors(s.parents, s.beams, c["B"], t), keys, values)
+        return dict(out=a, k=new[0].double(), v=new[1].double())
+    if kind == "linear":
+        y = s.x.double() @ s.w.double().T
+        return torch.relu(y) if c["relu"] else y
+    # selection: scores of the candidates and of the chosen; the rest are whole numbers
+    rng, g = _generators(seed)
+    B, M, V, t = c["B"], c["M"], c["V"], c["t"]
+    sids = _catalog(rng, c["n_sids"], V, 4 if V >= 256 else 3)
+    if kind == "select":
+        seen, matcher = _matcher(c["matcher"], rng, sids, V, B, int(api.grace_trie_count_nodes(sids, V)[-1]), 0.2)
+        marks = [None] * B
+    else:
+        seen, matcher = None, (api.MATCH_NONE, None, 0, 0)
+        marks = _targeted(sids, V, t + 1, *_targeting(rng, c["n_sids"], B, c["locations"]))
+    constraint = _Constraint(sids, V, seen, matcher)
+    first = int(api.grace_trie_count_nodes(sids, V)[t])
+    cand = torch.empty(B, M * V, device=DEV, dtype=torch.float64)
+    for b in range(B):
+        r = slice(b * M, (b + 1) * M)
+        allowed, _ = constraint.allowed(b, t, s.node[r].long() - first, marks[b])
+        cand[b] = torch.where(allowed, s.score[r, None].double() + s.logp[r].double(), -math.inf).view(-1)
+    return dict(score=_best(cand, c["K"])[0], flat=None, parent=None, token=None, node=None, key=None, cand=cand.view(B * M, V))
+
+
+def _targeted(sids, V, depth, ad_sid, bm, bl, ubm, ubl):
+    """Per request, bool over the distinct prefixes of `depth` tokens: the union of the attribute rows of the ads below
+    contains the request's, and the union of their location rows contains one of the request's."""
+    index, codes = _levels(sids, V, depth)
+    below = _up(index[ad_sid])
+
+    def bits(rows):
+        return _up(np.unpackbits(np.ascontiguousarray(rows).view(np.uint8), axis=1, bitorder="little"))
+
+    def union(rows):
+        r = bits(rows)
+        u = torch.zeros(codes.size, r.shape[1], dtype=torch.uint8, device=DEV)
+        return u.scatter_reduce_(0, below[:, None].expand_as(r), r, "amax")
+
+    lacking_bm, lacking_bl = (1 - union(bm)).half(), (1 - union(bl)).half()             # counts up to 448: exact in fp16
+    out = []
+    for b in range(ubm.shape[0]):
+        attributes = lacking_bm @ bits(ubm[b:b + 1]).half().T == 0
+        locations = lacking_bl @ bits(ubl[b]).half().T == 0
+        out.append(attributes[:, 0] & locations.any(dim=1))
+    return out
 
 
 # ------------------------------------------------------------------------------------------------
