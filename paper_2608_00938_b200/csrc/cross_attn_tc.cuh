@@ -89,8 +89,11 @@ cross_attn_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_con
   uint64_t* v_full = k_empty + kCaStages;     // [stages]  slot only after P V of its block
   uint64_t* v_empty = v_full + kCaStages;     // [stages]
   uint64_t* s_full = v_empty + kCaStages;
+  // [2] by block parity.  The softmax threads hand P of block g + 1 over without waiting for anything the issuer does
+  // after its wait for P of block g, so with a single barrier an issuer that comes late to that wait could find the
+  // phase after it complete as well and wait for good; with two, P of block g + 2 comes after P V of block g.
   uint64_t* p_full = s_full + 1;
-  uint64_t* o_full = p_full + 1;              // [2] by block parity: P V of the block is complete
+  uint64_t* o_full = p_full + 2;              // [2] by block parity: P V of the block is complete
   uint64_t* s_free = o_full + 2;
   uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(s_free + 1);
   volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_slot + 1);
@@ -108,6 +111,7 @@ cross_attn_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_con
     }
     tc::mbar_init(s_full, 1);
     tc::mbar_init(p_full, kCaSoftmaxWarps);    // one arrival per softmax warp
+    tc::mbar_init(p_full + 1, kCaSoftmaxWarps);
     tc::mbar_init(o_full, 1);
     tc::mbar_init(o_full + 1, 1);
     tc::mbar_init(s_free, kCaSoftmaxWarps);
@@ -261,7 +265,7 @@ cross_attn_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_con
         if (g + 1 < total_blocks && !issue_s(g + 1, j1, li1)) break;
         // p_full(g): P of block g is in its TMEM columns (and, on an item's first block, the
         // previous item's epilogue has read O).
-        if (!tc::mbar_wait(p_full, g & 1, abort_flag)) break;
+        if (!tc::mbar_wait(p_full + (g & 1), (g >> 1) & 1, abort_flag)) break;
         if (!tc::mbar_wait(v_full + s, (g >> 1) & 1, abort_flag)) break;
         tc::tc_fence_after();
         const uint32_t o_acc = tmem_o + (uint32_t)((li & 1) * DH), p_cols = tmem_p + (uint32_t)((g & 1) * 64);
@@ -448,7 +452,7 @@ cross_attn_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_con
         tc::tmem_st_wait();
         tc::tc_fence_before();
         __syncwarp();
-        if (lane == 0) tc::mbar_arrive(p_full);
+        if (lane == 0) tc::mbar_arrive(p_full + (g & 1));
         // the previous item's output, now that this block is with the tensor core
         if (pend_item >= 0) {
           ok = store_item(pend_item, pend_g, pend_li, pend_m, pend_l);
