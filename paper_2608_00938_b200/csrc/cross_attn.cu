@@ -6,9 +6,11 @@
 //     head size 64: the serving shapes.
 //   * cross_attn_tc_kernel (cross_attn_tc.cuh): tcgen05 / TMEM / TMA flash attention, head size 128.
 //   * cross_attn_row_kernel (below): a handful of query rows per request (step 0 of a decode).
-//   * cross_attn_small_kernel (below): a plain CUDA-core kernel for everything else (tiny
-//     configurations, d_h = 32, per-request encoder lengths at head size 128).  One warp per (row,
-//     head); lanes split the encoder positions for the scores and the head dimension for the sum.
+//   * cross_attn_small_kernel (below): a plain CUDA-core kernel for head size 32 (tiny configurations) and
+//     for more than 65535 requests or heads.  One warp per (row, head); lanes split the encoder
+//     positions for the scores and the head dimension for the sum.
+// Per-request encoder lengths take the same routes as full-length requests.  (Head size 128 with lengths ran the
+// CUDA-core kernel before: 16 x 1000 x 16 x 128, lengths 50..200: 7700 us; on the tensor cores 72.)
 #include "common.cuh"
 #include "cross_attn_tc.cuh"
 #include "cross_attn_ms.cuh"
@@ -20,7 +22,7 @@ struct CrossSmallParams {
   const uint16_t* q; const uint16_t* k; const uint16_t* v; uint16_t* out; float* lse;
   int64_t q_row_stride, out_row_stride, kv_stride_b, kv_stride_h, kv_stride_t;
   int R, M, H, T_ctx; float scale;
-  const int32_t* enc_len;        // nullable: valid encoder positions per request (small kernel only)
+  const int32_t* enc_len;        // nullable: valid encoder positions per request
 };
 
 template <int DH>
@@ -136,9 +138,11 @@ cross_attn_row_kernel(const CrossSmallParams p) {
     q[0] = bf16_lo(t4.x) * p.scale; q[1] = bf16_hi(t4.x) * p.scale; q[2] = bf16_lo(t4.y) * p.scale; q[3] = bf16_hi(t4.y) * p.scale;
     q[4] = bf16_lo(t4.z) * p.scale; q[5] = bf16_hi(t4.z) * p.scale; q[6] = bf16_lo(t4.w) * p.scale; q[7] = bf16_hi(t4.w) * p.scale;
   }
+  int T = p.T_ctx;                             // valid encoder positions of this request
+  if (p.enc_len != nullptr) { const int e = __ldg(p.enc_len + b); T = e < 0 ? 0 : (e < T ? e : T); }
   // this warp's contiguous slice of the encoder positions, RP at a time
-  const int per_warp = (p.T_ctx + kWarps - 1) / kWarps;
-  const int t_begin = warp * per_warp, t_end = min(p.T_ctx, t_begin + per_warp);
+  const int per_warp = (T + kWarps - 1) / kWarps;
+  const int t_begin = warp * per_warp, t_end = min(T, t_begin + per_warp);
   float m_run = -INFINITY, l_run = 0.f;
   float acc[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
   // The op is bound by reading K and V once (a row per request: nothing is reused), so loads never stop: the
@@ -195,15 +199,20 @@ cross_attn_row_kernel(const CrossSmallParams p) {
       l_all = fmaf(st_l[s2], f, l_all);
       o = fmaf(st_acc[s2][threadIdx.x], f, o);
     }
-    __nv_bfloat16 ob = __float2bfloat16_rn(o / l_all);
+    __nv_bfloat16 ob = __float2bfloat16_rn(l_all > 0.f ? o / l_all : 0.f);    // no encoder position: zero by definition
     p.out[(int64_t)r * p.out_row_stride + h * DH + threadIdx.x] = *reinterpret_cast<uint16_t*>(&ob);
-    if (p.lse != nullptr && threadIdx.x == 0) p.lse[(int64_t)r * p.H + h] = m_all + logf(l_all);
+    if (p.lse != nullptr && threadIdx.x == 0) p.lse[(int64_t)r * p.H + h] = l_all > 0.f ? m_all + logf(l_all) : -INFINITY;
   }
 }
 
 }  // namespace grace
 
 namespace grace {
+// Which kernel: 0: cross_attn_ms_kernel, 1: cross_attn_tc_kernel.
+static int cross_attn_form(int B, int M, int H, int d_h, int T_ctx, bool p32) {
+  (void)B; (void)M; (void)H; (void)T_ctx;
+  return d_h == 64 && !p32 ? 0 : 1;
+}
 int cross_attn_tc_timeouts() { return tc::tc_timeouts_read_and_clear(); }
 }  // namespace grace
 
@@ -229,20 +238,23 @@ extern "C" grace_status_t grace_cross_attn_varlen(const uint16_t* q, int64_t q_r
   p.q_row_stride = q_row_stride; p.out_row_stride = out_row_stride;
   p.kv_stride_b = kv_stride_b; p.kv_stride_h = kv_stride_h; p.kv_stride_t = kv_stride_t;
   p.R = B * M; p.M = M; p.H = H; p.T_ctx = T_ctx; p.scale = scale; p.enc_len = enc_len;
-  if (enc_len == nullptr && (d_h == 64 || d_h == 128) && M <= 8 && (int64_t)B * M * H <= 1184) {
+  if ((d_h == 64 || d_h == 128) && M <= 8 && (int64_t)B * M * H <= 1184) {
     // a few rows per request (step 0 of a decode): one CTA per (row, head), all resident at once
     if (d_h == 64) launch_pdl(cross_attn_row_kernel<64>, dim3(B * M * H), dim3(256), 0, s, p);
     else launch_pdl(cross_attn_row_kernel<128>, dim3(B * M * H), dim3(256), 0, s, p);
     GRACE_LAUNCH_CHECK();
     return GRACE_OK;
   }
-  if (cross_attn_ms_supported(B, M, H, d_h, T_ctx) && (enc_len == nullptr || M > 8)) {
-    return launch_cross_attn_ms(q, q_row_stride, k, v, kv_stride_b, kv_stride_h, kv_stride_t, out,
-                                out_row_stride, lse, enc_len, B, M, H, T_ctx, scale, s);
-  }
-  if (enc_len == nullptr && cross_attn_tc_supported(B, M, H, d_h, T_ctx)) {
-    return launch_cross_attn_tc(q, q_row_stride, k, v, kv_stride_b, kv_stride_h, kv_stride_t, out,
-                                out_row_stride, lse, B, M, H, d_h, T_ctx, scale, s);
+  if (cross_attn_tc_supported(B, M, H, d_h, T_ctx)) {
+    // probabilities as before the tensor cores took these over: fp32 (see cross_attn_tc_kernel)
+    const bool p32 = enc_len != nullptr && (d_h == 128 || M <= 8);
+    const int form = cross_attn_form(B, M, H, d_h, T_ctx, p32);
+    if (form == 0)
+      return launch_cross_attn_ms(q, q_row_stride, k, v, kv_stride_b, kv_stride_h, kv_stride_t, out,
+                                  out_row_stride, lse, enc_len, B, M, H, T_ctx, scale, s);
+    return (d_h == 64 ? launch_cross_attn_tc<64> : launch_cross_attn_tc<128>)(
+        q, q_row_stride, k, v, kv_stride_b, kv_stride_h, kv_stride_t, out, out_row_stride, lse, enc_len, B, M, H, T_ctx,
+        scale, form, p32, s);
   }
   const int64_t items = (int64_t)p.R * H;
   const unsigned blocks = (unsigned)((items + 3) / 4);

@@ -454,10 +454,6 @@ cross_attn_ms_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_con
   if (warp == kMsSoftmaxWarps) tc::tmem_dealloc(tmem_base, 512);
 }
 
-inline bool cross_attn_ms_supported(int B, int M, int H, int d_h, int T_ctx) {
-  return d_h == 64 && H <= 65535 && B <= 65535 && T_ctx >= 1 && M >= 1;
-}
-
 inline grace_status_t launch_cross_attn_ms(const uint16_t* q, int64_t q_row_stride, const uint16_t* k,
                                            const uint16_t* v, int64_t kv_stride_b, int64_t kv_stride_h,
                                            int64_t kv_stride_t, uint16_t* out, int64_t out_row_stride, float* lse,

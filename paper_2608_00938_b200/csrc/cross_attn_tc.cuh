@@ -37,21 +37,72 @@ constexpr int kCaHalfBytes = 128 * 64 * 2;                       // 16 KB: 128 r
 // through the TMEM load / barrier / TMEM store sequence per exponential; 168 registers).  Head size 64
 // runs TPR = 1 (4 % faster at 32 x 2048 x 1024); head size 128 keeps TPR = 2 for its wider output rows.
 constexpr int kCaBarBytes = 256;
-template <int DH> struct CaCfg {
+// SPLIT > 1: a cluster of SPLIT CTAs shares one work item, each taking a contiguous range of its K / V blocks; the
+// partial results (unnormalised output, maximum and sum per row) are merged through distributed shared memory:
+// every CTA owns DH / SPLIT of the output columns and receives the others' partial sums of them.
+template <int DH, int SPLIT> struct CaCfg {
   static constexpr int kHalves = DH / 64;
   static constexpr int kTileBytes = kCaHalfBytes * kHalves;      // Q, K_blk or V_blk
-  static constexpr int kSmemBytes = kTileBytes * (2 + 2 * kCaStages) + 1024 + kCaBarBytes + 2 * 2 * 128 * 4 + 2 * 2 * 128 * 4;
+  static constexpr int kQBufs = SPLIT > 1 ? 1 : 2;
+  static constexpr int kSlice = DH / SPLIT;                      // output columns a CTA finishes
+  static constexpr int kXBytes = SPLIT > 1 ? (SPLIT - 1) * 128 * kSlice * 4 + SPLIT * 128 * 8 : 0;
+  static constexpr int kSmemBytes = kTileBytes * (kQBufs + 2 * kCaStages) + 1024 + kCaBarBytes + 2 * 2 * 128 * 4 + 2 * 2 * 128 * 4 + kXBytes;
+  static_assert(kSmemBytes <= 227 * 1024, "");
   static constexpr uint32_t kTmemCols = 512;                     // S: 0..127, O: 2 x DH (by item parity), P: 2 x 64 (by block parity)
-  static constexpr int kCtasPerSm = 1;
 };
 
 struct CrossTcParams {
   uint16_t* out;
   float* lse;
+  const int32_t* enc_len;       // nullable: valid encoder positions per request (<= T)
   int64_t out_row_stride;
   int B, M, H, T;
   int tiles_m, total_items;
   float scale_log2;             // scale * log2(e)
+};
+
+// One work item: request, head, 128-row tile, encoder positions and the K / V blocks they take.  Every role of a
+// CTA walks the same sequence of items; those without any encoder position (nb == 0) are passed over by the loads
+// and the MMAs and written as zeros by the epilogue warps.
+// With SPLIT > 1 an item is a CTA's share of one: nb blocks from position t0 on (T counts from there).
+struct CaItem { int b, h, tile, t0, T, nb; };
+template <int SPLIT>
+__device__ __forceinline__ CaItem ca_item(const CrossTcParams& p, int item) {
+  CaItem it;
+  const int part = item % SPLIT;
+  item /= SPLIT;
+  const int bh = item / p.tiles_m;
+  it.tile = item - bh * p.tiles_m;
+  it.b = bh / p.H;
+  it.h = bh - it.b * p.H;
+  it.T = p.T;
+  if (p.enc_len != nullptr) { const int e = __ldg(p.enc_len + it.b); it.T = e < 0 ? 0 : (e < p.T ? e : p.T); }
+  it.nb = (it.T + kCaBN - 1) / kCaBN;
+  it.t0 = 0;
+  if (SPLIT > 1) {
+    const int first = it.nb * part / SPLIT;
+    it.nb = it.nb * (part + 1) / SPLIT - first;
+    it.t0 = first * kCaBN;
+    it.T -= it.t0;
+  }
+  return it;
+}
+// A position in that sequence: item, its place among the CTA's non-empty items (li), block inside the item.
+template <int SPLIT>
+struct CaCursor {
+  int item, li, j;
+  CaItem it;
+  __device__ __forceinline__ bool live(const CrossTcParams& p) const { return item < p.total_items; }
+  __device__ __forceinline__ void seek(const CrossTcParams& p) {       // to the first non-empty item from here on
+    for (; item < p.total_items; item += (int)gridDim.x) {
+      it = ca_item<SPLIT>(p, item);
+      if (it.nb > 0) return;
+    }
+  }
+  __device__ __forceinline__ void start(const CrossTcParams& p) { item = (int)blockIdx.x; li = 0; j = 0; seek(p); }
+  __device__ __forceinline__ void next(const CrossTcParams& p) {       // one block on
+    if (++j == it.nb) { j = 0; ++li; item += (int)gridDim.x; seek(p); }
+  }
 };
 
 __device__ __forceinline__ float ex2(float x) {
@@ -69,19 +120,25 @@ __device__ __forceinline__ float max3(float a, float b, float c) {
 // Persistent kernel: a flat grid of two CTAs per SM; CTA g takes the work items g, g + gridDim.x,
 // ...  An item is one (request, head, 128-row tile); consecutive items are the tiles of the same
 // (request, head), so the CTAs running at the same time read the same K/V from L2.
-template <int DH, int TPR>
-__global__ void __launch_bounds__((4 * TPR + 2) * 32, CaCfg<DH>::kCtasPerSm)
+// P32: the probabilities keep (at least) sixteen bits of their fp32 mantissa: P is stored as the sum of two bf16 values
+// and multiplied with V twice.  The two take the P columns of both block parities, so P of a block is stored
+// once P V of the block before it is complete.  Calls with per-request lengths run this form: they were computed with
+// fp32 probabilities before the tensor cores took them over, and one bf16 rounding of P shows in the result
+// (relative error against 64 bits 2.2e-3 instead of the output rounding's 1.7e-3).
+template <int DH, int TPR, int SPLIT, bool P32>
+__global__ void __launch_bounds__((4 * TPR + 2) * 32, 1)
 cross_attn_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant__ CUtensorMap map_k,
                      const __grid_constant__ CUtensorMap map_v, const CrossTcParams p) {
   constexpr int kCaSoftmaxWarps = 4 * TPR;
   constexpr int kCols = kCaBN / TPR;                       // score columns per softmax thread and block
-  constexpr int kCaTileBytes = CaCfg<DH>::kTileBytes, kHalves = CaCfg<DH>::kHalves;
-  constexpr uint32_t kCaTmemCols = CaCfg<DH>::kTmemCols;
+  constexpr int kCaTileBytes = CaCfg<DH, SPLIT>::kTileBytes, kHalves = CaCfg<DH, SPLIT>::kHalves;
+  constexpr uint32_t kCaTmemCols = CaCfg<DH, SPLIT>::kTmemCols;
+  constexpr int kQBufs = CaCfg<DH, SPLIT>::kQBufs, kSlice = CaCfg<DH, SPLIT>::kSlice;
   extern __shared__ uint8_t smem_raw[];
   uint8_t* tiles = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
-  uint8_t* q_tiles = tiles;                                      // two Q buffers
-  uint8_t* kv_tiles = tiles + 2 * kCaTileBytes;                  // stage s: K at 2s, V at 2s+1
-  uint64_t* bars = reinterpret_cast<uint64_t*>(tiles + kCaTileBytes * (2 + 2 * kCaStages));
+  uint8_t* q_tiles = tiles;                                      // two Q buffers (one if an item is all a CTA does)
+  uint8_t* kv_tiles = tiles + kQBufs * kCaTileBytes;             // stage s: K at 2s, V at 2s+1
+  uint64_t* bars = reinterpret_cast<uint64_t*>(tiles + kCaTileBytes * (kQBufs + 2 * kCaStages));
   uint64_t* q_full = bars;                    // [2]
   uint64_t* q_empty = bars + 2;               // [2]
   uint64_t* k_full = bars + 4;                // [stages]  K and V have separate rings: a K slot is
@@ -100,9 +157,12 @@ cross_attn_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_con
   float* half_max = reinterpret_cast<float*>(reinterpret_cast<uint8_t*>(bars) + kCaBarBytes);   // [2][2][128]
   float* half_sum = half_max + 2 * 2 * 128;                                                     // [2][128]
 
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int NB = (p.T + kCaBN - 1) / kCaBN;
+  float4* xbuf = reinterpret_cast<float4*>(half_sum + 2 * 2 * 128);                             // SPLIT: [SPLIT - 1][kSlice / 4][128]
+  float2* mlbuf = reinterpret_cast<float2*>(xbuf + (SPLIT - 1) * (kSlice / 4) * 128);           // SPLIT: [SPLIT][128] (maximum, sum)
 
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+
+  if (SPLIT > 1) asm volatile("barrier.cluster.arrive.relaxed.aligned;" ::: "memory");   // "this CTA has started"
   if (threadIdx.x == 0) {
     for (int i = 0; i < 2; ++i) { tc::mbar_init(q_full + i, 1); tc::mbar_init(q_empty + i, 1); }
     for (int s = 0; s < kCaStages; ++s) {
@@ -142,45 +202,44 @@ cross_attn_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_con
       // One thread feeds three queues (Q per item, K and V per block).  K of block g+2 can be
       // requested as soon as S of block g has run, long before the V slot of block g frees, so the
       // thread polls: whichever slot is free next gets its load, neither queue blocks the other.
-      const int my_items = (p.total_items - (int)blockIdx.x + (int)gridDim.x - 1) / (int)gridDim.x;
-      const int total_blocks = my_items * NB;
-      int gk = 0, gv = 0;                                    // next K block, next V block (global indices)
+      int gk = 0, gv = 0;                                    // next K block, next V block (counted over the CTA's items)
+      CaCursor<SPLIT> ck, cv;
+      ck.start(p);
+      cv = ck;
       int idle = 0;
-      while ((gk < total_blocks || gv < total_blocks) && !*abort_flag) {
+      while ((ck.live(p) || cv.live(p)) && !*abort_flag) {
         bool progressed = false;
-        if (gk < total_blocks) {
-          const int li = gk / NB, j = gk - li * NB, s = gk % kCaStages;
-          const int item = (int)blockIdx.x + li * (int)gridDim.x;
-          const int bh = item / p.tiles_m, h = bh % p.H, b = bh / p.H;
-          const bool need_q = (j == 0);
-          const int qb = li & 1;
+        if (ck.live(p)) {
+          const int s = gk % kCaStages;
+          const bool need_q = (ck.j == 0);
+          const int qb = ck.li & 1;
           if (tc::mbar_try_wait_now(k_empty + s, ((gk / kCaStages) & 1) ^ 1) &&
-              (!need_q || tc::mbar_try_wait_now(q_empty + qb, ((li >> 1) & 1) ^ 1))) {
+              (!need_q || tc::mbar_try_wait_now(q_empty + qb, ((ck.li >> 1) & 1) ^ 1))) {
             if (need_q) {
               tc::mbar_expect_tx(q_full + qb, kCaTileBytes);
 #pragma unroll
               for (int hf = 0; hf < kHalves; ++hf)
-                tc::tma_load_4d(q_tiles + qb * kCaTileBytes + hf * kCaHalfBytes, &map_q, q_full + qb, 64 * hf, h,
-                                (item % p.tiles_m) * kCaBM, b);
+                tc::tma_load_4d(q_tiles + qb * kCaTileBytes + hf * kCaHalfBytes, &map_q, q_full + qb, 64 * hf, ck.it.h,
+                                ck.it.tile * kCaBM, ck.it.b);
             }
             tc::mbar_expect_tx(k_full + s, kCaTileBytes);
 #pragma unroll
             for (int hf = 0; hf < kHalves; ++hf)
-              tc::tma_load_4d(kv_tiles + (2 * s) * kCaTileBytes + hf * kCaHalfBytes, &map_k, k_full + s, 64 * hf, j * kCaBN, h, b);
+              tc::tma_load_4d(kv_tiles + (2 * s) * kCaTileBytes + hf * kCaHalfBytes, &map_k, k_full + s, 64 * hf, ck.it.t0 + ck.j * kCaBN, ck.it.h, ck.it.b);
             ++gk;
+            ck.next(p);
             progressed = true;
           }
         }
-        if (gv < total_blocks && gv < gk) {
-          const int li = gv / NB, j = gv - li * NB, s = gv % kCaStages;
-          const int item = (int)blockIdx.x + li * (int)gridDim.x;
-          const int bh = item / p.tiles_m, h = bh % p.H, b = bh / p.H;
+        if (cv.live(p) && gv < gk) {
+          const int s = gv % kCaStages;
           if (tc::mbar_try_wait_now(v_empty + s, ((gv / kCaStages) & 1) ^ 1)) {
             tc::mbar_expect_tx(v_full + s, kCaTileBytes);
 #pragma unroll
             for (int hf = 0; hf < kHalves; ++hf)
-              tc::tma_load_4d(kv_tiles + (2 * s + 1) * kCaTileBytes + hf * kCaHalfBytes, &map_v, v_full + s, 64 * hf, j * kCaBN, h, b);
+              tc::tma_load_4d(kv_tiles + (2 * s + 1) * kCaTileBytes + hf * kCaHalfBytes, &map_v, v_full + s, 64 * hf, cv.it.t0 + cv.j * kCaBN, cv.it.h, cv.it.b);
             ++gv;
+            cv.next(p);
             progressed = true;
           }
         }
@@ -200,15 +259,13 @@ cross_attn_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_con
     if (lane == 0) {
       constexpr uint32_t idesc_s = tc::idesc_bf16(kCaBM, kCaBN, 0);     // Q K^T : B K-major
       constexpr uint32_t idesc_o = tc::idesc_bf16(kCaBM, 64, 1);        // P V   : B MN-major, 64 output columns at a time
-      const int my_items = (p.total_items - (int)blockIdx.x + (int)gridDim.x - 1) / (int)gridDim.x;
-      const int total_blocks = my_items * NB;
       // Every operand descriptor is fixed by (Q buffer, ring slot, k-step): build them once.  The
       // issuing thread shares its scheduler with busy softmax warps, so each instruction it does not
       // execute per block shortens the hand-off to the tensor core.
       // k-step k of Q or K: 16 of the DH columns = 32 bytes inside the 64-wide half (k / 4)
-      uint64_t q_desc[2][DH / 16], k_desc[kCaStages][DH / 16], v_desc[kCaStages][kHalves][kCaBN / 16];
+      uint64_t q_desc[kQBufs][DH / 16], k_desc[kCaStages][DH / 16], v_desc[kCaStages][kHalves][kCaBN / 16];
 #pragma unroll
-      for (int i = 0; i < 2; ++i)
+      for (int i = 0; i < kQBufs; ++i)
 #pragma unroll
         for (int k = 0; k < DH / 16; ++k)
           q_desc[i][k] = tc::smem_desc_sw128(tc::smem_addr(q_tiles + i * kCaTileBytes) + (k / 4) * kCaHalfBytes + 32 * (k % 4), 16, 1024);
@@ -224,12 +281,12 @@ cross_attn_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_con
             v_desc[st][hf][k] = tc::smem_desc_sw128(tc::smem_addr(kv_tiles + (2 * st + 1) * kCaTileBytes) + hf * kCaHalfBytes + 2048 * k, 1024, 1024);
       }
       // S of global block g: Q buffer of its item, K of ring slot g % stages
-      auto issue_s = [&](int g, int j, int li) -> bool {
-        const int qb = li & 1, s = g % kCaStages;
-        if (j == 0 && !tc::mbar_wait(q_full + qb, (li >> 1) & 1, abort_flag)) return false;
+      auto issue_s = [&](int g, const CaCursor<SPLIT>& c) -> bool {
+        const int qb = c.li & 1, s = g % kCaStages;
+        if (c.j == 0 && !tc::mbar_wait(q_full + qb, (c.li >> 1) & 1, abort_flag)) return false;
         if (!tc::mbar_wait(k_full + s, (g / kCaStages) & 1, abort_flag)) return false;
         tc::tc_fence_after();
-        if (qb == 0) {
+        if (kQBufs == 1 || qb == 0) {
           if (s == 0) {
 #pragma unroll
             for (int k = 0; k < DH / 16; ++k) tc::mma_ss(tmem_s, q_desc[0][k], k_desc[0][k], idesc_s, k ? 1u : 0u);
@@ -240,51 +297,58 @@ cross_attn_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_con
         } else {
           if (s == 0) {
 #pragma unroll
-            for (int k = 0; k < DH / 16; ++k) tc::mma_ss(tmem_s, q_desc[1][k], k_desc[0][k], idesc_s, k ? 1u : 0u);
+            for (int k = 0; k < DH / 16; ++k) tc::mma_ss(tmem_s, q_desc[kQBufs - 1][k], k_desc[0][k], idesc_s, k ? 1u : 0u);
           } else {
 #pragma unroll
-            for (int k = 0; k < DH / 16; ++k) tc::mma_ss(tmem_s, q_desc[1][k], k_desc[1][k], idesc_s, k ? 1u : 0u);
+            for (int k = 0; k < DH / 16; ++k) tc::mma_ss(tmem_s, q_desc[kQBufs - 1][k], k_desc[1][k], idesc_s, k ? 1u : 0u);
           }
         }
         tc::mma_commit(s_full);
         tc::mma_commit(k_empty + s);                         // K of block g is consumed
-        if (j == NB - 1) tc::mma_commit(q_empty + qb);       // last use of this item's Q tile
+        if (c.j == c.it.nb - 1) tc::mma_commit(q_empty + qb);       // last use of this item's Q tile
         return true;
       };
       static_assert(kCaStages == 2, "descriptor selection below is written for two ring slots");
-      bool ok = total_blocks > 0 && issue_s(0, 0, 0);
-      int j = 0, li = 0;                                     // block inside the item, local item index
-      for (int g = 0; ok && g < total_blocks; ++g) {
-        const int s = g & 1;
-        int j1 = j + 1, li1 = li;
-        if (j1 == NB) { j1 = 0; ++li1; }
+      CaCursor<SPLIT> cs;                                           // the block whose S is issued next; (j, li): the one whose P V is
+      cs.start(p);
+      bool ok = cs.live(p) && issue_s(0, cs);
+      for (int g = 0; ok; ++g) {
+        const int s = g & 1, j = cs.j, li = cs.li;
+        cs.next(p);
+        const bool more = cs.live(p);
         // s_free(g): every softmax thread holds its scores of block g in registers, so the S
         // columns can be overwritten: S of block g+1 (possibly the next item's first block) runs
         // on the tensor core while the exponentials of block g are computed.
         if (!tc::mbar_wait(s_free, g & 1, abort_flag)) break;
-        if (g + 1 < total_blocks && !issue_s(g + 1, j1, li1)) break;
+        if (more && !issue_s(g + 1, cs)) break;
         // p_full(g): P of block g is in its TMEM columns (and, on an item's first block, the
         // previous item's epilogue has read O).
         if (!tc::mbar_wait(p_full + (g & 1), (g >> 1) & 1, abort_flag)) break;
         if (!tc::mbar_wait(v_full + s, (g >> 1) & 1, abort_flag)) break;
         tc::tc_fence_after();
-        const uint32_t o_acc = tmem_o + (uint32_t)((li & 1) * DH), p_cols = tmem_p + (uint32_t)((g & 1) * 64);
+        const uint32_t o_acc = tmem_o + (uint32_t)((li & 1) * DH), p_cols = tmem_p + (uint32_t)(P32 ? 0 : (g & 1) * 64);
         if (s == 0) {
 #pragma unroll
           for (int hf = 0; hf < kHalves; ++hf)
 #pragma unroll
             for (int k = 0; k < kCaBN / 16; ++k)
-              tc::mma_ts(o_acc + 64 * hf, p_cols + 8 * k, v_desc[0][hf][k], idesc_o, (j | k) ? 1u : 0u);
+              {
+                tc::mma_ts(o_acc + 64 * hf, p_cols + 8 * k, v_desc[0][hf][k], idesc_o, (j | k) ? 1u : 0u);
+                if (P32) tc::mma_ts(o_acc + 64 * hf, p_cols + 64 + 8 * k, v_desc[0][hf][k], idesc_o, 1u);
+              }
         } else {
 #pragma unroll
           for (int hf = 0; hf < kHalves; ++hf)
 #pragma unroll
             for (int k = 0; k < kCaBN / 16; ++k)
-              tc::mma_ts(o_acc + 64 * hf, p_cols + 8 * k, v_desc[1][hf][k], idesc_o, (j | k) ? 1u : 0u);
+              {
+                tc::mma_ts(o_acc + 64 * hf, p_cols + 8 * k, v_desc[1][hf][k], idesc_o, (j | k) ? 1u : 0u);
+                if (P32) tc::mma_ts(o_acc + 64 * hf, p_cols + 64 + 8 * k, v_desc[1][hf][k], idesc_o, 1u);
+              }
         }
         tc::mma_commit(v_empty + s);                         // V of block g is consumed
         tc::mma_commit(o_full + (g & 1));                    // O includes block g
-        j = j1; li = li1;
+        ok = more;
       }
     }
   } else {
@@ -301,16 +365,16 @@ cross_attn_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_con
     bool ok = true;
     int g = 0, n_done = 0, li = 0;
     // the item whose output is still to be read from TMEM and stored (after the next block's P hand-over)
-    int pend_item = -1, pend_g = 0, pend_li = 0;
+    int pend_g = -1, pend_li = 0;
+    CaItem pend_it = {0, 0, 0, 0, 0, 0};
     float pend_m = 0.f, pend_l = 0.f;
     // wait for P V of global block gb (completion gb >> 1 of the barrier of its parity)
     auto wait_pv = [&](int gb) -> bool {
       bool w = tc::mbar_wait(o_full + (gb & 1), (gb >> 1) & 1, abort_flag);
       return __all_sync(kFullMask, w);
     };
-    auto store_item = [&](int item_e, int g_last, int li_e, float m_e, float l_e) -> bool {
-      const int tile = item_e % p.tiles_m, bh = item_e / p.tiles_m;
-      const int h = bh % p.H, b = bh / p.H;
+    auto store_item = [&](const CaItem& it_e, int g_last, int li_e, float m_e, float l_e) -> bool {
+      const int tile = it_e.tile, h = it_e.h, b = it_e.b;
       if (!wait_pv(g_last)) return false;
       tc::tc_fence_after();
       const uint32_t o_acc = tmem_o + (uint32_t)((li_e & 1) * DH);
@@ -355,10 +419,25 @@ cross_attn_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_con
       tc::tc_fence_before();
       return true;
     };
-    for (int item = blockIdx.x; ok && item < p.total_items; item += gridDim.x, ++li) {
+    for (int item = blockIdx.x; ok && item < p.total_items; item += gridDim.x) {
+      const CaItem it = ca_item<SPLIT>(p, item);
+      if (SPLIT > 1) pend_it = it;
+      if (it.nb == 0) {
+        if (SPLIT > 1) continue;                              // nothing of this item falls to this CTA
+        // no encoder position: the attention output is defined as zero
+        const int m = it.tile * kCaBM + row;
+        if (m < p.M) {
+          const int64_t r_out = (int64_t)it.b * p.M + m;
+          uint4* dst = reinterpret_cast<uint4*>(p.out + r_out * p.out_row_stride + it.h * DH + kOutCols * half);
+#pragma unroll
+          for (int i = 0; i < kOutCols / 8; ++i) dst[i] = make_uint4(0u, 0u, 0u, 0u);
+          if (p.lse != nullptr && half == 0) p.lse[r_out * p.H + it.h] = -INFINITY;
+        }
+        continue;
+      }
       const uint32_t o_acc = tmem_o + (uint32_t)((li & 1) * DH);
       float m_run = -INFINITY, l_run = 0.f;
-      for (int j = 0; j < NB; ++j, ++g) {
+      for (int j = 0; j < it.nb; ++j, ++g) {
         ok = ok && tc::mbar_wait(s_full, g & 1, abort_flag);
         ok = __all_sync(kFullMask, ok);
         if (!ok) break;
@@ -373,7 +452,7 @@ cross_attn_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_con
         tc::tc_fence_before();
         __syncwarp();
         if (lane == 0) tc::mbar_arrive(s_free);              // the scores now live in registers
-        const int valid = min(kCaBN, p.T - j * kCaBN) - col_base;   // this thread's columns that exist
+        const int valid = min(kCaBN, it.T - j * kCaBN) - col_base;   // this thread's columns that exist
         if (valid < kCols) {
 #pragma unroll
           for (int i = 0; i < kCols; ++i)
@@ -408,6 +487,7 @@ cross_attn_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_con
         // probabilities -> packed bf16 in the P columns; row sum in four independent accumulators
         const float neg_m = -m_new;
         float s0 = 0.f, s1 = 0.f, s2 = 0.f, s3 = 0.f;
+        uint32_t lo[P32 ? kCols / 2 : 1];
 #pragma unroll
         for (int i = 0; i < kCols / 4; ++i) {
           const float e0 = ex2(fmaf(__uint_as_float(r[4 * i]), p.scale_log2, neg_m));
@@ -415,21 +495,28 @@ cross_attn_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_con
           const float e2 = ex2(fmaf(__uint_as_float(r[4 * i + 2]), p.scale_log2, neg_m));
           const float e3 = ex2(fmaf(__uint_as_float(r[4 * i + 3]), p.scale_log2, neg_m));
           s0 += e0; s1 += e1; s2 += e2; s3 += e3;
-          r[2 * i] = pack_bf16x2(e0, e1);
-          r[2 * i + 1] = pack_bf16x2(e2, e3);
+          const uint32_t h0 = pack_bf16x2(e0, e1), h1 = pack_bf16x2(e2, e3);
+          r[2 * i] = h0;
+          r[2 * i + 1] = h1;
+          if (P32) {
+            lo[2 * i] = pack_bf16x2(e0 - bf16_lo(h0), e1 - bf16_hi(h0));
+            lo[2 * i + 1] = pack_bf16x2(e2 - bf16_lo(h1), e3 - bf16_hi(h1));
+          }
         }
         l_run = fmaf(l_run, alpha, (s0 + s1) + (s2 + s3));
-        if (g >= 2) {
-          // the P columns of this parity were read by P V of block g - 2: long finished, but it must be
-          ok = wait_pv(g - 2);
+        constexpr int kPBack = P32 ? 1 : 2;                   // the P columns were last read by P V of block g - kPBack
+        if (g >= kPBack) {
+          ok = wait_pv(g - kPBack);                           // (two blocks back: long finished, but it must be)
           if (!ok) break;
           tc::tc_fence_after();
         }
         {
+          const uint32_t p_cols = tmem_p + (uint32_t)(P32 ? 0 : (g & 1) * 64) + lane_addr + (kCols / 2) * half;
 #pragma unroll
-          for (int c = 0; c < kCols / 2; c += 16)
-            tc::tmem_st16(tmem_p + (uint32_t)((g & 1) * 64) + lane_addr + (kCols / 2) * half + c,
-                          *reinterpret_cast<uint32_t(*)[16]>(&r[c]));
+          for (int c = 0; c < kCols / 2; c += 16) {
+            tc::tmem_st16(p_cols + c, *reinterpret_cast<uint32_t(*)[16]>(&r[c]));
+            if (P32) tc::tmem_st16(p_cols + 64 + c, *reinterpret_cast<uint32_t(*)[16]>(&lo[P32 ? c : 0]));
+          }
         }
         if (j > 0 && __any_sync(kFullMask, grow)) {           // rare after the first blocks
           // O changes under the tensor core only here: P V of block g - 1 (the same item) must be complete
@@ -454,16 +541,111 @@ cross_attn_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_con
         __syncwarp();
         if (lane == 0) tc::mbar_arrive(p_full + (g & 1));
         // the previous item's output, now that this block is with the tensor core
-        if (pend_item >= 0) {
-          ok = store_item(pend_item, pend_g, pend_li, pend_m, pend_l);
-          pend_item = -1;
+        if (SPLIT == 1 && pend_g >= 0) {
+          ok = store_item(pend_it, pend_g, pend_li, pend_m, pend_l);
+          pend_g = -1;
           if (!ok) break;
         }
       }
       if (!ok) break;
-      pend_item = item; pend_g = g - 1; pend_li = li; pend_m = m_run; pend_l = l_run;
+      pend_it = it; pend_g = g - 1; pend_li = li; pend_m = m_run; pend_l = l_run;
+      ++li;
     }
-    if (ok && pend_item >= 0) store_item(pend_item, pend_g, pend_li, pend_m, pend_l);
+    if (SPLIT == 1) {
+      if (ok && pend_g >= 0) store_item(pend_it, pend_g, pend_li, pend_m, pend_l);
+    } else {
+      // ---- merge of the cluster's partial results ----
+      const int rank = (int)tc::cluster_cta_rank();
+      const bool have = pend_g >= 0;                          // this CTA had blocks of the item
+      if (have) { ok = wait_pv(pend_g) && ok; tc::tc_fence_after(); }
+      float l_tot = pend_l;
+      if (TPR == 2) {
+        half_sum[half * 128 + row] = pend_l;
+        tc::named_bar_sync(2 + quarter, 64);
+        l_tot += half_sum[(half ^ 1) * 128 + row];
+      }
+      const float2 ml = make_float2(have ? pend_m : -INFINITY, have ? l_tot : 0.f);
+      asm volatile("barrier.cluster.wait.aligned;" ::: "memory");        // the other CTAs have started
+      // A slice of kSlice columns goes to its owner (16 at a time; the two threads of a row take every second piece)
+      auto read_o = [&](int col, uint32_t (&o)[16]) {
+        if (have) {
+          tc::tmem_ld16(tmem_o + lane_addr + (uint32_t)col, o);
+          tc::tmem_ld_wait();
+        } else {
+#pragma unroll
+          for (int i = 0; i < 16; ++i) o[i] = 0u;
+        }
+      };
+      constexpr int kPieces = kSlice / 16;
+#pragma unroll 1
+      for (int o = 1; o < SPLIT; ++o) {
+        const int dst = (rank + o) % SPLIT, slot = rank < dst ? rank : rank - 1;
+#pragma unroll 1
+        for (int c = 0; c < kPieces; ++c) {
+          if (TPR == 2 && ((c + o) & 1) != half) continue;
+          uint32_t v[16];
+          read_o(dst * kSlice + 16 * c, v);
+          const uint32_t remote = tc::cluster_addr_of(xbuf + (slot * (kSlice / 4) + 4 * c) * 128 + row, (uint32_t)dst);
+#pragma unroll
+          for (int j = 0; j < 4; ++j)
+            asm volatile("st.shared::cluster.v4.b32 [%0], {%1, %2, %3, %4};"
+                         ::"r"(remote + (uint32_t)(j * 128 * 16)), "r"(v[4 * j]), "r"(v[4 * j + 1]), "r"(v[4 * j + 2]),
+                           "r"(v[4 * j + 3]) : "memory");
+        }
+        if (half == 0)
+          asm volatile("st.shared::cluster.v2.f32 [%0], {%1, %2};"
+                       ::"r"(tc::cluster_addr_of(mlbuf + rank * 128 + row, (uint32_t)dst)), "f"(ml.x), "f"(ml.y) : "memory");
+      }
+      if (half == 0) mlbuf[rank * 128 + row] = ml;
+      tc::cluster_sync_all();
+      float m_all = -INFINITY, l_all = 0.f, w[SPLIT];
+#pragma unroll
+      for (int s = 0; s < SPLIT; ++s) { w[s] = mlbuf[s * 128 + row].x; m_all = fmaxf(m_all, w[s]); }
+#pragma unroll
+      for (int s = 0; s < SPLIT; ++s) {
+        w[s] = w[s] == -INFINITY ? 0.f : ex2(w[s] - m_all);
+        l_all = fmaf(mlbuf[s * 128 + row].y, w[s], l_all);
+      }
+      const float inv = l_all > 0.f ? 1.f / l_all : 0.f;       // no encoder position: the output is defined as zero
+      const int m = pend_it.tile * kCaBM + row;
+      const int64_t r_out = (int64_t)pend_it.b * p.M + m;
+      const bool live = ok && m < p.M;
+#pragma unroll 1
+      for (int c = 0; c < kPieces; ++c) {
+        if (TPR == 2 && (c & 1) != half) continue;
+        uint32_t own[16];
+        read_o(rank * kSlice + 16 * c, own);
+        float v[16];
+#pragma unroll
+        for (int i = 0; i < 16; ++i) v[i] = 0.f;
+#pragma unroll
+        for (int s = 0; s < SPLIT; ++s) {                      // in rank order, whoever owns the columns
+#pragma unroll
+          for (int j = 0; j < 4; ++j) {
+            float4 t = make_float4(__uint_as_float(own[4 * j]), __uint_as_float(own[4 * j + 1]),
+                                   __uint_as_float(own[4 * j + 2]), __uint_as_float(own[4 * j + 3]));
+            if (s != rank) t = xbuf[((s < rank ? s : s - 1) * (kSlice / 4) + 4 * c + j) * 128 + row];
+            v[4 * j] = fmaf(t.x, w[s], v[4 * j]); v[4 * j + 1] = fmaf(t.y, w[s], v[4 * j + 1]);
+            v[4 * j + 2] = fmaf(t.z, w[s], v[4 * j + 2]); v[4 * j + 3] = fmaf(t.w, w[s], v[4 * j + 3]);
+          }
+        }
+        if (live) {
+          uint4* dst = reinterpret_cast<uint4*>(p.out + r_out * p.out_row_stride + pend_it.h * DH + rank * kSlice + 16 * c);
+#pragma unroll
+          for (int j = 0; j < 2; ++j)
+            dst[j] = make_uint4(pack_bf16x2(v[8 * j] * inv, v[8 * j + 1] * inv), pack_bf16x2(v[8 * j + 2] * inv, v[8 * j + 3] * inv),
+                                pack_bf16x2(v[8 * j + 4] * inv, v[8 * j + 5] * inv), pack_bf16x2(v[8 * j + 6] * inv, v[8 * j + 7] * inv));
+        }
+      }
+      if (live && p.lse != nullptr && rank == 0 && half == 0)
+        p.lse[r_out * p.H + pend_it.h] = l_all > 0.f ? (m_all + log2f(l_all)) * 0.6931471805599453f : -INFINITY;
+      tc::tc_fence_before();
+    }
+  }
+  if (SPLIT > 1 && warp >= kCaSoftmaxWarps) {                  // the producer's and the issuer's part in the two cluster barriers
+    __syncwarp();
+    asm volatile("barrier.cluster.wait.aligned;" ::: "memory");
+    tc::cluster_sync_all();
   }
   tc::tc_fence_before();
   __syncthreads();
@@ -471,15 +653,43 @@ cross_attn_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_con
 }
 
 inline bool cross_attn_tc_supported(int B, int M, int H, int d_h, int T_ctx) {
-  return d_h == 128 && H <= 65535 && B <= 65535 && T_ctx >= 1 && M >= 1;      // head size 64: cross_attn_ms.cuh
+  return (d_h == 64 || d_h == 128) && H <= 65535 && B <= 65535 && T_ctx >= 1 && M >= 1;
 }
 
-template <int DH, int TPR>
-inline grace_status_t launch_cross_attn_tc_dh(const uint16_t* q, int64_t q_row_stride, const uint16_t* k,
-                                              const uint16_t* v, int64_t kv_stride_b, int64_t kv_stride_h,
-                                              int64_t kv_stride_t, uint16_t* out, int64_t out_row_stride, float* lse,
-                                              int B, int M, int H, int T_ctx, float scale, cudaStream_t s) {
-  constexpr int kCaSmemBytes = CaCfg<DH>::kSmemBytes;
+template <int DH, int TPR, int SPLIT, bool P32>
+inline grace_status_t launch_cross_attn_tc_form(const CUtensorMap& mq, const CUtensorMap& mk, const CUtensorMap& mv,
+                                                const CrossTcParams& p, int items, cudaStream_t s) {
+  constexpr int kCaSmemBytes = CaCfg<DH, SPLIT>::kSmemBytes;
+  static unsigned long long attr_set_devices = 0;
+  static int n_sm_of[kMaxDevices] = {0};
+  DeviceSetup su(&attr_set_devices);
+  if (su) {
+    GRACE_CUDA_TRY(cudaFuncSetAttribute(cross_attn_tc_kernel<DH, TPR, SPLIT, P32>, cudaFuncAttributeMaxDynamicSharedMemorySize, kCaSmemBytes));
+    GRACE_CUDA_TRY(cudaDeviceGetAttribute(&n_sm_of[su.dev], cudaDevAttrMultiProcessorCount, su.dev));
+    su.done();
+  }
+  const int n_sm = n_sm_of[su.dev];
+  cudaLaunchConfig_t cfg = {};
+  cudaLaunchAttribute attr[2];
+  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  attr[1].id = cudaLaunchAttributeClusterDimension;
+  attr[1].val.clusterDim.x = SPLIT; attr[1].val.clusterDim.y = 1; attr[1].val.clusterDim.z = 1;
+  cfg.gridDim = dim3(SPLIT > 1 ? items * SPLIT : (items < n_sm ? items : n_sm));
+  cfg.blockDim = dim3((4 * TPR + 2) * 32); cfg.dynamicSmemBytes = kCaSmemBytes; cfg.stream = s;
+  cfg.attrs = attr; cfg.numAttrs = SPLIT > 1 ? 2 : 1;
+  cudaLaunchKernelEx(&cfg, cross_attn_tc_kernel<DH, TPR, SPLIT, P32>, mq, mk, mv, p);
+  GRACE_LAUNCH_CHECK();
+  return GRACE_OK;
+}
+
+// split: how many CTAs share a work item (1, 2 or 4); p32: fp32-like probabilities (above).
+template <int DH>
+inline grace_status_t launch_cross_attn_tc(const uint16_t* q, int64_t q_row_stride, const uint16_t* k,
+                                           const uint16_t* v, int64_t kv_stride_b, int64_t kv_stride_h,
+                                           int64_t kv_stride_t, uint16_t* out, int64_t out_row_stride, float* lse,
+                                           const int32_t* enc_len, int B, int M, int H, int T_ctx, float scale, int split, bool p32,
+                                           cudaStream_t s) {
   CUtensorMap mq, mk, mv;
   {
     const uint64_t dims[4] = {(uint64_t)DH, (uint64_t)H, (uint64_t)M, (uint64_t)B};
@@ -494,36 +704,22 @@ inline grace_status_t launch_cross_attn_tc_dh(const uint16_t* q, int64_t q_row_s
     if (!tc::make_tmap_bf16(&mk, k, 4, dims, str, box)) return GRACE_CUDA_ERROR;
     if (!tc::make_tmap_bf16(&mv, v, 4, dims, str, box)) return GRACE_CUDA_ERROR;
   }
-  static unsigned long long attr_set_devices = 0;
-  static int n_sm_of[kMaxDevices] = {0};
-  DeviceSetup su(&attr_set_devices);
-  if (su) {
-    GRACE_CUDA_TRY(cudaFuncSetAttribute(cross_attn_tc_kernel<DH, TPR>, cudaFuncAttributeMaxDynamicSharedMemorySize, kCaSmemBytes));
-    GRACE_CUDA_TRY(cudaDeviceGetAttribute(&n_sm_of[su.dev], cudaDevAttrMultiProcessorCount, su.dev));
-    su.done();
-  }
-  const int n_sm = n_sm_of[su.dev];
   CrossTcParams p;
-  p.out = out; p.lse = lse; p.out_row_stride = out_row_stride; p.B = B; p.M = M; p.H = H; p.T = T_ctx;
+  p.out = out; p.lse = lse; p.enc_len = enc_len; p.out_row_stride = out_row_stride; p.B = B; p.M = M; p.H = H; p.T = T_ctx;
   p.tiles_m = (M + kCaBM - 1) / kCaBM;
   const int64_t items = (int64_t)p.tiles_m * H * B;
-  if (items > 0x7fffffff) return GRACE_UNSUPPORTED_SHAPE;
-  p.total_items = (int)items;
+  if (items * split > 0x7fffffff) return GRACE_UNSUPPORTED_SHAPE;
+  p.total_items = (int)items * split;
   p.scale_log2 = scale * 1.4426950408889634f;
-  const int ctas = CaCfg<DH>::kCtasPerSm * n_sm;
-  const int grid = (int)(items < ctas ? items : ctas);
-  launch_pdl(cross_attn_tc_kernel<DH, TPR>, dim3(grid), dim3((4 * TPR + 2) * 32), kCaSmemBytes, s, mq, mk, mv, p);
-  GRACE_LAUNCH_CHECK();
-  return GRACE_OK;
-}
-
-inline grace_status_t launch_cross_attn_tc(const uint16_t* q, int64_t q_row_stride, const uint16_t* k,
-                                           const uint16_t* v, int64_t kv_stride_b, int64_t kv_stride_h,
-                                           int64_t kv_stride_t, uint16_t* out, int64_t out_row_stride, float* lse,
-                                           int B, int M, int H, int d_h, int T_ctx, float scale, cudaStream_t s) {
-  (void)d_h;                                                // 128 (cross_attn_tc_supported)
-  return launch_cross_attn_tc_dh<128, 2>(q, q_row_stride, k, v, kv_stride_b, kv_stride_h, kv_stride_t, out, out_row_stride,
-                                        lse, B, M, H, T_ctx, scale, s);
+  const int n = (int)items;
+  if (p32) {
+    if (split == 4) return launch_cross_attn_tc_form<DH, 2, 4, true>(mq, mk, mv, p, n, s);
+    if (split == 2) return launch_cross_attn_tc_form<DH, 2, 2, true>(mq, mk, mv, p, n, s);
+    return launch_cross_attn_tc_form<DH, 2, 1, true>(mq, mk, mv, p, n, s);
+  }
+  if (split == 4) return launch_cross_attn_tc_form<DH, 2, 4, false>(mq, mk, mv, p, n, s);
+  if (split == 2) return launch_cross_attn_tc_form<DH, 2, 2, false>(mq, mk, mv, p, n, s);
+  return launch_cross_attn_tc_form<DH, 2, 1, false>(mq, mk, mv, p, n, s);
 }
 
 }  // namespace grace

@@ -1,7 +1,11 @@
 """GPU parity at the sizes where a kernel or a dispatch rule can go wrong: tile edges, remainders, the smallest and the
 largest of its range, against the oracle (fp64) on the same seeded inputs."""
+import numpy as np
 import pytest
 import torch
+
+import synth
+from oracle import attention as OA
 
 pytestmark = pytest.mark.gpu
 
@@ -12,22 +16,54 @@ def api():
     return _api
 
 
-from gpu_util import DEV  # noqa: E402
+from gpu_util import DEV, assert_attention_close, dev, dev_bf16, f64  # noqa: E402
+
+
+# head size 128 with lengths: one block and several, several items per CTA with empty ones among them (more items than
+# SMs), few rows per request (a CTA per row and head) at every head size it serves, and too many pairs for that
+@pytest.mark.parametrize("B,M,H,d,T", [(7, 130, 16, 128, 260), (3, 257, 4, 128, 129), (40, 20, 9, 128, 130), (5, 8, 4, 64, 90),
+                                       (5, 1, 2, 128, 33), (6, 8, 30, 64, 70)])
+def test_cross_attn_lengths_on_every_route(api, B, M, H, d, T):
+    rng = synth.rng_for(2, 1300 + M + T)
+    q, k, v = (synth.normal_bf16(rng, s) for s in ((B, M, H, d), (B, H, T, d), (B, H, T, d)))
+    enc_len = np.array(([T, 0, 1, 128, T - 1, 64, 0] * B)[:B], dtype=np.int32)
+    enc_len = np.minimum(enc_len, T).astype(np.int32)
+    ref, lse_ref = OA.cross_attn_varlen(f64(q), f64(k), f64(v), enc_len, d ** -0.5)
+    kf, vf = synth.bf16_bits_to_f32(k).copy(), synth.bf16_bits_to_f32(v).copy()
+    for b in range(B):                                       # what lies past a request's length has no influence
+        kf[b, :, enc_len[b]:], vf[b, :, enc_len[b]:] = 50.0, -1000.0
+    out = torch.full((B * M, H, d), 7.0, dtype=torch.bfloat16, device=DEV)
+    lse = torch.zeros((B * M, H), dtype=torch.float32, device=DEV)
+    api.grace_cross_attn_varlen(dev_bf16(q).reshape(B * M, H, d), dev(kf).to(torch.bfloat16), dev(vf).to(torch.bfloat16),
+                                out, dev(enc_len), d ** -0.5, lse)
+    torch.cuda.synchronize()
+    got, got_lse = out.float().cpu().numpy().reshape(B, M, H, d), lse.cpu().numpy().reshape(B, M, H)
+    assert_attention_close(got, ref, "cross-attn lengths")
+    empty = enc_len == 0
+    assert (got[empty] == 0).all() and np.isneginf(got_lse[empty]).all()
+    np.testing.assert_allclose(got_lse[~empty], lse_ref[~empty], atol=2e-3, rtol=0)
 
 
 @pytest.mark.parametrize("B,M,H,T", [(16, 1000, 16, 200), (20, 300, 8, 640)])
 def test_cross_attn_waits_never_give_up_back_to_back(api, B, M, H, T):
-    """Head size 128, launches queued without a gap: no bounded wait runs out (the issuing
+    """Head size 128, launches queued without a gap, with and without lengths: no bounded wait runs out (the issuing
     thread may come arbitrarily late to its wait for a block's probabilities), and the last output is the first's."""
     d = 128
     g = torch.Generator(device=DEV)
     g.manual_seed(5)
     q, k, v = (torch.randn(*s, device=DEV, generator=g).to(torch.bfloat16) for s in ((B * M, H, d), (B, H, T, d), (B, H, T, d)))
+    lengths = torch.from_numpy(np.linspace(T // 4, T, B).astype(np.int32)).to(DEV)
     first, last = torch.empty_like(q), torch.empty_like(q)
     api.grace_wait_timeouts()
-    api.grace_cross_attn(q, k, v, first, d ** -0.5)
-    for _ in range(4000):
-        api.grace_cross_attn(q, k, v, last, d ** -0.5)
-    torch.cuda.synchronize()
-    assert api.grace_wait_timeouts() == 0
-    assert torch.equal(first, last)
+    for enc_len in (None, lengths):
+        def call(out):
+            if enc_len is None:
+                api.grace_cross_attn(q, k, v, out, d ** -0.5)
+            else:
+                api.grace_cross_attn_varlen(q, k, v, out, enc_len, d ** -0.5)
+        call(first)
+        for _ in range(4000):
+            call(last)
+        torch.cuda.synchronize()
+        assert api.grace_wait_timeouts() == 0
+        assert torch.equal(first, last)
