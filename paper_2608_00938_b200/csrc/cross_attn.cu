@@ -208,10 +208,20 @@ cross_attn_row_kernel(const CrossSmallParams p) {
 }  // namespace grace
 
 namespace grace {
-// Which kernel: 0: cross_attn_ms_kernel, 1: cross_attn_tc_kernel.
+// Which kernel and, for cross_attn_tc_kernel, how many CTAs share a work item (0: cross_attn_ms_kernel).  With at most
+// one 128-row tile per SM the GPU is idle beside them and an item's chain over its K / V blocks is what a call takes,
+// so the blocks are split as far as SMs and blocks go (d 64: 32 tiles, 8 blocks: ms 20.9 us, split 1 14.4, 2 9.2,
+// 4 7.6; 64 tiles, 4 blocks: 12.5 / 9.1 / 7.3; 128 tiles, 8 blocks: 21.2 / 15.1, 64 tiles, 1 block: 4.9 / 5.1);
+// clusters that do not all fit at once cost more than they give (64 tiles, 4 blocks, split 4: 12.4).  At head size 128 a
+// CTA keeps two blocks (16 tiles, 2 blocks: 6.2 / 6.7; 16 tiles, 8 blocks: 16.7 / 11.6 / 8.8).  Beyond one tile per SM
+// head size 64 takes the four-stream kernel (256 tiles, 8 blocks: ms 25.0 us, tc 27.6; 512 tiles: 36.6 / 50.6).
 static int cross_attn_form(int B, int M, int H, int d_h, int T_ctx, bool p32) {
-  (void)B; (void)M; (void)H; (void)T_ctx;
-  return d_h == 64 && !p32 ? 0 : 1;
+  const int64_t tiles = (int64_t)((M + kCaBM - 1) / kCaBM) * H * B;
+  const int blocks = (T_ctx + kCaBN - 1) / kCaBN, least = d_h == 128 ? 2 : 1;
+  if (tiles > 148) return d_h == 64 && !p32 ? 0 : 1;
+  if (tiles * 4 <= 148 && blocks >= 4 * least) return 4;
+  if (tiles * 2 <= 148 && blocks >= 2 * least) return 2;
+  return 1;
 }
 int cross_attn_tc_timeouts() { return tc::tc_timeouts_read_and_clear(); }
 }  // namespace grace

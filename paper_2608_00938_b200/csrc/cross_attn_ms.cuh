@@ -129,9 +129,11 @@ cross_attn_ms_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_con
   const uint32_t tmem_base = *tmem_slot;
   pdl_wait();                                  // barrier set-up and TMEM allocation overlapped the previous kernel's tail
   pdl_trigger();
-  // Half `hf` of CTA c works on the items 2 (c + k gridDim) + hf, k = 0, 1, ...: the two halves of a
-  // CTA and neighbouring CTAs run neighbouring items, which share K/V in L2.
+  // Half `hf` of CTA c works on the items c + (2 k + hf) gridDim, k = 0, 1, ...: neighbouring CTAs run
+  // neighbouring items, which share K/V in L2, and with fewer items than halves every SM gets one before any
+  // gets two.
   const int item_step = 2 * (int)gridDim.x;
+  auto first_item = [](int hf) { return (int)blockIdx.x + hf * (int)gridDim.x; };
 
   if (warp >= kMsSoftmaxWarps) {
     // ---------------- MMA issuer and TMA producer, one warp per stream ----------------
@@ -158,7 +160,7 @@ cross_attn_ms_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_con
     if (lane == 0) { tc::tma_prefetch_desc(&map_q); tc::tma_prefetch_desc(&map_k); tc::tma_prefetch_desc(&map_v); }
 
     // ---- loads ----
-    int lq_item = 2 * (int)blockIdx.x + hf, lq_cnt = 0;           // Q: next item to look at; tiles requested
+    int lq_item = first_item(hf), lq_cnt = 0;           // Q: next item to look at; tiles requested
     int lk_item = lq_item, lk_j = 0, lk_cnt = 0;                  // K/V (first stream of the half only): item, block, blocks requested
     MsItem lk_it = lk_item < p.total_items ? ms_item(p, lk_item) : MsItem{0, 0, 0, 0, 0, 0};
     MsItem lq_it = lk_it;                                          // an item is decoded when a queue moves on to it
@@ -233,7 +235,7 @@ cross_attn_ms_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_con
         c.item += item_step;
       }
     };
-    Cursor cs = {2 * (int)blockIdx.x + hf, 0, 0}, cp = cs;
+    Cursor cs = {first_item(hf), 0, 0}, cp = cs;
     uint32_t kc = 0, vc = 0;                      // blocks whose S / whose P V has been issued (ring slot = count % stages)
     uint32_t qs = 0;                              // Q tiles started by the S cursor (buffer = qs & 1)
     uint32_t pw = 0;                              // p_full phases consumed
@@ -323,7 +325,7 @@ cross_attn_ms_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_con
         release = -1;
       }
     };
-    for (int item = 2 * (int)blockIdx.x + hf; ok && item < p.total_items; item += item_step) {
+    for (int item = first_item(hf); ok && item < p.total_items; item += item_step) {
       const MsItem it = ms_item(p, item);
       if (tile >= it.ntiles) continue;
       const int m = it.row0 + tile * kMsBM + row;
@@ -493,8 +495,7 @@ inline grace_status_t launch_cross_attn_ms(const uint16_t* q, int64_t q_row_stri
   if (items > 0x3fffffff) return GRACE_UNSUPPORTED_SHAPE;
   p.total_items = (int)items;
   p.scale_log2 = scale * 1.4426950408889634f;
-  const int64_t ctas = (items + 1) / 2;
-  const int grid = (int)(ctas < n_sm ? ctas : n_sm);
+  const int grid = (int)(items < n_sm ? items : n_sm);
   launch_pdl(cross_attn_ms_kernel, dim3(grid), dim3(kMsThreads), kMsSmemBytes, s, mq, mk, mv, mo, p);
   GRACE_LAUNCH_CHECK();
   return GRACE_OK;
