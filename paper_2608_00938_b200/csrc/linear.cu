@@ -1,14 +1,16 @@
 // y = act(x @ w^T) (+ residual): the projection / feed-forward / logits GEMMs of the decoder
 // layer (Section 3.2), on tcgen05 tensor cores.
 //
-// One CTA computes a 128 x BN output tile.  A producer thread streams 128 x 64 bf16 tiles of x
-// and BN x 64 tiles of w through a ring of shared-memory stages with TMA (128-byte swizzle,
-// out-of-range rows read as zero, so ragged M and N need no special path).  One thread issues
-// tcgen05.mma (M = 128, N = BN, K = 16 per instruction) with the fp32 accumulator in TMEM;
-// tcgen05.commit frees each stage as soon as the tensor core has consumed it.  All four warps then
-// read the accumulator back (each warp its own 32 TMEM lanes = 32 output rows), apply ReLU /
-// residual, and store bf16 or fp32.  Two CTAs fit on an SM, so one CTA's epilogue overlaps the
-// other's main loop.
+// Two kernels: linear_kernel (one 128 x BN tile per CTA or per cluster, for the problems whose tiles do
+// not fill the GPU with 256 x 256 pair tiles) and linear_pair_kernel (persistent CTA pairs, further down).
+//
+// linear_kernel: a producer thread streams 128 x 64 bf16 tiles of x and BN x 64 tiles of w through a ring
+// of shared-memory stages with TMA (128-byte swizzle, out-of-range rows read as zero, so ragged M and N
+// need no special path).  One thread issues tcgen05.mma (M = 128, N = BN, K = 16 per instruction) with the
+// fp32 accumulator in TMEM; tcgen05.commit frees each stage as soon as the tensor core has consumed it.
+// Four warps own the tile's rows (thread = row = TMEM lane): where a LayerNorm is folded in they form the
+// rows' statistics from the operand tiles while the tensor core works on them, then they read the
+// accumulator back, apply LayerNorm / ReLU / residual and store bf16 or fp32.
 #include "common.cuh"
 #include "tc.cuh"
 
@@ -23,15 +25,24 @@ __device__ __forceinline__ float fast_ex2(float x) {
 constexpr int kGemmBM = 128;
 constexpr int kGemmBK = 64;
 
-// STAGES = 3: throughput form (several CTAs per SM).  STAGES = 8 with BN = 32: latency form for launches whose grid
-// does not fill the GPU (step 0 of a decode: 32 rows): the whole K = 512 of a tile is in flight at once, and the
-// narrow tile spreads the weight stream over twice as many SMs as BN = 64 did (step 0: 382 -> 352 us; BN = 16: same).
-template <int BN, int STAGES>
-struct GemmSmem {
+// What bounds the small problems of a decode (1 .. a few thousand rows) is latency and the 64 bytes per clock that
+// an SM can pull from L2: a 128 x BN tile takes (128 + BN) * K * 2 bytes.  SPLIT > 1: a cluster of SPLIT CTAs shares
+// a tile, each taking a range of K; every CTA then owns BN / SPLIT of the tile's columns, receives the other CTAs'
+// partial sums of them through distributed shared memory, adds them in rank order and finishes them (the row
+// statistics, which each CTA has for its range of K, travel the same way).  The K loop and the epilogue both
+// shrink by SPLIT and the grid grows by it.  Stages: the whole K range of a CTA in flight where it fits (latency
+// forms), three where several CTAs share an SM (throughput form).
+template <int BN, int STAGES, int SPLIT>
+struct GemmCfg {
   static constexpr int kABytes = kGemmBM * kGemmBK * 2;
   static constexpr int kBBytes = BN * kGemmBK * 2;
   static constexpr int kStageBytes = kABytes + kBBytes;
-  static constexpr int kTotal = STAGES * kStageBytes + 1024 /*alignment slack*/ + 256 /*barriers*/;
+  static constexpr int kSlice = BN / SPLIT;                                   // columns a CTA finishes
+  static constexpr int kXBytes = (SPLIT - 1) * kGemmBM * kSlice * 4;          // the other CTAs' partial sums of them
+  static constexpr int kStatBytes = SPLIT > 1 ? SPLIT * kGemmBM * 8 : 0;      // (sum, sum of squares) per row and CTA
+  static constexpr int kColBytes = kSlice * 8;                                // (col_sum, col_bias) of those columns
+  static constexpr int kTotal = STAGES * kStageBytes + kXBytes + kStatBytes + kColBytes + 1024 /*alignment slack*/ + 256 /*barriers*/;
+  static_assert(kSlice % 16 == 0 && kTotal <= 227 * 1024, "");
 };
 
 struct GemmParams {
@@ -40,165 +51,311 @@ struct GemmParams {
   const float* residual;
   const uint16_t* residual_bf16;   // bf16 residual stream (added in fp32, result rounded to bf16)
   // LayerNorm folded into the GEMM (x is the raw stream, w carries the gain): y = row.x * acc + row.y * col_sum + col_bias
-  const float2* aff_row;           // [M]: (rstd, -rstd * mean) of the row; nullptr = plain GEMM
+  const float2* aff_row;           // [M]: (rstd, -rstd * mean) of the row; nullptr = none given
   const float* aff_cs;             // [N]: sum over k of w[n][k]
-  const float* aff_cb;             // [N]: sum over k of beta[k] * w0[n][k]
+  const float* aff_cb;             // [N]: sum over k of beta[k] * w0[n][k]; nullptr = plain GEMM
+  float ln_eps;                    // aff_cb given, aff_row not: the kernel forms the rows' statistics itself,
+  float2* aff_out;                 //   and leaves them here too (if not NULL)
   int64_t ldy;
   int M, N, K, relu;
 };
 
-template <int BN, int STAGES>
-__global__ void __launch_bounds__(128)
+constexpr int kGemmThreads = 192;                           // four row warps, TMA producer, MMA issuer
+
+template <int BN, int STAGES, int SPLIT>
+__global__ void __launch_bounds__(kGemmThreads, 2)
 linear_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_constant__ CUtensorMap map_w,
               const GemmParams p) {
   // The weights do not depend on the kernel before this one: their first tiles are requested before the wait
   // on that kernel, so their trip from HBM overlaps its tail; every thread waits before its first access to
   // anything an earlier kernel wrote (activations, row statistics, the residual).
   pdl_trigger();
-  constexpr int kGemmStages = STAGES;
-  using S = GemmSmem<BN, STAGES>;
+  using S = GemmCfg<BN, STAGES, SPLIT>;
+  constexpr int kSlice = S::kSlice;
   extern __shared__ uint8_t smem_raw[];
   uint8_t* tiles = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
-  uint64_t* full = reinterpret_cast<uint64_t*>(tiles + kGemmStages * S::kStageBytes);
-  uint64_t* empty = full + kGemmStages;
-  uint64_t* accum_bar = empty + kGemmStages;
+  float4* xbuf = reinterpret_cast<float4*>(tiles + STAGES * S::kStageBytes);            // [SPLIT - 1][kSlice / 4][128]
+  float2* sbuf = reinterpret_cast<float2*>(tiles + STAGES * S::kStageBytes + S::kXBytes);   // [SPLIT][128]
+  float* col_s = reinterpret_cast<float*>(tiles + STAGES * S::kStageBytes + S::kXBytes + S::kStatBytes);   // [kSlice] bias, [kSlice] sum
+  uint64_t* full = reinterpret_cast<uint64_t*>(tiles + STAGES * S::kStageBytes + S::kXBytes + S::kStatBytes + S::kColBytes);
+  uint64_t* empty = full + STAGES;
+  uint64_t* accum_bar = empty + STAGES;
   uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(accum_bar + 1);
   volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_slot + 1);
 
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int m0 = blockIdx.y * kGemmBM, n0 = blockIdx.x * BN;
-  const int KB = p.K / kGemmBK;
+  const int rank = SPLIT > 1 ? (int)(blockIdx.x % SPLIT) : 0;
+  const int m0 = blockIdx.y * kGemmBM, n0 = (int)(blockIdx.x / SPLIT) * BN;
+  const int KB_all = p.K / kGemmBK;
+  const int kb0 = KB_all * rank / SPLIT, KB = KB_all * (rank + 1) / SPLIT - kb0;        // this CTA's k-blocks (>= 1)
+  const bool folded = p.aff_cb != nullptr;
+  const bool stats = folded && p.aff_row == nullptr;
 
+  if (SPLIT > 1) asm volatile("barrier.cluster.arrive.relaxed.aligned;" ::: "memory");   // "this CTA has started"
   if (threadIdx.x == 0) {
-    for (int s = 0; s < kGemmStages; ++s) { tc::mbar_init(full + s, 1); tc::mbar_init(empty + s, 1); }
+    for (int s = 0; s < STAGES; ++s) { tc::mbar_init(full + s, 1); tc::mbar_init(empty + s, stats ? 5 : 1); }
     tc::mbar_init(accum_bar, 1);
     *abort_flag = 0;
     tc::fence_mbar_init();
-    tc::tma_prefetch_desc(&map_x);
-    tc::tma_prefetch_desc(&map_w);
   }
-  if (warp == 0) tc::tmem_alloc(tmem_slot, BN < 32 ? 32 : BN);
+  if (warp == 4) {
+    if (lane == 0) { tc::tma_prefetch_desc(&map_x); tc::tma_prefetch_desc(&map_w); }
+    __syncwarp();
+    tc::tmem_alloc(tmem_slot, BN < 32 ? 32 : BN);
+  }
   tc::tc_fence_before();
   __syncthreads();
   tc::tc_fence_after();
   const uint32_t tmem_base = *tmem_slot;
 
-  if (warp == 0 && lane == 0) {
-    // ---- TMA producer ----
-    const int first = KB < kGemmStages ? KB : kGemmStages;  // the ring's first pass needs no empty-slot wait
-    for (int kb = 0; kb < first; ++kb) {
-      tc::mbar_expect_tx(full + kb, S::kStageBytes);
-      tc::tma_load_2d(tiles + kb * S::kStageBytes + S::kABytes, &map_w, full + kb, kb * kGemmBK, n0);
-    }
-    pdl_wait();
-    for (int kb = 0; kb < first; ++kb)
-      tc::tma_load_2d(tiles + kb * S::kStageBytes, &map_x, full + kb, kb * kGemmBK, m0);
-    for (int kb = first; kb < KB; ++kb) {
-      const int s = kb % kGemmStages;
-      if (!tc::mbar_wait(empty + s, ((kb / kGemmStages) & 1) ^ 1, abort_flag)) break;
-      tc::mbar_expect_tx(full + s, S::kStageBytes);
-      uint8_t* a = tiles + s * S::kStageBytes;
-      tc::tma_load_2d(a, &map_x, full + s, kb * kGemmBK, m0);
-      tc::tma_load_2d(a + S::kABytes, &map_w, full + s, kb * kGemmBK, n0);
-    }
-  } else if (warp == 1 && lane == 0) {
-    // ---- MMA issuer ----
-    constexpr uint32_t idesc = tc::idesc_bf16(kGemmBM, BN, 0);
-    for (int kb = 0; kb < KB; ++kb) {
-      const int s = kb % kGemmStages;
-      if (!tc::mbar_wait(full + s, (kb / kGemmStages) & 1, abort_flag)) break;
-      tc::tc_fence_after();
-      const uint32_t a_addr = tc::smem_addr(tiles + s * S::kStageBytes);
-      const uint64_t a_desc = tc::smem_desc_sw128(a_addr, 16, 1024);
-      const uint64_t b_desc = tc::smem_desc_sw128(a_addr + S::kABytes, 16, 1024);
-#pragma unroll
-      for (int k = 0; k < kGemmBK / 16; ++k)
-        tc::mma_ss(tmem_base, a_desc + (uint64_t)(2 * k), b_desc + (uint64_t)(2 * k), idesc, (kb | k) ? 1u : 0u);
-      tc::mma_commit(empty + s);
-    }
-    tc::mma_commit(accum_bar);
-  }
-  __syncwarp();
-  pdl_wait();
-
-  // ---- epilogue: warp w owns TMEM lanes 32w .. 32w+31 = rows m0 + 32w + lane ----
-  // Folded LayerNorm: the row's pair and the column vectors of a chunk are fetched (from clamped addresses,
-  // unconditionally) one chunk ahead of their use, the first while the accumulator is still filling.
-  const bool folded = p.aff_row != nullptr;
-  const float* cs_or_cb = p.aff_cs != nullptr ? p.aff_cs : p.aff_cb;
+  bool ok = true;
+  float2 row_sums = make_float2(0.f, 0.f);                 // this CTA's share of the row's (sum, sum of squares)
+  const int row = warp * 32 + lane;                        // warps 0..3: TMEM lane = row of the tile
+  const int m = m0 + row;
+  // The slice is finished kChunk columns at a time.  Its column vectors wait in shared memory (fetched while the
+  // accumulator fills: read from global memory one chunk ahead they were the epilogue's critical path, 550 clocks per
+  // 16 columns); the residual is fetched one chunk ahead, from clamped addresses, so that nothing waits for it before
+  // its use.
+  constexpr int kChunk = kSlice < 32 ? kSlice : 32;
   float2 ar = make_float2(1.f, 0.f);
-  float4 cs_next[4], cb_next[4];
-  auto fetch_cols = [&](int c) {
-    if (!folded) return;
-    const int n = min(n0 + c, p.N - 16);
+  uint4 res_next[kChunk / 4];
+  const int slice0 = n0 + rank * kSlice;                   // first of the columns this CTA finishes
+  auto fetch_residual = [&](int c) {
+    const int64_t at = (int64_t)min(m, p.M - 1) * p.ldy;
+    if (p.residual != nullptr) {
 #pragma unroll
-    for (int j = 0; j < 4; ++j) {
-      cb_next[j] = __ldg(reinterpret_cast<const float4*>(p.aff_cb + n) + j);
-      cs_next[j] = __ldg(reinterpret_cast<const float4*>(cs_or_cb + n) + j);
+      for (int j = 0; j < kChunk / 4; ++j)
+        res_next[j] = *reinterpret_cast<const uint4*>(p.residual + at + min(slice0 + c + 4 * j, p.N - 4));
+    } else if (p.residual_bf16 != nullptr) {
+#pragma unroll
+      for (int j = 0; j < kChunk / 8; ++j)
+        res_next[j] = *reinterpret_cast<const uint4*>(p.residual_bf16 + at + min(slice0 + c + 8 * j, p.N - 8));
     }
   };
-  if (folded) ar = __ldg(p.aff_row + min(m0 + warp * 32 + lane, p.M - 1));
-  fetch_cols(0);
-  const bool ok = tc::mbar_wait(accum_bar, 0, abort_flag);
-  tc::tc_fence_after();
-  __syncwarp();
-  if (ok) {
-    const int m = m0 + warp * 32 + lane;
-#pragma unroll 1
-    for (int c = 0; c < BN; c += 16) {
-      uint32_t acc[16];
-      tc::tmem_ld16(tmem_base + ((uint32_t)(warp * 32) << 16) + (uint32_t)c, acc);
-      float cs[16], cb[16];
-      if (folded) {
-#pragma unroll
-        for (int j = 0; j < 4; ++j) {
-          cs[4 * j] = cs_next[j].x; cs[4 * j + 1] = cs_next[j].y; cs[4 * j + 2] = cs_next[j].z; cs[4 * j + 3] = cs_next[j].w;
-          cb[4 * j] = cb_next[j].x; cb[4 * j + 1] = cb_next[j].y; cb[4 * j + 2] = cb_next[j].z; cb[4 * j + 3] = cb_next[j].w;
-        }
-        if (c + 16 < BN) fetch_cols(c + 16);
+
+  if (warp == 4) {
+    if (lane == 0) {
+      // ---- TMA producer ----
+      const int first = KB < STAGES ? KB : STAGES;          // the ring's first pass needs no empty-slot wait
+      for (int kb = 0; kb < first; ++kb) {
+        tc::mbar_expect_tx(full + kb, S::kStageBytes);
+        tc::tma_load_2d(tiles + kb * S::kStageBytes + S::kABytes, &map_w, full + kb, (kb0 + kb) * kGemmBK, n0);
       }
-      tc::tmem_ld_wait();
-      const int n = n0 + c;
-      if (m < p.M && n < p.N) {           // N % 16 == 0: the 16 columns are all in or all out
-        float v[16];
+      pdl_wait();
+      for (int kb = 0; kb < first; ++kb)
+        tc::tma_load_2d(tiles + kb * S::kStageBytes, &map_x, full + kb, (kb0 + kb) * kGemmBK, m0);
+      for (int kb = first; kb < KB; ++kb) {
+        const int s = kb % STAGES;
+        if (!tc::mbar_wait(empty + s, ((kb / STAGES) & 1) ^ 1, abort_flag)) break;
+        tc::mbar_expect_tx(full + s, S::kStageBytes);
+        uint8_t* a = tiles + s * S::kStageBytes;
+        tc::tma_load_2d(a, &map_x, full + s, (kb0 + kb) * kGemmBK, m0);
+        tc::tma_load_2d(a + S::kABytes, &map_w, full + s, (kb0 + kb) * kGemmBK, n0);
+      }
+    }
+    __syncwarp();
+  } else if (warp == 5) {
+    if (lane == 0) {
+      // ---- MMA issuer ----
+      constexpr uint32_t idesc = tc::idesc_bf16(kGemmBM, BN, 0);
+      for (int kb = 0; kb < KB; ++kb) {
+        const int s = kb % STAGES;
+        if (!tc::mbar_wait(full + s, (kb / STAGES) & 1, abort_flag)) break;
+        tc::tc_fence_after();
+        const uint32_t a_addr = tc::smem_addr(tiles + s * S::kStageBytes);
+        const uint64_t a_desc = tc::smem_desc_sw128(a_addr, 16, 1024);
+        const uint64_t b_desc = tc::smem_desc_sw128(a_addr + S::kABytes, 16, 1024);
 #pragma unroll
-        for (int j = 0; j < 16; ++j) {
-          v[j] = __uint_as_float(acc[j]);
-          if (folded) v[j] = fmaf(ar.x, v[j], p.aff_cs != nullptr ? fmaf(ar.y, cs[j], cb[j]) : cb[j]);
-          if (p.relu) v[j] = fmaxf(v[j], 0.f);
+        for (int k = 0; k < kGemmBK / 16; ++k)
+          tc::mma_ss(tmem_base, a_desc + (uint64_t)(2 * k), b_desc + (uint64_t)(2 * k), idesc, (kb | k) ? 1u : 0u);
+        tc::mma_commit(empty + s);
+      }
+      tc::mma_commit(accum_bar);
+    }
+    __syncwarp();
+  } else {
+    pdl_wait();
+    if (folded && threadIdx.x < kSlice) {
+      const int n = min(slice0 + (int)threadIdx.x, p.N - 1);
+      col_s[threadIdx.x] = __ldg(p.aff_cb + n);
+      col_s[kSlice + threadIdx.x] = p.aff_cs != nullptr ? __ldg(p.aff_cs + n) : 0.f;
+    }
+    fetch_residual(0);
+    if (folded && !stats) ar = __ldg(p.aff_row + min(m, p.M - 1));
+    if (stats) {
+      f32x2_t acc[2], sq[4];                                // independent chains: a row is one thread's work
+#pragma unroll
+      for (int i = 0; i < 4; ++i) { acc[i & 1] = f2_pack(0.f, 0.f); sq[i] = f2_pack(0.f, 0.f); }
+      for (int kb = 0; kb < KB; ++kb) {
+        const int s = kb % STAGES;
+        ok = tc::mbar_wait(full + s, (kb / STAGES) & 1, abort_flag);
+        ok = __all_sync(kFullMask, ok);
+        if (!ok) break;
+        // 128 bytes of the row, in the order that keeps eight neighbouring rows on different banks
+        const uint4* a_row = reinterpret_cast<const uint4*>(tiles + s * S::kStageBytes + row * 128);
+#pragma unroll
+        for (int j = 0; j < 8; ++j) {
+          const uint4 t = a_row[j ^ (row & 7)];
+          const f32x2_t a = f2_from_bf16x2(t.x), b = f2_from_bf16x2(t.y), c = f2_from_bf16x2(t.z), d = f2_from_bf16x2(t.w);
+          acc[j & 1] = f2_add(acc[j & 1], f2_add(f2_add(a, b), f2_add(c, d)));
+          sq[0] = f2_fma(a, a, sq[0]); sq[1] = f2_fma(b, b, sq[1]); sq[2] = f2_fma(c, c, sq[2]); sq[3] = f2_fma(d, d, sq[3]);
+        }
+        __syncwarp();
+        if (lane == 0) tc::mbar_arrive(empty + s);
+      }
+      float lo, hi, qlo, qhi;
+      f2_unpack(f2_add(acc[0], acc[1]), lo, hi);
+      f2_unpack(f2_add(f2_add(sq[0], sq[1]), f2_add(sq[2], sq[3])), qlo, qhi);
+      row_sums = make_float2(lo + hi, qlo + qhi);
+    }
+    ok = tc::mbar_wait(accum_bar, 0, abort_flag) && ok;
+    ok = __all_sync(kFullMask, ok);
+    tc::tc_fence_after();
+    if (folded) tc::named_bar_sync(1, 128);                 // the column vectors of all four warps
+  }
+  const uint32_t t_acc = tmem_base + ((uint32_t)((warp & 3) * 32) << 16);
+  if (SPLIT > 1) {
+    // partial sums of the other CTAs' columns to their owners; every CTA of the cluster has long started
+    asm volatile("barrier.cluster.wait.aligned;" ::: "memory");
+    if (warp < 4 && ok) {
+#pragma unroll 1
+      for (int o = 1; o < SPLIT; ++o) {
+        const int dst = (rank + o) % SPLIT;
+        const int slot = rank < dst ? rank : rank - 1;     // this CTA's place among the owner's SPLIT - 1 sources
+        const uint32_t remote = tc::cluster_addr_of(xbuf + slot * (kSlice / 4) * 128 + row, (uint32_t)dst);
+#pragma unroll
+        for (int c = 0; c < kSlice; c += 16) {
+          uint32_t acc[16];
+          tc::tmem_ld16(t_acc + (uint32_t)(dst * kSlice + c), acc);
+          tc::tmem_ld_wait();
+          if (m < p.M) {
+#pragma unroll
+            for (int j = 0; j < 4; ++j)
+              asm volatile("st.shared::cluster.v4.b32 [%0], {%1, %2, %3, %4};"
+                           ::"r"(remote + (uint32_t)((c / 4 + j) * 128 * 16)), "r"(acc[4 * j]), "r"(acc[4 * j + 1]),
+                             "r"(acc[4 * j + 2]), "r"(acc[4 * j + 3]) : "memory");
+          }
+        }
+        if (stats)
+          asm volatile("st.shared::cluster.v2.f32 [%0], {%1, %2};"
+                       ::"r"(tc::cluster_addr_of(sbuf + rank * 128 + row, (uint32_t)dst)), "f"(row_sums.x), "f"(row_sums.y) : "memory");
+      }
+      if (stats) sbuf[rank * 128 + row] = row_sums;
+    }
+    __syncwarp();
+    tc::cluster_sync_all();
+    if (stats && warp < 4) {
+      row_sums = sbuf[row];
+#pragma unroll
+      for (int s = 1; s < SPLIT; ++s) {
+        const float2 t = sbuf[s * 128 + row];
+        row_sums.x += t.x;
+        row_sums.y += t.y;
+      }
+    }
+  }
+
+  if (warp < 4 && ok) {
+    if (stats) {
+      const float inv_k = 1.f / (float)p.K;
+      const float mean = row_sums.x * inv_k;
+      const float var = fmaxf(row_sums.y * inv_k - mean * mean, 0.f);
+      const float rstd = rsqrtf(var + p.ln_eps);
+      ar = make_float2(rstd, -rstd * mean);
+      if (blockIdx.x == 0 && p.aff_out != nullptr && m < p.M) p.aff_out[m] = ar;
+    }
+    const bool sectors = ((reinterpret_cast<uintptr_t>(p.y_bf16) | reinterpret_cast<uintptr_t>(p.y_f32) | (uintptr_t)p.ldy * 2) & 31) == 0;
+#pragma unroll 1
+    for (int c = 0; c < kSlice; c += kChunk) {
+      uint32_t acc[kChunk];
+      if constexpr (kChunk == 32) tc::tmem_ld32(t_acc + (uint32_t)(rank * kSlice + c), acc);
+      else tc::tmem_ld16(t_acc + (uint32_t)(rank * kSlice + c), acc);
+      uint4 res[kChunk / 4];
+#pragma unroll
+      for (int j = 0; j < kChunk / 4; ++j) res[j] = res_next[j];
+      if (c + kChunk < kSlice) fetch_residual(c + kChunk);
+      tc::tmem_ld_wait();
+#pragma unroll
+      for (int h = 0; h < kChunk; h += 16) {
+        const int n = slice0 + c + h;
+        if (m >= p.M || n >= p.N) continue;                // N % 16 == 0: the 16 columns are all in or all out
+        float v[16];
+        if (SPLIT == 1) {
+#pragma unroll
+          for (int j = 0; j < 16; ++j) v[j] = __uint_as_float(acc[h + j]);
+        } else {
+          // in rank order, whoever owns the columns
+#pragma unroll
+          for (int j = 0; j < 16; ++j) v[j] = 0.f;
+#pragma unroll
+          for (int s = 0; s < SPLIT; ++s) {
+#pragma unroll
+            for (int j = 0; j < 4; ++j) {
+              float4 t = make_float4(__uint_as_float(acc[h + 4 * j]), __uint_as_float(acc[h + 4 * j + 1]),
+                                     __uint_as_float(acc[h + 4 * j + 2]), __uint_as_float(acc[h + 4 * j + 3]));
+              if (s != rank) t = xbuf[((s < rank ? s : s - 1) * (kSlice / 4) + (c + h) / 4 + j) * 128 + row];
+              v[4 * j] += t.x; v[4 * j + 1] += t.y; v[4 * j + 2] += t.z; v[4 * j + 3] += t.w;
+            }
+          }
+        }
+        if (folded) {
+#pragma unroll
+          for (int j = 0; j < 16; j += 4) {
+            const float4 cb = *reinterpret_cast<const float4*>(col_s + c + h + j);
+            const float4 cs = *reinterpret_cast<const float4*>(col_s + kSlice + c + h + j);
+            v[j] = fmaf(ar.x, v[j], fmaf(ar.y, cs.x, cb.x)); v[j + 1] = fmaf(ar.x, v[j + 1], fmaf(ar.y, cs.y, cb.y));
+            v[j + 2] = fmaf(ar.x, v[j + 2], fmaf(ar.y, cs.z, cb.z)); v[j + 3] = fmaf(ar.x, v[j + 3], fmaf(ar.y, cs.w, cb.w));
+          }
+        }
+        if (p.relu) {
+#pragma unroll
+          for (int j = 0; j < 16; ++j) v[j] = fmaxf(v[j], 0.f);
         }
         if (p.residual != nullptr) {
-          const float4* res = reinterpret_cast<const float4*>(p.residual + (int64_t)m * p.ldy + n);
 #pragma unroll
           for (int j = 0; j < 4; ++j) {
-            const float4 r4 = res[j];
-            v[4 * j] += r4.x; v[4 * j + 1] += r4.y; v[4 * j + 2] += r4.z; v[4 * j + 3] += r4.w;
+            const uint4 r4 = res[h / 4 + j];
+            v[4 * j] += __uint_as_float(r4.x); v[4 * j + 1] += __uint_as_float(r4.y);
+            v[4 * j + 2] += __uint_as_float(r4.z); v[4 * j + 3] += __uint_as_float(r4.w);
           }
         }
         if (p.residual_bf16 != nullptr) {
-          const uint4* res = reinterpret_cast<const uint4*>(p.residual_bf16 + (int64_t)m * p.ldy + n);
 #pragma unroll
           for (int j = 0; j < 2; ++j) {
-            const uint4 r4 = res[j];
+            const uint4 r4 = res[h / 8 + j];
             v[8 * j] += bf16_lo(r4.x); v[8 * j + 1] += bf16_hi(r4.x); v[8 * j + 2] += bf16_lo(r4.y); v[8 * j + 3] += bf16_hi(r4.y);
             v[8 * j + 4] += bf16_lo(r4.z); v[8 * j + 5] += bf16_hi(r4.z); v[8 * j + 6] += bf16_lo(r4.w); v[8 * j + 7] += bf16_hi(r4.w);
           }
         }
+        // a thread owns a row: whole 32-byte sectors where the output's alignment allows
+        uint4 o[4];
+        void* dst;
         if (p.y_f32 != nullptr) {
-          float4* dst = reinterpret_cast<float4*>(p.y_f32 + (int64_t)m * p.ldy + n);
+          dst = p.y_f32 + (int64_t)m * p.ldy + n;
 #pragma unroll
-          for (int j = 0; j < 4; ++j) dst[j] = make_float4(v[4 * j], v[4 * j + 1], v[4 * j + 2], v[4 * j + 3]);
+          for (int j = 0; j < 4; ++j)
+            o[j] = make_uint4(__float_as_uint(v[4 * j]), __float_as_uint(v[4 * j + 1]), __float_as_uint(v[4 * j + 2]), __float_as_uint(v[4 * j + 3]));
         } else {
-          uint4* dst = reinterpret_cast<uint4*>(p.y_bf16 + (int64_t)m * p.ldy + n);
-          dst[0] = make_uint4(pack_bf16x2(v[0], v[1]), pack_bf16x2(v[2], v[3]), pack_bf16x2(v[4], v[5]), pack_bf16x2(v[6], v[7]));
-          dst[1] = make_uint4(pack_bf16x2(v[8], v[9]), pack_bf16x2(v[10], v[11]), pack_bf16x2(v[12], v[13]), pack_bf16x2(v[14], v[15]));
+          dst = p.y_bf16 + (int64_t)m * p.ldy + n;
+#pragma unroll
+          for (int j = 0; j < 2; ++j)
+            o[j] = make_uint4(pack_bf16x2(v[8 * j], v[8 * j + 1]), pack_bf16x2(v[8 * j + 2], v[8 * j + 3]),
+                              pack_bf16x2(v[8 * j + 4], v[8 * j + 5]), pack_bf16x2(v[8 * j + 6], v[8 * j + 7]));
+        }
+        if (sectors) {
+          st_global_32B(dst, o[0], o[1]);
+          if (p.y_f32 != nullptr) st_global_32B(reinterpret_cast<uint4*>(dst) + 2, o[2], o[3]);
+        } else {
+          reinterpret_cast<uint4*>(dst)[0] = o[0];
+          reinterpret_cast<uint4*>(dst)[1] = o[1];
+          if (p.y_f32 != nullptr) { reinterpret_cast<uint4*>(dst)[2] = o[2]; reinterpret_cast<uint4*>(dst)[3] = o[3]; }
         }
       }
     }
   }
   tc::tc_fence_before();
   __syncthreads();
-  if (warp == 0) tc::tmem_dealloc(tmem_base, BN < 32 ? 32 : BN);
+  if (warp == 4) tc::tmem_dealloc(tmem_base, BN < 32 ? 32 : BN);
 }
 
 // ---------------------------------------------------------------------------------------------
@@ -644,7 +801,8 @@ struct Affine {                                            // LayerNorm folded i
   const float* cs;
   const float* cb;
   float eps = 0.f;                                         // in_kernel_stats only
-  bool in_kernel_stats = false;                            // the pair kernel forms (rstd, -rstd * mean) itself
+  float2* out = nullptr;                                   // in_kernel_stats, linear_kernel: receives them
+  bool in_kernel_stats = false;                            // the GEMM kernel forms (rstd, -rstd * mean) itself
 };
 struct AllowedStores {                                     // kOutF32LseAllowed
   const uint64_t* bits = nullptr;
@@ -686,20 +844,85 @@ static grace_status_t launch_pair(const CUtensorMap& mx, const CUtensorMap& mw, 
   return GRACE_OK;
 }
 
-template <int BN, int STAGES>
+template <int BN, int STAGES, int SPLIT>
 static grace_status_t launch_linear(const CUtensorMap& mx, const CUtensorMap& mw, const GemmParams& p, cudaStream_t s) {
+  using S = GemmCfg<BN, STAGES, SPLIT>;
   static unsigned long long attr_set_devices = 0;
   DeviceSetup su(&attr_set_devices);
   if (su) {
-    GRACE_CUDA_TRY(cudaFuncSetAttribute(linear_kernel<BN, STAGES>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                        GemmSmem<BN, STAGES>::kTotal));
+    GRACE_CUDA_TRY(cudaFuncSetAttribute(linear_kernel<BN, STAGES, SPLIT>, cudaFuncAttributeMaxDynamicSharedMemorySize, S::kTotal));
     su.done();
   }
-  dim3 grid((p.N + BN - 1) / BN, (p.M + kGemmBM - 1) / kGemmBM);
-  launch_pdl(linear_kernel<BN, STAGES>, grid, dim3(128), GemmSmem<BN, STAGES>::kTotal, s, mx, mw, p);
+  cudaLaunchConfig_t cfg = {};
+  cudaLaunchAttribute attr[2];
+  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  attr[1].id = cudaLaunchAttributeClusterDimension;
+  attr[1].val.clusterDim.x = SPLIT; attr[1].val.clusterDim.y = 1; attr[1].val.clusterDim.z = 1;
+  cfg.gridDim = dim3((p.N + BN - 1) / BN * SPLIT, (p.M + kGemmBM - 1) / kGemmBM);
+  cfg.blockDim = dim3(kGemmThreads); cfg.dynamicSmemBytes = S::kTotal; cfg.stream = s;
+  cfg.attrs = attr; cfg.numAttrs = SPLIT > 1 ? 2 : 1;
+  cudaLaunchKernelEx(&cfg, linear_kernel<BN, STAGES, SPLIT>, mx, mw, p);
   GRACE_LAUNCH_CHECK();
   return GRACE_OK;
 }
+
+// Which kernel runs a problem: the estimate below, in microseconds, of every form that can, and the least of them.
+// linear_kernel: a wave of CTAs takes a fixed part (launch, first loads, epilogue: it grows with the columns a CTA
+// finishes) and a part per k-block of its range of K; CTAs beyond a wave wait for it.  The constants are fits to
+// chains of dependent launches on a B200 (x [M][K] times [N][K], M 1 .. 4096, N 128 .. 8192, K 128 .. 8192; most
+// estimates are within 10 %).  What it gives against the rule before (pair kernel from M = 1024 on, else 32- or 128-wide
+// tiles without a split), LayerNorm included: 512 x 1536 x 512: 10.3 -> 5.8 us, 512 x 2048 x 512: 10.5 -> 6.1,
+// 512 x 512 x 2048: 10.3 -> 5.8, 16 x 512 x 2048: 9.9 -> 4.3, 1024 x 512 x 2048: 13.1 -> 7.1, 1024 x 512 x 512:
+// 7.6 -> 5.0, 2048 x 512 x 2048: 13.1 -> 9.1.
+struct LinearForm { int bn, split, per_sm; float fixed, per_kb; };     // bn = 0: the CTA-pair kernel
+constexpr LinearForm kLinearForms[] = {
+    {32, 1, 1, 2.3f, 0.24f}, {32, 2, 1, 2.7f, 0.24f},                                // whole K range in flight
+    {64, 1, 1, 2.9f, 0.245f}, {64, 2, 1, 3.1f, 0.25f}, {64, 4, 1, 3.0f, 0.28f},
+    {128, 1, 1, 4.0f, 0.255f}, {128, 2, 1, 4.2f, 0.25f}, {128, 4, 1, 4.1f, 0.25f},
+    {64, 1, 2, 4.2f, 0.28f}, {128, 1, 2, 5.0f, 0.46f}};                              // two CTAs per SM, three or four stages
+static grace_status_t run_linear(const LinearForm& f, const CUtensorMap& mx, const CUtensorMap& mw, const GemmParams& p, cudaStream_t s) {
+  switch (f.bn * 16 + f.split * 2 + f.per_sm - 1) {
+    case 32 * 16 + 2: return launch_linear<32, 8, 1>(mx, mw, p, s);
+    case 32 * 16 + 4: return launch_linear<32, 8, 2>(mx, mw, p, s);
+    case 64 * 16 + 2: return launch_linear<64, 8, 1>(mx, mw, p, s);
+    case 64 * 16 + 4: return launch_linear<64, 8, 2>(mx, mw, p, s);
+    case 64 * 16 + 8: return launch_linear<64, 8, 4>(mx, mw, p, s);
+    case 128 * 16 + 2: return launch_linear<128, 6, 1>(mx, mw, p, s);
+    case 128 * 16 + 4: return launch_linear<128, 4, 2>(mx, mw, p, s);
+    case 128 * 16 + 8: return launch_linear<128, 4, 4>(mx, mw, p, s);
+    case 64 * 16 + 3: return launch_linear<64, 4, 1>(mx, mw, p, s);
+    case 128 * 16 + 3: return launch_linear<128, 3, 1>(mx, mw, p, s);
+  }
+  return GRACE_UNSUPPORTED_SHAPE;
+}
+
+// stats_launch: the pair kernel would need the statistics kernel in front.  whole_k: no split of K, so that the sums are
+// those of the pair kernel bit for bit (fp32 products: grace_linear_f32_lse promises those of grace_linear).
+static LinearForm linear_form(int M, int N, int K, bool pair_possible, bool stats_launch, bool whole_k) {
+  const int64_t tiles_m = (M + kGemmBM - 1) / kGemmBM;
+  const int kb = K / kGemmBK;
+  LinearForm best = {0, 0, 0, 0.f, 0.f};
+  float least = 3.4e38f;
+  if (pair_possible) {
+    const int64_t waves = ((int64_t)((M + 255) / 256) * ((N + 255) / 256) + 73) / 74;
+    least = 2.7f + (float)waves * (1.0f + 0.33f * (float)kb) + (stats_launch ? 3.2f + 3.6e-7f * (float)M * (float)K : 0.f);
+  }
+  for (const LinearForm& f : kLinearForms) {
+    if (f.split > kb || (whole_k && f.split > 1)) continue;
+    const int64_t ctas = tiles_m * ((N + f.bn - 1) / f.bn) * f.split;
+    const int wave = f.split == 1 ? 148 * f.per_sm : (f.split == 2 ? 144 : 132);       // clusters lie within a GPC
+    const float t = (float)((ctas + wave - 1) / wave) * (f.fixed + f.per_kb * (float)((kb + f.split - 1) / f.split));
+    if (t < least) { least = t; best = f; }
+  }
+  return best;
+}
+// The pair kernel takes whole 256 x 256 tiles and adds into the residual stream by TMA only in place.
+static bool linear_pair_possible(int M, int N, bool residual_elsewhere) { return M >= 1024 && N >= 256 && !residual_elsewhere; }
+
+static bool linear_whole_k(int M, int N, bool plain_f32) { return plain_f32 && M >= 1024 && N >= 256; }
+// Centred rows and at most two 256-wide tiles: the pair kernel forms the LayerNorm statistics itself.
+static bool linear_narrow_centred(int M, int N, const float* col_sum) { return M >= 1024 && N >= 256 && N <= 512 && col_sum == nullptr; }
 
 }  // namespace grace
 
@@ -722,7 +945,11 @@ static grace_status_t linear_impl(const uint16_t* x, int64_t ldx, const uint16_t
     return GRACE_UNSUPPORTED_SHAPE;
   if (allow_bits != nullptr && (lse_part == nullptr || (reinterpret_cast<uintptr_t>(allow_bits) & 15)))
     return GRACE_UNSUPPORTED_SHAPE;                          // allowed-only stores exist in the large-problem kernel only
-  if (M >= 1024 && N >= 256 && (residual == nullptr || aliased)) {
+  LinearForm form = {0, 0, 0, 0.f, 0.f};
+  if (lse_part == nullptr)
+    form = linear_form(M, N, K, linear_pair_possible(M, N, residual != nullptr && !aliased),
+                       aff.row != nullptr && !linear_narrow_centred(M, N, aff.cs), linear_whole_k(M, N, y_f32 != nullptr && residual == nullptr));
+  if (form.bn == 0) {
     // large GEMM: persistent CTA-pair kernel, TMA-store epilogue (add-reduction when y is the residual stream)
     CUtensorMap mx, mw, my;
     const uint64_t dx[2] = {(uint64_t)K, (uint64_t)M}, sx[1] = {(uint64_t)ldx};
@@ -753,9 +980,6 @@ static grace_status_t linear_impl(const uint16_t* x, int64_t ldx, const uint16_t
     return launch_pair<kOutF32>(mx, mw, my, M, N, K, relu, s, nullptr, aff);
   }
   CUtensorMap mx, mw;
-  // a grid that leaves most SMs idle is latency-bound: narrower tiles (more CTAs) and the whole K in flight
-  const bool latency_form = (int64_t)((M + kGemmBM - 1) / kGemmBM) * ((N + 127) / 128) < 74;
-  const int BN = (N >= 128 && !latency_form) ? 128 : (latency_form ? 32 : 64);
   {
     const uint64_t dims[2] = {(uint64_t)K, (uint64_t)M}, str[1] = {(uint64_t)ldx};
     const uint32_t box[2] = {(uint32_t)kGemmBK, (uint32_t)kGemmBM};
@@ -763,15 +987,14 @@ static grace_status_t linear_impl(const uint16_t* x, int64_t ldx, const uint16_t
   }
   {
     const uint64_t dims[2] = {(uint64_t)K, (uint64_t)N}, str[1] = {(uint64_t)ldw};
-    const uint32_t box[2] = {(uint32_t)kGemmBK, (uint32_t)BN};
+    const uint32_t box[2] = {(uint32_t)kGemmBK, (uint32_t)form.bn};
     if (!tc::make_tmap_bf16(&mw, w, 2, dims, str, box)) return GRACE_CUDA_ERROR;
   }
   GemmParams p;
   p.y_bf16 = y_bf16; p.y_f32 = y_f32; p.residual = residual; p.residual_bf16 = add_into_bf16 ? y_bf16 : nullptr;
-  p.aff_row = aff.row; p.aff_cs = aff.cs; p.aff_cb = aff.cb;
+  p.aff_row = aff.in_kernel_stats ? nullptr : aff.row; p.aff_cs = aff.cs; p.aff_cb = aff.cb; p.ln_eps = aff.eps; p.aff_out = aff.out;
   p.ldy = ldy; p.M = M; p.N = N; p.K = K; p.relu = relu;
-  if (BN == 128) return launch_linear<128, 3>(mx, mw, p, s);
-  return latency_form ? launch_linear<32, 8>(mx, mw, p, s) : launch_linear<64, 3>(mx, mw, p, s);
+  return run_linear(form, mx, mw, p, s);
 }
 
 extern "C" grace_status_t grace_linear(const uint16_t* x, int64_t ldx, const uint16_t* w, int64_t ldw,
@@ -809,18 +1032,23 @@ extern "C" grace_status_t grace_linear_layer_norm(const uint16_t* x, int64_t ldx
   if (lse_part != nullptr && (reinterpret_cast<uintptr_t>(lse_part) & 7)) return GRACE_INVALID_ARG;
   if (M <= 0 || N <= 0 || K <= 0 || ldx != K) return GRACE_INVALID_ARG;     // the LayerNorm is over the whole row of x
   grace::Affine aff = {reinterpret_cast<const float2*>(row_affine), col_sum, col_bias};
-  // The statistics come out of the GEMM's own operand tiles where the CTA-pair kernel runs, the rows are centred
-  // (no col_sum) and the output is at most two tiles wide; otherwise the statistics kernel runs first, into
-  // row_affine.  Every n-tile forms the statistics of its rows again, and the shared-memory reads that takes
-  // (16 KB per k-block on top of the 32 KB the tensor cores read and the 32 KB TMA writes) slow the main loop by a
-  // fifth: measured at 65536 x 512 -> N, one kernel against two: N = 512: 36 us against 43; N = 1536: 99 against
-  // 95; N = 2048: 130 against 122.
-  const bool pair_kernel = (M >= 1024 && N >= 256);
+  // The statistics come out of the GEMM's own operand tiles in linear_kernel, and where the CTA-pair kernel runs if
+  // the rows are centred (no col_sum) and the output is at most two tiles wide; otherwise the statistics kernel
+  // runs first, into row_affine.  In the pair kernel every n-tile forms the statistics of its rows again, and the
+  // shared-memory reads that takes (16 KB per k-block on top of the 32 KB the tensor cores read and the 32 KB TMA
+  // writes) slow the main loop by a fifth: measured at 65536 x 512 -> N, one kernel against two: N = 512: 36 us
+  // against 43; N = 1536: 99 against 95; N = 2048: 130 against 122.
+  const bool narrow_centred = lse_part == nullptr && grace::linear_narrow_centred(M, N, col_sum);
+  const bool pair_kernel = lse_part != nullptr ||
+                           grace::linear_form(M, N, K, grace::linear_pair_possible(M, N, false), !narrow_centred,
+                                              grace::linear_whole_k(M, N, y_f32 != nullptr)).bn == 0;
   // (not for a logits GEMM with log-sum-exp partials: grace_linear_logits_allowed takes its statistics from the
   // statistics kernel, and the two forms of a decode step are to agree bit for bit)
-  if (pair_kernel && col_sum == nullptr && N <= 512 && lse_part == nullptr) {
+  if (!narrow_centred && K > 2048) return GRACE_UNSUPPORTED_SHAPE;           // what grace_row_stats_bf16 takes
+  if (!pair_kernel || narrow_centred) {
     aff.eps = eps;
     aff.in_kernel_stats = true;
+    if (!narrow_centred) aff.out = reinterpret_cast<float2*>(row_affine);
   } else {
     const grace_status_t st = grace_row_stats_bf16(x, M, K, eps, row_affine, stream);
     if (st != GRACE_OK) return st;
