@@ -3,17 +3,20 @@
 //
 // The candidates are read from HBM once.  Three launches:
 //   1. sample   : per request, 4096 sample points x 8 consecutive floats (one 32-byte sector per
-//                 point, one point per N/4096-element stratum).  The r-th largest sample, with r
+//                 point, one point per 4096th of the candidates).  The r-th largest sample, with r
 //                 a few standard deviations above K * (samples / N), becomes a threshold that
 //                 with high probability has between K and `kCap` candidates above it.
 //   2. collect  : the one full pass.  Every candidate above the threshold is appended to the
 //                 request's list (warp-aggregated atomics; hits are a fraction of a percent).
-//   3. finalize : requests whose list came out short or overflowed (and every request when N is
-//                 small) are first redone by a three-level radix select that resolves ties by
-//                 index (one CTA per request, exact for any input).  Then: bitonic sort of the list on (key, index), write the first K; if the threshold
-//                 was -inf and fewer than K finite candidates exist, the remaining slots are the
-//                 lowest-index -inf candidates.
+//   3. finalize : a counting sort (bitonic where keys are clustered) of the list on (key, index), writes the
+//                 first K; if the threshold was -inf and fewer than K finite candidates exist, the remaining
+//                 slots are the lowest-index -inf candidates.  Requests whose list came out short or
+//                 overflowed are first redone by a three-level radix select that resolves ties by index (one
+//                 CTA per request, exact for any input).
+// Small requests (N <= kDirectMax) are finalize alone: it takes the finite candidates straight into shared memory,
+// or selects exactly if they are more than fit.  In a decode step finalize also updates the beam state.
 // The result is exact whatever the threshold; the threshold only decides which path runs.
+#include "beam_state.cuh"
 #include "common.cuh"
 
 namespace grace {
@@ -24,6 +27,7 @@ constexpr int kSamplePoints = 4096;
 constexpr int kSampleSize = kSamplePoints * 8;
 constexpr int kTopkThreads = 1024;
 constexpr int kMaxK = 4096;              // largest K supported
+constexpr int kDirectMax = 4 * kCap;     // finalize alone up to here
 constexpr int kBucketMax = 128;          // finalize: largest bucket the counting sort ranks by comparison
 
 struct TopkHeader {                      // lives in the workspace, one per request
@@ -149,15 +153,15 @@ topk_sample_kernel(const CandSrc src, uint32_t rank, TopkHeader* hdr) {
   __shared__ uint32_t red[64];
   const int b = blockIdx.x;
   const int64_t N = src.N;
-  const uint32_t stratum = (uint32_t)(N / kSamplePoints) & ~7u;     // multiple of 8 elements (N < 2^31)
-  const uint32_t slots = stratum >> 3;
+  const uint64_t n8 = (uint64_t)(N >> 3);                            // groups of 8 candidates, at least kSamplePoints
   float4 v[2 * (kSamplePoints / kTopkThreads)];
 #pragma unroll
   for (int q = 0; q < kSamplePoints / kTopkThreads; ++q) {
     const uint32_t p = q * kTopkThreads + threadIdx.x;
     uint32_t h = p * 0x9e3779b1u + (uint32_t)b * 0x85ebca77u;      // where in its stratum point p of request b lies
     h ^= h >> 16; h *= 0x85ebca6bu; h ^= h >> 13; h *= 0xc2b2ae35u; h ^= h >> 16;
-    const uint32_t at4 = (p * stratum + __umulhi(h, slots) * 8u) >> 2;
+    const uint32_t lo = (uint32_t)(p * n8 / kSamplePoints), hi = (uint32_t)((p + 1) * n8 / kSamplePoints);
+    const int64_t at4 = 2ll * (lo + __umulhi(h, hi - lo));
     v[2 * q] = src.load4(b, at4, false);
     v[2 * q + 1] = src.load4(b, at4 + 1, false);
   }
@@ -216,13 +220,6 @@ topk_sample_kernel(const CandSrc src, uint32_t rank, TopkHeader* hdr) {
     hdr[b].need_exact = 0;
     hdr[b].t_excl = (prefix <= kKeyNegInf) ? kKeyNegInf : prefix - 1;
   }
-}
-
-__global__ void topk_reset_kernel(TopkHeader* hdr, int B) {
-  pdl_wait();
-  pdl_trigger();
-  const int b = blockIdx.x * blockDim.x + threadIdx.x;
-  if (b < B) { hdr[b].count = 0; hdr[b].t_excl = 0; hdr[b].need_exact = 1; }
 }
 
 // ---- 2. collect ------------------------------------------------------------------------------
@@ -459,16 +456,23 @@ __device__ void topk_exact_select(const CandSrc& src, int K, uint2* lists, int b
     __syncthreads();
     const int hi_shift = shifts[level] + bits[level];
     uint32_t n_ninf = 0;            // -inf dominates masked rows: count it in a register
-    for (int64_t i = threadIdx.x; i < n4; i += kTopkThreads) {
-      const float4 v = src.load4(b, i, false);
-      const float x[4] = {v.x, v.y, v.z, v.w};
+    constexpr int U = 4;                                    // loads in flight: one CTA reads the whole request
+    for (int64_t i0 = threadIdx.x; i0 < n4; i0 += U * kTopkThreads) {
+      float4 v[U];
 #pragma unroll
-      for (int j = 0; j < 4; ++j) {
-        if (level == 0 && x[j] != x[j]) saw_nan = true;
-        const uint32_t u = ordered_key(x[j]);
-        if (u == kKeyNegInf) { ++n_ninf; continue; }
-        const bool match = (level == 0) || ((u >> hi_shift) == prefix);
-        if (match) atomicAdd(&hist[(u >> shifts[level]) & (nb - 1)], 1u);
+      for (int e = 0; e < U; ++e) if (i0 + e * kTopkThreads < n4) v[e] = src.load4(b, i0 + e * kTopkThreads, false);
+#pragma unroll
+      for (int e = 0; e < U; ++e) {
+        if (i0 + e * kTopkThreads >= n4) break;
+        const float x[4] = {v[e].x, v[e].y, v[e].z, v[e].w};
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+          if (level == 0 && x[j] != x[j]) saw_nan = true;
+          const uint32_t u = ordered_key(x[j]);
+          if (u == kKeyNegInf) { ++n_ninf; continue; }
+          const bool match = (level == 0) || ((u >> hi_shift) == prefix);
+          if (match) atomicAdd(&hist[(u >> shifts[level]) & (nb - 1)], 1u);
+        }
       }
     }
     if (n_ninf != 0 && ((level == 0) || ((kKeyNegInf >> hi_shift) == prefix)))
@@ -586,10 +590,14 @@ __device__ void block_bitonic_sort_desc(unsigned long long* keys) {
   __syncthreads();
 }
 
+// What finalize starts from: the list that the collecting pass left, the candidates themselves (if they fit: small
+// requests), or the exact selection.
+enum { kFinalizeList = 0, kFinalizeExact = 1, kFinalizeDirect = 2 };
+
 __global__ void __launch_bounds__(kTopkThreads)
 topk_finalize_kernel(const CandSrc src, int K, int K_out, int V, TopkHeader* hdr,
-                     uint2* lists, int force_exact, float* out_score, int32_t* out_flat, int32_t* out_parent,
-                     int32_t* out_token, int32_t* d_status) {
+                     uint2* lists, int mode, float* out_score, int32_t* out_flat, int32_t* out_parent,
+                     int32_t* out_token, const BeamUpdate upd, int32_t* d_status) {
   // K = min(requested, N) entries are selected; rows of the outputs are K_out = requested wide.
   pdl_wait();
   pdl_trigger();
@@ -599,32 +607,87 @@ topk_finalize_kernel(const CandSrc src, int K, int K_out, int V, TopkHeader* hdr
   __shared__ uint32_t result[2];
   __shared__ uint32_t red[64];
   const int b = blockIdx.x;
-  uint32_t c = hdr[b].count;
-  // Exact multi-pass selection when the sampled threshold did not deliver (list short although the
-  // threshold was not -inf, or list overflow) and for shapes that skip sampling altogether.
-  const bool need_exact = force_exact || c > (uint32_t)kCap || (c < (uint32_t)K && hdr[b].t_excl != kKeyNegInf);
-  if (need_exact) {
-    if (!force_exact && threadIdx.x == 0) flag_status(d_status, GRACE_DEV_TOPK_EXACT_PATH);
-    topk_exact_select(src, K, lists, b, reinterpret_cast<uint32_t*>(sort_keys), scratch, result, d_status);
-    __syncthreads();
-    c = (uint32_t)K;
-  }
-  c = min(c, (uint32_t)kCap);
-  const uint2* list = lists + (int64_t)b * kCap;
   unsigned long long* all_keys = sort_keys;                 // c composite keys (value key, ~index)
   unsigned long long* top_keys = sort_keys + kCap;          // the K winners (fast path: plus one bucket's overhang)
   uint32_t* hist = reinterpret_cast<uint32_t*>(top_keys + kMaxK + kBucketMax);
   uint32_t* offs = hist + 4096;
   const int64_t N = src.N;
-  const uint32_t n_out = min(c, (uint32_t)K);
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   uint32_t kmin = 0xffffffffu, kmax = 0u;
-  for (uint32_t i = threadIdx.x; i < c; i += kTopkThreads) {
-    const uint2 e = list[i];
-    all_keys[i] = ((unsigned long long)e.x << 32) | (unsigned long long)(0xffffffffu - e.y);
-    kmin = min(kmin, e.x);
-    kmax = max(kmax, e.x);
+  uint32_t c = 0;
+  bool need_exact = mode == kFinalizeExact, from_list = true;
+  if (mode == kFinalizeDirect) {
+    // every finite candidate straight into shared memory, in any order (the keys carry the index)
+    if (threadIdx.x == 0) result[0] = 0;
+    __syncthreads();
+    bool saw_nan = false;
+    const int n4 = (int)(N >> 2);
+    constexpr int U = 4;
+    for (int i0 = 0; i0 < n4; i0 += U * kTopkThreads) {
+      float4 v[U];
+#pragma unroll
+      for (int e = 0; e < U; ++e) {
+        const int i = i0 + e * kTopkThreads + (int)threadIdx.x;
+        v[e] = i < n4 ? src.load4(b, i, false) : make_float4(-INFINITY, -INFINITY, -INFINITY, -INFINITY);
+      }
+#pragma unroll
+      for (int e = 0; e < U; ++e) {
+        const int i = i0 + e * kTopkThreads + (int)threadIdx.x;
+        const float x[4] = {v[e].x, v[e].y, v[e].z, v[e].w};
+        uint32_t key[4];
+        int n = 0;
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+          if (x[j] != x[j]) saw_nan = true;
+          key[j] = ordered_key(x[j]);
+          n += key[j] > kKeyNegInf;
+        }
+        if (!__any_sync(kFullMask, n != 0)) continue;
+        const uint32_t incl = warp_incl_scan((uint32_t)n);
+        uint32_t at = 0;
+        if (lane == 31) at = atomicAdd(&result[0], incl);
+        at = __shfl_sync(kFullMask, at, 31) + incl - (uint32_t)n;
+#pragma unroll
+        for (int j = 0; j < 4; ++j)
+          if (key[j] > kKeyNegInf) {
+            if (at < (uint32_t)kCap)
+              all_keys[at] = ((unsigned long long)key[j] << 32) | (unsigned long long)(0xffffffffu - (uint32_t)(4 * i + j));
+            kmin = min(kmin, key[j]);
+            kmax = max(kmax, key[j]);
+            ++at;
+          }
+      }
+    }
+    if (saw_nan) flag_status(d_status, GRACE_DEV_NAN);
+    __syncthreads();
+    c = result[0];
+    __syncthreads();                                        // (the scratch is reused below)
+    need_exact = c > (uint32_t)kCap;
+    from_list = need_exact;
+  } else if (mode == kFinalizeList) {
+    // Exact multi-pass selection when the sampled threshold did not deliver (list short although the
+    // threshold was not -inf, or list overflow).
+    c = hdr[b].count;
+    need_exact = c > (uint32_t)kCap || (c < (uint32_t)K && hdr[b].t_excl != kKeyNegInf);
+    if (need_exact && threadIdx.x == 0) flag_status(d_status, GRACE_DEV_TOPK_EXACT_PATH);
   }
+  if (need_exact) {
+    topk_exact_select(src, K, lists, b, reinterpret_cast<uint32_t*>(sort_keys), scratch, result, d_status);
+    __syncthreads();
+    c = (uint32_t)K;
+    kmin = 0xffffffffu;
+    kmax = 0u;
+  }
+  c = min(c, (uint32_t)kCap);
+  const uint2* list = lists + (int64_t)b * kCap;
+  const uint32_t n_out = min(c, (uint32_t)K);
+  if (from_list)
+    for (uint32_t i = threadIdx.x; i < c; i += kTopkThreads) {
+      const uint2 e = list[i];
+      all_keys[i] = ((unsigned long long)e.x << 32) | (unsigned long long)(0xffffffffu - e.y);
+      kmin = min(kmin, e.x);
+      kmax = max(kmax, e.x);
+    }
   for (int i = threadIdx.x; i < 4096; i += kTopkThreads) hist[i] = 0;
 #pragma unroll
   for (int d = 16; d >= 1; d >>= 1) {
@@ -799,16 +862,24 @@ topk_finalize_kernel(const CandSrc src, int K, int K_out, int V, TopkHeader* hdr
     if (out_parent) out_parent[o] = 0;
     if (out_token) out_token[o] = 0;
   }
+  if (upd.new_node != nullptr) {                            // the new beam's nodes and keys, from this CTA's own outputs
+    __syncthreads();
+    for (int i = (int)threadIdx.x; i < K_out; i += kTopkThreads) {
+      const int64_t o = (int64_t)b * K_out + i;
+      beam_update_one(upd, o, b, out_parent[o], out_token[o], out_score[o], d_status);
+    }
+  }
 }
 
 // Sampling plan: rank r of the sample whose value is the threshold, or 0 if sampling is not
 // worthwhile / not safe for this shape (then the exact path handles every request).
 static uint32_t sample_rank(int64_t N, int K) {
-  if (N < (int64_t)kSampleSize * 8 || (N & 7)) return 0;
+  if (N <= (int64_t)kDirectMax || (N & 7)) return 0;
   const double frac = (double)kSampleSize / (double)N;
   const double expect = K * frac;
   const double r = ceil(expect + 4.0 * sqrt(expect) + 8.0);
-  if (r / frac > 0.75 * kCap || r > kSampleSize / 4) return 0;
+  // (a thread of the sampling kernel keeps its two largest of 32 keys: far below 1024, few of the r are lost)
+  if (r / frac > 0.75 * kCap || r > 700) return 0;
   return (uint32_t)r;
 }
 
@@ -824,7 +895,7 @@ namespace grace {
 // Shared by the public entry point and the variant that owns its scratch.
 grace_status_t launch_beam_topk(const CandSrc& src_in, int B, int K, int V, float* out_score,
                                 int32_t* out_flat, int32_t* out_parent, int32_t* out_token,
-                                void* ws, int32_t* d_status, cudaStream_t s) {
+                                void* ws, const BeamUpdate& upd, int32_t* d_status, cudaStream_t s) {
   CandSrc src = src_in;
   const int64_t N = src.N;
   TopkHeader* hdr = reinterpret_cast<TopkHeader*>(ws);
@@ -848,7 +919,7 @@ grace_status_t launch_beam_topk(const CandSrc& src_in, int B, int K, int V, floa
     su.done();
   }
   const int collect_grid = collect_grid_of[su.dev];
-  int force_exact = 1;
+  int mode = N <= (int64_t)kDirectMax ? kFinalizeDirect : kFinalizeExact;
   if (rank != 0) {
     launch_pdl(topk_sample_kernel, dim3(B), dim3(kTopkThreads), 0, s, src, rank, hdr);
     GRACE_LAUNCH_CHECK();
@@ -871,37 +942,33 @@ grace_status_t launch_beam_topk(const CandSrc& src_in, int B, int K, int V, floa
       launch_pdl(topk_collect_kernel, dim3(grid), dim3(kCollectThreads), 0, s, src, hdr, lists, d_status);
       GRACE_LAUNCH_CHECK();
     }
-    force_exact = 0;
-  } else {
-    launch_pdl(topk_reset_kernel, dim3((B + 255) / 256), dim3(256), 0, s, hdr, B);
-    GRACE_LAUNCH_CHECK();
+    mode = kFinalizeList;
   }
-  launch_pdl(topk_finalize_kernel, dim3(B), dim3(kTopkThreads), final_smem, s, src, K, K_out, V, hdr, lists, force_exact, out_score, out_flat,
-                                                          out_parent, out_token, d_status);
+  launch_pdl(topk_finalize_kernel, dim3(B), dim3(kTopkThreads), final_smem, s, src, K, K_out, V, hdr, lists, mode, out_score, out_flat,
+             out_parent, out_token, upd, d_status);
   GRACE_LAUNCH_CHECK();
   return GRACE_OK;
 }
 }  // namespace grace
 
-extern "C" grace_status_t grace_beam_topk(const float* cand, int B, int64_t N, int K, int V,
-                                          float* out_score, int32_t* out_flat, int32_t* out_parent,
-                                          int32_t* out_token, void* ws, size_t ws_bytes,
-                                          int32_t* d_status, void* stream) {
+namespace grace {
+// The public entry points without an update; grace_decode_step passes the one that follows its selection.
+grace_status_t beam_topk_update(const float* cand, int B, int64_t N, int K, int V, float* out_score, int32_t* out_flat,
+                                int32_t* out_parent, int32_t* out_token, void* ws, size_t ws_bytes,
+                                const BeamUpdate& upd, int32_t* d_status, void* stream) {
   if (!cand || !out_score || !ws) return GRACE_INVALID_ARG;
   if (B <= 0 || N <= 0 || N >= (1ll << 31) || K < 1 || V <= 0) return GRACE_INVALID_ARG;
   if (K > 4096 || (N & 3)) return GRACE_UNSUPPORTED_SHAPE;
   if (!grace_aligned16(cand) || (reinterpret_cast<uintptr_t>(ws) & 255u)) return GRACE_INVALID_ARG;
   if (ws_bytes < grace_beam_topk_workspace_bytes(B, N, K)) return GRACE_WORKSPACE_TOO_SMALL;
-  grace::CandSrc src = {cand, nullptr, nullptr, nullptr, N, V, -1};
-  return grace::launch_beam_topk(src, B, K, V, out_score, out_flat, out_parent, out_token, ws,
-                                 d_status, (cudaStream_t)stream);
+  CandSrc src = {cand, nullptr, nullptr, nullptr, N, V, -1};
+  return launch_beam_topk(src, B, K, V, out_score, out_flat, out_parent, out_token, ws, upd, d_status, (cudaStream_t)stream);
 }
 
-extern "C" grace_status_t grace_beam_topk_masked(const float* logits, const uint64_t* allow_bits,
-                                                 const float* row_score, const float* row_lse, int B, int M, int V,
-                                                 int K, float* out_score, int32_t* out_flat, int32_t* out_parent,
-                                                 int32_t* out_token, void* ws, size_t ws_bytes, int32_t* d_status,
-                                                 void* stream) {
+grace_status_t beam_topk_masked_update(const float* logits, const uint64_t* allow_bits, const float* row_score,
+                                       const float* row_lse, int B, int M, int V, int K, float* out_score,
+                                       int32_t* out_flat, int32_t* out_parent, int32_t* out_token, void* ws,
+                                       size_t ws_bytes, const BeamUpdate& upd, int32_t* d_status, void* stream) {
   if (!logits || !allow_bits || !row_score || !row_lse || !out_score || !ws) return GRACE_INVALID_ARG;
   if (B <= 0 || M <= 0 || V <= 0 || (V & 63) || K < 1) return GRACE_INVALID_ARG;
   const int64_t N = (int64_t)M * V;
@@ -912,12 +979,27 @@ extern "C" grace_status_t grace_beam_topk_masked(const float* logits, const uint
   int log2_V = -1;
   if ((V & (V - 1)) == 0)
     for (log2_V = 0; (1 << log2_V) < V; ++log2_V) {}
-  grace::CandSrc src = {logits, allow_bits, row_score, row_lse, N, V, log2_V};
-  return grace::launch_beam_topk(src, B, K, V, out_score, out_flat, out_parent, out_token, ws, d_status,
-                                 (cudaStream_t)stream);
+  CandSrc src = {logits, allow_bits, row_score, row_lse, N, V, log2_V};
+  return launch_beam_topk(src, B, K, V, out_score, out_flat, out_parent, out_token, ws, upd, d_status, (cudaStream_t)stream);
+}
+}  // namespace grace
+
+extern "C" grace_status_t grace_beam_topk(const float* cand, int B, int64_t N, int K, int V,
+                                          float* out_score, int32_t* out_flat, int32_t* out_parent,
+                                          int32_t* out_token, void* ws, size_t ws_bytes,
+                                          int32_t* d_status, void* stream) {
+  return grace::beam_topk_update(cand, B, N, K, V, out_score, out_flat, out_parent, out_token, ws, ws_bytes,
+                                 grace::BeamUpdate{}, d_status, stream);
 }
 
-
+extern "C" grace_status_t grace_beam_topk_masked(const float* logits, const uint64_t* allow_bits,
+                                                 const float* row_score, const float* row_lse, int B, int M, int V,
+                                                 int K, float* out_score, int32_t* out_flat, int32_t* out_parent,
+                                                 int32_t* out_token, void* ws, size_t ws_bytes, int32_t* d_status,
+                                                 void* stream) {
+  return grace::beam_topk_masked_update(logits, allow_bits, row_score, row_lse, B, M, V, K, out_score, out_flat, out_parent,
+                                        out_token, ws, ws_bytes, grace::BeamUpdate{}, d_status, stream);
+}
 
 // ---------------------------------------------------------------------------------------------
 // grace_beam_topk_static: the same selection with the scratch memory owned by the library.
@@ -971,6 +1053,6 @@ extern "C" grace_status_t grace_beam_topk_static(const float* cand, int B, int64
   // The kernels (re)initialise every header word they read, so the previous call's contents do not
   // matter; nothing here has to start at zero.
   grace::CandSrc src = {cand, nullptr, nullptr, nullptr, N, V, -1};
-  return grace::launch_beam_topk(src, B, K, V, out_score, out_flat, out_parent, out_token, scratch, d_status,
+  return grace::launch_beam_topk(src, B, K, V, out_score, out_flat, out_parent, out_token, scratch, grace::BeamUpdate{}, d_status,
                                  (cudaStream_t)stream);
 }

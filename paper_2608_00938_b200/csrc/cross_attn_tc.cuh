@@ -565,6 +565,7 @@ cross_attn_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_con
         l_tot += half_sum[(half ^ 1) * 128 + row];
       }
       const float2 ml = make_float2(have ? pend_m : -INFINITY, have ? l_tot : 0.f);
+      __syncwarp();
       asm volatile("barrier.cluster.wait.aligned;" ::: "memory");        // the other CTAs have started
       // A slice of kSlice columns goes to its owner (16 at a time; the two threads of a row take every second piece)
       auto read_o = [&](int col, uint32_t (&o)[16]) {

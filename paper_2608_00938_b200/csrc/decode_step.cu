@@ -2,6 +2,7 @@
 // current beam rows, log-probabilities, CD + GTM mask with score add, beam top-k, state update.
 // Host-side sequencing only; every stage is one of the library's own kernels on the caller's
 // stream, with no allocation and no synchronisation, so the loop can be enqueued back to back.
+#include "beam_state.cuh"
 #include "common.cuh"
 
 extern "C" grace_status_t grace_decoder_validate(const grace_decoder_t* d) {
@@ -61,6 +62,16 @@ extern "C" grace_status_t grace_decode_begin(const grace_decoder_t* d, void* str
   GRACE_LAUNCH_CHECK();
   return GRACE_OK;
 }
+
+namespace grace {                                           // beam_topk.cu: a selection that ends with the state update
+grace_status_t beam_topk_update(const float* cand, int B, int64_t N, int K, int V, float* out_score, int32_t* out_flat,
+                                int32_t* out_parent, int32_t* out_token, void* ws, size_t ws_bytes,
+                                const BeamUpdate& upd, int32_t* d_status, void* stream);
+grace_status_t beam_topk_masked_update(const float* logits, const uint64_t* allow_bits, const float* row_score,
+                                       const float* row_lse, int B, int M, int V, int K, float* out_score,
+                                       int32_t* out_flat, int32_t* out_parent, int32_t* out_token, void* ws,
+                                       size_t ws_bytes, const BeamUpdate& upd, int32_t* d_status, void* stream);
+}  // namespace grace
 
 #define GRACE_TRY(expr)                         \
   do {                                          \
@@ -131,6 +142,8 @@ extern "C" grace_status_t grace_decode_step(const grace_decoder_t* d, int t, voi
   const int n_parts = d->V / 256;
   const bool parts = d->lse_part != nullptr && d->row_lse != nullptr && R >= 1024 && (d->V % 256) == 0 && n_parts <= 32;
   int32_t* parent_out = d->parents + (int64_t)(t + 1) * d->R_max;
+  const grace::BeamUpdate update = {d->node[cur], d->key[cur], d->trie.child_bits, d->trie.child_base, d->node[nxt],
+                                    d->key[nxt], d->trie.num_internal, M, d->V, t};
   if (parts && d->logits_allowed_only && d->allow_bits != nullptr && t >= d->masked_from_step) {
     // The constraint first (it needs the beam state only), then a logits GEMM that stores only the allowed logits
     // and the rows' log-sum-exp partials, their merge, and the selection through the allow bits: neither the
@@ -146,10 +159,9 @@ extern "C" grace_status_t grace_decode_step(const grace_decoder_t* d, int t, voi
                                             d->V, d->lse_part, R, d->V, D, stream));
     }
     GRACE_TRY(grace_row_lse_from_parts(d->lse_part, n_parts, d->node[cur], &d->trie, d->row_lse, R, stream));
-    GRACE_TRY(grace_beam_topk_masked(d->logp, d->allow_bits, d->score[cur], d->row_lse, B, M, d->V, K, d->score[nxt],
-                                     d->out_flat, parent_out, d->token[nxt], d->topk_ws, d->topk_ws_bytes, st, stream));
-    GRACE_TRY(grace_beam_update(parent_out, d->token[nxt], d->score[nxt], d->node[cur], d->key[cur], &d->trie,
-                                d->node[nxt], d->key[nxt], B, K, M, t, st, stream));
+    GRACE_TRY(grace::beam_topk_masked_update(d->logp, d->allow_bits, d->score[cur], d->row_lse, B, M, d->V, K, d->score[nxt],
+                                             d->out_flat, parent_out, d->token[nxt], d->topk_ws, d->topk_ws_bytes, update,
+                                             st, stream));
     return GRACE_OK;
   }
   GRACE_TRY(ln_linear(d->lnf_g, d->lnf_b, d->w_out, d->cs_out, d->cb_out, nullptr, d->logp, d->V, d->V, 0,
@@ -161,10 +173,9 @@ extern "C" grace_status_t grace_decode_step(const grace_decoder_t* d, int t, voi
     GRACE_TRY(grace_gtm_mask_logits_parts(d->logp, d->row_lse, d->score[cur], d->node[cur], d->key[cur], &d->trie,
                                           &d->matcher, nullptr, d->allow_bits, B, M, d->V, t,
                                           parts ? d->lse_part : nullptr, n_parts, st, stream));
-    GRACE_TRY(grace_beam_topk_masked(d->logp, d->allow_bits, d->score[cur], d->row_lse, B, M, d->V, K, d->score[nxt],
-                                     d->out_flat, parent_out, d->token[nxt], d->topk_ws, d->topk_ws_bytes, st, stream));
-    GRACE_TRY(grace_beam_update(parent_out, d->token[nxt], d->score[nxt], d->node[cur], d->key[cur], &d->trie,
-                                d->node[nxt], d->key[nxt], B, K, M, t, st, stream));
+    GRACE_TRY(grace::beam_topk_masked_update(d->logp, d->allow_bits, d->score[cur], d->row_lse, B, M, d->V, K, d->score[nxt],
+                                             d->out_flat, parent_out, d->token[nxt], d->topk_ws, d->topk_ws_bytes, update,
+                                             st, stream));
     return GRACE_OK;
   }
   if (d->row_lse != nullptr) {
@@ -177,10 +188,8 @@ extern "C" grace_status_t grace_decode_step(const grace_decoder_t* d, int t, voi
                              nullptr, B, M, d->V, t, st, stream));
   }
   // parents of step t+1 live in slab t+1; tokens become the next step's input tokens
-  GRACE_TRY(grace_beam_topk(d->cand, B, (int64_t)M * d->V, K, d->V, d->score[nxt], d->out_flat, parent_out,
-                            d->token[nxt], d->topk_ws, d->topk_ws_bytes, st, stream));
-  GRACE_TRY(grace_beam_update(parent_out, d->token[nxt], d->score[nxt], d->node[cur], d->key[cur], &d->trie,
-                              d->node[nxt], d->key[nxt], B, K, M, t, st, stream));
+  GRACE_TRY(grace::beam_topk_update(d->cand, B, (int64_t)M * d->V, K, d->V, d->score[nxt], d->out_flat, parent_out,
+                                    d->token[nxt], d->topk_ws, d->topk_ws_bytes, update, st, stream));
   return GRACE_OK;
 }
 

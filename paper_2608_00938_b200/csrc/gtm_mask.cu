@@ -9,6 +9,7 @@
 // 4 bytes in per candidate); with the Bloom matcher the random 8-byte probes into the request's
 // 512 KB filter (L2-resident) add a latency/L2-bandwidth term.
 #include <cstdlib>
+#include "beam_state.cuh"
 #include "common.cuh"
 
 namespace grace {
@@ -49,7 +50,7 @@ __device__ __forceinline__ int nth_set_bit64(uint64_t word, int n) {
 }
 
 constexpr int kMaskWarpsPerBlock = 8;
-constexpr int kMaskSplitWarps = 32;      // SPLIT: warps that share one row (a CTA of 1024 threads)
+constexpr int kMaskSplitWarps = 32;      // SPLIT: at most so many warps share one row (a CTA)
 
 // The log-sum-exp of a row from per-lane (maximum, sum of e^(x - maximum)) pairs (lanes without a pair pass
 // (-inf, 0)): every lane returns the same value.  One definition, with the roundings spelled out, for the mask
@@ -76,9 +77,10 @@ __device__ __forceinline__ float warp_merge_lse(float m_l, float s_l) {
 //      log-probabilities is read only if one of its tokens is allowed.
 // LOGITS = true: `logp` holds raw logits; the row's log-sum-exp is taken in a first streaming pass
 // and cand = score + (logit - lse) for allowed tokens.
-// SPLIT = true (few rows, e.g. step 0 with one beam per request): the 32 warps of a 1024-thread CTA share ONE
-// row: each takes every 32nd group of 32 children in phase 1 and every 32nd group of 128 tokens in
-// the streaming passes; the warp-level synchronisation points become CTA barriers.
+// SPLIT = true (few rows, e.g. step 0 with one beam per request): the warps of a CTA share ONE row: each takes
+// every blockDim.x / 32-th group of 32 children in phase 1 and of 128 tokens in the streaming passes; the warp-level
+// synchronisation points become CTA barriers.  The CTA has as many warps (4 .. 32) as keep all rows resident at once:
+// a chain of dependent look-ups and barriers is what a row takes, so a second wave of CTAs costs as much again.
 template <int KIND, bool LOGITS, bool SPLIT>
 __global__ void __launch_bounds__((SPLIT ? kMaskSplitWarps : kMaskWarpsPerBlock) * 32)
 gtm_mask_kernel(const MaskParams p) {
@@ -92,7 +94,7 @@ gtm_mask_kernel(const MaskParams p) {
   const int r = SPLIT ? (int)blockIdx.x : (int)blockIdx.x * kMaskWarpsPerBlock + wib;
   if (r >= p.R) return;
   const int part = SPLIT ? wib : 0;                      // this warp's share of the row's work
-  constexpr int kParts = SPLIT ? kMaskSplitWarps : 1;
+  const int kParts = SPLIT ? (int)(blockDim.x >> 5) : 1;
   auto sync_row = [&]() { if (SPLIT) __syncthreads(); else __syncwarp(); };
   const int V = p.V;
   const int W = V >> 6;
@@ -158,12 +160,8 @@ gtm_mask_kernel(const MaskParams p) {
   if (SPLIT && LOGITS) {                                 // merge the warps' (maximum, rescaled sum) pairs
     __syncthreads();
     if (!dead) {
-      float m_c = -INFINITY;
-      for (int w = 0; w < kParts; ++w) m_c = fmaxf(m_c, s_lse[0][w]);
-      float s_c = 0.f;
-      for (int w = 0; w < kParts; ++w)
-        if (s_lse[0][w] > -INFINITY) s_c += s_lse[1][w] * expf(s_lse[0][w] - m_c);
-      lse = m_c + logf(s_c);
+      const float m_p = lane < kParts ? s_lse[0][lane] : -INFINITY;
+      lse = warp_merge_lse(m_p, lane < kParts ? s_lse[1][lane] : 0.f);
     }
   }
   if (LOGITS && lane == 0 && part == 0 && p.row_lse != nullptr) p.row_lse[r] = lse;
@@ -592,39 +590,12 @@ __global__ void beam_update_csr_kernel(const int32_t* __restrict__ parent, const
 }
 
 __global__ void beam_update_kernel(const int32_t* __restrict__ parent, const int32_t* __restrict__ token,
-                                   const float* __restrict__ score, const int32_t* __restrict__ prev_node,
-                                   const uint64_t* __restrict__ prev_key, const uint64_t* __restrict__ child_bits,
-                                   const int32_t* __restrict__ child_base, int64_t num_internal,
-                                   int32_t* __restrict__ new_node, uint64_t* __restrict__ new_key,
-                                   int B, int K, int M_prev, int V, int prefix_len, int32_t* d_status) {
+                                   const float* __restrict__ score, const BeamUpdate u, int B, int K, int32_t* d_status) {
   pdl_wait();
   pdl_trigger();
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= B * K) return;
-  const int b = i / K;
-  int par = parent[i];
-  const int tok = token[i];
-  if (par < 0 || par >= M_prev || tok < 0 || tok >= V) {
-    flag_status(d_status, GRACE_DEV_BAD_INDEX);
-    new_node[i] = -1;
-    new_key[i] = 0;
-    return;
-  }
-  const int64_t src = (int64_t)b * M_prev + par;
-  new_key[i] = prev_key[src] | ((uint64_t)(tok + 1) << (16 * prefix_len));
-  const int node = prev_node[src];
-  int out = -1;
-  if (node >= 0 && node < num_internal && score[i] != __int_as_float(0xff800000)) {
-    const int W = V >> 6;
-    const uint64_t* row = child_bits + (int64_t)node * W;
-    const uint64_t word = row[tok >> 6];
-    if ((word >> (tok & 63)) & 1ull) {
-      int rank = __popcll(word & ((1ull << (tok & 63)) - 1ull));
-      for (int w = 0; w < (tok >> 6); ++w) rank += __popcll(row[w]);
-      out = child_base[node] + rank;
-    }
-  }
-  new_node[i] = out;
+  beam_update_one(u, i, i / K, parent[i], token[i], score[i], d_status);
 }
 
 }  // namespace grace
@@ -661,15 +632,18 @@ static grace_status_t launch_mask(const float* logp, bool logits, float* row_lse
   cudaStream_t s = (cudaStream_t)stream;
   // Plain launches (no early scheduling under the previous kernel's tail): starting this kernel's CTAs while the
   // logits GEMM drains made the dense trie level 0.3 ms slower in the decode loop.
-  // few rows: a CTA per row, so that the row's matcher look-ups and its streaming passes use eight warps
+  // Few rows: a CTA per row, so that the row's matcher look-ups and its streaming passes use several warps
+  // (these launches are scheduled early: nothing else fills the GPU under them).
   const bool split = p.R <= 2048;
+  int split_warps = kMaskSplitWarps;
+  while (split_warps > 4 && p.R * split_warps > 148 * 64) split_warps >>= 1;
   const int blocks = split ? p.R : (p.R + kMaskWarpsPerBlock - 1) / kMaskWarpsPerBlock;
-  const int threads = (split ? kMaskSplitWarps : kMaskWarpsPerBlock) * 32;
+  const int threads = (split ? split_warps : kMaskWarpsPerBlock) * 32;
 #define GRACE_MASK_LAUNCH(K)                                                      \
   do {                                                                            \
-    if (logits && split) gtm_mask_kernel<K, true, true><<<blocks, threads, 0, s>>>(p);        \
+    if (logits && split) launch_pdl(gtm_mask_kernel<K, true, true>, dim3(blocks), dim3(threads), 0, s, p);   \
     else if (logits) gtm_mask_kernel<K, true, false><<<blocks, threads, 0, s>>>(p);           \
-    else if (split) gtm_mask_kernel<K, false, true><<<blocks, threads, 0, s>>>(p);            \
+    else if (split) launch_pdl(gtm_mask_kernel<K, false, true>, dim3(blocks), dim3(threads), 0, s, p);       \
     else gtm_mask_kernel<K, false, false><<<blocks, threads, 0, s>>>(p);                      \
   } while (0)
   switch (matcher->kind) {
@@ -784,9 +758,10 @@ extern "C" grace_status_t grace_beam_update(const int32_t* parent, const int32_t
   if (!trie || !trie_ok(trie, trie->V)) return GRACE_INVALID_ARG;
   if (B <= 0 || K <= 0 || M_prev <= 0 || prefix_len < 0 || prefix_len >= 4) return GRACE_INVALID_ARG;
   const int n = B * K;
+  const grace::BeamUpdate u = {prev_node, prev_key, trie->child_bits, trie->child_base, new_node, new_key,
+                               trie->num_internal, M_prev, trie->V, prefix_len};
   grace::launch_pdl(grace::beam_update_kernel, dim3((n + 255) / 256), dim3(256), 0, (cudaStream_t)stream,
-      parent, token, score, prev_node, prev_key, trie->child_bits, trie->child_base, trie->num_internal,
-      new_node, new_key, B, K, M_prev, trie->V, prefix_len, d_status);
+      parent, token, score, u, B, K, d_status);
   GRACE_LAUNCH_CHECK();
   return GRACE_OK;
 }

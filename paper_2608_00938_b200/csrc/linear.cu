@@ -216,6 +216,7 @@ linear_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_constant__
   const uint32_t t_acc = tmem_base + ((uint32_t)((warp & 3) * 32) << 16);
   if (SPLIT > 1) {
     // partial sums of the other CTAs' columns to their owners; every CTA of the cluster has long started
+    __syncwarp();
     asm volatile("barrier.cluster.wait.aligned;" ::: "memory");
     if (warp < 4 && ok) {
 #pragma unroll 1

@@ -6,6 +6,7 @@ import torch
 
 import synth
 from oracle import attention as OA
+from oracle import topk as OT
 
 pytestmark = pytest.mark.gpu
 
@@ -67,3 +68,58 @@ def test_cross_attn_waits_never_give_up_back_to_back(api, B, M, H, T):
         torch.cuda.synchronize()
         assert api.grace_wait_timeouts() == 0
         assert torch.equal(first, last)
+
+
+@pytest.mark.parametrize("N,V,K", [(64, 64, 16), (8192, 64, 4096), (8196, 4, 512), (32768, 2048, 1000), (32772, 4, 64),
+                                   (40960, 64, 300), (65536, 1024, 4096), (100000, 1000, 700)])
+@pytest.mark.parametrize("finite", [0.0, 0.001, 0.2, 1.0])
+def test_topk_between_its_paths(api, N, V, K, finite):
+    """Sizes around the limits of the one-kernel selection and of the sampled one, with few, some and all candidates
+    finite (more than fit in shared memory among them), ties included: exact against the oracle."""
+    rng = np.random.default_rng(N + K + int(1000 * finite))
+    B = 3
+    cand = np.where(rng.random((B, N)) < finite, np.round(rng.standard_normal((B, N)) * 50) / 16, -np.inf).astype(np.float32)
+    sc, flat, par, tok = OT.beam_topk(cand, K, V)
+    out = [torch.zeros(B, K, device=DEV), *(torch.zeros(B, K, device=DEV, dtype=torch.int32) for _ in range(3))]
+    ws = torch.full((api.grace_beam_topk_workspace_bytes(B, N, K),), 255, device=DEV, dtype=torch.uint8)
+    api.grace_beam_topk(dev(cand), K, V, *out, ws)
+    torch.cuda.synchronize()
+    for got, want in zip(out, (sc, flat, par, tok)):
+        assert np.array_equal(got.cpu().numpy(), want)
+
+
+@pytest.mark.parametrize("M,N,K", [(1, 64, 64), (17, 96, 128), (130, 512, 512), (129, 528, 2048), (512, 1536, 512), (1025, 512, 512),
+                                   (1030, 2048, 512), (300, 2048, 1088), (2049, 272, 320), (5, 2048, 2048)])
+@pytest.mark.parametrize("centred", [True, False])
+def test_layer_norm_gemm_in_every_form(api, M, N, K, centred):
+    """grace_linear_layer_norm (statistics inside the GEMM, K shared by the CTAs of a cluster) and the additions into
+    both residual streams, at tile edges and remainders, against fp64 on the same bf16 operands.
+
+    Bounds: LayerNorm: one rounding of the result to bf16 (2^-9 relative) and fp32 sums (a few 2^-24 of the row's absolute
+    sum, scaled by rstd); additions likewise."""
+    g = torch.Generator(device=DEV)
+    g.manual_seed(M + N + K)
+    x = torch.randn(M, K, device=DEV, generator=g)
+    x = (x - x.mean(1, keepdim=True) + (0.0 if centred else 0.7)).to(torch.bfloat16)
+    w = (torch.randn(N, K, device=DEV, generator=g) * 0.05).to(torch.bfloat16)
+    cs, cb = w.double().sum(1).float(), torch.randn(N, device=DEV, generator=g)
+    x64, w64 = x.double(), w.double()
+    mean, var = x64.mean(1, keepdim=True), x64.var(1, unbiased=False, keepdim=True)
+    rstd = (var + 1e-5).rsqrt()
+    prod, absolute = x64 @ w64.T, x64.abs() @ w64.abs().T
+    shift = 0.0 if centred else -rstd * mean * cs.double()
+    want = torch.relu(rstd * prod + shift + cb.double())
+    y, aff = torch.empty(M, N, device=DEV, dtype=torch.bfloat16), torch.empty(M, 2, device=DEV)
+    api.grace_linear_layer_norm(x, w, 1e-5, aff, None if centred else cs, cb, y, relu=True)
+    bound = 2.0 ** -8 * want.abs() + 2.0 ** -17 * (rstd * absolute + (0 if centred else (rstd * mean * cs.double()).abs())) + 1e-5
+    assert ((y.double() - want).abs() <= bound).all()
+    for dtype in (torch.bfloat16, torch.float32):
+        r = torch.randn(M, N, device=DEV, generator=g).to(dtype)
+        want = r.double() + prod
+        if dtype == torch.bfloat16:
+            api.grace_linear_add_bf16(x, w, r)
+            bound = 2.0 ** -8 * (want.abs() + prod.abs()) + 2.0 ** -19 * absolute
+        else:
+            api.grace_linear(x, w, r, residual=r)
+            bound = 2.0 ** -19 * absolute + 2.0 ** -22 * want.abs()
+        assert ((r.double() - want).abs() <= bound + 1e-30).all()
