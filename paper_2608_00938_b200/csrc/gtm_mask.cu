@@ -419,8 +419,11 @@ row_lse_from_parts_kernel(const float2* __restrict__ lse_part, int n_parts, cons
 // bitmask and its N_loc location rows are staged in shared memory once and reused by every
 // candidate of those beams.  One warp per beam; lanes take the child entries of the beam's node.
 // Evaluation order as in the paper: bitmask first (stop at the first failing word), Bloom only for
-// entries that pass, inner scan stops at the first word that is not contained, outer scan at the
-// first location that is.
+// entries that pass, outer scan stops at the first location that is contained.  A word that holds none of the
+// request's bits passes whatever the row holds and is not read; the others are read in the order of the request's
+// bits in them, most first, so that most entries fail on their first read: the rows lie scattered over L2 and the
+// stage is bound by the cache lines that its reads touch (one line per entry and word).  Two entries per lane are
+// in flight.
 // ---------------------------------------------------------------------------------------------
 struct LookupParams {
   const float* logp;
@@ -440,15 +443,31 @@ __global__ void __launch_bounds__(kMaskWarpsPerBlock * 32)
 gtm_lookup_kernel(const LookupParams p) {
   extern __shared__ uint64_t s_user[];                         // [WBM] bitmask, then [N_loc][WBL]
   __shared__ unsigned long long s_allow[kMaskWarpsPerBlock][kLookupMaxWords];
-  __shared__ int s_queue[kMaskWarpsPerBlock][64];
+  __shared__ int s_queue[kMaskWarpsPerBlock][96];
+  __shared__ int s_order[WBM + 1];                             // number of words to read, then which, in that order
   const grace_gtm_index_t& ix = p.idx;
   const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
   const int b = blockIdx.y;
   const int V = ix.V, W = V >> 6;
+  pdl_wait();
+  pdl_trigger();
   for (int i = threadIdx.x; i < WBM; i += blockDim.x) s_user[i] = ix.user_bitmask[(int64_t)b * WBM + i];
   for (int i = threadIdx.x; i < ix.N_loc * WBL; i += blockDim.x)
     s_user[WBM + i] = ix.user_blooms[(int64_t)b * ix.N_loc * WBL + i];
+  if (threadIdx.x == 0) s_order[0] = 0;
   __syncthreads();
+  if (threadIdx.x < WBM) {
+    const int i = threadIdx.x, bits = __popcll(s_user[i]);
+    int before = 0;
+    for (int j = 0; j < WBM; ++j) {
+      const int other = __popcll(s_user[j]);
+      before += other > bits || (other == bits && j < i);
+    }
+    s_order[1 + before] = i;
+    if (bits != 0) atomicAdd(&s_order[0], 1);
+  }
+  __syncthreads();
+  const int n_words = s_order[0];
   const int m = blockIdx.x * kMaskWarpsPerBlock + wib;
   if (m >= p.M) return;
   const int64_t r = (int64_t)b * p.M + m;
@@ -470,26 +489,39 @@ gtm_lookup_kernel(const LookupParams p) {
     const int end = kway ? __ldg(ix.part_offsets + e_end) : e_end;
     int* queue = s_queue[wib];                 // slots that passed the bitmask, waiting for Bloom
     int queued = 0;
-    for (int j0 = start; j0 < end || queued > 0; j0 += 32) {
-      // ---- bitmask stage: one entry per lane, first failing word ends it ----
-      const int j = j0 + lane;
-      bool pass = false;
-      if (j < end) {
-        const uint64_t* bm = ix.bitmask_table + (int64_t)__ldg(ix.bitmask_index + j) * WBM;
-        pass = true;
+    int id[2];                                 // row ids of this round's entries, fetched a round ahead
 #pragma unroll
-        for (int w = 0; w < WBM; ++w) {
-          if (!pass) break;
-          const uint64_t u = s_user[w];
-          pass = (__ldg(bm + w) & u) == u;
-        }
+    for (int e = 0; e < 2; ++e) id[e] = start + 32 * e + lane < end ? __ldg(ix.bitmask_index + start + 32 * e + lane) : 0;
+    for (int j0 = start; j0 < end || queued > 0; j0 += 64) {
+      // ---- bitmask stage: two entries per lane, first failing word ends an entry ----
+      const uint64_t* bm[2];
+      bool pass[2];
+#pragma unroll
+      for (int e = 0; e < 2; ++e) {
+        const int j = j0 + 32 * e + lane;
+        pass[e] = j < end;
+        bm[e] = ix.bitmask_table + (int64_t)id[e] * WBM;
+        id[e] = j + 64 < end ? __ldg(ix.bitmask_index + j + 64) : 0;
+      }
+      for (int i = 1; i <= n_words; ++i) {
+        if (!__any_sync(kFullMask, pass[0] || pass[1])) break;
+        const int w = s_order[i];
+        const uint64_t u = s_user[w];
+        uint64_t row[2] = {0ull, 0ull};
+#pragma unroll
+        for (int e = 0; e < 2; ++e) if (pass[e]) row[e] = __ldg(bm[e] + w);
+#pragma unroll
+        for (int e = 0; e < 2; ++e) pass[e] = pass[e] && (row[e] & u) == u;
       }
       // survivors are queued so that the (much longer) Bloom stage always runs with full warps
-      const uint32_t votes = __ballot_sync(kFullMask, pass);
-      if (pass) queue[queued + __popc(votes & ((1u << lane) - 1u))] = j;
-      queued += __popc(votes);
+#pragma unroll
+      for (int e = 0; e < 2; ++e) {
+        const uint32_t votes = __ballot_sync(kFullMask, pass[e]);
+        if (pass[e]) queue[queued + __popc(votes & ((1u << lane) - 1u))] = j0 + 32 * e + lane;
+        queued += __popc(votes);
+      }
       __syncwarp();
-      const bool last_round = (j0 + 32 >= end);
+      const bool last_round = (j0 + 64 >= end);
       while (queued >= 32 || (last_round && queued > 0)) {
         const int take = min(queued, 32);
         const int e = (lane < take) ? queue[queued - take + lane] : -1;
@@ -538,21 +570,31 @@ gtm_lookup_kernel(const LookupParams p) {
   if (p.allow_bits != nullptr)
     for (int w = lane; w < W; w += 32) p.allow_bits[r * W + w] = allow[w];
   if (p.cand != nullptr) {
-    for (int g = 0; g < V; g += 128) {
-      const int tok0 = g + 4 * lane;
-      if (tok0 >= V) continue;
-      const uint32_t nib = (uint32_t)(allow[tok0 >> 6] >> (tok0 & 63)) & 0xfu;
-      float4 lp = make_float4(0.f, 0.f, 0.f, 0.f);
-      if (nib != 0u) lp = __ldg(reinterpret_cast<const float4*>(lrow + tok0));
-      const float vals[4] = {lp.x, lp.y, lp.z, lp.w};
-      float outv[4];
+    constexpr int U = 4;                       // groups of 128 tokens whose log-probabilities are requested together
+    for (int g = 0; g < V; g += U * 128) {
+      uint32_t nib[U];
+      float4 lp[U];
 #pragma unroll
-      for (int j = 0; j < 4; ++j) {
-        const bool okj = (nib >> j) & 1u;
-        outv[j] = okj ? (score + vals[j]) : ninf;
-        if (okj && vals[j] != vals[j]) saw_nan = true;
+      for (int u = 0; u < U; ++u) {
+        const int tok0 = g + u * 128 + 4 * lane;
+        nib[u] = tok0 < V ? (uint32_t)(allow[tok0 >> 6] >> (tok0 & 63)) & 0xfu : 0u;
+        lp[u] = make_float4(0.f, 0.f, 0.f, 0.f);
+        if (nib[u] != 0u) lp[u] = __ldg(reinterpret_cast<const float4*>(lrow + tok0));
       }
-      *reinterpret_cast<float4*>(p.cand + r * V + tok0) = make_float4(outv[0], outv[1], outv[2], outv[3]);
+#pragma unroll
+      for (int u = 0; u < U; ++u) {
+        const int tok0 = g + u * 128 + 4 * lane;
+        if (tok0 >= V) continue;
+        const float vals[4] = {lp[u].x, lp[u].y, lp[u].z, lp[u].w};
+        float outv[4];
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+          const bool okj = (nib[u] >> j) & 1u;
+          outv[j] = okj ? (score + vals[j]) : ninf;
+          if (okj && vals[j] != vals[j]) saw_nan = true;
+        }
+        *reinterpret_cast<float4*>(p.cand + r * V + tok0) = make_float4(outv[0], outv[1], outv[2], outv[3]);
+      }
     }
   }
   if (saw_nan) flag_status(p.d_status, GRACE_DEV_NAN);
@@ -563,6 +605,8 @@ __global__ void beam_update_csr_kernel(const int32_t* __restrict__ parent, const
                                        const uint64_t* __restrict__ prev_key, const grace_gtm_index_t ix,
                                        int32_t* __restrict__ new_node, uint64_t* __restrict__ new_key, int B, int K,
                                        int M_prev, int prefix_len, int32_t* d_status) {
+  pdl_wait();
+  pdl_trigger();
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= B * K) return;
   const int b = i / K;
@@ -789,10 +833,10 @@ extern "C" grace_status_t grace_gtm_lookup(const float* logp, const float* beam_
   const size_t smem = (size_t)(index->W_bm + (size_t)index->N_loc * index->W_bl) * sizeof(uint64_t);
   cudaStream_t s = (cudaStream_t)stream;
   const int threads = kMaskWarpsPerBlock * 32;
-  if (index->W_bm == 7 && index->W_bl == 4) gtm_lookup_kernel<7, 4><<<grid, threads, smem, s>>>(p);
-  else if (index->W_bm == 2 && index->W_bl == 4) gtm_lookup_kernel<2, 4><<<grid, threads, smem, s>>>(p);
-  else if (index->W_bm == 1 && index->W_bl == 1) gtm_lookup_kernel<1, 1><<<grid, threads, smem, s>>>(p);
-  else if (index->W_bm == 4 && index->W_bl == 4) gtm_lookup_kernel<4, 4><<<grid, threads, smem, s>>>(p);
+  if (index->W_bm == 7 && index->W_bl == 4) launch_pdl(gtm_lookup_kernel<7, 4>, grid, dim3(threads), smem, s, p);
+  else if (index->W_bm == 2 && index->W_bl == 4) launch_pdl(gtm_lookup_kernel<2, 4>, grid, dim3(threads), smem, s, p);
+  else if (index->W_bm == 1 && index->W_bl == 1) launch_pdl(gtm_lookup_kernel<1, 1>, grid, dim3(threads), smem, s, p);
+  else if (index->W_bm == 4 && index->W_bl == 4) launch_pdl(gtm_lookup_kernel<4, 4>, grid, dim3(threads), smem, s, p);
   else return GRACE_UNSUPPORTED_SHAPE;      // row widths are compile-time: (7,4) as in the paper, plus (1,1), (2,4), (4,4)
   GRACE_LAUNCH_CHECK();
   return GRACE_OK;
@@ -807,7 +851,7 @@ extern "C" grace_status_t grace_beam_update_csr(const int32_t* parent, const int
     return GRACE_INVALID_ARG;
   if (B <= 0 || K <= 0 || M_prev <= 0 || prefix_len < 0 || prefix_len >= 4) return GRACE_INVALID_ARG;
   const int n = B * K;
-  grace::beam_update_csr_kernel<<<(n + 255) / 256, 256, 0, (cudaStream_t)stream>>>(
+  grace::launch_pdl(grace::beam_update_csr_kernel, dim3((n + 255) / 256), dim3(256), 0, (cudaStream_t)stream,
       parent, token, score, prev_node, prev_key, *index, new_node, new_key, B, K, M_prev, prefix_len, d_status);
   GRACE_LAUNCH_CHECK();
   return GRACE_OK;
