@@ -442,6 +442,12 @@ grace_status_t grace_linear(const uint16_t* x, int64_t ldx, const uint16_t* w, i
                             uint16_t* y_bf16, float* y_f32, int64_t ldy, const float* residual,
                             int M, int N, int K, int relu, void* stream);
 
+/* y[i] = x @ w[i]^T for count products of one shape that share x (the cross-attention K and V of every layer from
+ * one encoder output): the products of grace_linear with bf16 outputs, up to eight of them in one launch.  w and
+ * y_bf16: host arrays of count device pointers, each [N][K] (row stride ldw) and [M][N] (row stride ldy). */
+grace_status_t grace_linear_multi(const uint16_t* x, int64_t ldx, int count, const uint16_t* const* w, int64_t ldw,
+                                  uint16_t* const* y_bf16, int64_t ldy, int M, int N, int K, void* stream);
+
 /* y += x @ w^T with a bf16 residual stream y [M][N] (row stride ldy): the product is accumulated in
  * fp32, rounded to bf16 and added to y in bf16 (large problems: by a TMA add-reduction, y is never read
  * into the SM).  Same shape and alignment rules as grace_linear. */
@@ -474,12 +480,13 @@ grace_status_t grace_linear_folded_ln(const uint16_t* x, int64_t ldx, const uint
                                       int M, int N, int K, int relu, void* stream);
 
 /* grace_row_stats_bf16 (over D = K, with eps) followed by grace_linear_folded_ln, as one call: the LayerNorm over
- * the rows of x [M][K] (ldx == K) and the GEMM behind it.  For M >= 1024 and 256 <= N <= 512 with centred rows
- * (col_sum NULL) and no lse_part it is ONE kernel: the row statistics are formed from the GEMM's own operand tiles in shared
- * memory while the tensor cores work on them, so the residual stream is not read a second time; row_affine
- * (device, fp32 [M][2], 8-byte aligned) is then not touched.  Otherwise (wider outputs, where forming the
+ * the rows of x [M][K] (ldx == K) and the GEMM behind it.  Where the GEMM's tiles are few (up to a few thousand rows) or its
+ * output is narrow (256 <= N <= 512, centred rows: col_sum NULL) and there is no lse_part it is ONE kernel: the row
+ * statistics are formed from the GEMM's own operand tiles in shared memory while the tensor cores work on them, so the
+ * residual stream is not read a second time.  Otherwise (large problems with wide outputs, where forming the
  * statistics once per 256-column tile costs more than reading the stream once) the statistics kernel runs
- * first, into row_affine.  Other arguments and errors as grace_linear_folded_ln. */
+ * first.  Either way the statistics end up in row_affine (device, fp32 [M][2], 8-byte aligned), except for M >= 1024
+ * and 256 <= N <= 512 with centred rows and no lse_part, where it is not touched.  Other arguments and errors as grace_linear_folded_ln. */
 grace_status_t grace_linear_layer_norm(const uint16_t* x, int64_t ldx, const uint16_t* w, int64_t ldw, float eps,
                                        float* row_affine, const float* col_sum, const float* col_bias,
                                        uint16_t* y_bf16, float* y_f32, int64_t ldy, float* lse_part,

@@ -140,6 +140,7 @@ _beam_topk_static_max = _sig("grace_beam_topk_static_max_requests", _i32, [])
 _beam_update = _sig("grace_beam_update", _i32, [_vp, _vp, _vp, _vp, _vp, C.POINTER(TrieStruct), _vp, _vp,
                                                _i32, _i32, _i32, _i32, _vp, _vp])
 _linear = _sig("grace_linear", _i32, [_vp, _i64, _vp, _i64, _vp, _vp, _i64, _vp, _i32, _i32, _i32, _i32, _vp])
+_linear_multi = _sig("grace_linear_multi", _i32, [_vp, _i64, _i32, C.POINTER(_vp), _i64, C.POINTER(_vp), _i64, _i32, _i32, _i32, _vp])
 _linear_add_bf16 = _sig("grace_linear_add_bf16", _i32, [_vp, _i64, _vp, _i64, _vp, _i64, _i32, _i32, _i32, _vp])
 _layer_norm_bf16 = _sig("grace_layer_norm_bf16", _i32, [_vp, _vp, _vp, _vp, _i32, _i32, _f32, _vp])
 _embed_bf16 = _sig("grace_embed_bf16", _i32, [_vp, _vp, _vp, _vp, _i32, _i32, _i32, _vp, _vp])
@@ -601,6 +602,18 @@ def grace_linear(x, w, y, residual=None, relu: bool = False):
     _check(_linear(x.data_ptr(), x.stride(0), w.data_ptr(), w.stride(0), yb, yf, y.stride(0),
                    _dp(residual), M, N, K, int(relu), _stream()), "grace_linear")
     return y
+
+
+def grace_linear_multi(x, ws, ys):
+    """ys[i] = x @ ws[i].T; x [M, K] bf16, ws [N, K] bf16 and ys [M, N] bf16, all of one shape and row stride."""
+    M, K = x.shape
+    N, n = ws[0].shape[0], len(ws)
+    wp, yp = (_vp * n)(*(w.data_ptr() for w in ws)), (_vp * n)(*(_dp(y) for y in ys))
+    assert len(ys) == n and all(w.shape == ws[0].shape and w.stride() == ws[0].stride() for w in ws)
+    assert all(y.shape == (M, N) and y.stride() == ys[0].stride() for y in ys)
+    _check(_linear_multi(x.data_ptr(), x.stride(0), n, wp, ws[0].stride(0), yp, ys[0].stride(0), M, N, K, _stream()),
+           "grace_linear_multi")
+    return ys
 
 
 def grace_linear_add_bf16(x, w, y):

@@ -62,10 +62,19 @@ struct GemmParams {
 
 constexpr int kGemmThreads = 192;                           // four row warps, TMA producer, MMA issuer
 
-template <int BN, int STAGES, int SPLIT>
+// The weights and outputs of G products that share x (grace_linear_multi: one launch, more tiles); G = 1: one product.
+constexpr int kMultiMost = 8;
+template <int G>
+struct GemmSet {
+  CUtensorMap w[G];
+  CUtensorMap y[G];              // linear_pair_kernel
+  uint16_t* y_bf16[G];           // linear_kernel, G > 1
+  int count;                     // of them in use
+};
+
+template <int BN, int STAGES, int SPLIT, int G>
 __global__ void __launch_bounds__(kGemmThreads, 2)
-linear_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_constant__ CUtensorMap map_w,
-              const GemmParams p) {
+linear_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_constant__ GemmSet<G> set, const GemmParams p) {
   // The weights do not depend on the kernel before this one: their first tiles are requested before the wait
   // on that kernel, so their trip from HBM overlaps its tail; every thread waits before its first access to
   // anything an earlier kernel wrote (activations, row statistics, the residual).
@@ -85,7 +94,11 @@ linear_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_constant__
 
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int rank = SPLIT > 1 ? (int)(blockIdx.x % SPLIT) : 0;
-  const int m0 = blockIdx.y * kGemmBM, n0 = (int)(blockIdx.x / SPLIT) * BN;
+  const int n_tiles = G > 1 ? (p.N + BN - 1) / BN : 0;
+  const int which = G > 1 ? (int)(blockIdx.x / SPLIT) / n_tiles : 0;                    // of the products
+  const CUtensorMap& map_w = set.w[which];
+  uint16_t* const y_bf16 = G > 1 ? set.y_bf16[which] : p.y_bf16;
+  const int m0 = blockIdx.y * kGemmBM, n0 = ((int)(blockIdx.x / SPLIT) - which * n_tiles) * BN;
   const int KB_all = p.K / kGemmBK;
   const int kb0 = KB_all * rank / SPLIT, KB = KB_all * (rank + 1) / SPLIT - kb0;        // this CTA's k-blocks (>= 1)
   const bool folded = p.aff_cb != nullptr;
@@ -265,7 +278,7 @@ linear_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_constant__
       ar = make_float2(rstd, -rstd * mean);
       if (blockIdx.x == 0 && p.aff_out != nullptr && m < p.M) p.aff_out[m] = ar;
     }
-    const bool sectors = ((reinterpret_cast<uintptr_t>(p.y_bf16) | reinterpret_cast<uintptr_t>(p.y_f32) | (uintptr_t)p.ldy * 2) & 31) == 0;
+    const bool sectors = ((reinterpret_cast<uintptr_t>(y_bf16) | reinterpret_cast<uintptr_t>(p.y_f32) | (uintptr_t)p.ldy * 2) & 31) == 0;
 #pragma unroll 1
     for (int c = 0; c < kSlice; c += kChunk) {
       uint32_t acc[kChunk];
@@ -337,7 +350,7 @@ linear_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_constant__
           for (int j = 0; j < 4; ++j)
             o[j] = make_uint4(__float_as_uint(v[4 * j]), __float_as_uint(v[4 * j + 1]), __float_as_uint(v[4 * j + 2]), __float_as_uint(v[4 * j + 3]));
         } else {
-          dst = p.y_bf16 + (int64_t)m * p.ldy + n;
+          dst = y_bf16 + (int64_t)m * p.ldy + n;
 #pragma unroll
           for (int j = 0; j < 2; ++j)
             o[j] = make_uint4(pack_bf16x2(v[8 * j], v[8 * j + 1]), pack_bf16x2(v[8 * j + 2], v[8 * j + 3]),
@@ -429,10 +442,10 @@ __device__ __forceinline__ float2 lse_merge_halves(float m_a, float s_a, float m
   return make_float2(m, __fmaf_rn(s_a, ea, __fmul_rn(s_b, eb)));
 }
 
-template <int OUT, bool STATS>
+template <int OUT, bool STATS, int G>
 __global__ void __launch_bounds__((STATS || OUT == kOutF32LseAllowed) ? 320 : 192, 1)
-linear_pair_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_constant__ CUtensorMap map_w,
-                   const __grid_constant__ CUtensorMap map_y, int M, int N, int K, int relu, float2* lse_part,
+linear_pair_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_constant__ GemmSet<G> set,
+                   int M, int N, int K, int relu, float2* lse_part,
                    const float2* __restrict__ aff_row, const float* __restrict__ aff_cs,
                    const float* __restrict__ aff_cb, float ln_eps, const uint64_t* __restrict__ allow_bits,
                    float* __restrict__ y_direct, int64_t ldy) {
@@ -463,7 +476,10 @@ linear_pair_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_const
   const uint32_t rank = tc::cluster_cta_rank();            // 0: issues the MMAs; 1: peer
   const int pair = blockIdx.x >> 1, n_pairs = gridDim.x >> 1;
   const int KB = K / kPBK;
-  const int n_tiles = (N + 255) / 256, m_tiles = (M + 255) / 256;
+  // (G > 1: the n-tiles of all products side by side, so that neighbouring pairs share a row panel of x)
+  const int n_tiles_one = (N + 255) / 256, n_tiles = G > 1 ? n_tiles_one * set.count : n_tiles_one, m_tiles = (M + 255) / 256;
+  auto product_of = [&](int tile) { return G > 1 ? (tile % n_tiles) / n_tiles_one : 0; };
+  auto column_of = [&](int tile) { return (G > 1 ? (tile % n_tiles) % n_tiles_one : tile % n_tiles) * 256; };
   const int total = n_tiles * m_tiles;
 
   if (threadIdx.x == 0) {
@@ -476,7 +492,7 @@ linear_pair_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_const
     }
     *abort_flag = 0;
     tc::fence_mbar_init();
-    tc::tma_prefetch_desc(&map_x); tc::tma_prefetch_desc(&map_w); tc::tma_prefetch_desc(&map_y);
+    tc::tma_prefetch_desc(&map_x); tc::tma_prefetch_desc(&set.w[0]); tc::tma_prefetch_desc(&set.y[0]);
   }
   if (warp == 0) tc::tmem_alloc_pair(tmem_slot, 512);
   tc::tc_fence_before();
@@ -491,7 +507,8 @@ linear_pair_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_const
     if (lane == 0) {                                        // ---- TMA producer (both CTAs) ----
       int it = 0;
       for (int tile = pair; tile < total; tile += n_pairs) {
-        const int m0 = (tile / n_tiles) * 256 + (int)rank * 128, n0 = (tile % n_tiles) * 256 + (int)rank * 128;
+        const int m0 = (tile / n_tiles) * 256 + (int)rank * 128, n0 = column_of(tile) + (int)rank * 128;
+        const CUtensorMap* map_w = &set.w[product_of(tile)];
         for (int kb = 0; kb < KB; ++kb, ++it) {
           const int s = it % kQStages;
           if (!tc::mbar_wait_cluster(empty + s, ((it / kQStages) & 1) ^ 1, abort_flag)) { tile = total; break; }
@@ -499,7 +516,7 @@ linear_pair_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_const
           uint8_t* a = tiles + s * kQStageBytes;
           const uint32_t bar = tc::cluster_addr_of(full + s, 0);
           tc::tma_load_2d_pair(a, &map_x, bar, kb * kPBK, m0);
-          tc::tma_load_2d_pair(a + kQABytes, &map_w, bar, kb * kPBK, n0);
+          tc::tma_load_2d_pair(a + kQABytes, map_w, bar, kb * kPBK, n0);
         }
       }
     }
@@ -612,7 +629,8 @@ linear_pair_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_const
     };
     fetch_affine(pair);
     for (int tile = pair; tile < total; tile += n_pairs, ++local) {
-      const int m0 = (tile / n_tiles) * 256 + (int)rank * 128, n0 = (tile % n_tiles) * 256;
+      const int m0 = (tile / n_tiles) * 256 + (int)rank * 128, n0 = column_of(tile);
+      const CUtensorMap* map_y = &set.y[product_of(tile)];
       const int ab = local & 1;
       float2 ar = ar_next;                                 // rows and columns past the edge: values never stored
       const ulonglong2 aw_lo = aw_lo_next, aw_hi = aw_hi_next;
@@ -782,8 +800,8 @@ linear_pair_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_const
         tc::fence_proxy_async_smem();
         tc::named_bar_sync(1, 128);
         if (issuer && m0 < M) {
-          if (OUT == kOutF32Add || OUT == kOutBf16Add) tc::tma_reduce_add_2d(&map_y, buf, n0 + c * kColsPerChunk, m0);
-          else tc::tma_store_2d(&map_y, buf, n0 + c * kColsPerChunk, m0);
+          if (OUT == kOutF32Add || OUT == kOutBf16Add) tc::tma_reduce_add_2d(map_y, buf, n0 + c * kColsPerChunk, m0);
+          else tc::tma_store_2d(map_y, buf, n0 + c * kColsPerChunk, m0);
         }
         if (issuer) tc::bulk_commit();
       }
@@ -811,8 +829,8 @@ struct AllowedStores {                                     // kOutF32LseAllowed
   int64_t ldy = 0;
 };
 
-template <int OUT, bool STATS = false>
-static grace_status_t launch_pair(const CUtensorMap& mx, const CUtensorMap& mw, const CUtensorMap& my, int M, int N,
+template <int OUT, bool STATS = false, int G = 1>
+static grace_status_t launch_pair(const CUtensorMap& mx, const GemmSet<G>& set, int M, int N,
                                   int K, int relu, cudaStream_t s, float2* lse_part = nullptr,
                                   Affine aff = Affine{nullptr, nullptr, nullptr}, AllowedStores al = AllowedStores{}) {
   static unsigned long long attr_set_devices = 0;
@@ -826,32 +844,32 @@ static grace_status_t launch_pair(const CUtensorMap& mx, const CUtensorMap& mw, 
   cfg.blockDim = dim3((STATS || OUT == kOutF32LseAllowed) ? 320 : 192); cfg.dynamicSmemBytes = kQSmem; cfg.stream = s; cfg.attrs = attr; cfg.numAttrs = 2;
   DeviceSetup su(&attr_set_devices);
   if (su) {
-    GRACE_CUDA_TRY(cudaFuncSetAttribute(linear_pair_kernel<OUT, STATS>, cudaFuncAttributeMaxDynamicSharedMemorySize, kQSmem));
+    GRACE_CUDA_TRY(cudaFuncSetAttribute(linear_pair_kernel<OUT, STATS, G>, cudaFuncAttributeMaxDynamicSharedMemorySize, kQSmem));
     int n_sm = 0, clusters = 0;
     GRACE_CUDA_TRY(cudaDeviceGetAttribute(&n_sm, cudaDevAttrMultiProcessorCount, su.dev));
     cfg.gridDim = dim3(n_sm & ~1);
-    GRACE_CUDA_TRY(cudaOccupancyMaxActiveClusters(&clusters, linear_pair_kernel<OUT, STATS>, &cfg));
+    GRACE_CUDA_TRY(cudaOccupancyMaxActiveClusters(&clusters, linear_pair_kernel<OUT, STATS, G>, &cfg));
     if (clusters <= 0) return GRACE_CUDA_ERROR;
     if (clusters > n_sm / 2) clusters = n_sm / 2;
     max_clusters_of[su.dev] = clusters;
     su.done();
   }
   const int max_clusters = max_clusters_of[su.dev];
-  const int total = ((N + 255) / 256) * ((M + 255) / 256);
-  cfg.gridDim = dim3(2 * (total < max_clusters ? total : max_clusters));
-  GRACE_CUDA_TRY(cudaLaunchKernelEx(&cfg, linear_pair_kernel<OUT, STATS>, mx, mw, my, M, N, K, relu, lse_part, aff.row, aff.cs, aff.cb, aff.eps,
+  const int64_t total = (int64_t)((N + 255) / 256) * ((M + 255) / 256) * set.count;
+  cfg.gridDim = dim3(2 * (unsigned)(total < max_clusters ? total : max_clusters));
+  GRACE_CUDA_TRY(cudaLaunchKernelEx(&cfg, linear_pair_kernel<OUT, STATS, G>, mx, set, M, N, K, relu, lse_part, aff.row, aff.cs, aff.cb, aff.eps,
                                     al.bits, al.y, al.ldy));
   GRACE_LAUNCH_CHECK();
   return GRACE_OK;
 }
 
-template <int BN, int STAGES, int SPLIT>
-static grace_status_t launch_linear(const CUtensorMap& mx, const CUtensorMap& mw, const GemmParams& p, cudaStream_t s) {
+template <int BN, int STAGES, int SPLIT, int G>
+static grace_status_t launch_linear(const CUtensorMap& mx, const GemmSet<G>& set, const GemmParams& p, cudaStream_t s) {
   using S = GemmCfg<BN, STAGES, SPLIT>;
   static unsigned long long attr_set_devices = 0;
   DeviceSetup su(&attr_set_devices);
   if (su) {
-    GRACE_CUDA_TRY(cudaFuncSetAttribute(linear_kernel<BN, STAGES, SPLIT>, cudaFuncAttributeMaxDynamicSharedMemorySize, S::kTotal));
+    GRACE_CUDA_TRY(cudaFuncSetAttribute(linear_kernel<BN, STAGES, SPLIT, G>, cudaFuncAttributeMaxDynamicSharedMemorySize, S::kTotal));
     su.done();
   }
   cudaLaunchConfig_t cfg = {};
@@ -860,10 +878,10 @@ static grace_status_t launch_linear(const CUtensorMap& mx, const CUtensorMap& mw
   attr[0].val.programmaticStreamSerializationAllowed = 1;
   attr[1].id = cudaLaunchAttributeClusterDimension;
   attr[1].val.clusterDim.x = SPLIT; attr[1].val.clusterDim.y = 1; attr[1].val.clusterDim.z = 1;
-  cfg.gridDim = dim3((p.N + BN - 1) / BN * SPLIT, (p.M + kGemmBM - 1) / kGemmBM);
+  cfg.gridDim = dim3((p.N + BN - 1) / BN * SPLIT * set.count, (p.M + kGemmBM - 1) / kGemmBM);
   cfg.blockDim = dim3(kGemmThreads); cfg.dynamicSmemBytes = S::kTotal; cfg.stream = s;
   cfg.attrs = attr; cfg.numAttrs = SPLIT > 1 ? 2 : 1;
-  cudaLaunchKernelEx(&cfg, linear_kernel<BN, STAGES, SPLIT>, mx, mw, p);
+  cudaLaunchKernelEx(&cfg, linear_kernel<BN, STAGES, SPLIT, G>, mx, set, p);
   GRACE_LAUNCH_CHECK();
   return GRACE_OK;
 }
@@ -882,36 +900,37 @@ constexpr LinearForm kLinearForms[] = {
     {64, 1, 1, 2.9f, 0.245f}, {64, 2, 1, 3.1f, 0.25f}, {64, 4, 1, 3.0f, 0.28f},
     {128, 1, 1, 4.0f, 0.255f}, {128, 2, 1, 4.2f, 0.25f}, {128, 4, 1, 4.1f, 0.25f},
     {64, 1, 2, 4.2f, 0.28f}, {128, 1, 2, 5.0f, 0.46f}};                              // two CTAs per SM, three or four stages
-static grace_status_t run_linear(const LinearForm& f, const CUtensorMap& mx, const CUtensorMap& mw, const GemmParams& p, cudaStream_t s) {
+template <int G>
+static grace_status_t run_linear(const LinearForm& f, const CUtensorMap& mx, const GemmSet<G>& set, const GemmParams& p, cudaStream_t s) {
   switch (f.bn * 16 + f.split * 2 + f.per_sm - 1) {
-    case 32 * 16 + 2: return launch_linear<32, 8, 1>(mx, mw, p, s);
-    case 32 * 16 + 4: return launch_linear<32, 8, 2>(mx, mw, p, s);
-    case 64 * 16 + 2: return launch_linear<64, 8, 1>(mx, mw, p, s);
-    case 64 * 16 + 4: return launch_linear<64, 8, 2>(mx, mw, p, s);
-    case 64 * 16 + 8: return launch_linear<64, 8, 4>(mx, mw, p, s);
-    case 128 * 16 + 2: return launch_linear<128, 6, 1>(mx, mw, p, s);
-    case 128 * 16 + 4: return launch_linear<128, 4, 2>(mx, mw, p, s);
-    case 128 * 16 + 8: return launch_linear<128, 4, 4>(mx, mw, p, s);
-    case 64 * 16 + 3: return launch_linear<64, 4, 1>(mx, mw, p, s);
-    case 128 * 16 + 3: return launch_linear<128, 3, 1>(mx, mw, p, s);
+    case 32 * 16 + 2: return launch_linear<32, 8, 1, G>(mx, set, p, s);
+    case 32 * 16 + 4: return launch_linear<32, 8, 2, G>(mx, set, p, s);
+    case 64 * 16 + 2: return launch_linear<64, 8, 1, G>(mx, set, p, s);
+    case 64 * 16 + 4: return launch_linear<64, 8, 2, G>(mx, set, p, s);
+    case 64 * 16 + 8: return launch_linear<64, 8, 4, G>(mx, set, p, s);
+    case 128 * 16 + 2: return launch_linear<128, 6, 1, G>(mx, set, p, s);
+    case 128 * 16 + 4: return launch_linear<128, 4, 2, G>(mx, set, p, s);
+    case 128 * 16 + 8: return launch_linear<128, 4, 4, G>(mx, set, p, s);
+    case 64 * 16 + 3: return launch_linear<64, 4, 1, G>(mx, set, p, s);
+    case 128 * 16 + 3: return launch_linear<128, 3, 1, G>(mx, set, p, s);
   }
   return GRACE_UNSUPPORTED_SHAPE;
 }
 
 // stats_launch: the pair kernel would need the statistics kernel in front.  whole_k: no split of K, so that the sums are
 // those of the pair kernel bit for bit (fp32 products: grace_linear_f32_lse promises those of grace_linear).
-static LinearForm linear_form(int M, int N, int K, bool pair_possible, bool stats_launch, bool whole_k) {
+static LinearForm linear_form(int M, int N, int K, bool pair_possible, bool stats_launch, bool whole_k, int products = 1) {
   const int64_t tiles_m = (M + kGemmBM - 1) / kGemmBM;
   const int kb = K / kGemmBK;
   LinearForm best = {0, 0, 0, 0.f, 0.f};
   float least = 3.4e38f;
   if (pair_possible) {
-    const int64_t waves = ((int64_t)((M + 255) / 256) * ((N + 255) / 256) + 73) / 74;
+    const int64_t waves = ((int64_t)((M + 255) / 256) * ((N + 255) / 256) * products + 73) / 74;
     least = 2.7f + (float)waves * (1.0f + 0.33f * (float)kb) + (stats_launch ? 3.2f + 3.6e-7f * (float)M * (float)K : 0.f);
   }
   for (const LinearForm& f : kLinearForms) {
     if (f.split > kb || (whole_k && f.split > 1)) continue;
-    const int64_t ctas = tiles_m * ((N + f.bn - 1) / f.bn) * f.split;
+    const int64_t ctas = tiles_m * ((N + f.bn - 1) / f.bn) * f.split * products;
     const int wave = f.split == 1 ? 148 * f.per_sm : (f.split == 2 ? 144 : 132);       // clusters lie within a GPC
     const float t = (float)((ctas + wave - 1) / wave) * (f.fixed + f.per_kb * (float)((kb + f.split - 1) / f.split));
     if (t < least) { least = t; best = f; }
@@ -952,7 +971,9 @@ static grace_status_t linear_impl(const uint16_t* x, int64_t ldx, const uint16_t
                        aff.row != nullptr && !linear_narrow_centred(M, N, aff.cs), linear_whole_k(M, N, y_f32 != nullptr && residual == nullptr));
   if (form.bn == 0) {
     // large GEMM: persistent CTA-pair kernel, TMA-store epilogue (add-reduction when y is the residual stream)
-    CUtensorMap mx, mw, my;
+    CUtensorMap mx;
+    GemmSet<1> set;
+    set.count = 1;
     const uint64_t dx[2] = {(uint64_t)K, (uint64_t)M}, sx[1] = {(uint64_t)ldx};
     const uint32_t bx[2] = {(uint32_t)kPBK, 128u};
     const uint64_t dw[2] = {(uint64_t)K, (uint64_t)N}, sw[1] = {(uint64_t)ldw};
@@ -960,27 +981,29 @@ static grace_status_t linear_impl(const uint16_t* x, int64_t ldx, const uint16_t
     const uint64_t dy[2] = {(uint64_t)N, (uint64_t)M}, sy[1] = {(uint64_t)ldy};
     const bool f32 = (y_f32 != nullptr);
     const uint32_t by[2] = {f32 ? 32u : 64u, 128u};
-    if (!tc::make_tmap_bf16(&mx, x, 2, dx, sx, bx) || !tc::make_tmap_bf16(&mw, w, 2, dw, sw, bw) ||
-        !tc::make_tmap(&my, f32 ? (const void*)y_f32 : (const void*)y_bf16, 2, dy, sy, by, f32))
+    if (!tc::make_tmap_bf16(&mx, x, 2, dx, sx, bx) || !tc::make_tmap_bf16(&set.w[0], w, 2, dw, sw, bw) ||
+        !tc::make_tmap(&set.y[0], f32 ? (const void*)y_f32 : (const void*)y_bf16, 2, dy, sy, by, f32))
       return GRACE_CUDA_ERROR;
     if (aff.row != nullptr && (add_into_bf16 || aliased)) return GRACE_INVALID_ARG;
     if (allow_bits != nullptr)
-      return launch_pair<kOutF32LseAllowed>(mx, mw, my, M, N, K, relu, s, reinterpret_cast<float2*>(lse_part), aff,
+      return launch_pair<kOutF32LseAllowed>(mx, set, M, N, K, relu, s, reinterpret_cast<float2*>(lse_part), aff,
                                             AllowedStores{allow_bits, y_f32, ldy});
     if (aff.in_kernel_stats) {
       if (f32) return lse_part != nullptr
-                          ? launch_pair<kOutF32Lse, true>(mx, mw, my, M, N, K, relu, s, reinterpret_cast<float2*>(lse_part), aff)
-                          : launch_pair<kOutF32, true>(mx, mw, my, M, N, K, relu, s, nullptr, aff);
-      return launch_pair<kOutBf16, true>(mx, mw, my, M, N, K, relu, s, nullptr, aff);
+                          ? launch_pair<kOutF32Lse, true>(mx, set, M, N, K, relu, s, reinterpret_cast<float2*>(lse_part), aff)
+                          : launch_pair<kOutF32, true>(mx, set, M, N, K, relu, s, nullptr, aff);
+      return launch_pair<kOutBf16, true>(mx, set, M, N, K, relu, s, nullptr, aff);
     }
-    if (!f32) return add_into_bf16 ? launch_pair<kOutBf16Add>(mx, mw, my, M, N, K, relu, s)
-                                   : launch_pair<kOutBf16>(mx, mw, my, M, N, K, relu, s, nullptr, aff);
+    if (!f32) return add_into_bf16 ? launch_pair<kOutBf16Add>(mx, set, M, N, K, relu, s)
+                                   : launch_pair<kOutBf16>(mx, set, M, N, K, relu, s, nullptr, aff);
     if (lse_part != nullptr)
-      return launch_pair<kOutF32Lse>(mx, mw, my, M, N, K, relu, s, reinterpret_cast<float2*>(lse_part), aff);
-    if (aliased) return launch_pair<kOutF32Add>(mx, mw, my, M, N, K, relu, s);
-    return launch_pair<kOutF32>(mx, mw, my, M, N, K, relu, s, nullptr, aff);
+      return launch_pair<kOutF32Lse>(mx, set, M, N, K, relu, s, reinterpret_cast<float2*>(lse_part), aff);
+    if (aliased) return launch_pair<kOutF32Add>(mx, set, M, N, K, relu, s);
+    return launch_pair<kOutF32>(mx, set, M, N, K, relu, s, nullptr, aff);
   }
-  CUtensorMap mx, mw;
+  CUtensorMap mx;
+  GemmSet<1> set;
+  set.count = 1;
   {
     const uint64_t dims[2] = {(uint64_t)K, (uint64_t)M}, str[1] = {(uint64_t)ldx};
     const uint32_t box[2] = {(uint32_t)kGemmBK, (uint32_t)kGemmBM};
@@ -989,19 +1012,59 @@ static grace_status_t linear_impl(const uint16_t* x, int64_t ldx, const uint16_t
   {
     const uint64_t dims[2] = {(uint64_t)K, (uint64_t)N}, str[1] = {(uint64_t)ldw};
     const uint32_t box[2] = {(uint32_t)kGemmBK, (uint32_t)form.bn};
-    if (!tc::make_tmap_bf16(&mw, w, 2, dims, str, box)) return GRACE_CUDA_ERROR;
+    if (!tc::make_tmap_bf16(&set.w[0], w, 2, dims, str, box)) return GRACE_CUDA_ERROR;
   }
   GemmParams p;
   p.y_bf16 = y_bf16; p.y_f32 = y_f32; p.residual = residual; p.residual_bf16 = add_into_bf16 ? y_bf16 : nullptr;
   p.aff_row = aff.in_kernel_stats ? nullptr : aff.row; p.aff_cs = aff.cs; p.aff_cb = aff.cb; p.ln_eps = aff.eps; p.aff_out = aff.out;
   p.ldy = ldy; p.M = M; p.N = N; p.K = K; p.relu = relu;
-  return run_linear(form, mx, mw, p, s);
+  return run_linear<1>(form, mx, set, p, s);
 }
 
 extern "C" grace_status_t grace_linear(const uint16_t* x, int64_t ldx, const uint16_t* w, int64_t ldw,
                                        uint16_t* y_bf16, float* y_f32, int64_t ldy, const float* residual,
                                        int M, int N, int K, int relu, void* stream) {
   return linear_impl(x, ldx, w, ldw, y_bf16, y_f32, ldy, residual, false, M, N, K, relu, stream);
+}
+
+extern "C" grace_status_t grace_linear_multi(const uint16_t* x, int64_t ldx, int count, const uint16_t* const* w, int64_t ldw,
+                                             uint16_t* const* y_bf16, int64_t ldy, int M, int N, int K, void* stream) {
+  using namespace grace;
+  if (!x || !w || !y_bf16 || count <= 0 || M <= 0 || N <= 0 || K <= 0) return GRACE_INVALID_ARG;
+  if ((K % kGemmBK) || (N % 16)) return GRACE_UNSUPPORTED_SHAPE;
+  if (!grace_aligned16(x) || (ldx & 7) || (ldw & 7) || (ldy & 7) || ldx < K || ldw < K || ldy < N) return GRACE_INVALID_ARG;
+  for (int i = 0; i < count; ++i)
+    if (!w[i] || !y_bf16[i] || !grace_aligned16(w[i]) || !grace_aligned16(y_bf16[i])) return GRACE_INVALID_ARG;
+  cudaStream_t s = (cudaStream_t)stream;
+  for (int first = 0; first < count; first += kMultiMost) {
+    const int here = count - first < kMultiMost ? count - first : kMultiMost;
+    const LinearForm form = linear_form(M, N, K, linear_pair_possible(M, N, false), false, false, here);
+    CUtensorMap mx;
+    GemmSet<kMultiMost> set;
+    set.count = here;
+    const uint64_t dx[2] = {(uint64_t)K, (uint64_t)M}, sx[1] = {(uint64_t)ldx};
+    const uint64_t dw[2] = {(uint64_t)K, (uint64_t)N}, sw[1] = {(uint64_t)ldw};
+    const uint64_t dy[2] = {(uint64_t)N, (uint64_t)M}, sy[1] = {(uint64_t)ldy};
+    const uint32_t bx[2] = {64u, 128u}, by[2] = {64u, 128u};
+    const uint32_t bw[2] = {64u, form.bn == 0 ? 128u : (uint32_t)form.bn};
+    if (!tc::make_tmap_bf16(&mx, x, 2, dx, sx, bx)) return GRACE_CUDA_ERROR;
+    for (int i = 0; i < here; ++i) {
+      set.y_bf16[i] = y_bf16[first + i];
+      if (!tc::make_tmap_bf16(&set.w[i], w[first + i], 2, dw, sw, bw) ||
+          (form.bn == 0 && !tc::make_tmap_bf16(&set.y[i], y_bf16[first + i], 2, dy, sy, by)))
+        return GRACE_CUDA_ERROR;
+    }
+    grace_status_t st;
+    if (form.bn == 0) {
+      st = launch_pair<kOutBf16, false, kMultiMost>(mx, set, M, N, K, 0, s);
+    } else {
+      GemmParams p = {};
+      p.ldy = ldy; p.M = M; p.N = N; p.K = K;
+      st = run_linear<kMultiMost>(form, mx, set, p, s);
+    }
+    if (st != GRACE_OK) return st;
+  }
+  return GRACE_OK;
 }
 
 extern "C" grace_status_t grace_linear_f32_lse(const uint16_t* x, int64_t ldx, const uint16_t* w, int64_t ldw,

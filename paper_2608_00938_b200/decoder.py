@@ -215,9 +215,7 @@ class Decoder:
         """enc bf16 [B, T_ctx, d_enc] -> k_cross / v_cross [B, T_ctx, H, d_h] per layer."""
         B, T, d_enc = enc.shape
         x = enc.reshape(B * T, d_enc)
-        for li in range(self.n_layers):
-            api.grace_linear(x, self.w_kc[li], self.k_cross[li].view(B * T, -1))
-            api.grace_linear(x, self.w_vc[li], self.v_cross[li].view(B * T, -1))
+        api.grace_linear_multi(x, self.w_kc + self.w_vc, [y.view(B * T, -1) for y in self.k_cross + self.v_cross])
 
     def reset(self) -> None:
         """Start state (Section 3.3: M_0 = 1): start token, score 0, root node, empty key."""

@@ -123,3 +123,19 @@ def test_layer_norm_gemm_in_every_form(api, M, N, K, centred):
             api.grace_linear(x, w, r, residual=r)
             bound = 2.0 ** -19 * absolute + 2.0 ** -22 * want.abs()
         assert ((r.double() - want).abs() <= bound + 1e-30).all()
+
+
+@pytest.mark.parametrize("M,N,K,count", [(1, 64, 64, 2), (129, 512, 128, 4), (1024, 512, 512, 8), (2000, 512, 512, 9), (33, 528, 320, 17),
+                                         (9000, 256, 192, 8)])
+def test_linear_multi_is_the_single_products(api, M, N, K, count):
+    """Every product of grace_linear_multi against fp64 (fp32 sums, one rounding to bf16), with more products than a
+    launch takes, tiles that cut the last rows and columns, and neighbours' outputs that must stay apart."""
+    g = torch.Generator(device=DEV)
+    g.manual_seed(M + N + K)
+    x = torch.randn(M, K, device=DEV, generator=g).to(torch.bfloat16)
+    ws = [(torch.randn(N, K, device=DEV, generator=g) * 0.1).to(torch.bfloat16) for _ in range(count)]
+    ys = [torch.full((M, N), float("nan"), device=DEV, dtype=torch.bfloat16) for _ in range(count)]
+    api.grace_linear_multi(x, ws, ys)
+    for w, y in zip(ws, ys):
+        want, absolute = x.double() @ w.double().T, x.double().abs() @ w.double().abs().T
+        assert ((y.double() - want).abs() <= 2.0 ** -8 * want.abs() + 2.0 ** -19 * absolute + 1e-30).all()
