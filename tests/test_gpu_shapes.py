@@ -139,3 +139,21 @@ def test_linear_multi_is_the_single_products(api, M, N, K, count):
     for w, y in zip(ws, ys):
         want, absolute = x.double() @ w.double().T, x.double().abs() @ w.double().abs().T
         assert ((y.double() - want).abs() <= 2.0 ** -8 * want.abs() + 2.0 ** -19 * absolute + 1e-30).all()
+
+
+# a (row, head) pair on its own: 32, 8 and 1 warps per pair at every head size that takes them; slices of the positions that
+# some warps or lane groups have none of; a last CTA with fewer pairs than it has warps
+@pytest.mark.parametrize("B,M,H,d,T", [(1, 1, 8, 64, 1030), (2, 3, 5, 128, 513), (1, 16, 4, 32, 700), (1, 8, 8, 64, 5), (3, 2, 2, 128, 1),
+                                       (2, 100, 3, 32, 37), (7, 61, 3, 32, 129), (4, 300, 1, 32, 1)])
+def test_cross_attn_pairs(api, B, M, H, d, T):
+    rng = synth.rng_for(2, 1400 + M + T)
+    q, k, v = (synth.normal_bf16(rng, s) for s in ((B, M, H, d), (B, H, T, d), (B, H, T, d)))
+    ref, lse_ref = OA.cross_attn(f64(q), f64(k), f64(v), d ** -0.5)
+    out = torch.full((B * M, H, d), 7.0, dtype=torch.bfloat16, device=DEV)
+    lse = torch.zeros((B * M, H), dtype=torch.float32, device=DEV)
+    api.grace_cross_attn(dev_bf16(q).reshape(B * M, H, d), dev_bf16(k), dev_bf16(v), out, d ** -0.5, lse)
+    torch.cuda.synchronize()
+    # fp32 throughout: the output's rounding to bf16 alone
+    got = out.double().cpu().numpy().reshape(B, M, H, d)
+    assert (np.abs(got - ref) <= 2.0 ** -8 * np.abs(ref) + 1e-5).all()
+    np.testing.assert_allclose(lse.cpu().numpy().reshape(B, M, H), lse_ref, atol=1e-4, rtol=0)
