@@ -21,7 +21,7 @@
 // therefore never wait for P V: they hand P of a block over and go on to the next block (whose S the tensor
 // core produced under their exponentials), and an item's output is read from TMEM and stored one block later.
 // A 128-wide tile is held as two 64-wide halves (the 128-byte swizzle spans 64 bf16), each with its own TMA
-// box and its own MMA k-steps (Q, K) or output-column half (V).
+// box and its own MMA k-steps (Q, K) or half of the output columns (V: one MMA spans both).
 #pragma once
 #include "common.cuh"
 #include "tc.cuh"
@@ -258,12 +258,12 @@ cross_attn_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_con
     // ---------------- MMA issuer ----------------
     if (lane == 0) {
       constexpr uint32_t idesc_s = tc::idesc_bf16(kCaBM, kCaBN, 0);     // Q K^T : B K-major
-      constexpr uint32_t idesc_o = tc::idesc_bf16(kCaBM, 64, 1);        // P V   : B MN-major, 64 output columns at a time
+      constexpr uint32_t idesc_o = tc::idesc_bf16(kCaBM, DH, 1);        // P V   : B MN-major, all output columns at once
       // Every operand descriptor is fixed by (Q buffer, ring slot, k-step): build them once.  The
       // issuing thread shares its scheduler with busy softmax warps, so each instruction it does not
       // execute per block shortens the hand-off to the tensor core.
       // k-step k of Q or K: 16 of the DH columns = 32 bytes inside the 64-wide half (k / 4)
-      uint64_t q_desc[kQBufs][DH / 16], k_desc[kCaStages][DH / 16], v_desc[kCaStages][kHalves][kCaBN / 16];
+      uint64_t q_desc[kQBufs][DH / 16], k_desc[kCaStages][DH / 16], v_desc[kCaStages][kCaBN / 16];
 #pragma unroll
       for (int i = 0; i < kQBufs; ++i)
 #pragma unroll
@@ -274,11 +274,10 @@ cross_attn_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_con
 #pragma unroll
         for (int k = 0; k < DH / 16; ++k)
           k_desc[st][k] = tc::smem_desc_sw128(tc::smem_addr(kv_tiles + (2 * st) * kCaTileBytes) + (k / 4) * kCaHalfBytes + 32 * (k % 4), 16, 1024);
+        // (the second 64-wide half of V's columns lies kCaHalfBytes further)
 #pragma unroll
-        for (int hf = 0; hf < kHalves; ++hf)
-#pragma unroll
-          for (int k = 0; k < kCaBN / 16; ++k)
-            v_desc[st][hf][k] = tc::smem_desc_sw128(tc::smem_addr(kv_tiles + (2 * st + 1) * kCaTileBytes) + hf * kCaHalfBytes + 2048 * k, 1024, 1024);
+        for (int k = 0; k < kCaBN / 16; ++k)
+          v_desc[st][k] = tc::smem_desc_sw128(tc::smem_addr(kv_tiles + (2 * st + 1) * kCaTileBytes) + 2048 * k, kHalves > 1 ? kCaHalfBytes : 1024, 1024);
       }
       // S of global block g: Q buffer of its item, K of ring slot g % stages
       auto issue_s = [&](int g, const CaCursor<SPLIT>& c) -> bool {
@@ -329,22 +328,16 @@ cross_attn_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_con
         const uint32_t o_acc = tmem_o + (uint32_t)((li & 1) * DH), p_cols = tmem_p + (uint32_t)(P32 ? 0 : (g & 1) * 64);
         if (s == 0) {
 #pragma unroll
-          for (int hf = 0; hf < kHalves; ++hf)
-#pragma unroll
-            for (int k = 0; k < kCaBN / 16; ++k)
-              {
-                tc::mma_ts(o_acc + 64 * hf, p_cols + 8 * k, v_desc[0][hf][k], idesc_o, (j | k) ? 1u : 0u);
-                if (P32) tc::mma_ts(o_acc + 64 * hf, p_cols + 64 + 8 * k, v_desc[0][hf][k], idesc_o, 1u);
-              }
+          for (int k = 0; k < kCaBN / 16; ++k) {
+            tc::mma_ts(o_acc, p_cols + 8 * k, v_desc[0][k], idesc_o, (j | k) ? 1u : 0u);
+            if (P32) tc::mma_ts(o_acc, p_cols + 64 + 8 * k, v_desc[0][k], idesc_o, 1u);
+          }
         } else {
 #pragma unroll
-          for (int hf = 0; hf < kHalves; ++hf)
-#pragma unroll
-            for (int k = 0; k < kCaBN / 16; ++k)
-              {
-                tc::mma_ts(o_acc + 64 * hf, p_cols + 8 * k, v_desc[1][hf][k], idesc_o, (j | k) ? 1u : 0u);
-                if (P32) tc::mma_ts(o_acc + 64 * hf, p_cols + 64 + 8 * k, v_desc[1][hf][k], idesc_o, 1u);
-              }
+          for (int k = 0; k < kCaBN / 16; ++k) {
+            tc::mma_ts(o_acc, p_cols + 8 * k, v_desc[1][k], idesc_o, (j | k) ? 1u : 0u);
+            if (P32) tc::mma_ts(o_acc, p_cols + 64 + 8 * k, v_desc[1][k], idesc_o, 1u);
+          }
         }
         tc::mma_commit(v_empty + s);                         // V of block g is consumed
         tc::mma_commit(o_full + (g & 1));                    // O includes block g
