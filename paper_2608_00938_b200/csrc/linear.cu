@@ -894,12 +894,17 @@ static grace_status_t launch_linear(const CUtensorMap& mx, const GemmSet<G>& set
 // tiles without a split), LayerNorm included: 512 x 1536 x 512: 10.3 -> 5.8 us, 512 x 2048 x 512: 10.5 -> 6.1,
 // 512 x 512 x 2048: 10.3 -> 5.8, 16 x 512 x 2048: 9.9 -> 4.3, 1024 x 512 x 2048: 13.1 -> 7.1, 1024 x 512 x 512:
 // 7.6 -> 5.0, 2048 x 512 x 2048: 13.1 -> 9.1.
-struct LinearForm { int bn, split, per_sm; float fixed, per_kb; };     // bn = 0: the CTA-pair kernel
+// Rows beyond the problem's last cost no exchange and no stores: both parts grow from few rows to a full tile of 128.
+struct LinearForm {
+  int bn, split, per_sm;                   // bn = 0: the CTA-pair kernel
+  float fixed, per_kb;                     // with few rows
+  float fixed_rows, per_kb_rows;           // added with 128 rows or more
+};
 constexpr LinearForm kLinearForms[] = {
-    {32, 1, 1, 2.3f, 0.24f}, {32, 2, 1, 2.7f, 0.24f},                                // whole K range in flight
-    {64, 1, 1, 2.9f, 0.245f}, {64, 2, 1, 3.1f, 0.25f}, {64, 4, 1, 3.0f, 0.28f},
-    {128, 1, 1, 4.0f, 0.255f}, {128, 2, 1, 4.2f, 0.25f}, {128, 4, 1, 4.1f, 0.25f},
-    {64, 1, 2, 4.2f, 0.28f}, {128, 1, 2, 5.0f, 0.46f}};                              // two CTAs per SM, three or four stages
+    {32, 1, 1, 1.9f, 0.243f, 0.1f, 0.f}, {32, 2, 1, 2.35f, 0.235f, 0.4f, 0.02f},     // whole K range in flight
+    {64, 1, 1, 2.35f, 0.243f, 0.4f, 0.f}, {64, 2, 1, 2.55f, 0.236f, 0.7f, 0.014f}, {64, 4, 1, 2.4f, 0.233f, 0.9f, 0.08f},
+    {128, 1, 1, 3.25f, 0.245f, 0.85f, 0.f}, {128, 2, 1, 3.15f, 0.246f, 1.2f, 0.f}, {128, 4, 1, 2.95f, 0.237f, 1.4f, 0.01f},
+    {64, 1, 2, 3.85f, 0.318f, 0.f, 0.f}, {128, 1, 2, 5.0f, 0.46f, 0.f, 0.f}};        // two CTAs per SM, three or four stages
 template <int G>
 static grace_status_t run_linear(const LinearForm& f, const CUtensorMap& mx, const GemmSet<G>& set, const GemmParams& p, cudaStream_t s) {
   switch (f.bn * 16 + f.split * 2 + f.per_sm - 1) {
@@ -922,7 +927,8 @@ static grace_status_t run_linear(const LinearForm& f, const CUtensorMap& mx, con
 static LinearForm linear_form(int M, int N, int K, bool pair_possible, bool stats_launch, bool whole_k, int products = 1) {
   const int64_t tiles_m = (M + kGemmBM - 1) / kGemmBM;
   const int kb = K / kGemmBK;
-  LinearForm best = {0, 0, 0, 0.f, 0.f};
+  LinearForm best = {};
+  const float rows = M < kGemmBM ? (float)M / (float)kGemmBM : 1.f;
   float least = 3.4e38f;
   if (pair_possible) {
     const int64_t waves = ((int64_t)((M + 255) / 256) * ((N + 255) / 256) * products + 73) / 74;
@@ -932,7 +938,8 @@ static LinearForm linear_form(int M, int N, int K, bool pair_possible, bool stat
     if (f.split > kb || (whole_k && f.split > 1)) continue;
     const int64_t ctas = tiles_m * ((N + f.bn - 1) / f.bn) * f.split * products;
     const int wave = f.split == 1 ? 148 * f.per_sm : (f.split == 2 ? 144 : 132);       // clusters lie within a GPC
-    const float t = (float)((ctas + wave - 1) / wave) * (f.fixed + f.per_kb * (float)((kb + f.split - 1) / f.split));
+    const float t = (float)((ctas + wave - 1) / wave) * (f.fixed + rows * f.fixed_rows +
+                                                         (f.per_kb + rows * f.per_kb_rows) * (float)((kb + f.split - 1) / f.split));
     if (t < least) { least = t; best = f; }
   }
   return best;
@@ -965,7 +972,7 @@ static grace_status_t linear_impl(const uint16_t* x, int64_t ldx, const uint16_t
     return GRACE_UNSUPPORTED_SHAPE;
   if (allow_bits != nullptr && (lse_part == nullptr || (reinterpret_cast<uintptr_t>(allow_bits) & 15)))
     return GRACE_UNSUPPORTED_SHAPE;                          // allowed-only stores exist in the large-problem kernel only
-  LinearForm form = {0, 0, 0, 0.f, 0.f};
+  LinearForm form = {};
   if (lse_part == nullptr)
     form = linear_form(M, N, K, linear_pair_possible(M, N, residual != nullptr && !aliased),
                        aff.row != nullptr && !linear_narrow_centred(M, N, aff.cs), linear_whole_k(M, N, y_f32 != nullptr && residual == nullptr));
