@@ -63,6 +63,7 @@ struct CrossMsParams {
   int64_t out_row_stride;
   int B, M, H, T;
   int pairs_m, total_items;     // 256-row items per (request, head); items = B * H * pairs_m
+  int full_m, full_items;       // of them with two live tiles; B * H * full_m
   float scale_log2;             // scale * log2(e)
 };
 
@@ -78,11 +79,15 @@ __device__ __forceinline__ float ms_max3(float a, float b, float c) {
 }
 
 // One 256-row item: request, head, first query row, encoder positions, blocks, live tiles.
+// Items whose rows fill one tile only (the last of a (request, head) whose M leaves 1 .. 128 rows) come after all others:
+// the second stream of a half takes no part in them and counts neither their blocks nor their phases of the ring, so it
+// must not meet an item with two tiles afterwards.
 struct MsItem { int b, h, row0, T, nb, ntiles; };
 __device__ __forceinline__ MsItem ms_item(const CrossMsParams& p, int item) {
   MsItem it;
-  const int bh = item / p.pairs_m;
-  const int pair = item - bh * p.pairs_m;
+  const bool full = item < p.full_items;
+  const int bh = full ? item / p.full_m : item - p.full_items;
+  const int pair = full ? item - bh * p.full_m : p.full_m;
   it.b = bh / p.H;
   it.h = bh - it.b * p.H;
   it.row0 = pair * 2 * kMsBM;
@@ -494,6 +499,8 @@ inline grace_status_t launch_cross_attn_ms(const uint16_t* q, int64_t q_row_stri
   const int64_t items = (int64_t)p.pairs_m * H * B;
   if (items > 0x3fffffff) return GRACE_UNSUPPORTED_SHAPE;
   p.total_items = (int)items;
+  p.full_m = (M + kMsBM - 1) / (2 * kMsBM);                  // (an item has a second tile from its 129th row on)
+  p.full_items = p.full_m * H * B;
   p.scale_log2 = scale * 1.4426950408889634f;
   const int grid = (int)(items < n_sm ? items : n_sm);
   launch_pdl(cross_attn_ms_kernel, dim3(grid), dim3(kMsThreads), kMsSmemBytes, s, mq, mk, mv, mo, p);

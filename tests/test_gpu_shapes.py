@@ -157,3 +157,30 @@ def test_cross_attn_pairs(api, B, M, H, d, T):
     got = out.double().cpu().numpy().reshape(B, M, H, d)
     assert (np.abs(got - ref) <= 2.0 ** -8 * np.abs(ref) + 1e-5).all()
     np.testing.assert_allclose(lse.cpu().numpy().reshape(B, M, H), lse_ref, atol=1e-4, rtol=0)
+
+
+# head size 64 beyond one tile per SM (the four-stream kernel), several items per half, the last rows of a request in one
+# tile of two: items with one live tile and with two in the same half
+@pytest.mark.parametrize("B,M,H,T", [(16, 600, 8, 130), (20, 300, 8, 200), (13, 1100, 5, 70), (30, 100, 10, 65)])
+@pytest.mark.parametrize("lengths", [False, True])
+def test_cross_attn_items_with_one_tile_and_with_two(api, B, M, H, T, lengths):
+    d = 64
+    rng = synth.rng_for(2, 1500 + M + T)
+    q, k, v = (synth.normal_bf16(rng, s) for s in ((B, M, H, d), (B, H, T, d), (B, H, T, d)))
+    enc_len = np.minimum(np.array([T, 0, 1, 64, T - 1, 65, 0, 63] * B)[:B], T).astype(np.int32)
+    out = torch.full((B * M, H, d), 7.0, dtype=torch.bfloat16, device=DEV)
+    lse = torch.zeros((B * M, H), dtype=torch.float32, device=DEV)
+    args = dev_bf16(q).reshape(B * M, H, d), dev_bf16(k), dev_bf16(v), out
+    if lengths:
+        ref, lse_ref = OA.cross_attn_varlen(f64(q), f64(k), f64(v), enc_len, d ** -0.5)
+        api.grace_cross_attn_varlen(*args, dev(enc_len), d ** -0.5, lse)
+    else:
+        ref, lse_ref = OA.cross_attn(f64(q), f64(k), f64(v), d ** -0.5)
+        api.grace_cross_attn(*args, d ** -0.5, lse)
+    torch.cuda.synchronize()
+    assert api.grace_wait_timeouts() == 0
+    got, got_lse = out.float().cpu().numpy().reshape(B, M, H, d), lse.cpu().numpy().reshape(B, M, H)
+    assert_attention_close(got, ref, "one tile and two")
+    some = enc_len > 0 if lengths else np.ones(B, bool)
+    assert (got[~some] == 0).all() and np.isneginf(got_lse[~some]).all()
+    np.testing.assert_allclose(got_lse[some], lse_ref[some], atol=2e-3, rtol=0)
