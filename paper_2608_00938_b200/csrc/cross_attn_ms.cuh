@@ -35,7 +35,8 @@
 //     them with a TMA store per warp (rows beyond M are clipped by the tensor map).
 //
 // Ragged M and T are zero-filled by TMA and masked in the softmax; `enc_len` (optional) gives a
-// per-request number of valid encoder positions (0: the output rows are zero).  Every wait is
+// per-request number of valid encoder positions (0: the output rows are zero), and what lies past it has no
+// influence whatever it holds: scores are masked, rows of V cleared before P V reads them.  Every wait is
 // bounded (tc::mbar_wait); a wait that gives up sets the CTA's abort flag, every role leaves its
 // loops, TMEM is freed and the kernel returns.
 #pragma once
@@ -411,6 +412,18 @@ cross_attn_ms_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_con
         l_run = fmaf(l_run, alpha, (s0 + s1) + (s2 + s3));
 #pragma unroll
         for (int c = 0; c < kMsBN / 2; c += 16) tc::tmem_st16(tmem_s + c, *reinterpret_cast<uint32_t(*)[16]>(&r[c]));
+        // Positions past the request's length: their probabilities are 0, but 0 times what the padding holds (NaN, Inf) is
+        // not, so this stream clears those rows of V in the ring slot before its P V.  (The half's other stream
+        // clears them too; the tile is its own again only after both.  Past p.T the loads left zeros.)
+        if (valid < kMsBN && it.T < p.T) {
+          const uint32_t slot = g % kMsStages;                      // a stream takes part in every block of its half so far
+          ok = tc::mbar_wait_likely_done(kv_full + hf * kMsStages + slot, (g / kMsStages) & 1, abort_flag);
+          ok = __all_sync(kFullMask, ok);
+          if (!ok) break;
+          uint4* v_rows = reinterpret_cast<uint4*>(kv_tiles + (hf * kMsStages + (int)slot) * 2 * kMsKVBytes + kMsKVBytes);
+          for (int i = valid * 8 + row; i < kMsBN * 8; i += kMsBM) v_rows[i] = make_uint4(0u, 0u, 0u, 0u);
+          tc::fence_proxy_async_smem();
+        }
         tc::tmem_st_wait();
         tc::tc_fence_before();
         __syncwarp();

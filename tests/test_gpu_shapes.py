@@ -184,3 +184,24 @@ def test_cross_attn_items_with_one_tile_and_with_two(api, B, M, H, T, lengths):
     some = enc_len > 0 if lengths else np.ones(B, bool)
     assert (got[~some] == 0).all() and np.isneginf(got_lse[~some]).all()
     np.testing.assert_allclose(got_lse[some], lse_ref[some], atol=2e-3, rtol=0)
+
+
+# the four-stream kernel (head size 64, more than one tile per SM)
+PADDED = [(20, 300, 8, 64, 200), (16, 600, 8, 64, 130)]
+
+
+@pytest.mark.parametrize("B,M,H,d,T", PADDED)
+@pytest.mark.parametrize("padding", [float("nan"), float("inf")])
+def test_cross_attn_padding_has_no_influence_whatever_it_holds(api, B, M, H, d, T, padding):
+    """K and V past a request's length: NaN or infinities there give the bits that zeros give."""
+    rng = synth.rng_for(2, 1600 + M + T)
+    q, k, v = (dev_bf16(synth.normal_bf16(rng, s)) for s in ((B * M, H, d), (B, H, T, d), (B, H, T, d)))
+    enc_len = np.minimum(np.array([T, 0, 1, 64, T - 1, 65, 17, 127, 128, 15] * B)[:B], T).astype(np.int32)
+    past = torch.arange(T, device=DEV)[None, None, :, None] >= dev(enc_len)[:, None, None, None]
+    results = []
+    for fill in (0.0, padding):
+        out, lse = torch.empty_like(q), torch.empty(B * M, H, device=DEV)
+        api.grace_cross_attn_varlen(q, k.masked_fill(past, fill), v.masked_fill(past, fill), out, dev(enc_len), d ** -0.5, lse)
+        results.append((out, lse))
+    assert not results[0][0].isnan().any()
+    assert torch.equal(results[0][0], results[1][0]) and torch.equal(results[0][1], results[1][1])
