@@ -14,7 +14,7 @@
 // K and V blocks arrive by TMA through two separate two-slot rings; Q, K and V are addressed with 4-D tensor
 // maps over the caller's strides, so the beam-major Q / O layout is never permuted (the view /
 // permute / reshape chain of Section 5.1 costs nothing).  Ragged M and T are zero-filled by TMA
-// and masked in the softmax.  Warp roles: softmax + epilogue warps first, then the TMA producer warp, then
+// and masked in the softmax; K and V past a request's length have no influence whatever they hold.  Warp roles: softmax + epilogue warps first, then the TMA producer warp, then
 // the MMA issuer warp.
 // The kernel is persistent (each CTA loops over work items; Q is double-buffered), one CTA per SM with all
 // 512 TMEM columns: S (128), O twice (by item parity) and P twice (by block parity).  The softmax threads
@@ -313,6 +313,7 @@ cross_attn_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_con
       bool ok = cs.live(p) && issue_s(0, cs);
       for (int g = 0; ok; ++g) {
         const int s = g & 1, j = cs.j, li = cs.li;
+        const int left = cs.it.T - j * kCaBN;                // positions of the request from this block on
         cs.next(p);
         const bool more = cs.live(p);
         // s_free(g): every softmax thread holds its scores of block g in registers, so the S
@@ -326,7 +327,14 @@ cross_attn_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_con
         if (!tc::mbar_wait(v_full + s, (g >> 1) & 1, abort_flag)) break;
         tc::tc_fence_after();
         const uint32_t o_acc = tmem_o + (uint32_t)((li & 1) * DH), p_cols = tmem_p + (uint32_t)(P32 ? 0 : (g & 1) * 64);
-        if (s == 0) {
+        if (left <= kCaBN - 16) {                            // (on its own: a test per k-step slows the full blocks)
+          const uint64_t v0 = s == 0 ? v_desc[0][0] : v_desc[1][0];
+#pragma unroll 1
+          for (int k = 0; 16 * k < left; ++k) {
+            tc::mma_ts(o_acc, p_cols + 8 * k, v0 + (uint64_t)(k * 2048 / 16), idesc_o, (j | k) ? 1u : 0u);
+            if (P32) tc::mma_ts(o_acc, p_cols + 64 + 8 * k, v0 + (uint64_t)(k * 2048 / 16), idesc_o, 1u);
+          }
+        } else if (s == 0) {
 #pragma unroll
           for (int k = 0; k < kCaBN / 16; ++k) {
             tc::mma_ts(o_acc, p_cols + 8 * k, v_desc[0][k], idesc_o, (j | k) ? 1u : 0u);
@@ -527,6 +535,23 @@ cross_attn_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_con
             uint32_t (&o1)[16] = *reinterpret_cast<uint32_t(*)[16]>(&o[16]);
             tc::tmem_st16(o_acc + lane_addr + kOutCols * half + c, o0);
             tc::tmem_st16(o_acc + lane_addr + kOutCols * half + c + 16, o1);
+          }
+        }
+        // Positions past the request's length: their probabilities are 0, but 0 times what the padding holds (NaN, Inf) is
+        // not.  P V leaves out whole k-steps of them; the rest of a k-step's rows of V is cleared here.  (Past p.T the
+        // loads left zeros.)  16 x 1000 x 16 x 128 x 50..200: 57.5 us without, 59.2 so; cleared by the issuing thread
+        // 62, by a warp of its own 64, not loaded at all (boxes of 64, 32 .. 1 rows) 65; without leaving k-steps out 61.
+        const int left = it.T - j * kCaBN;
+        if (left < kCaBN && it.t0 + it.T < p.T && (left & 15) != 0) {
+          ok = tc::mbar_wait(v_full + (g & 1), (g >> 1) & 1, abort_flag);
+          ok = __all_sync(kFullMask, ok);
+          if (!ok) break;
+          const int i = left * 8 + (int)threadIdx.x;          // 16-byte pieces of the half's 128-byte rows
+          if (i < ((left + 15) & ~15) * 8) {
+#pragma unroll
+            for (int hf = 0; hf < kHalves; ++hf)
+              reinterpret_cast<uint4*>(kv_tiles + (2 * (g & 1) + 1) * kCaTileBytes + hf * kCaHalfBytes)[i] = make_uint4(0u, 0u, 0u, 0u);
+            tc::fence_proxy_async_smem();
           }
         }
         tc::tmem_st_wait();

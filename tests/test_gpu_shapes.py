@@ -186,8 +186,12 @@ def test_cross_attn_items_with_one_tile_and_with_two(api, B, M, H, T, lengths):
     np.testing.assert_allclose(got_lse[some], lse_ref[some], atol=2e-3, rtol=0)
 
 
-# the four-stream kernel (head size 64, more than one tile per SM)
-PADDED = [(20, 300, 8, 64, 200), (16, 600, 8, 64, 130)]
+# the four-stream kernel (head size 64, more than one tile per SM); the one-stream kernel: head size 128, items of a CTA
+# alone and shared by clusters of two and four (CTAs of them without any block), head size 64 shared by two and four, few
+# rows per request with more pairs than the pair kernel takes; a (row, head) pair per CTA and per warp
+PADDED = [(20, 300, 8, 64, 200), (16, 600, 8, 64, 130), (10, 257, 8, 128, 300), (10, 20, 7, 128, 700), (10, 130, 1, 128, 1100),
+          (10, 130, 3, 64, 300), (10, 40, 3, 64, 600), (20, 8, 8, 64, 200), (20, 8, 8, 128, 200), (10, 2, 3, 64, 200),
+          (10, 5, 3, 32, 200), (10, 200, 3, 32, 130), (10, 1, 3, 128, 530)]
 
 
 @pytest.mark.parametrize("B,M,H,d,T", PADDED)
