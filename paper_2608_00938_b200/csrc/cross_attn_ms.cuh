@@ -59,7 +59,7 @@ constexpr int kMsSmemBytes = 1024 + 8 * kMsQBytes + 2 * kMsStages * 2 * kMsKVByt
 
 struct CrossMsParams {
   float* lse;
-  const int32_t* enc_len;       // nullable: valid encoder positions per request (<= T)
+  const int32_t* enc_len;       // LENGTHS: valid encoder positions per request (<= T)
   uint16_t* out;                // only for rows without any encoder position (written as zeros)
   int64_t out_row_stride;
   int B, M, H, T;
@@ -84,6 +84,7 @@ __device__ __forceinline__ float ms_max3(float a, float b, float c) {
 // the second stream of a half takes no part in them and counts neither their blocks nor their phases of the ring, so it
 // must not meet an item with two tiles afterwards.
 struct MsItem { int b, h, row0, T, nb, ntiles; };
+template <bool LENGTHS>
 __device__ __forceinline__ MsItem ms_item(const CrossMsParams& p, int item) {
   MsItem it;
   const bool full = item < p.full_items;
@@ -93,13 +94,15 @@ __device__ __forceinline__ MsItem ms_item(const CrossMsParams& p, int item) {
   it.h = bh - it.b * p.H;
   it.row0 = pair * 2 * kMsBM;
   int t = p.T;
-  if (p.enc_len != nullptr) { const int e = __ldg(p.enc_len + it.b); t = e < 0 ? 0 : (e < t ? e : t); }
+  if (LENGTHS) { const int e = __ldg(p.enc_len + it.b); t = e < 0 ? 0 : (e < t ? e : t); }
   it.T = t;
   it.nb = (t + kMsBN - 1) / kMsBN;
   it.ntiles = p.M - it.row0 > kMsBM ? 2 : 1;
   return it;
 }
 
+// LENGTHS: per-request lengths are given (without them the loop that decides the pace does not carry their code: 1 to 2 %).
+template <bool LENGTHS>
 __global__ void __launch_bounds__(kMsThreads, 1)
 cross_attn_ms_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant__ CUtensorMap map_k,
                      const __grid_constant__ CUtensorMap map_v, const __grid_constant__ CUtensorMap map_o,
@@ -168,7 +171,7 @@ cross_attn_ms_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_con
     // ---- loads ----
     int lq_item = first_item(hf), lq_cnt = 0;           // Q: next item to look at; tiles requested
     int lk_item = lq_item, lk_j = 0, lk_cnt = 0;                  // K/V (first stream of the half only): item, block, blocks requested
-    MsItem lk_it = lk_item < p.total_items ? ms_item(p, lk_item) : MsItem{0, 0, 0, 0, 0, 0};
+    MsItem lk_it = lk_item < p.total_items ? ms_item<LENGTHS>(p, lk_item) : MsItem{0, 0, 0, 0, 0, 0};
     MsItem lq_it = lk_it;                                          // an item is decoded when a queue moves on to it
     auto refill = [&]() -> bool {
       bool progressed = false;
@@ -189,13 +192,13 @@ cross_attn_ms_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_con
         }
         if (advance) {
           lq_item += item_step; progressed = true;
-          if (lq_item < p.total_items) lq_it = ms_item(p, lq_item);
+          if (lq_item < p.total_items) lq_it = ms_item<LENGTHS>(p, lq_item);
         }
       }
       if (tile == 0 && lk_item < p.total_items) {
         if (lk_j >= lk_it.nb) {
           lk_item += item_step; lk_j = 0; progressed = true;
-          if (lk_item < p.total_items) lk_it = ms_item(p, lk_item);
+          if (lk_item < p.total_items) lk_it = ms_item<LENGTHS>(p, lk_item);
         } else {
           const int slot = lk_cnt % kMsStages;
           if (tc::mbar_try_wait_now(kve + slot, ((lk_cnt / kMsStages) & 1) ^ 1)) {
@@ -236,7 +239,7 @@ cross_attn_ms_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_con
     auto seek = [&](Cursor& c) {
       c.u = 0; c.nb = 0;
       while (c.item < p.total_items) {
-        const MsItem it = ms_item(p, c.item);
+        const MsItem it = ms_item<LENGTHS>(p, c.item);
         if (tile < it.ntiles && it.nb > 0) { c.nb = it.nb; return; }
         c.item += item_step;
       }
@@ -332,7 +335,7 @@ cross_attn_ms_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_con
       }
     };
     for (int item = first_item(hf); ok && item < p.total_items; item += item_step) {
-      const MsItem it = ms_item(p, item);
+      const MsItem it = ms_item<LENGTHS>(p, item);
       if (tile >= it.ntiles) continue;
       const int m = it.row0 + tile * kMsBM + row;
       const bool row_live = m < p.M;
@@ -415,7 +418,7 @@ cross_attn_ms_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_con
         // Positions past the request's length: their probabilities are 0, but 0 times what the padding holds (NaN, Inf) is
         // not, so this stream clears those rows of V in the ring slot before its P V.  (The half's other stream
         // clears them too; the tile is its own again only after both.  Past p.T the loads left zeros.)
-        if (valid < kMsBN && it.T < p.T) {
+        if (LENGTHS && valid < kMsBN && it.T < p.T) {
           const uint32_t slot = g % kMsStages;                      // a stream takes part in every block of its half so far
           ok = tc::mbar_wait_likely_done(kv_full + hf * kMsStages + slot, (g / kMsStages) & 1, abort_flag);
           ok = __all_sync(kFullMask, ok);
@@ -500,7 +503,8 @@ inline grace_status_t launch_cross_attn_ms(const uint16_t* q, int64_t q_row_stri
   static int n_sm_of[kMaxDevices] = {0};
   DeviceSetup su(&attr_set_devices);
   if (su) {
-    GRACE_CUDA_TRY(cudaFuncSetAttribute(cross_attn_ms_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kMsSmemBytes));
+    GRACE_CUDA_TRY(cudaFuncSetAttribute(cross_attn_ms_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, kMsSmemBytes));
+    GRACE_CUDA_TRY(cudaFuncSetAttribute(cross_attn_ms_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, kMsSmemBytes));
     GRACE_CUDA_TRY(cudaDeviceGetAttribute(&n_sm_of[su.dev], cudaDevAttrMultiProcessorCount, su.dev));
     su.done();
   }
@@ -516,7 +520,7 @@ inline grace_status_t launch_cross_attn_ms(const uint16_t* q, int64_t q_row_stri
   p.full_items = p.full_m * H * B;
   p.scale_log2 = scale * 1.4426950408889634f;
   const int grid = (int)(items < n_sm ? items : n_sm);
-  launch_pdl(cross_attn_ms_kernel, dim3(grid), dim3(kMsThreads), kMsSmemBytes, s, mq, mk, mv, mo, p);
+  launch_pdl(enc_len != nullptr ? cross_attn_ms_kernel<true> : cross_attn_ms_kernel<false>, dim3(grid), dim3(kMsThreads), kMsSmemBytes, s, mq, mk, mv, mo, p);
   GRACE_LAUNCH_CHECK();
   return GRACE_OK;
 }
