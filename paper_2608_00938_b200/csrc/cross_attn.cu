@@ -96,7 +96,11 @@ cross_attn_row_kernel(const CrossRowParams p) {
       if (t0 + u * RP + grp >= t_end) d[u] = -INFINITY;
       m_new = fmaxf(m_new, d[u]);
     }
-    if (m_new > -INFINITY) {                                // (a group past the slice's end has seen nothing yet)
+    if (m_new == -INFINITY) {
+      // a group past the slice's end, or scores of -inf only: no weight yet; but a maximum drops NaN, the sum must not
+#pragma unroll
+      for (int u = 0; u < U; ++u) if (d[u] != d[u]) l_run = d[u];
+    } else {
       const float corr = __expf(m_run - m_new);              // 0 the first time (m_run = -inf)
       l_run *= corr;
 #pragma unroll
@@ -132,12 +136,12 @@ cross_attn_row_kernel(const CrossRowParams p) {
     for (int i = 0; i < 8; ++i) acc[i] += __shfl_xor_sync(kFullMask, acc[i], o);
   }
   if (WARPS == 1) {
-    const float inv = l_run > 0.f ? 1.f / l_run : 0.f;      // no encoder position: the output is defined as zero
+    const float inv = T > 0 ? 1.f / l_run : 0.f;            // no encoder position: the output is defined as zero
     if (grp == 0)
       *reinterpret_cast<uint4*>(p.out + (int64_t)r * p.out_row_stride + h * DH + piece * 8) =
           make_uint4(pack_bf16x2(acc[0] * inv, acc[1] * inv), pack_bf16x2(acc[2] * inv, acc[3] * inv),
                      pack_bf16x2(acc[4] * inv, acc[5] * inv), pack_bf16x2(acc[6] * inv, acc[7] * inv));
-    if (p.lse != nullptr && lane == 0) p.lse[(int64_t)r * p.H + h] = l_run > 0.f ? m_w + logf(l_run) : -INFINITY;
+    if (p.lse != nullptr && lane == 0) p.lse[(int64_t)r * p.H + h] = T > 0 ? m_w + logf(l_run) : -INFINITY;
     return;
   }
   if (grp == 0) {
@@ -159,9 +163,9 @@ cross_attn_row_kernel(const CrossRowParams p) {
     float o = 0.f;
 #pragma unroll
     for (int s2 = 0; s2 < WARPS; ++s2) o = fmaf(st_acc[s2][threadIdx.x], __shfl_sync(kFullMask, f, s2), o);
-    __nv_bfloat16 ob = __float2bfloat16_rn(l_all > 0.f ? o / l_all : 0.f);    // no encoder position: zero by definition
+    __nv_bfloat16 ob = __float2bfloat16_rn(T > 0 ? o / l_all : 0.f);    // no encoder position: zero by definition
     p.out[(int64_t)r * p.out_row_stride + h * DH + threadIdx.x] = *reinterpret_cast<uint16_t*>(&ob);
-    if (p.lse != nullptr && threadIdx.x == 0) p.lse[(int64_t)r * p.H + h] = l_all > 0.f ? m_all + logf(l_all) : -INFINITY;
+    if (p.lse != nullptr && threadIdx.x == 0) p.lse[(int64_t)r * p.H + h] = T > 0 ? m_all + logf(l_all) : -INFINITY;
   }
 }
 

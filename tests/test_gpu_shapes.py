@@ -209,3 +209,40 @@ def test_cross_attn_padding_has_no_influence_whatever_it_holds(api, B, M, H, d, 
         results.append((out, lse))
     assert not results[0][0].isnan().any()
     assert torch.equal(results[0][0], results[1][0]) and torch.equal(results[0][1], results[1][1])
+
+
+# a (row, head) pair on 32, 8 and 1 warps; lane groups whose positions are all NaN, and others that saw none
+NAN_SHAPES = [(1, 2, 3, 64, 700), (2, 3, 2, 128, 20), (5, 100, 3, 32, 40), (64, 5, 3, 64, 9)]
+
+
+@pytest.mark.parametrize("B,M,H,d,T", NAN_SHAPES)
+@pytest.mark.parametrize("lengths", [False, True])
+def test_cross_attn_does_not_hide_nan(api, B, M, H, d, T, lengths):
+    """A NaN in a query row, a NaN key and a score that overflows to +inf leave NaN in the outputs and the log-sum-exp they
+    have a part in, whichever kernel runs, and nothing in the others: not the zeros of a request without positions."""
+    rng = synth.rng_for(2, 1700 + M + T)
+    q, k, v = (dev_bf16(synth.normal_bf16(rng, s)) for s in ((B * M, H, d), (B, H, T, d), (B, H, T, d)))
+    enc_len = torch.full((B,), T, device=DEV, dtype=torch.int32)
+
+    def run(q, k):
+        out, lse = torch.zeros_like(q), torch.zeros(B * M, H, device=DEV)
+        if lengths:
+            api.grace_cross_attn_varlen(q, k, v, out, enc_len, d ** -0.5, lse)
+        else:
+            api.grace_cross_attn(q, k, v, out, d ** -0.5, lse)
+        return out, lse
+
+    good, good_lse = run(q, k)
+    assert good.isfinite().all() and good_lse.isfinite().all()
+    bad_q = q.clone()
+    bad_q[M - 1, 0, 3] = float("nan")                                    # one row of request 0, one head
+    bad_k = k.clone()
+    bad_k[0, 0, T - 1, 5] = float("nan")
+    big_q, big_k = q.clone(), k.clone()
+    big_q[:M, 0, 1], big_k[0, 0, T // 2, :], big_k[0, 0, T // 2, 1] = 64.0, 0.0, 3e38
+    for case, (out, lse), rows in (("query", run(bad_q, k), slice(M - 1, M)), ("key", run(q, bad_k), slice(0, M)),
+                                   ("overflow", run(big_q, big_k), slice(0, M))):
+        hit = torch.zeros(B * M, H, dtype=torch.bool, device=DEV)
+        hit[rows, 0] = True
+        assert out[hit].isnan().all() and lse[hit].isnan().all(), case
+        assert torch.equal(out[~hit], good[~hit]) and torch.equal(lse[~hit], good_lse[~hit]), case
