@@ -69,9 +69,10 @@ cross_attn_row_kernel(const CrossRowParams p) {
 #pragma unroll
     for (int u = 0; u < U; ++u) {
       const int t = t0 + u * RP + grp;
-      const int64_t off = (int64_t)(t < t_end ? t : t_begin) * p.kv_stride_t;
-      kd[u] = __ldg(reinterpret_cast<const uint4*>(kb + off));
-      vd[u] = __ldg(reinterpret_cast<const uint4*>(vb + off));
+      const int64_t off = (int64_t)t * p.kv_stride_t;
+      // (past the slice zeros: a weight of 0 times an infinite value of some other position would be NaN)
+      kd[u] = t < t_end ? __ldg(reinterpret_cast<const uint4*>(kb + off)) : make_uint4(0u, 0u, 0u, 0u);
+      vd[u] = t < t_end ? __ldg(reinterpret_cast<const uint4*>(vb + off)) : make_uint4(0u, 0u, 0u, 0u);
     }
   };
   if (kAhead && t_begin < t_end) fetch(t_begin, kk, vv);

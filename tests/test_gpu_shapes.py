@@ -246,3 +246,19 @@ def test_cross_attn_does_not_hide_nan(api, B, M, H, d, T, lengths):
         hit[rows, 0] = True
         assert out[hit].isnan().all() and lse[hit].isnan().all(), case
         assert torch.equal(out[~hit], good[~hit]) and torch.equal(lse[~hit], good_lse[~hit]), case
+
+
+@pytest.mark.parametrize("B,M,H,d,T", [(1, 2, 3, 64, 5), (2, 3, 2, 128, 21), (5, 100, 3, 32, 7), (1, 1, 2, 64, 515)])
+def test_cross_attn_pairs_with_an_infinite_value(api, B, M, H, d, T):
+    """An infinite value at any one position gives the infinity in its column and leaves the other columns alone: no lane
+    that has run out of positions multiplies it with a weight of zero."""
+    rng = synth.rng_for(2, 1800 + M + T)
+    q, k, v = (dev_bf16(synth.normal_bf16(rng, s)) for s in ((B * M, H, d), (B, H, T, d), (B, H, T, d)))
+    good, out = torch.zeros_like(q), torch.zeros_like(q)
+    api.grace_cross_attn(q, k, v, good, d ** -0.5)
+    for t in sorted({0, 1, T // 2, T - 1}):
+        w = v.clone()
+        w[:, :, t, 2] = float("inf")
+        api.grace_cross_attn(q, k, w, out, d ** -0.5)
+        assert (out[:, :, 2] == float("inf")).all()
+        assert torch.equal(out[:, :, 3:], good[:, :, 3:]) and torch.equal(out[:, :, :2], good[:, :, :2])
