@@ -625,7 +625,7 @@ cross_attn_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_con
         w[s] = w[s] == -INFINITY ? 0.f : ex2(w[s] - m_all);
         l_all = fmaf(mlbuf[s * 128 + row].y, w[s], l_all);
       }
-      const float inv = l_all > 0.f ? 1.f / l_all : 0.f;       // no encoder position: the output is defined as zero
+      const float inv = l_all == 0.f ? 0.f : 1.f / l_all;      // no encoder position: the output is defined as zero (NaN stays)
       const int m = pend_it.tile * kCaBM + row;
       const int64_t r_out = (int64_t)pend_it.b * p.M + m;
       const bool live = ok && m < p.M;
@@ -657,7 +657,7 @@ cross_attn_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_con
         }
       }
       if (live && p.lse != nullptr && rank == 0 && half == 0)
-        p.lse[r_out * p.H + pend_it.h] = l_all > 0.f ? (m_all + log2f(l_all)) * 0.6931471805599453f : -INFINITY;
+        p.lse[r_out * p.H + pend_it.h] = l_all == 0.f ? -INFINITY : (m_all + log2f(l_all)) * 0.6931471805599453f;
       tc::tc_fence_before();
     }
   }

@@ -211,8 +211,11 @@ def test_cross_attn_padding_has_no_influence_whatever_it_holds(api, B, M, H, d, 
     assert torch.equal(results[0][0], results[1][0]) and torch.equal(results[0][1], results[1][1])
 
 
-# a (row, head) pair on 32, 8 and 1 warps; lane groups whose positions are all NaN, and others that saw none
-NAN_SHAPES = [(1, 2, 3, 64, 700), (2, 3, 2, 128, 20), (5, 100, 3, 32, 40), (64, 5, 3, 64, 9)]
+# a (row, head) pair on 32, 8 and 1 warps; lane groups whose positions are all NaN, and others that saw none; the
+# one-stream kernel alone and in clusters of two and four at both head sizes; the four-stream kernel
+NAN_SHAPES = [(1, 2, 3, 64, 700), (2, 3, 2, 128, 20), (5, 100, 3, 32, 40), (64, 5, 3, 64, 9), (2, 130, 3, 128, 130),
+              (2, 130, 3, 128, 600), (2, 130, 3, 128, 1100), (2, 40, 3, 64, 100), (30, 40, 2, 64, 200), (2, 40, 3, 64, 600),
+              (20, 300, 8, 64, 100)]
 
 
 @pytest.mark.parametrize("B,M,H,d,T", NAN_SHAPES)
