@@ -238,13 +238,18 @@ extern "C" grace_status_t grace_cross_attn_varlen(const uint16_t* q, int64_t q_r
   if (cross_attn_tc_supported(B, M, H, d_h, T_ctx)) {
     // probabilities as before the tensor cores took these over: fp32 (see cross_attn_tc_kernel)
     const bool p32 = enc_len != nullptr && (d_h == 128 || M <= 8);
+    // ... and any stride and any scale: what a tensor map cannot say (negative and huge strides) and scales that are not
+    // positive (the softmax threads take the maximum before they scale) still run on the CUDA cores.
+    if (p32 && !(scale >= 1e-30f)) return run_pairs(false);
     const int form = cross_attn_form(B, M, H, d_h, T_ctx, p32);
     if (form == 0)
       return launch_cross_attn_ms(q, q_row_stride, k, v, kv_stride_b, kv_stride_h, kv_stride_t, out,
                                   out_row_stride, lse, enc_len, B, M, H, T_ctx, scale, s);
-    return (d_h == 64 ? launch_cross_attn_tc<64> : launch_cross_attn_tc<128>)(
+    const grace_status_t st = (d_h == 64 ? launch_cross_attn_tc<64> : launch_cross_attn_tc<128>)(
         q, q_row_stride, k, v, kv_stride_b, kv_stride_h, kv_stride_t, out, out_row_stride, lse, enc_len, B, M, H, T_ctx,
         scale, form, p32, s);
+    if (p32 && st == GRACE_UNSUPPORTED_SHAPE) return run_pairs(false);
+    return st;
   }
   return run_pairs(false);
 }

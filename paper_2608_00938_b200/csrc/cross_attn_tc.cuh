@@ -702,7 +702,8 @@ inline grace_status_t launch_cross_attn_tc_form(const CUtensorMap& mq, const CUt
   return GRACE_OK;
 }
 
-// split: how many CTAs share a work item (1, 2 or 4); p32: fp32-like probabilities (above).
+// split: how many CTAs share a work item (1, 2 or 4); p32: fp32-like probabilities (above).  GRACE_UNSUPPORTED_SHAPE, with
+// nothing launched: too many items, or (p32) strides that a tensor map cannot express.
 template <int DH>
 inline grace_status_t launch_cross_attn_tc(const uint16_t* q, int64_t q_row_stride, const uint16_t* k,
                                            const uint16_t* v, int64_t kv_stride_b, int64_t kv_stride_h,
@@ -710,18 +711,19 @@ inline grace_status_t launch_cross_attn_tc(const uint16_t* q, int64_t q_row_stri
                                            const int32_t* enc_len, int B, int M, int H, int T_ctx, float scale, int split, bool p32,
                                            cudaStream_t s) {
   CUtensorMap mq, mk, mv;
+  const grace_status_t no_map = p32 ? GRACE_UNSUPPORTED_SHAPE : GRACE_CUDA_ERROR;
   {
     const uint64_t dims[4] = {(uint64_t)DH, (uint64_t)H, (uint64_t)M, (uint64_t)B};
     const uint64_t str[3] = {(uint64_t)DH, (uint64_t)q_row_stride, (uint64_t)M * (uint64_t)q_row_stride};
     const uint32_t box[4] = {64u, 1u, (uint32_t)kCaBM, 1u};
-    if (!tc::make_tmap_bf16(&mq, q, 4, dims, str, box)) return GRACE_CUDA_ERROR;
+    if (!tc::make_tmap_bf16(&mq, q, 4, dims, str, box)) return no_map;
   }
   {
     const uint64_t dims[4] = {(uint64_t)DH, (uint64_t)T_ctx, (uint64_t)H, (uint64_t)B};
     const uint64_t str[3] = {(uint64_t)kv_stride_t, (uint64_t)kv_stride_h, (uint64_t)kv_stride_b};
     const uint32_t box[4] = {64u, (uint32_t)kCaBN, 1u, 1u};
-    if (!tc::make_tmap_bf16(&mk, k, 4, dims, str, box)) return GRACE_CUDA_ERROR;
-    if (!tc::make_tmap_bf16(&mv, v, 4, dims, str, box)) return GRACE_CUDA_ERROR;
+    if (!tc::make_tmap_bf16(&mk, k, 4, dims, str, box)) return no_map;
+    if (!tc::make_tmap_bf16(&mv, v, 4, dims, str, box)) return no_map;
   }
   CrossTcParams p;
   p.out = out; p.lse = lse; p.enc_len = enc_len; p.out_row_stride = out_row_stride; p.B = B; p.M = M; p.H = H; p.T = T_ctx;

@@ -265,3 +265,34 @@ def test_cross_attn_pairs_with_an_infinite_value(api, B, M, H, d, T):
         api.grace_cross_attn(q, k, w, out, d ** -0.5)
         assert (out[:, :, 2] == float("inf")).all()
         assert torch.equal(out[:, :, 3:], good[:, :, 3:]) and torch.equal(out[:, :, :2], good[:, :, :2])
+
+
+@pytest.mark.parametrize("B,M,H,d,T", [(3, 40, 2, 128, 150), (4, 20, 9, 128, 300), (20, 8, 8, 64, 70)])
+@pytest.mark.parametrize("form", ["shared context", "shared heads", "heads backwards", "no scale", "negative scale"])
+def test_cross_attn_lengths_with_any_strides_and_scale(api, B, M, H, d, T, form):
+    """Calls with lengths take strides of zero, negative strides (which no tensor map can express) and scales that are not
+    positive."""
+    rng = synth.rng_for(2, 1900 + M + T)
+    kvB, kvH = 1 if form == "shared context" else B, 1 if form == "shared heads" else H
+    q, k, v = (synth.normal_bf16(rng, s) for s in ((B, M, H, d), (kvB, kvH, T, d), (kvB, kvH, T, d)))
+    enc_len = np.minimum(np.array([T, 0, 1, 128, T - 1, 65] * B)[:B], T).astype(np.int32)
+    scale = {"no scale": 0.0, "negative scale": -(d ** -0.5)}.get(form, d ** -0.5)
+    kr, vr = (np.broadcast_to(f64(a), (B, H, T, d)) for a in (k, v))
+    if form == "heads backwards":
+        kr, vr = kr[:, ::-1], vr[:, ::-1]
+    ref, lse_ref = OA.cross_attn_varlen(f64(q), kr, vr, enc_len, scale)
+    qd, kd, vd, lens = dev_bf16(q).reshape(B * M, H, d), dev_bf16(k), dev_bf16(v), dev(enc_len)
+    out, lse = torch.full_like(qd, 7.0), torch.zeros(B * M, H, device=DEV)
+    if form == "heads backwards":
+        last = [a[0, H - 1].data_ptr() for a in (kd, vd)]
+        st = api._cross_attn_varlen(qd.data_ptr(), H * d, *last, H * T * d, -T * d, d, out.data_ptr(), H * d, lse.data_ptr(),
+                                    lens.data_ptr(), B, M, H, d, T, scale, None, torch.cuda.current_stream().cuda_stream)
+        assert st == api.GRACE_OK
+    else:
+        api.grace_cross_attn_varlen(qd, kd.expand(B, H, T, d), vd.expand(B, H, T, d), out, lens, scale, lse)
+    torch.cuda.synchronize()
+    some = enc_len > 0
+    got, got_lse = out.float().cpu().numpy().reshape(B, M, H, d), lse.cpu().numpy().reshape(B, M, H)
+    assert_attention_close(got, ref, form)
+    assert (got[~some] == 0).all()
+    np.testing.assert_allclose(got_lse[some], lse_ref[some], atol=2e-3, rtol=0)
