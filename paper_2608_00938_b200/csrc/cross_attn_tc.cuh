@@ -1,6 +1,6 @@
 // Cross-attention on tcgen05 tensor cores (Section 5.1: beams of a request are the M dimension of
-// a dense contraction against that request's shared K/V).  Written for head size 64 or 128; the library
-// uses it for head size 128 (head size 64 runs the four-stream kernel of cross_attn_ms.cuh).
+// a dense contraction against that request's shared K/V): head size 128, and head size 64 with at most one
+// 128-row tile per SM or with lengths and few rows per request (otherwise the four-stream kernel of cross_attn_ms.cuh).
 //
 // A work item is 128 query rows of one (request, head); its encoder positions are streamed in
 // blocks of 128:
@@ -32,10 +32,8 @@ constexpr int kCaBM = 128;        // query rows per work item
 constexpr int kCaBN = 128;        // encoder positions per block
 constexpr int kCaStages = 2;
 constexpr int kCaHalfBytes = 128 * 64 * 2;                       // 16 KB: 128 rows x 64 bf16, one swizzle span wide
-// TPR = softmax threads per query row: 2 (eight softmax warps, each thread half of a block's columns) or
-// 1 (four softmax warps, a thread owns the whole row: no exchange between threads, half as many trips
-// through the TMEM load / barrier / TMEM store sequence per exponential; 168 registers).  Head size 64
-// runs TPR = 1 (4 % faster at 32 x 2048 x 1024); head size 128 keeps TPR = 2 for its wider output rows.
+constexpr int kCaSoftmaxWarps = 8;   // two threads per query row: each half of a block's score columns and of the output columns
+constexpr int kCaThreads = (kCaSoftmaxWarps + 2) * 32;
 constexpr int kCaBarBytes = 256;
 // SPLIT > 1: a cluster of SPLIT CTAs shares one work item, each taking a contiguous range of its K / V blocks; the
 // partial results (unnormalised output, maximum and sum per row) are merged through distributed shared memory:
@@ -117,7 +115,7 @@ __device__ __forceinline__ float max3(float a, float b, float c) {
   return m;
 }
 
-// Persistent kernel: a flat grid of two CTAs per SM; CTA g takes the work items g, g + gridDim.x,
+// Persistent kernel: a flat grid of one CTA per SM; CTA g takes the work items g, g + gridDim.x,
 // ...  An item is one (request, head, 128-row tile); consecutive items are the tiles of the same
 // (request, head), so the CTAs running at the same time read the same K/V from L2.
 // P32: the probabilities keep (at least) sixteen bits of their fp32 mantissa: P is stored as the sum of two bf16 values
@@ -125,12 +123,11 @@ __device__ __forceinline__ float max3(float a, float b, float c) {
 // once P V of the block before it is complete.  Calls with per-request lengths run this form: they were computed with
 // fp32 probabilities before the tensor cores took them over, and one bf16 rounding of P shows in the result
 // (relative error against 64 bits 2.2e-3 instead of the output rounding's 1.7e-3).
-template <int DH, int TPR, int SPLIT, bool P32>
-__global__ void __launch_bounds__((4 * TPR + 2) * 32, 1)
+template <int DH, int SPLIT, bool P32>
+__global__ void __launch_bounds__(kCaThreads, 1)
 cross_attn_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant__ CUtensorMap map_k,
                      const __grid_constant__ CUtensorMap map_v, const CrossTcParams p) {
-  constexpr int kCaSoftmaxWarps = 4 * TPR;
-  constexpr int kCols = kCaBN / TPR;                       // score columns per softmax thread and block
+  constexpr int kCols = kCaBN / 2;                         // score columns per softmax thread and block
   constexpr int kCaTileBytes = CaCfg<DH, SPLIT>::kTileBytes, kHalves = CaCfg<DH, SPLIT>::kHalves;
   constexpr uint32_t kCaTmemCols = CaCfg<DH, SPLIT>::kTmemCols;
   constexpr int kQBufs = CaCfg<DH, SPLIT>::kQBufs, kSlice = CaCfg<DH, SPLIT>::kSlice;
@@ -362,7 +359,7 @@ cross_attn_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_con
     const int row = quarter * 32 + lane;
     const uint32_t lane_addr = (uint32_t)(quarter * 32) << 16;
     const int col_base = kCols * half;
-    constexpr int kOutCols = DH / TPR;                     // output columns per thread
+    constexpr int kOutCols = DH / 2;                       // output columns per thread
     bool ok = true;
     int g = 0, n_done = 0, li = 0;
     // the item whose output is still to be read from TMEM and stored (after the next block's P hand-over)
@@ -384,13 +381,10 @@ cross_attn_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_con
       for (int c = 0; c < kOutCols; c += 32)
         tc::tmem_ld32(o_acc + lane_addr + kOutCols * half + c, *reinterpret_cast<uint32_t(*)[32]>(&o[c]));
       tc::tmem_ld_wait();
-      float l_tot = l_e;
-      if (TPR == 2) {
-        float* hs = half_sum + (n_done & 1) * 256;            // double-buffered by item parity
-        hs[half * 128 + row] = l_e;
-        tc::named_bar_sync(2 + quarter, 64);
-        l_tot += hs[(half ^ 1) * 128 + row];
-      }
+      float* hs = half_sum + (n_done & 1) * 256;              // double-buffered by item parity
+      hs[half * 128 + row] = l_e;
+      tc::named_bar_sync(2 + quarter, 64);
+      const float l_tot = l_e + hs[(half ^ 1) * 128 + row];
       ++n_done;
       const int m = tile * kCaBM + row;
       if (m < p.M) {
@@ -474,12 +468,10 @@ cross_attn_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_con
         mx0 = max3(mx0, __uint_as_float(r[kCols - 4]), __uint_as_float(r[kCols - 3]));
         mx1 = max3(mx1, __uint_as_float(r[kCols - 2]), __uint_as_float(r[kCols - 1]));
         float mx = fmaxf(max3(mx0, mx1, mx2), mx3);
-        if (TPR == 2) {
-          float* hm = half_max + (g & 1) * 256;
-          hm[half * 128 + row] = mx;
-          tc::named_bar_sync(2 + quarter, 64);                // the two warps of this row quarter
-          mx = fmaxf(mx, hm[(half ^ 1) * 128 + row]);
-        }
+        float* hm = half_max + (g & 1) * 256;
+        hm[half * 128 + row] = mx;
+        tc::named_bar_sync(2 + quarter, 64);                  // the two warps of this row quarter
+        mx = fmaxf(mx, hm[(half ^ 1) * 128 + row]);
         const float m_blk = mx * p.scale_log2;
         const bool grow = m_blk > m_run + 8.0f;               // always true on an item's first block
         const float m_new = grow ? m_blk : m_run;
@@ -576,12 +568,9 @@ cross_attn_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_con
       const int rank = (int)tc::cluster_cta_rank();
       const bool have = pend_g >= 0;                          // this CTA had blocks of the item
       if (have) { ok = wait_pv(pend_g) && ok; tc::tc_fence_after(); }
-      float l_tot = pend_l;
-      if (TPR == 2) {
-        half_sum[half * 128 + row] = pend_l;
-        tc::named_bar_sync(2 + quarter, 64);
-        l_tot += half_sum[(half ^ 1) * 128 + row];
-      }
+      half_sum[half * 128 + row] = pend_l;
+      tc::named_bar_sync(2 + quarter, 64);
+      const float l_tot = pend_l + half_sum[(half ^ 1) * 128 + row];
       const float2 ml = make_float2(have ? pend_m : -INFINITY, have ? l_tot : 0.f);
       __syncwarp();
       asm volatile("barrier.cluster.wait.aligned;" ::: "memory");        // the other CTAs have started
@@ -601,7 +590,7 @@ cross_attn_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_con
         const int dst = (rank + o) % SPLIT, slot = rank < dst ? rank : rank - 1;
 #pragma unroll 1
         for (int c = 0; c < kPieces; ++c) {
-          if (TPR == 2 && ((c + o) & 1) != half) continue;
+          if (((c + o) & 1) != half) continue;
           uint32_t v[16];
           read_o(dst * kSlice + 16 * c, v);
           const uint32_t remote = tc::cluster_addr_of(xbuf + (slot * (kSlice / 4) + 4 * c) * 128 + row, (uint32_t)dst);
@@ -631,7 +620,7 @@ cross_attn_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_con
       const bool live = ok && m < p.M;
 #pragma unroll 1
       for (int c = 0; c < kPieces; ++c) {
-        if (TPR == 2 && (c & 1) != half) continue;
+        if ((c & 1) != half) continue;
         uint32_t own[16];
         read_o(rank * kSlice + 16 * c, own);
         float v[16];
@@ -675,7 +664,7 @@ inline bool cross_attn_tc_supported(int B, int M, int H, int d_h, int T_ctx) {
   return (d_h == 64 || d_h == 128) && H <= 65535 && B <= 65535 && T_ctx >= 1 && M >= 1;
 }
 
-template <int DH, int TPR, int SPLIT, bool P32>
+template <int DH, int SPLIT, bool P32>
 inline grace_status_t launch_cross_attn_tc_form(const CUtensorMap& mq, const CUtensorMap& mk, const CUtensorMap& mv,
                                                 const CrossTcParams& p, int items, cudaStream_t s) {
   constexpr int kCaSmemBytes = CaCfg<DH, SPLIT>::kSmemBytes;
@@ -683,7 +672,7 @@ inline grace_status_t launch_cross_attn_tc_form(const CUtensorMap& mq, const CUt
   static int n_sm_of[kMaxDevices] = {0};
   DeviceSetup su(&attr_set_devices);
   if (su) {
-    GRACE_CUDA_TRY(cudaFuncSetAttribute(cross_attn_tc_kernel<DH, TPR, SPLIT, P32>, cudaFuncAttributeMaxDynamicSharedMemorySize, kCaSmemBytes));
+    GRACE_CUDA_TRY(cudaFuncSetAttribute(cross_attn_tc_kernel<DH, SPLIT, P32>, cudaFuncAttributeMaxDynamicSharedMemorySize, kCaSmemBytes));
     GRACE_CUDA_TRY(cudaDeviceGetAttribute(&n_sm_of[su.dev], cudaDevAttrMultiProcessorCount, su.dev));
     su.done();
   }
@@ -695,9 +684,9 @@ inline grace_status_t launch_cross_attn_tc_form(const CUtensorMap& mq, const CUt
   attr[1].id = cudaLaunchAttributeClusterDimension;
   attr[1].val.clusterDim.x = SPLIT; attr[1].val.clusterDim.y = 1; attr[1].val.clusterDim.z = 1;
   cfg.gridDim = dim3(SPLIT > 1 ? items * SPLIT : (items < n_sm ? items : n_sm));
-  cfg.blockDim = dim3((4 * TPR + 2) * 32); cfg.dynamicSmemBytes = kCaSmemBytes; cfg.stream = s;
+  cfg.blockDim = dim3(kCaThreads); cfg.dynamicSmemBytes = kCaSmemBytes; cfg.stream = s;
   cfg.attrs = attr; cfg.numAttrs = SPLIT > 1 ? 2 : 1;
-  cudaLaunchKernelEx(&cfg, cross_attn_tc_kernel<DH, TPR, SPLIT, P32>, mq, mk, mv, p);
+  cudaLaunchKernelEx(&cfg, cross_attn_tc_kernel<DH, SPLIT, P32>, mq, mk, mv, p);
   GRACE_LAUNCH_CHECK();
   return GRACE_OK;
 }
@@ -734,13 +723,15 @@ inline grace_status_t launch_cross_attn_tc(const uint16_t* q, int64_t q_row_stri
   p.scale_log2 = scale * 1.4426950408889634f;
   const int n = (int)items;
   if (p32) {
-    if (split == 4) return launch_cross_attn_tc_form<DH, 2, 4, true>(mq, mk, mv, p, n, s);
-    if (split == 2) return launch_cross_attn_tc_form<DH, 2, 2, true>(mq, mk, mv, p, n, s);
-    return launch_cross_attn_tc_form<DH, 2, 1, true>(mq, mk, mv, p, n, s);
+    if constexpr (DH == 128) {                               // (at head size 64 these are more items than SMs)
+      if (split == 4) return launch_cross_attn_tc_form<DH, 4, true>(mq, mk, mv, p, n, s);
+      if (split == 2) return launch_cross_attn_tc_form<DH, 2, true>(mq, mk, mv, p, n, s);
+    }
+    return launch_cross_attn_tc_form<DH, 1, true>(mq, mk, mv, p, n, s);
   }
-  if (split == 4) return launch_cross_attn_tc_form<DH, 2, 4, false>(mq, mk, mv, p, n, s);
-  if (split == 2) return launch_cross_attn_tc_form<DH, 2, 2, false>(mq, mk, mv, p, n, s);
-  return launch_cross_attn_tc_form<DH, 2, 1, false>(mq, mk, mv, p, n, s);
+  if (split == 4) return launch_cross_attn_tc_form<DH, 4, false>(mq, mk, mv, p, n, s);
+  if (split == 2) return launch_cross_attn_tc_form<DH, 2, false>(mq, mk, mv, p, n, s);
+  return launch_cross_attn_tc_form<DH, 1, false>(mq, mk, mv, p, n, s);
 }
 
 }  // namespace grace
