@@ -52,7 +52,7 @@ template <int DH, int SPLIT> struct CaCfg {
 struct CrossTcParams {
   uint16_t* out;
   float* lse;
-  const int32_t* enc_len;       // nullable: valid encoder positions per request (<= T)
+  const int32_t* enc_len;       // LENGTHS: valid encoder positions per request (<= T)
   int64_t out_row_stride;
   int B, M, H, T;
   int tiles_m, total_items;
@@ -64,7 +64,7 @@ struct CrossTcParams {
 // and the MMAs and written as zeros by the epilogue warps.
 // With SPLIT > 1 an item is a CTA's share of one: nb blocks from position t0 on (T counts from there).
 struct CaItem { int b, h, tile, t0, T, nb; };
-template <int SPLIT>
+template <int SPLIT, bool LENGTHS>
 __device__ __forceinline__ CaItem ca_item(const CrossTcParams& p, int item) {
   CaItem it;
   const int part = item % SPLIT;
@@ -74,7 +74,7 @@ __device__ __forceinline__ CaItem ca_item(const CrossTcParams& p, int item) {
   it.b = bh / p.H;
   it.h = bh - it.b * p.H;
   it.T = p.T;
-  if (p.enc_len != nullptr) { const int e = __ldg(p.enc_len + it.b); it.T = e < 0 ? 0 : (e < p.T ? e : p.T); }
+  if (LENGTHS) { const int e = __ldg(p.enc_len + it.b); it.T = e < 0 ? 0 : (e < p.T ? e : p.T); }
   it.nb = (it.T + kCaBN - 1) / kCaBN;
   it.t0 = 0;
   if (SPLIT > 1) {
@@ -86,14 +86,14 @@ __device__ __forceinline__ CaItem ca_item(const CrossTcParams& p, int item) {
   return it;
 }
 // A position in that sequence: item, its place among the CTA's non-empty items (li), block inside the item.
-template <int SPLIT>
+template <int SPLIT, bool LENGTHS>
 struct CaCursor {
   int item, li, j;
   CaItem it;
   __device__ __forceinline__ bool live(const CrossTcParams& p) const { return item < p.total_items; }
   __device__ __forceinline__ void seek(const CrossTcParams& p) {       // to the first non-empty item from here on
     for (; item < p.total_items; item += (int)gridDim.x) {
-      it = ca_item<SPLIT>(p, item);
+      it = ca_item<SPLIT, LENGTHS>(p, item);
       if (it.nb > 0) return;
     }
   }
@@ -123,7 +123,8 @@ __device__ __forceinline__ float max3(float a, float b, float c) {
 // once P V of the block before it is complete.  Calls with per-request lengths run this form: they were computed with
 // fp32 probabilities before the tensor cores took them over, and one bf16 rounding of P shows in the result
 // (relative error against 64 bits 2.2e-3 instead of the output rounding's 1.7e-3).
-template <int DH, int SPLIT, bool P32>
+// LENGTHS: per-request lengths are given (without them no code for them: it costs a split call 2 to 3 %).
+template <int DH, int SPLIT, bool P32, bool LENGTHS>
 __global__ void __launch_bounds__(kCaThreads, 1)
 cross_attn_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant__ CUtensorMap map_k,
                      const __grid_constant__ CUtensorMap map_v, const CrossTcParams p) {
@@ -200,7 +201,7 @@ cross_attn_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_con
       // requested as soon as S of block g has run, long before the V slot of block g frees, so the
       // thread polls: whichever slot is free next gets its load, neither queue blocks the other.
       int gk = 0, gv = 0;                                    // next K block, next V block (counted over the CTA's items)
-      CaCursor<SPLIT> ck, cv;
+      CaCursor<SPLIT, LENGTHS> ck, cv;
       ck.start(p);
       cv = ck;
       int idle = 0;
@@ -277,7 +278,7 @@ cross_attn_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_con
           v_desc[st][k] = tc::smem_desc_sw128(tc::smem_addr(kv_tiles + (2 * st + 1) * kCaTileBytes) + 2048 * k, kHalves > 1 ? kCaHalfBytes : 1024, 1024);
       }
       // S of global block g: Q buffer of its item, K of ring slot g % stages
-      auto issue_s = [&](int g, const CaCursor<SPLIT>& c) -> bool {
+      auto issue_s = [&](int g, const CaCursor<SPLIT, LENGTHS>& c) -> bool {
         const int qb = c.li & 1, s = g % kCaStages;
         if (c.j == 0 && !tc::mbar_wait(q_full + qb, (c.li >> 1) & 1, abort_flag)) return false;
         if (!tc::mbar_wait(k_full + s, (g / kCaStages) & 1, abort_flag)) return false;
@@ -305,7 +306,7 @@ cross_attn_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_con
         return true;
       };
       static_assert(kCaStages == 2, "descriptor selection below is written for two ring slots");
-      CaCursor<SPLIT> cs;                                           // the block whose S is issued next; (j, li): the one whose P V is
+      CaCursor<SPLIT, LENGTHS> cs;                                           // the block whose S is issued next; (j, li): the one whose P V is
       cs.start(p);
       bool ok = cs.live(p) && issue_s(0, cs);
       for (int g = 0; ok; ++g) {
@@ -415,7 +416,7 @@ cross_attn_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_con
       return true;
     };
     for (int item = blockIdx.x; ok && item < p.total_items; item += gridDim.x) {
-      const CaItem it = ca_item<SPLIT>(p, item);
+      const CaItem it = ca_item<SPLIT, LENGTHS>(p, item);
       if (SPLIT > 1) pend_it = it;
       if (it.nb == 0) {
         if (SPLIT > 1) continue;                              // nothing of this item falls to this CTA
@@ -534,7 +535,7 @@ cross_attn_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_con
         // loads left zeros.)  16 x 1000 x 16 x 128 x 50..200: 57.5 us without, 59.2 so; cleared by the issuing thread
         // 62, by a warp of its own 64, not loaded at all (boxes of 64, 32 .. 1 rows) 65; without leaving k-steps out 61.
         const int left = it.T - j * kCaBN;
-        if (left < kCaBN && it.t0 + it.T < p.T && (left & 15) != 0) {
+        if (LENGTHS && left < kCaBN && it.t0 + it.T < p.T && (left & 15) != 0) {
           ok = tc::mbar_wait(v_full + (g & 1), (g >> 1) & 1, abort_flag);
           ok = __all_sync(kFullMask, ok);
           if (!ok) break;
@@ -664,7 +665,7 @@ inline bool cross_attn_tc_supported(int B, int M, int H, int d_h, int T_ctx) {
   return (d_h == 64 || d_h == 128) && H <= 65535 && B <= 65535 && T_ctx >= 1 && M >= 1;
 }
 
-template <int DH, int SPLIT, bool P32>
+template <int DH, int SPLIT, bool P32, bool LENGTHS>
 inline grace_status_t launch_cross_attn_tc_form(const CUtensorMap& mq, const CUtensorMap& mk, const CUtensorMap& mv,
                                                 const CrossTcParams& p, int items, cudaStream_t s) {
   constexpr int kCaSmemBytes = CaCfg<DH, SPLIT>::kSmemBytes;
@@ -672,7 +673,7 @@ inline grace_status_t launch_cross_attn_tc_form(const CUtensorMap& mq, const CUt
   static int n_sm_of[kMaxDevices] = {0};
   DeviceSetup su(&attr_set_devices);
   if (su) {
-    GRACE_CUDA_TRY(cudaFuncSetAttribute(cross_attn_tc_kernel<DH, SPLIT, P32>, cudaFuncAttributeMaxDynamicSharedMemorySize, kCaSmemBytes));
+    GRACE_CUDA_TRY(cudaFuncSetAttribute(cross_attn_tc_kernel<DH, SPLIT, P32, LENGTHS>, cudaFuncAttributeMaxDynamicSharedMemorySize, kCaSmemBytes));
     GRACE_CUDA_TRY(cudaDeviceGetAttribute(&n_sm_of[su.dev], cudaDevAttrMultiProcessorCount, su.dev));
     su.done();
   }
@@ -686,7 +687,7 @@ inline grace_status_t launch_cross_attn_tc_form(const CUtensorMap& mq, const CUt
   cfg.gridDim = dim3(SPLIT > 1 ? items * SPLIT : (items < n_sm ? items : n_sm));
   cfg.blockDim = dim3(kCaThreads); cfg.dynamicSmemBytes = kCaSmemBytes; cfg.stream = s;
   cfg.attrs = attr; cfg.numAttrs = SPLIT > 1 ? 2 : 1;
-  cudaLaunchKernelEx(&cfg, cross_attn_tc_kernel<DH, SPLIT, P32>, mq, mk, mv, p);
+  cudaLaunchKernelEx(&cfg, cross_attn_tc_kernel<DH, SPLIT, P32, LENGTHS>, mq, mk, mv, p);
   GRACE_LAUNCH_CHECK();
   return GRACE_OK;
 }
@@ -722,16 +723,23 @@ inline grace_status_t launch_cross_attn_tc(const uint16_t* q, int64_t q_row_stri
   p.total_items = (int)items * split;
   p.scale_log2 = scale * 1.4426950408889634f;
   const int n = (int)items;
-  if (p32) {
-    if constexpr (DH == 128) {                               // (at head size 64 these are more items than SMs)
-      if (split == 4) return launch_cross_attn_tc_form<DH, 4, true>(mq, mk, mv, p, n, s);
-      if (split == 2) return launch_cross_attn_tc_form<DH, 2, true>(mq, mk, mv, p, n, s);
+  if (enc_len != nullptr) {
+    if (p32) {
+      if constexpr (DH == 128) {                             // (at head size 64 these are more items than SMs)
+        if (split == 4) return launch_cross_attn_tc_form<DH, 4, true, true>(mq, mk, mv, p, n, s);
+        if (split == 2) return launch_cross_attn_tc_form<DH, 2, true, true>(mq, mk, mv, p, n, s);
+      }
+      return launch_cross_attn_tc_form<DH, 1, true, true>(mq, mk, mv, p, n, s);
     }
-    return launch_cross_attn_tc_form<DH, 1, true>(mq, mk, mv, p, n, s);
+    if constexpr (DH == 64) {                                // (at head size 128 lengths mean p32)
+      if (split == 4) return launch_cross_attn_tc_form<DH, 4, false, true>(mq, mk, mv, p, n, s);
+      if (split == 2) return launch_cross_attn_tc_form<DH, 2, false, true>(mq, mk, mv, p, n, s);
+      return launch_cross_attn_tc_form<DH, 1, false, true>(mq, mk, mv, p, n, s);
+    }
   }
-  if (split == 4) return launch_cross_attn_tc_form<DH, 4, false>(mq, mk, mv, p, n, s);
-  if (split == 2) return launch_cross_attn_tc_form<DH, 2, false>(mq, mk, mv, p, n, s);
-  return launch_cross_attn_tc_form<DH, 1, false>(mq, mk, mv, p, n, s);
+  if (split == 4) return launch_cross_attn_tc_form<DH, 4, false, false>(mq, mk, mv, p, n, s);
+  if (split == 2) return launch_cross_attn_tc_form<DH, 2, false, false>(mq, mk, mv, p, n, s);
+  return launch_cross_attn_tc_form<DH, 1, false, false>(mq, mk, mv, p, n, s);
 }
 
 }  // namespace grace
