@@ -63,7 +63,17 @@ extern "C" grace_status_t grace_decode_begin(const grace_decoder_t* d, void* str
   return GRACE_OK;
 }
 
-namespace grace {                                           // beam_topk.cu: a selection that ends with the state update
+namespace grace {
+// linear.cu: grace_linear, grace_linear_add_bf16 and grace_linear_layer_norm with weights that no kernel in flight writes
+// (they are at rest during a step: its first kernel waits for everything enqueued before it).
+grace_status_t step_linear(const uint16_t* x, int64_t ldx, const uint16_t* w, int64_t ldw, uint16_t* y_bf16, float* y_f32,
+                           int64_t ldy, const float* residual, int M, int N, int K, int relu, void* stream);
+grace_status_t step_linear_add_bf16(const uint16_t* x, int64_t ldx, const uint16_t* w, int64_t ldw, uint16_t* y_inout, int64_t ldy,
+                                    int M, int N, int K, void* stream);
+grace_status_t step_linear_layer_norm(const uint16_t* x, int64_t ldx, const uint16_t* w, int64_t ldw, float eps, float* row_affine,
+                                      const float* col_sum, const float* col_bias, uint16_t* y_bf16, float* y_f32, int64_t ldy,
+                                      float* lse_part, int M, int N, int K, int relu, void* stream);
+// beam_topk.cu: a selection that ends with the state update
 grace_status_t beam_topk_update(const float* cand, int B, int64_t N, int K, int V, float* out_score, int32_t* out_flat,
                                 int32_t* out_parent, int32_t* out_token, void* ws, size_t ws_bytes,
                                 const BeamUpdate& upd, int32_t* d_status, void* stream);
@@ -101,16 +111,16 @@ extern "C" grace_status_t grace_decode_step(const grace_decoder_t* d, int t, voi
   auto ln_linear = [&](const float* g, const float* b, const uint16_t* w, const float* cs, const float* cb,
                        uint16_t* y_bf16, float* y_f32, int64_t ldy, int N, int relu, float* lse_part) -> grace_status_t {
     if (folded)
-      return grace_linear_layer_norm(d->x_bf16, D, w, D, d->ln_eps, d->row_affine, cs, cb, y_bf16, y_f32, ldy, lse_part, R,
+      return grace::step_linear_layer_norm(d->x_bf16, D, w, D, d->ln_eps, d->row_affine, cs, cb, y_bf16, y_f32, ldy, lse_part, R,
                                      N, D, relu, stream);
     grace_status_t s1 = layer_norm(g, b);
     if (s1 != GRACE_OK) return s1;
     if (lse_part != nullptr) return grace_linear_f32_lse(d->h, D, w, D, y_f32, ldy, lse_part, R, N, D, stream);
-    return grace_linear(d->h, D, w, D, y_bf16, y_f32, ldy, nullptr, R, N, D, relu, stream);
+    return grace::step_linear(d->h, D, w, D, y_bf16, y_f32, ldy, nullptr, R, N, D, relu, stream);
   };
   auto add_into_x = [&](const uint16_t* a, int64_t lda, const uint16_t* w, int K) -> grace_status_t {
-    return xb ? grace_linear_add_bf16(a, lda, w, K, d->x_bf16, D, R, D, K, stream)
-              : grace_linear(a, lda, w, K, nullptr, d->x, D, d->x, R, D, K, 0, stream);
+    return xb ? grace::step_linear_add_bf16(a, lda, w, K, d->x_bf16, D, R, D, K, stream)
+              : grace::step_linear(a, lda, w, K, nullptr, d->x, D, d->x, R, D, K, 0, stream);
   };
   if (xb) GRACE_TRY(grace_embed_bf16(d->token[cur], d->embed, d->pos + (int64_t)t * D, d->x_bf16, R, D, d->V + 1, st, stream));
   else GRACE_TRY(grace_embed(d->token[cur], d->embed, d->pos + (int64_t)t * D, d->x, R, D, d->V + 1, st, stream));

@@ -58,6 +58,7 @@ struct GemmParams {
   float2* aff_out;                 //   and leaves them here too (if not NULL)
   int64_t ldy;
   int M, N, K, relu;
+  int fixed_w;                     // no kernel that may still be running writes w
 };
 
 constexpr int kGemmThreads = 192;                           // four row warps, TMA producer, MMA issuer
@@ -75,9 +76,10 @@ struct GemmSet {
 template <int BN, int STAGES, int SPLIT, int G>
 __global__ void __launch_bounds__(kGemmThreads, 2)
 linear_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_constant__ GemmSet<G> set, const GemmParams p) {
-  // The weights do not depend on the kernel before this one: their first tiles are requested before the wait
-  // on that kernel, so their trip from HBM overlaps its tail; every thread waits before its first access to
-  // anything an earlier kernel wrote (activations, row statistics, the residual).
+  // In a decode step the weights do not depend on the kernel before this one: their first tiles are requested before
+  // the wait on that kernel, so their trip from HBM overlaps its tail.  (The step's first kernel has waited for everything
+  // in front of the step.)  Otherwise, and for whatever else an earlier kernel may have written (activations, row
+  // statistics, the residual), every thread waits before its first access.
   pdl_trigger();
   using S = GemmCfg<BN, STAGES, SPLIT>;
   constexpr int kSlice = S::kSlice;
@@ -150,6 +152,7 @@ linear_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_constant__
     if (lane == 0) {
       // ---- TMA producer ----
       const int first = KB < STAGES ? KB : STAGES;          // the ring's first pass needs no empty-slot wait
+      if (!p.fixed_w) pdl_wait();
       for (int kb = 0; kb < first; ++kb) {
         tc::mbar_expect_tx(full + kb, S::kStageBytes);
         tc::tma_load_2d(tiles + kb * S::kStageBytes + S::kABytes, &map_w, full + kb, (kb0 + kb) * kGemmBK, n0);
@@ -958,7 +961,7 @@ static grace_status_t linear_impl(const uint16_t* x, int64_t ldx, const uint16_t
                                   bool add_into_bf16, int M, int N, int K, int relu, void* stream,
                                   float* lse_part = nullptr,
                                   grace::Affine aff = grace::Affine{nullptr, nullptr, nullptr},
-                                  const uint64_t* allow_bits = nullptr) {
+                                  const uint64_t* allow_bits = nullptr, bool fixed_w = false) {
   using namespace grace;
   if (!x || !w || ((y_bf16 == nullptr) == (y_f32 == nullptr))) return GRACE_INVALID_ARG;
   if (M <= 0 || N <= 0 || K <= 0) return GRACE_INVALID_ARG;
@@ -1024,7 +1027,7 @@ static grace_status_t linear_impl(const uint16_t* x, int64_t ldx, const uint16_t
   GemmParams p;
   p.y_bf16 = y_bf16; p.y_f32 = y_f32; p.residual = residual; p.residual_bf16 = add_into_bf16 ? y_bf16 : nullptr;
   p.aff_row = aff.in_kernel_stats ? nullptr : aff.row; p.aff_cs = aff.cs; p.aff_cb = aff.cb; p.ln_eps = aff.eps; p.aff_out = aff.out;
-  p.ldy = ldy; p.M = M; p.N = N; p.K = K; p.relu = relu;
+  p.ldy = ldy; p.M = M; p.N = N; p.K = K; p.relu = relu; p.fixed_w = fixed_w;
   return run_linear<1>(form, mx, set, p, s);
 }
 
@@ -1093,10 +1096,9 @@ extern "C" grace_status_t grace_linear_folded_ln(const uint16_t* x, int64_t ldx,
   return linear_impl(x, ldx, w, ldw, y_bf16, y_f32, ldy, nullptr, false, M, N, K, relu, stream, lse_part, aff);
 }
 
-extern "C" grace_status_t grace_linear_layer_norm(const uint16_t* x, int64_t ldx, const uint16_t* w, int64_t ldw,
-                                                  float eps, float* row_affine, const float* col_sum,
-                                                  const float* col_bias, uint16_t* y_bf16, float* y_f32, int64_t ldy,
-                                                  float* lse_part, int M, int N, int K, int relu, void* stream) {
+static grace_status_t layer_norm_impl(const uint16_t* x, int64_t ldx, const uint16_t* w, int64_t ldw, float eps, float* row_affine,
+                                      const float* col_sum, const float* col_bias, uint16_t* y_bf16, float* y_f32,
+                                      int64_t ldy, float* lse_part, int M, int N, int K, int relu, void* stream, bool fixed_w) {
   if (!row_affine || !col_bias || (reinterpret_cast<uintptr_t>(row_affine) & 7) ||
       !grace_aligned16(col_sum) || !grace_aligned16(col_bias))
     return GRACE_INVALID_ARG;
@@ -1124,7 +1126,14 @@ extern "C" grace_status_t grace_linear_layer_norm(const uint16_t* x, int64_t ldx
     const grace_status_t st = grace_row_stats_bf16(x, M, K, eps, row_affine, stream);
     if (st != GRACE_OK) return st;
   }
-  return linear_impl(x, ldx, w, ldw, y_bf16, y_f32, ldy, nullptr, false, M, N, K, relu, stream, lse_part, aff);
+  return linear_impl(x, ldx, w, ldw, y_bf16, y_f32, ldy, nullptr, false, M, N, K, relu, stream, lse_part, aff, nullptr, fixed_w);
+}
+
+extern "C" grace_status_t grace_linear_layer_norm(const uint16_t* x, int64_t ldx, const uint16_t* w, int64_t ldw,
+                                                  float eps, float* row_affine, const float* col_sum,
+                                                  const float* col_bias, uint16_t* y_bf16, float* y_f32, int64_t ldy,
+                                                  float* lse_part, int M, int N, int K, int relu, void* stream) {
+  return layer_norm_impl(x, ldx, w, ldw, eps, row_affine, col_sum, col_bias, y_bf16, y_f32, ldy, lse_part, M, N, K, relu, stream, false);
 }
 
 extern "C" grace_status_t grace_linear_logits_allowed(const uint16_t* x, int64_t ldx, const uint16_t* w, int64_t ldw,
@@ -1151,6 +1160,24 @@ extern "C" grace_status_t grace_linear_add_bf16(const uint16_t* x, int64_t ldx, 
                                                 uint16_t* y_inout, int64_t ldy, int M, int N, int K, void* stream) {
   return linear_impl(x, ldx, w, ldw, y_inout, nullptr, ldy, nullptr, true, M, N, K, 0, stream);
 }
+
+namespace grace {
+grace_status_t step_linear(const uint16_t* x, int64_t ldx, const uint16_t* w, int64_t ldw, uint16_t* y_bf16, float* y_f32,
+                           int64_t ldy, const float* residual, int M, int N, int K, int relu, void* stream) {
+  return linear_impl(x, ldx, w, ldw, y_bf16, y_f32, ldy, residual, false, M, N, K, relu, stream, nullptr,
+                     Affine{nullptr, nullptr, nullptr}, nullptr, true);
+}
+grace_status_t step_linear_add_bf16(const uint16_t* x, int64_t ldx, const uint16_t* w, int64_t ldw, uint16_t* y_inout, int64_t ldy,
+                                    int M, int N, int K, void* stream) {
+  return linear_impl(x, ldx, w, ldw, y_inout, nullptr, ldy, nullptr, true, M, N, K, 0, stream, nullptr,
+                     Affine{nullptr, nullptr, nullptr}, nullptr, true);
+}
+grace_status_t step_linear_layer_norm(const uint16_t* x, int64_t ldx, const uint16_t* w, int64_t ldw, float eps, float* row_affine,
+                                      const float* col_sum, const float* col_bias, uint16_t* y_bf16, float* y_f32, int64_t ldy,
+                                      float* lse_part, int M, int N, int K, int relu, void* stream) {
+  return layer_norm_impl(x, ldx, w, ldw, eps, row_affine, col_sum, col_bias, y_bf16, y_f32, ldy, lse_part, M, N, K, relu, stream, true);
+}
+}  // namespace grace
 
 // ---------------------------------------------------------------------------------------------
 // Bounded waits, checked without hanging anything: a one-block kernel waits on a barrier that

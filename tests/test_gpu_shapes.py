@@ -296,3 +296,29 @@ def test_cross_attn_lengths_with_any_strides_and_scale(api, B, M, H, d, T, form)
     assert_attention_close(got, ref, form)
     assert (got[~some] == 0).all()
     np.testing.assert_allclose(got_lse[some], lse_ref[some], atol=2e-3, rtol=0)
+
+
+@pytest.mark.parametrize("N,K,M", [(1008, 512, 16), (1024, 512, 1024), (512, 512, 2048), (64, 1024, 300)])
+def test_linear_reads_weights_that_the_call_before_wrote(api, N, K, M):
+    """w of one product is the output of the product in front of it on the stream, long in its K loop when the second call
+    is launched: whatever the form, the second reads what the first left."""
+    g = torch.Generator(device=DEV)
+    g.manual_seed(N + K + M)
+    a = torch.randn(N, 8192, device=DEV, generator=g).to(torch.bfloat16)
+    b = (torch.randn(K, 8192, device=DEV, generator=g) * 0.02).to(torch.bfloat16)
+    x = torch.randn(M, K, device=DEV, generator=g).to(torch.bfloat16)
+    w = torch.empty(N, K, device=DEV, dtype=torch.bfloat16)
+    want, y = torch.empty(M, N, device=DEV, dtype=torch.bfloat16), torch.empty(M, N, device=DEV, dtype=torch.bfloat16)
+    aff, cb = torch.empty(M, 2, device=DEV), torch.zeros(N, device=DEV)
+    calls = (lambda out: api.grace_linear(x, w, out), lambda out: api.grace_linear_multi(x, [w, w], [out, torch.empty_like(out)]),
+             lambda out: api.grace_linear_layer_norm(x, w, 1e-5, aff, None, cb, out),
+             lambda out: api.grace_linear_add_bf16(x, w, out.zero_()))
+    for call in calls:
+        api.grace_linear(a, b, w)
+        torch.cuda.synchronize()
+        call(want)
+        for _ in range(20):
+            w.fill_(float("nan"))
+            api.grace_linear(a, b, w)
+            call(y)
+            assert torch.equal(y, want)
