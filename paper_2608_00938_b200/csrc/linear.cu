@@ -936,6 +936,7 @@ static LinearForm linear_form(int M, int N, int K, bool pair_possible, bool stat
   if (pair_possible) {
     const int64_t waves = ((int64_t)((M + 255) / 256) * ((N + 255) / 256) * products + 73) / 74;
     least = 2.7f + (float)waves * (1.0f + 0.33f * (float)kb) + (stats_launch ? 3.2f + 3.6e-7f * (float)M * (float)K : 0.f);
+    if (tiles_m > 65535) return best;                        // more row tiles than gridDim.y takes: the persistent kernel
   }
   for (const LinearForm& f : kLinearForms) {
     if (f.split > kb || (whole_k && f.split > 1)) continue;

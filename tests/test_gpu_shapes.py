@@ -322,3 +322,24 @@ def test_linear_reads_weights_that_the_call_before_wrote(api, N, K, M):
             api.grace_linear(a, b, w)
             call(y)
             assert torch.equal(y, want)
+
+
+def test_layer_norm_gemm_of_more_row_tiles_than_a_grid_is_high(api):
+    """65536 x 128 rows and one more: the form whose row tiles are gridDim.y cannot run them."""
+    M, N, K = 65536 * 128 + 1, 256, 1024
+    g = torch.Generator(device=DEV)
+    g.manual_seed(3)
+    some = torch.tensor([0, 1, 128 * 65535 - 1, 128 * 65535, M - 2, M - 1], device=DEV)
+    x = torch.zeros(M, K, device=DEV, dtype=torch.bfloat16)
+    x[some] = torch.randn(some.numel(), K, device=DEV, generator=g).to(torch.bfloat16)
+    w = (torch.randn(N, K, device=DEV, generator=g) * 0.05).to(torch.bfloat16)
+    cs, cb = w.double().sum(1).float(), torch.randn(N, device=DEV, generator=g)
+    y, aff = torch.empty(M, N, device=DEV, dtype=torch.bfloat16), torch.empty(M, 2, device=DEV)
+    api.grace_linear_layer_norm(x, w, 1e-5, aff, cs, cb, y)
+    x64 = x[some].double()
+    mean, rstd = x64.mean(1, keepdim=True), (x64.var(1, unbiased=False, keepdim=True) + 1e-5).rsqrt()
+    prod, absolute = x64 @ w.double().T, x64.abs() @ w.double().abs().T
+    want = rstd * (prod - mean * cs.double()) + cb.double()
+    bound = 2.0 ** -8 * want.abs() + 2.0 ** -17 * rstd * (absolute + (mean * cs.double()).abs()) + 1e-5
+    assert ((y[some].double() - want).abs() <= bound).all()
+    assert (y[2].double() - cb.double()).abs().max() <= 2.0 ** -8 * cb.abs().max()        # a row of zeros: the bias
