@@ -343,3 +343,23 @@ def test_layer_norm_gemm_of_more_row_tiles_than_a_grid_is_high(api):
     bound = 2.0 ** -8 * want.abs() + 2.0 ** -17 * rstd * (absolute + (mean * cs.double()).abs()) + 1e-5
     assert ((y[some].double() - want).abs() <= bound).all()
     assert (y[2].double() - cb.double()).abs().max() <= 2.0 ** -8 * cb.abs().max()        # a row of zeros: the bias
+
+
+@pytest.mark.parametrize("M,K", [(4, 512), (1000, 512), (1024, 2048), (3000, 1088), (70, 128)])
+@pytest.mark.parametrize("mean", [0.0, 0.7, 10.0])
+def test_row_statistics_of_a_gemm_that_forms_them(api, M, K, mean):
+    """row_affine as the GEMM leaves it against 64 bits.  Bound: (rstd, -rstd mean) are rounded to fp32 a few times each
+    (2^-25 rms a rounding) and E[x^2] - mean^2 enlarges the error of the two sums by 1 + mean^2 / var; the sums themselves may
+    add no more than that.  rms over the rows, three such roundings."""
+    g = torch.Generator(device=DEV)
+    g.manual_seed(M + K)
+    x = (torch.randn(M, K, device=DEV, generator=g) + mean).to(torch.bfloat16)
+    w = (torch.randn(256, K, device=DEV, generator=g) * 0.05).to(torch.bfloat16)
+    cs, cb = w.double().sum(1).float(), torch.zeros(256, device=DEV)
+    y, aff = torch.empty(M, 256, device=DEV), torch.zeros(M, 2, device=DEV)
+    api.grace_linear_layer_norm(x, w, 1e-5, aff, cs, cb, y)
+    mu, var = x.double().mean(1), x.double().var(1, unbiased=False)
+    rstd = (var + 1e-5).rsqrt()
+    bound = 3 * 2.0 ** -25 * (1 + (mu * mu / var).mean().item())
+    assert (((aff[:, 0].double() - rstd) / rstd) ** 2).mean().sqrt() <= bound
+    assert ((aff[:, 1].double() + rstd * mu).norm() / (rstd * mu).norm().clamp_min(1e-30)) <= 2 * bound
