@@ -853,6 +853,7 @@ struct Affine {                                            // LayerNorm folded i
   float eps = 0.f;                                         // in_kernel_stats only
   float2* out = nullptr;                                   // in_kernel_stats, linear_kernel: receives them
   bool in_kernel_stats = false;                            // the GEMM kernel forms (rstd, -rstd * mean) itself
+  bool forms_stats = false;                                // the call forms them, there or in the statistics kernel
 };
 struct AllowedStores {                                     // kOutF32LseAllowed
   const uint64_t* bits = nullptr;
@@ -925,6 +926,10 @@ static grace_status_t launch_linear(const CUtensorMap& mx, const GemmSet<G>& set
 // tiles without a split), LayerNorm included: 512 x 1536 x 512: 10.3 -> 5.8 us, 512 x 2048 x 512: 10.5 -> 6.1,
 // 512 x 512 x 2048: 10.3 -> 5.8, 16 x 512 x 2048: 9.9 -> 4.3, 1024 x 512 x 2048: 13.1 -> 7.1, 1024 x 512 x 512:
 // 7.6 -> 5.0, 2048 x 512 x 2048: 13.1 -> 9.1.
+// Row statistics formed from the operand tiles are free for eight k-blocks, which are in flight at once; beyond, the ring
+// waits for the warps that form them (as if free: 10000 x 512 x 2048 45 us where the pair kernel behind the statistics
+// kernel takes 28, 16384 x 512 x 2048 45 / 33, 4096 x 1024 x 2048 23 / 19).  Two CTAs per SM take an SM's time from each other: a last
+// wave of one per SM is shorter (1000 x 6144 x 2048: 36.3 us in the form estimated before, 28.7 so); seen with long K only.
 // Rows beyond the problem's last cost no exchange and no stores: both parts grow from few rows to a full tile of 128.
 struct LinearForm {
   int bn, split, per_sm;                   // bn = 0: the CTA-pair kernel
@@ -953,9 +958,11 @@ static grace_status_t run_linear(const LinearForm& f, const CUtensorMap& mx, con
   return GRACE_UNSUPPORTED_SHAPE;
 }
 
-// stats_launch: the pair kernel would need the statistics kernel in front.  whole_k: no split of K, so that the sums are
-// those of the pair kernel bit for bit (fp32 products: grace_linear_f32_lse promises those of grace_linear).
-static LinearForm linear_form(int M, int N, int K, bool pair_possible, bool stats_launch, bool whole_k, int products = 1) {
+enum LinearStats { kStatsNone, kStatsFormed, kStatsFormedNarrow };
+// stats: whether the call's row statistics are still to be formed, and if so whether the pair kernel would form them itself
+// (narrow) or need the statistics kernel in front.  whole_k: no split of K, so that the sums are those of the pair kernel bit
+// for bit (fp32 products: grace_linear_f32_lse promises those of grace_linear).
+static LinearForm linear_form(int M, int N, int K, bool pair_possible, LinearStats stats, bool whole_k, int products = 1) {
   const int64_t tiles_m = (M + kGemmBM - 1) / kGemmBM;
   const int kb = K / kGemmBK;
   LinearForm best = {};
@@ -963,15 +970,19 @@ static LinearForm linear_form(int M, int N, int K, bool pair_possible, bool stat
   float least = 3.4e38f;
   if (pair_possible) {
     const int64_t waves = ((int64_t)((M + 255) / 256) * ((N + 255) / 256) * products + 73) / 74;
-    least = 2.7f + (float)waves * (1.0f + 0.33f * (float)kb) + (stats_launch ? 3.2f + 3.6e-7f * (float)M * (float)K : 0.f);
+    least = 2.7f + (float)waves * (1.0f + 0.33f * (float)kb) + (stats == kStatsFormed ? 3.2f + 3.6e-7f * (float)M * (float)K : 0.f);
     if (tiles_m > 65535) return best;                        // more row tiles than gridDim.y takes: the persistent kernel
   }
   for (const LinearForm& f : kLinearForms) {
     if (f.split > kb || (whole_k && f.split > 1)) continue;
     const int64_t ctas = tiles_m * ((N + f.bn - 1) / f.bn) * f.split * products;
     const int wave = f.split == 1 ? 148 * f.per_sm : (f.split == 2 ? 144 : 132);       // clusters lie within a GPC
-    const float t = (float)((ctas + wave - 1) / wave) * (f.fixed + rows * f.fixed_rows +
-                                                         (f.per_kb + rows * f.per_kb_rows) * (float)((kb + f.split - 1) / f.split));
+    const int64_t waves = (ctas + wave - 1) / wave;
+    const int long_kb = (kb + f.split - 1) / f.split;
+    float one = f.fixed + rows * f.fixed_rows + (f.per_kb + rows * f.per_kb_rows) * (float)long_kb;
+    if (stats != kStatsNone && long_kb > 8) one += (f.per_sm == 1 ? 0.07f : 0.15f) * (float)(long_kb - 8);
+    float t = (float)waves * one;
+    if (f.per_sm == 2 && waves > 1 && long_kb > 8 && ctas - (waves - 1) * wave <= 148) t -= 0.35f * one;
     if (t < least) { least = t; best = f; }
   }
   return best;
@@ -982,6 +993,9 @@ static bool linear_pair_possible(int M, int N, bool residual_elsewhere) { return
 static bool linear_whole_k(int M, int N, bool plain_f32) { return plain_f32 && M >= 1024 && N >= 256; }
 // Centred rows and at most two 256-wide tiles: the pair kernel forms the LayerNorm statistics itself.
 static bool linear_narrow_centred(int M, int N, const float* col_sum) { return M >= 1024 && N >= 256 && N <= 512 && col_sum == nullptr; }
+static LinearStats linear_stats(int M, int N, const float* col_sum) {
+  return linear_narrow_centred(M, N, col_sum) ? kStatsFormedNarrow : kStatsFormed;
+}
 
 }  // namespace grace
 
@@ -1007,7 +1021,7 @@ static grace_status_t linear_impl(const uint16_t* x, int64_t ldx, const uint16_t
   LinearForm form = {};
   if (lse_part == nullptr)
     form = linear_form(M, N, K, linear_pair_possible(M, N, residual != nullptr && !aliased),
-                       aff.row != nullptr && !linear_narrow_centred(M, N, aff.cs), linear_whole_k(M, N, y_f32 != nullptr && residual == nullptr));
+                       aff.forms_stats ? linear_stats(M, N, aff.cs) : kStatsNone, linear_whole_k(M, N, y_f32 != nullptr && residual == nullptr));
   if (form.bn == 0) {
     // large GEMM: persistent CTA-pair kernel, TMA-store epilogue (add-reduction when y is the residual stream)
     CUtensorMap mx;
@@ -1077,7 +1091,7 @@ extern "C" grace_status_t grace_linear_multi(const uint16_t* x, int64_t ldx, int
   cudaStream_t s = (cudaStream_t)stream;
   for (int first = 0; first < count; first += kMultiMost) {
     const int here = count - first < kMultiMost ? count - first : kMultiMost;
-    const LinearForm form = linear_form(M, N, K, linear_pair_possible(M, N, false), false, false, here);
+    const LinearForm form = linear_form(M, N, K, linear_pair_possible(M, N, false), kStatsNone, false, here);
     CUtensorMap mx;
     GemmSet<kMultiMost> set;
     set.count = here;
@@ -1134,6 +1148,7 @@ static grace_status_t layer_norm_impl(const uint16_t* x, int64_t ldx, const uint
   if (lse_part != nullptr && (reinterpret_cast<uintptr_t>(lse_part) & 7)) return GRACE_INVALID_ARG;
   if (M <= 0 || N <= 0 || K <= 0 || ldx != K) return GRACE_INVALID_ARG;     // the LayerNorm is over the whole row of x
   grace::Affine aff = {reinterpret_cast<const float2*>(row_affine), col_sum, col_bias};
+  aff.forms_stats = true;
   // The statistics come out of the GEMM's own operand tiles in linear_kernel, and where the CTA-pair kernel runs if
   // the rows are centred (no col_sum) and the output is at most two tiles wide; otherwise the statistics kernel
   // runs first, into row_affine.  In the pair kernel every n-tile forms the statistics of its rows again, and the
@@ -1142,7 +1157,7 @@ static grace_status_t layer_norm_impl(const uint16_t* x, int64_t ldx, const uint
   // against 43; N = 1536: 99 against 95; N = 2048: 130 against 122.
   const bool narrow_centred = lse_part == nullptr && grace::linear_narrow_centred(M, N, col_sum);
   const bool pair_kernel = lse_part != nullptr ||
-                           grace::linear_form(M, N, K, grace::linear_pair_possible(M, N, false), !narrow_centred,
+                           grace::linear_form(M, N, K, grace::linear_pair_possible(M, N, false), grace::linear_stats(M, N, col_sum),
                                               grace::linear_whole_k(M, N, y_f32 != nullptr)).bn == 0;
   // (not for a logits GEMM with log-sum-exp partials: grace_linear_logits_allowed takes its statistics from the
   // statistics kernel, and the two forms of a decode step are to agree bit for bit)
