@@ -238,17 +238,25 @@ extern "C" grace_status_t grace_cross_attn_varlen(const uint16_t* q, int64_t q_r
     return GRACE_OK;
   };
   // Few pairs, or long ones: a CTA each, all resident at once; 32 warps each while there is one pair
-  // per SM (32 x 1 x 8 x 64 x 1024: 8 warps 15.9 us, 32 warps 16.4).  Otherwise a warp each, except at head size 128, where
-  // a warp has two lane groups only (32 x 1 x 16 x 200: 8 warps 15.5 us, one 23.6).  (1 x 1 x 8 x 64 x 1024: 8.8 us with 8 warps and states merged one by one, 5.3 now;
+  // per SM (32 x 1 x 8 x 64 x 1024: 8 warps 15.9 us, 32 warps 16.4).  A warp each when there are more and they are short:
+  // eight warps win from T = pairs / 3 on at head size 64 (512 x 511 positions: 18.3 us with one warp, 11 with eight;
+  // 1184: 200 positions 10 / 14, 333 23 / 22, 511 38 / 32), pairs / 2 at 32 (592 x 256: 6.6 / 5.6), pairs / 9 at 128, where a
+  // warp has two lane groups only (592 x 64: 7 / 5; 1184 x 128: 12 / 15).  (1 x 1 x 8 x 64 x 1024: 8.8 us with 8 warps and states merged one by one, 5.3 now;
   // head size 32 against the kernel before, which read K and V two bytes at a time: 1 x 16 x 4 x 64: 6.0 -> 2.3 us,
   // 1 x 16 x 4 x 1024: 66 -> 4.4, 8 x 200 x 4 x 128: 31 -> 13.8, 64 x 16 x 4 x 512: 78 -> 30.)
-  if ((M <= 8 || d_h == 32) && pairs <= 1184) return run_pairs(pairs <= 2 * 148 || T_ctx >= 512 || d_h == 128);
+  if ((M <= 8 || d_h == 32) && pairs <= 8 * 148)
+    return run_pairs(pairs <= 2 * 148 || (int64_t)T_ctx * (d_h == 128 ? 9 : d_h == 64 ? 3 : 2) >= pairs);
   if (cross_attn_tc_supported(B, M, H, d_h, T_ctx)) {
     // probabilities as before the tensor cores took these over: fp32 (see cross_attn_tc_kernel)
     const bool p32 = enc_len != nullptr && (d_h == 128 || M <= 8);
     // ... and any stride and any scale: what a tensor map cannot say (negative and huge strides) and scales that are not
     // positive (the softmax threads take the maximum before they scale) still run on the CUDA cores.
     if (p32 && !(scale >= 1e-30f)) return run_pairs(false);
+    // A 128-row tile with a few live rows is no faster than a warp per pair while rows x positions are few (with lengths,
+    // one / the tensor cores: 1 row, head size 64: 2400 pairs x 33 positions 5 / 42 us, x 1024 94 / 204; head size 128: 2368 x 33
+    // 7 / 45, x 511 80 / 109; 2 rows, 64: 4800 x 1024 131 / 205, 128: 2368 x 256 36 / 38, x 511 68 / 58; 8 rows, 64: 4736 x 64
+    // 10 / 12, x 128 17 / 13, 128: 2432 x 64 10 / 10).
+    if (p32 && M <= 8 && ((d_h == 64 && M <= 2) || M * (int64_t)T_ctx <= 512)) return run_pairs(false);
     const int form = cross_attn_form(B, M, H, d_h, T_ctx, p32);
     if (form == 0)
       return launch_cross_attn_ms(q, q_row_stride, k, v, kv_stride_b, kv_stride_h, kv_stride_t, out,
