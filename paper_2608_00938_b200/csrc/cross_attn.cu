@@ -191,9 +191,9 @@ namespace grace {
 static int cross_attn_form(int B, int M, int H, int d_h, int T_ctx, bool p32) {
   const int64_t tiles = (int64_t)((M + kCaBM - 1) / kCaBM) * H * B;
   const int blocks = (T_ctx + kCaBN - 1) / kCaBN, least = d_h == 128 ? 2 : 1;
-  if (tiles > 148) return d_h == 64 && !p32 ? 0 : 1;
-  if (tiles * 4 <= 148 && blocks >= 4 * least) return 4;
-  if (tiles * 2 <= 148 && blocks >= 2 * least) return 2;
+  if (tiles > kSms) return d_h == 64 && !p32 ? 0 : 1;
+  if (tiles * 4 <= kSmsInFours && blocks >= 4 * least) return 4;
+  if (tiles * 2 <= kSmsInTwos && blocks >= 2 * least) return 2;
   return 1;
 }
 int cross_attn_tc_timeouts() { return tc::tc_timeouts_read_and_clear(); }
@@ -225,7 +225,7 @@ extern "C" grace_status_t grace_cross_attn_varlen(const uint16_t* q, int64_t q_r
   auto run_pairs = [&](bool few) -> grace_status_t {
 #define GRACE_PAIR_LAUNCH(D)                                                                                              \
   do {                                                                                                                  \
-    if (few && pairs <= 148 && T_ctx >= 512)                                                                            \
+    if (few && pairs <= kSms && T_ctx >= 512)                                                                            \
       launch_pdl(cross_attn_row_kernel<D, 32, 1>, dim3((unsigned)pairs), dim3(1024), 0, s, p);                          \
     else if (few) launch_pdl(cross_attn_row_kernel<D, 8, 1>, dim3((unsigned)pairs), dim3(256), 0, s, p);                \
     else launch_pdl(cross_attn_row_kernel<D, 1, 8>, dim3((unsigned)((pairs + 7) / 8)), dim3(256), 0, s, p);             \
@@ -244,8 +244,8 @@ extern "C" grace_status_t grace_cross_attn_varlen(const uint16_t* q, int64_t q_r
   // warp has two lane groups only (592 x 64: 7 / 5; 1184 x 128: 12 / 15).  (1 x 1 x 8 x 64 x 1024: 8.8 us with 8 warps and states merged one by one, 5.3 now;
   // head size 32 against the kernel before, which read K and V two bytes at a time: 1 x 16 x 4 x 64: 6.0 -> 2.3 us,
   // 1 x 16 x 4 x 1024: 66 -> 4.4, 8 x 200 x 4 x 128: 31 -> 13.8, 64 x 16 x 4 x 512: 78 -> 30.)
-  if ((M <= 8 || d_h == 32) && pairs <= 8 * 148)
-    return run_pairs(pairs <= 2 * 148 || (int64_t)T_ctx * (d_h == 128 ? 9 : d_h == 64 ? 3 : 2) >= pairs);
+  if ((M <= 8 || d_h == 32) && pairs <= 8 * kSms)
+    return run_pairs(pairs <= 2 * kSms || (int64_t)T_ctx * (d_h == 128 ? 9 : d_h == 64 ? 3 : 2) >= pairs);
   if (cross_attn_tc_supported(B, M, H, d_h, T_ctx)) {
     // probabilities as before the tensor cores took these over: fp32 (see cross_attn_tc_kernel)
     const bool p32 = enc_len != nullptr && (d_h == 128 || M <= 8);

@@ -680,7 +680,7 @@ static grace_status_t launch_mask(const float* logp, bool logits, float* row_lse
   // (these launches are scheduled early: nothing else fills the GPU under them).
   const bool split = p.R <= 2048;
   int split_warps = kMaskSplitWarps;
-  while (split_warps > 4 && p.R * split_warps > 148 * 64) split_warps >>= 1;
+  while (split_warps > 4 && p.R * split_warps > kSms * 64) split_warps >>= 1;
   const int blocks = split ? p.R : (p.R + kMaskWarpsPerBlock - 1) / kMaskWarpsPerBlock;
   const int threads = (split ? split_warps : kMaskWarpsPerBlock) * 32;
 #define GRACE_MASK_LAUNCH(K)                                                      \

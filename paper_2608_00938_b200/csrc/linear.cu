@@ -969,20 +969,20 @@ static LinearForm linear_form(int M, int N, int K, bool pair_possible, LinearSta
   const float rows = M < kGemmBM ? (float)M / (float)kGemmBM : 1.f;
   float least = 3.4e38f;
   if (pair_possible) {
-    const int64_t waves = ((int64_t)((M + 255) / 256) * ((N + 255) / 256) * products + 73) / 74;
+    const int64_t waves = ((int64_t)((M + 255) / 256) * ((N + 255) / 256) * products + kSmsInTwos / 2 - 1) / (kSmsInTwos / 2);
     least = 2.7f + (float)waves * (1.0f + 0.33f * (float)kb) + (stats == kStatsFormed ? 3.2f + 3.6e-7f * (float)M * (float)K : 0.f);
     if (tiles_m > 65535) return best;                        // more row tiles than gridDim.y takes: the persistent kernel
   }
   for (const LinearForm& f : kLinearForms) {
     if (f.split > kb || (whole_k && f.split > 1)) continue;
     const int64_t ctas = tiles_m * ((N + f.bn - 1) / f.bn) * f.split * products;
-    const int wave = f.split == 1 ? 148 * f.per_sm : (f.split == 2 ? 144 : 132);       // clusters lie within a GPC
+    const int wave = f.split == 1 ? kSms * f.per_sm : (f.split == 2 ? kSmsInTwos : kSmsInFours);
     const int64_t waves = (ctas + wave - 1) / wave;
     const int long_kb = (kb + f.split - 1) / f.split;
     float one = f.fixed + rows * f.fixed_rows + (f.per_kb + rows * f.per_kb_rows) * (float)long_kb;
     if (stats != kStatsNone && long_kb > 8) one += (f.per_sm == 1 ? 0.07f : 0.15f) * (float)(long_kb - 8);
     float t = (float)waves * one;
-    if (f.per_sm == 2 && waves > 1 && long_kb > 8 && ctas - (waves - 1) * wave <= 148) t -= 0.35f * one;
+    if (f.per_sm == 2 && waves > 1 && long_kb > 8 && ctas - (waves - 1) * wave <= kSms) t -= 0.35f * one;
     if (t < least) { least = t; best = f; }
   }
   return best;
