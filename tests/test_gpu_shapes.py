@@ -88,8 +88,13 @@ def test_topk_between_its_paths(api, N, V, K, finite):
         assert np.array_equal(got.cpu().numpy(), want)
 
 
+# the forms of linear_kernel (columns / split): 32/1, 32/1, 32/2, 64/4, 64/1, 32/1, 128/1, 128/2, 64/1, 64/4, 128/1, 128/4, 64/2, 128/1
+# two CTAs per SM (centred and the additions: the pair kernel), 128/1, 128/1 two per SM, 64/1 two per SM; the pair kernel
+# with the statistics kernel in front
 @pytest.mark.parametrize("M,N,K", [(1, 64, 64), (17, 96, 128), (130, 512, 512), (129, 528, 2048), (512, 1536, 512), (1025, 512, 512),
-                                   (1030, 2048, 512), (300, 2048, 1088), (2049, 272, 320), (5, 2048, 2048)])
+                                   (1030, 2048, 512), (300, 2048, 1088), (2049, 272, 320), (5, 2048, 2048), (513, 2064, 1088),
+                                   (5, 4096, 1088), (513, 528, 1088), (5001, 528, 320), (1500, 1040, 512), (700, 6160, 1088),
+                                   (1025, 1040, 128), (5001, 1040, 64)])
 @pytest.mark.parametrize("centred", [True, False])
 def test_layer_norm_gemm_in_every_form(api, M, N, K, centred):
     """grace_linear_layer_norm (statistics inside the GEMM, K shared by the CTAs of a cluster) and the additions into
@@ -125,8 +130,10 @@ def test_layer_norm_gemm_in_every_form(api, M, N, K, centred):
         assert ((r.double() - want).abs() <= bound + 1e-30).all()
 
 
+# 32/1, 32/1, the pair kernel twice (the ninth: 64/1), 32/1, the pair kernel, 128/4, 64/4, 128/1, 64/2, 32/2, 128/4, 128/1 two CTAs per SM
 @pytest.mark.parametrize("M,N,K,count", [(1, 64, 64, 2), (129, 512, 128, 4), (1024, 512, 512, 8), (2000, 512, 512, 9), (33, 528, 320, 17),
-                                         (9000, 256, 192, 8)])
+                                         (9000, 256, 192, 8), (1, 512, 512, 8), (130, 512, 1088, 2), (500, 512, 512, 8),
+                                         (40, 528, 1088, 8), (130, 128, 512, 3), (700, 144, 2048, 2), (900, 272, 512, 8)])
 def test_linear_multi_is_the_single_products(api, M, N, K, count):
     """Every product of grace_linear_multi against fp64 (fp32 sums, one rounding to bf16), with more products than a
     launch takes, tiles that cut the last rows and columns, and neighbours' outputs that must stay apart."""
@@ -363,3 +370,53 @@ def test_row_statistics_of_a_gemm_that_forms_them(api, M, K, mean):
     bound = 3 * 2.0 ** -25 * (1 + (mu * mu / var).mean().item())
     assert (((aff[:, 0].double() - rstd) / rstd) ** 2).mean().sqrt() <= bound
     assert ((aff[:, 1].double() + rstd * mu).norm() / (rstd * mu).norm().clamp_min(1e-30)) <= 2 * bound
+
+
+# an item shared by a cluster of two and of four CTAs at both head sizes, ragged, with and without lengths (CTAs of a cluster
+# that have no block of a short request)
+@pytest.mark.parametrize("B,M,H,d,T", [(1, 130, 4, 128, 600), (1, 130, 4, 128, 1100), (7, 20, 2, 128, 1030), (7, 20, 5, 128, 520),
+                                       (3, 70, 2, 64, 600), (7, 130, 4, 64, 300)])
+@pytest.mark.parametrize("lengths", [False, True])
+def test_cross_attn_items_shared_by_clusters(api, B, M, H, d, T, lengths):
+    rng = synth.rng_for(2, 2000 + M + T)
+    q, k, v = (synth.normal_bf16(rng, s) for s in ((B, M, H, d), (B, H, T, d), (B, H, T, d)))
+    enc_len = np.minimum(np.array([T - 3, 0, 1, 128, T, 257, 130]), T).astype(np.int32)[:B]
+    out, lse = torch.full((B * M, H, d), 7.0, dtype=torch.bfloat16, device=DEV), torch.zeros((B * M, H), device=DEV)
+    args = dev_bf16(q).reshape(B * M, H, d), dev_bf16(k), dev_bf16(v), out
+    if lengths:
+        ref, lse_ref = OA.cross_attn_varlen(f64(q), f64(k), f64(v), enc_len, d ** -0.5)
+        api.grace_cross_attn_varlen(*args, dev(enc_len), d ** -0.5, lse)
+    else:
+        ref, lse_ref = OA.cross_attn(f64(q), f64(k), f64(v), d ** -0.5)
+        api.grace_cross_attn(*args, d ** -0.5, lse)
+    torch.cuda.synchronize()
+    got, got_lse = out.float().cpu().numpy().reshape(B, M, H, d), lse.cpu().numpy().reshape(B, M, H)
+    assert_attention_close(got, ref, "shared by clusters")
+    some = enc_len > 0 if lengths else np.ones(B, bool)
+    assert (got[~some] == 0).all() and np.isneginf(got_lse[~some]).all()
+    np.testing.assert_allclose(got_lse[some], lse_ref[some], atol=2e-3, rtol=0)
+
+
+# the four-stream kernel, and items shared by clusters of two and four at both head sizes
+@pytest.mark.parametrize("B,M,H,d,T", [(20, 300, 4, 64, 640), (1, 130, 2, 128, 640), (1, 130, 2, 128, 1152), (2, 130, 2, 64, 640),
+                                       (2, 130, 12, 64, 300)])
+@pytest.mark.parametrize("lengths", [False, True])
+def test_cross_attn_growing_scores_on_the_other_routes(api, B, M, H, d, T, lengths):
+    """Scores that rise along the positions by more than the lazy-rescaling threshold, and rows where they fall: the
+    accumulator is rescaled under way, and CTAs that share an item merge very different maxima."""
+    rng = synth.rng_for(2, 2100 + M + T)
+    q = np.abs(synth.bf16_bits_to_f32(synth.normal_bf16(rng, (B, M, H, d)))) + 0.5
+    q[:, ::2] *= -1.0
+    k = synth.bf16_bits_to_f32(synth.normal_bf16(rng, (B, H, T, d))) * 0.1 + np.linspace(0.0, 9.0, T, dtype=np.float32)[None, None, :, None]
+    qb, kb, vb = synth.f32_to_bf16_bits(q), synth.f32_to_bf16_bits(k), synth.normal_bf16(rng, (B, H, T, d))
+    scale = 0.125 if d == 64 else 0.0625
+    enc_len = np.full(B, T - 5, np.int32) if lengths else np.full(B, T, np.int32)
+    ref, _ = OA.cross_attn_varlen(f64(qb), f64(kb), f64(vb), enc_len, scale)
+    out = torch.zeros((B * M, H, d), dtype=torch.bfloat16, device=DEV)
+    args = dev_bf16(qb).reshape(B * M, H, d), dev_bf16(kb), dev_bf16(vb), out
+    if lengths:
+        api.grace_cross_attn_varlen(*args, dev(enc_len), scale)
+    else:
+        api.grace_cross_attn(*args, scale)
+    torch.cuda.synchronize()
+    assert_attention_close(out.float().cpu().numpy().reshape(B, M, H, d), ref, "growing scores")
