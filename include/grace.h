@@ -187,7 +187,8 @@ grace_status_t grace_cross_attn(const uint16_t* q, int64_t q_row_stride,
 
 /* The same with padded encoder outputs (an extension; the paper fixes T_ctx per batch, Section 3.2):
  *   enc_len : device int32 [B] or NULL; request b attends to positions 0 .. enc_len[b]-1 only
- *             (values are clamped to [0, T_ctx]); NULL = all T_ctx positions.
+ *             (values are clamped to [0, T_ctx]; K and V past them have no influence whatever they hold,
+ *             NaN included); NULL = all T_ctx positions.
  * A request with enc_len 0 gets zero output rows and lse = -inf (the softmax over an empty set is
  * left undefined by the paper).  grace_cross_attn is this call with enc_len = NULL. */
 grace_status_t grace_cross_attn_varlen(const uint16_t* q, int64_t q_row_stride,
