@@ -140,9 +140,9 @@ struct DeviceSetup {
   explicit operator bool() const { return needed; }
   void done() { if (bit) __atomic_fetch_or(mask, bit, __ATOMIC_RELEASE); }
 };
-// CTAs of a kernel with one per SM that a B200 holds at once: alone, in clusters of two and of four (a cluster lies within a
+// CTAs of a kernel with one per SM that a B200 holds at once: alone, in clusters of two, four and eight (a cluster lies within a
 // GPC; cudaOccupancyMaxActiveClusters).  The dispatch rules count in these; grids that have to fit ask the device.
-constexpr int kSms = 148, kSmsInTwos = 148, kSmsInFours = 132;
+constexpr int kSms = 148, kSmsInTwos = 148, kSmsInFours = 132, kSmsInEights = 120;
 inline int current_device_index() {
   int dev = 0;
   if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= kMaxDevices) return 0;

@@ -73,6 +73,9 @@ grace_status_t step_linear_add_bf16(const uint16_t* x, int64_t ldx, const uint16
 grace_status_t step_linear_layer_norm(const uint16_t* x, int64_t ldx, const uint16_t* w, int64_t ldw, float eps, float* row_affine,
                                       const float* col_sum, const float* col_bias, uint16_t* y_bf16, float* y_f32, int64_t ldy,
                                       float* lse_part, int M, int N, int K, int relu, void* stream);
+// layer_chain.cu: the layers of steps of few rows, without their cross-attention
+bool layer_chain_takes(const grace_decoder_t* d, int t);
+grace_status_t layer_chain(const grace_decoder_t* d, int t, int post, void* stream);
 // beam_topk.cu: a selection that ends with the state update
 grace_status_t beam_topk_update(const float* cand, int B, int64_t N, int K, int V, float* out_score, int32_t* out_flat,
                                 int32_t* out_parent, int32_t* out_token, void* ws, size_t ws_bytes,
@@ -122,9 +125,17 @@ extern "C" grace_status_t grace_decode_step(const grace_decoder_t* d, int t, voi
     return xb ? grace::step_linear_add_bf16(a, lda, w, K, d->x_bf16, D, R, D, K, stream)
               : grace::step_linear(a, lda, w, K, nullptr, d->x, D, d->x, R, D, K, 0, stream);
   };
-  if (xb) GRACE_TRY(grace_embed_bf16(d->token[cur], d->embed, d->pos + (int64_t)t * D, d->x_bf16, R, D, d->V + 1, st, stream));
+  const bool chain = grace::layer_chain_takes(d, t);
+  if (chain) {
+    for (int l = 0; l < d->n_layers; ++l) {
+      GRACE_TRY(grace::layer_chain(d, t, l - 1, stream));
+      GRACE_TRY(grace_cross_attn(d->qkv, HD, d->layers[l].k_cross, d->layers[l].v_cross, (int64_t)d->T_ctx * HD, d->d_h, HD,
+                                 d->attn, HD, nullptr, B, M, d->H, d->d_h, d->T_ctx, scale, st, stream));
+    }
+    GRACE_TRY(grace::layer_chain(d, t, d->n_layers - 1, stream));
+  } else if (xb) GRACE_TRY(grace_embed_bf16(d->token[cur], d->embed, d->pos + (int64_t)t * D, d->x_bf16, R, D, d->V + 1, st, stream));
   else GRACE_TRY(grace_embed(d->token[cur], d->embed, d->pos + (int64_t)t * D, d->x, R, D, d->V + 1, st, stream));
-  for (int l = 0; l < d->n_layers; ++l) {
+  for (int l = 0; l < d->n_layers && !chain; ++l) {
     const grace_layer_t& w = d->layers[l];
     // self-attention block
     if (w.qkv_slabs != nullptr) {                          // the projection lands in the cache slab of this step
@@ -206,11 +217,12 @@ extern "C" grace_status_t grace_decode_step(const grace_decoder_t* d, int t, voi
 namespace grace {
 int linear_tc_timeouts();
 int cross_attn_tc_timeouts();
+int layer_chain_timeouts();
 }  // namespace grace
 
 extern "C" int grace_wait_timeouts(void) {
-  const int a = grace::linear_tc_timeouts(), b = grace::cross_attn_tc_timeouts();
-  return (a < 0 || b < 0) ? -1 : a + b;
+  const int a = grace::linear_tc_timeouts(), b = grace::cross_attn_tc_timeouts(), c = grace::layer_chain_timeouts();
+  return (a < 0 || b < 0 || c < 0) ? -1 : a + b + c;
 }
 
 // Keeps part of a buffer that many kernels of a step re-read (the residual stream: three add-reductions,

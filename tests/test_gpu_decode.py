@@ -242,3 +242,64 @@ def test_decode_without_materialised_candidates_equals_the_materialised_path(kin
     assert torch.equal(outs[0][0].view(torch.int32), outs[1][0].view(torch.int32))
     assert torch.equal(outs[0][1], outs[1][1]) and torch.equal(outs[0][2], outs[1][2])
     assert torch.equal(outs[0][3], outs[1][3])
+
+
+@pytest.mark.parametrize("B,schedule,residual_bf16,shape", [
+    (1, (1, 1, 16, 16), True, (2, 128, 4, 32, 512, 128)),              # one row, one tile with few live rows
+    (1, (1, 63, 64, 65), True, (2, 512, 8, 64, 2048, 512)),            # around a tile of 64 rows; all eight CTAs
+    (3, (1, 64, 43, 65), "uncentred", (2, 512, 8, 64, 2048, 512)),     # requests across tiles, column sums
+    (3, (1, 64, 43, 65), False, (2, 512, 8, 64, 2048, 512)),
+    (2, (1, 33, 100, 64), True, (3, 256, 4, 64, 1024, 256)),           # four CTAs
+    (2, (1, 33, 100, 64), False, (1, 256, 8, 32, 512, 256)),           # a layer on its own, two heads a CTA, 128 hidden columns each
+    (2, (1, 33, 100, 64), True, (2, 512, 16, 32, 1536, 512)),          # 192 hidden columns a CTA: a pass of 128, one of 64
+    (2, (1, 33, 60, 64), False, (2, 128, 2, 64, 128, 128)),            # 64 hidden columns a CTA
+])
+def test_layers_in_one_kernel_equal_the_layers_as_launches(B, schedule, residual_bf16, shape):
+    """Steps of few rows run what lies between two cross-attentions as one kernel where the cache is kept in place; with a
+    cache of its own (kv_in_place=False) every stage is a launch.  Same inputs, step by step: residual stream, K and V.
+    Both round the same values to bf16 (three additions into the stream per layer, or three LayerNorms and as many
+    products in front of the fp32 stream), and a sum in another order moves a rounding by at most 2^-8 of the value:
+    relative difference <= 2^-8 sqrt(3 layers)."""
+    from paper_2608_00938_b200 import api
+    from paper_2608_00938_b200.decoder import Decoder
+    cfg = _config1(B=B, matcher_kind="node", schedule=schedule, final_k=16, n_sids=4000, shape=shape, ln_affine=True, T_ctx=40)
+    made = []
+    dec, _ = _make_gpu_decoder(cfg, residual_bf16=residual_bf16)
+    made.append(dec)
+    shp, trie = cfg["shp"], cfg["trie"]
+    bits, base, _ = api.grace_trie_build_dense(cfg["sids"], shp.V)
+    mb = np.stack([api.grace_node_bitmask_build(cfg["sids"], shp.V, e, trie.num_nodes) for e in cfg["elig"]])
+    made.append(Decoder(n_layers=shp.n_layers, d_model=shp.d_model, n_heads=shp.n_heads, d_head=shp.d_head, d_ffn=shp.d_ffn,
+                        V=shp.V, L=shp.L, T_ctx=40, B=B, beam_sizes=list(schedule) + [16], weights=cfg["w"], trie_bits=bits,
+                        trie_base=base, num_nodes=trie.num_nodes, matcher=(api.MATCH_NODE_BITMASK, mb, 0, 0), device=DEV,
+                        separate_cand=True, residual_bf16=bool(residual_bf16), kv_in_place=False,
+                        centre_stream=False if residual_bf16 == "uncentred" else None))
+    one, many = made
+    enc = torch.from_numpy(cfg["enc"]).to(DEV).to(torch.bfloat16)
+    for d in made:
+        d.project_cross_kv(enc)
+        d.reset()
+    bound = 2.0 ** -8 * (3 * shp.n_layers) ** 0.5
+
+    def differ(a, b):
+        return ((a.double() - b.double()).norm() / b.double().norm()).item()
+
+    for t in range(shp.L):
+        R, cur = B * schedule[t], t & 1
+        launches = []
+        for d in made:
+            n = api.grace_kernel_launch_count()
+            if d is many:                                    # the same beam
+                for name in ("token", "score", "node", "key"):
+                    getattr(many, name)[cur].copy_(getattr(one, name)[cur])
+                many.parents[t].copy_(one.parents[t])
+            d.step(t)
+            torch.cuda.synchronize()
+            assert d.d_status.item() & ~api.DEV_TOPK_EXACT_PATH == 0
+            launches.append(api.grace_kernel_launch_count() - n)
+        assert launches[0] < launches[1]
+        assert differ(one.x[:R], many.x[:R]) <= bound, f"step {t}: residual stream"
+        for li in range(shp.n_layers):
+            assert differ(one.qkv_slabs[li][t][:R, 1], many.k_cache[li][t][:R]) <= bound, f"step {t}: K of layer {li}"
+            assert differ(one.qkv_slabs[li][t][:R, 2], many.v_cache[li][t][:R]) <= bound, f"step {t}: V of layer {li}"
+    assert api.grace_wait_timeouts() == 0
