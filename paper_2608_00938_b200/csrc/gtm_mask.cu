@@ -441,7 +441,8 @@ constexpr int kLookupMaxWords = 64;          // V <= 4096
 template <int WBM, int WBL>
 __global__ void __launch_bounds__(kMaskWarpsPerBlock * 32)
 gtm_lookup_kernel(const LookupParams p) {
-  extern __shared__ uint64_t s_user[];                         // [WBM] bitmask, then [N_loc][WBL]
+  extern __shared__ __align__(16) uint64_t s_user[];           // [WBM] bitmask, then, from an even word on, [N_loc][WBL]
+  uint64_t* const s_loc = s_user + ((WBM + 1) & ~1);
   __shared__ unsigned long long s_allow[kMaskWarpsPerBlock][kLookupMaxWords];
   __shared__ int s_queue[kMaskWarpsPerBlock][96];
   __shared__ int s_order[WBM + 1];                             // number of words to read, then which, in that order
@@ -453,7 +454,7 @@ gtm_lookup_kernel(const LookupParams p) {
   pdl_trigger();
   for (int i = threadIdx.x; i < WBM; i += blockDim.x) s_user[i] = ix.user_bitmask[(int64_t)b * WBM + i];
   for (int i = threadIdx.x; i < ix.N_loc * WBL; i += blockDim.x)
-    s_user[WBM + i] = ix.user_blooms[(int64_t)b * ix.N_loc * WBL + i];
+    s_loc[i] = ix.user_blooms[(int64_t)b * ix.N_loc * WBL + i];
   if (threadIdx.x == 0) s_order[0] = 0;
   __syncthreads();
   if (threadIdx.x < WBM) {
@@ -523,8 +524,12 @@ gtm_lookup_kernel(const LookupParams p) {
       __syncwarp();
       const bool last_round = (j0 + 64 >= end);
       while (queued >= 32 || (last_round && queued > 0)) {
+        // A row has a few survivors: with at most 16 or 8 of them, two or four lanes share one, each a part of the
+        // locations (a request's 64 locations, lane by lane, were a quarter of what the SM's load unit did for a row).
         const int take = min(queued, 32);
-        const int e = (lane < take) ? queue[queued - take + lane] : -1;
+        const int wide = take > 16 ? 32 : take > 8 ? 16 : 8;             // survivors side by side
+        const int slot = lane & (wide - 1), share = (ix.N_loc * wide + 31) >> 5;
+        const int e = (slot < take) ? queue[queued - take + slot] : -1;
         queued -= take;
         bool ok = false;
         if (e >= 0) {
@@ -533,17 +538,28 @@ gtm_lookup_kernel(const LookupParams p) {
 #pragma unroll
           for (int w = 0; w < WBL; ++w) nbl[w] = ~__ldg(blp + w);
           // ANY-of-N_loc, branch-free inside a group of eight locations, early exit between groups
-          for (int q0 = 0; q0 < ix.N_loc && !ok; q0 += 8) {
-            const int qn = min(8, ix.N_loc - q0);
+          const int q_first = (lane / wide) * share, q_end = min(ix.N_loc, q_first + share);
+          for (int q0 = q_first; q0 < q_end && !ok; q0 += 8) {
+            const int qn = min(8, q_end - q0);
             for (int q = 0; q < qn; ++q) {
-              const uint64_t* qr = s_user + WBM + (q0 + q) * WBL;
+              const uint64_t* qr = s_loc + (q0 + q) * WBL;
               uint64_t outside = 0ull;
+              if (WBL % 2 == 0) {
 #pragma unroll
-              for (int w = 0; w < WBL; ++w) outside |= qr[w] & nbl[w];
+                for (int w = 0; w < WBL; w += 2) {
+                  const ulonglong2 u = *reinterpret_cast<const ulonglong2*>(qr + w);
+                  outside |= (u.x & nbl[w]) | (u.y & nbl[(w + 1) % WBL]);
+                }
+              } else {
+#pragma unroll
+                for (int w = 0; w < WBL; ++w) outside |= qr[w] & nbl[w];
+              }
               ok = ok || (outside == 0ull);
             }
           }
         }
+        const uint32_t votes = __ballot_sync(kFullMask, ok);
+        ok = slot == lane && e >= 0 && (wide == 32 ? ok : ((wide == 16 ? votes | (votes >> 16) : votes | (votes >> 8) | (votes >> 16) | (votes >> 24)) >> slot) & 1u);
         if (ok) {
           int entry = e;
           if (kway) {                          // the entry that owns slot e: last one whose first slot is <= e
@@ -830,7 +846,7 @@ extern "C" grace_status_t grace_gtm_lookup(const float* logp, const float* beam_
   p.logp = logp; p.beam_score = beam_score; p.beam_node = beam_node; p.idx = *index; p.cand = cand;
   p.allow_bits = allow_bits; p.d_status = d_status; p.M = M;
   dim3 grid((unsigned)((M + kMaskWarpsPerBlock - 1) / kMaskWarpsPerBlock), (unsigned)B);
-  const size_t smem = (size_t)(index->W_bm + (size_t)index->N_loc * index->W_bl) * sizeof(uint64_t);
+  const size_t smem = (size_t)(((index->W_bm + 1) & ~1) + (size_t)index->N_loc * index->W_bl) * sizeof(uint64_t);
   cudaStream_t s = (cudaStream_t)stream;
   const int threads = kMaskWarpsPerBlock * 32;
   if (index->W_bm == 7 && index->W_bl == 4) launch_pdl(gtm_lookup_kernel<7, 4>, grid, dim3(threads), smem, s, p);

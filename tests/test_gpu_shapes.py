@@ -420,3 +420,11 @@ def test_cross_attn_growing_scores_on_the_other_routes(api, B, M, H, d, T, lengt
         api.grace_cross_attn(*args, scale)
     torch.cuda.synchronize()
     assert_attention_close(out.float().cpu().numpy().reshape(B, M, H, d), ref, "growing scores")
+
+
+# a few survivors of the attributes share the locations among the lanes of a warp: fewer locations than lanes that share
+# them, counts that no share divides, one past a whole group of eight; a request that every entry's attributes let through
+@pytest.mark.parametrize("n_loc", [1, 3, 9, 33])
+def test_gtm_lookup_with_any_number_of_locations(api, n_loc):
+    from test_gpu_ops import test_gtm_lookup_paper_form_matches_oracle as paper_form
+    paper_form(api, 256, 4, 9000, 3, 21, 1, n_loc)
