@@ -108,6 +108,7 @@ extern "C" grace_status_t grace_decode_step(const grace_decoder_t* d, int t, voi
     return xb ? grace_layer_norm_bf16(d->x_bf16, g, b, d->h, R, D, d->ln_eps, stream)
               : grace_layer_norm(d->x, g, b, d->h, R, D, d->ln_eps, stream);
   };
+  bool normed = false;                                      // d->h already holds the rows of the final LayerNorm
   // LayerNorm + the GEMM that consumes it: either the two kernels, or (folded) row statistics + a GEMM on the
   // raw stream whose epilogue applies them
   const bool folded = xb && d->row_affine != nullptr;
@@ -116,8 +117,10 @@ extern "C" grace_status_t grace_decode_step(const grace_decoder_t* d, int t, voi
     if (folded)
       return grace::step_linear_layer_norm(d->x_bf16, D, w, D, d->ln_eps, d->row_affine, cs, cb, y_bf16, y_f32, ldy, lse_part, R,
                                      N, D, relu, stream);
-    grace_status_t s1 = layer_norm(g, b);
-    if (s1 != GRACE_OK) return s1;
+    if (!normed) {
+      const grace_status_t s1 = layer_norm(g, b);
+      if (s1 != GRACE_OK) return s1;
+    }
     if (lse_part != nullptr) return grace_linear_f32_lse(d->h, D, w, D, y_f32, ldy, lse_part, R, N, D, stream);
     return grace::step_linear(d->h, D, w, D, y_bf16, y_f32, ldy, nullptr, R, N, D, relu, stream);
   };
@@ -133,6 +136,7 @@ extern "C" grace_status_t grace_decode_step(const grace_decoder_t* d, int t, voi
                                  d->attn, HD, nullptr, B, M, d->H, d->d_h, d->T_ctx, scale, st, stream));
     }
     GRACE_TRY(grace::layer_chain(d, t, d->n_layers - 1, stream));
+    normed = !xb;
   } else if (xb) GRACE_TRY(grace_embed_bf16(d->token[cur], d->embed, d->pos + (int64_t)t * D, d->x_bf16, R, D, d->V + 1, st, stream));
   else GRACE_TRY(grace_embed(d->token[cur], d->embed, d->pos + (int64_t)t * D, d->x, R, D, d->V + 1, st, stream));
   for (int l = 0; l < d->n_layers && !chain; ++l) {
@@ -175,7 +179,7 @@ extern "C" grace_status_t grace_decode_step(const grace_decoder_t* d, int t, voi
       GRACE_TRY(grace_linear_logits_allowed(d->x_bf16, D, d->w_out, D, d->ln_eps, d->row_affine, d->cs_out, d->cb_out,
                                             d->allow_bits, d->logp, d->V, d->lse_part, R, d->V, D, stream));
     else {
-      GRACE_TRY(layer_norm(d->lnf_g, d->lnf_b));
+      if (!normed) GRACE_TRY(layer_norm(d->lnf_g, d->lnf_b));
       GRACE_TRY(grace_linear_logits_allowed(d->h, D, d->w_out, D, 0.f, nullptr, nullptr, nullptr, d->allow_bits, d->logp,
                                             d->V, d->lse_part, R, d->V, D, stream));
     }

@@ -27,6 +27,9 @@
 // Measured and left out: sixteen epilogue warps of 16 columns (167 -> 204 us), a deeper ring (165), all columns of a k-block in
 // one MMA (164, d_model 128: 47 -> 50).
 //
+// With an fp32 stream the final LayerNorm comes out of the last launch as well (2 x 128, three steps of up to 16 rows: 174 -> 168
+// us a search); the bf16 stream's is folded into the output head.
+//
 // Row statistics travel with the tiles as (mean, sum of squared deviations) per 32 columns and are merged by the reader.
 #include "common.cuh"
 #include "tc.cuh"
@@ -58,7 +61,8 @@ struct LayerChainParams {
   const int32_t* parents;                                  // [L + 1][R_max]
   int32_t* d_status;
   const float *cb_1, *cs_1, *cb_qkv, *cs_qkv, *cb_qc, *cs_qc;              // folded: bias, column sums (or NULL)
-  const float *ln1_g, *ln1_b, *ln2_g, *ln2_b, *ln3_g, *ln3_b;              // not folded
+  const float *ln1_g, *ln1_b, *ln2_g, *ln2_b, *ln3_g, *ln3_b;              // not folded; behind the last layer ln1 is the final one,
+  uint16_t* h_final;                                       //   whose rows go here, [R][D]
 };
 
 template <int C>
@@ -301,7 +305,7 @@ layer_chain_kernel(const __grid_constant__ LayerChainMaps maps, const __grid_con
       for (int i = threadIdx.x; i < 384; i += 256) {
         const int which = i >> 6, n = rank * 64 + (i & 63);
         const float* src = which == 0 ? p.ln1_g : which == 1 ? p.ln1_b : which == 2 ? p.ln2_g : which == 3 ? p.ln2_b : which == 4 ? p.ln3_g : p.ln3_b;
-        vec[i] = ((which < 4) ? p.pre : p.post) ? __ldg(src + n) : 0.f;
+        vec[i] = (which < 2 || (which < 4 ? p.pre : p.post)) ? __ldg(src + n) : 0.f;
       }
     }
     if (threadIdx.x == 0) {
@@ -610,7 +614,15 @@ layer_chain_kernel(const __grid_constant__ LayerChainMaps maps, const __grid_con
       }
       // The CTA's 64 columns become k-block `rank` of every CTA's operand tile: x for a LayerNorm (the raw bf16 rows with
       // their statistics, or, F32, the normalised rows), or the self-attention's output.
-      if (step != 2 || p.pre) {
+      // a warp per destination: copies that eight lanes of one warp send are issued one after the other
+      auto send_stats = [&]() {
+        const float2* mine = stats + rank * 2 * kLcRows;
+        if (warp == rank) tc::mbar_expect_tx(stats_full, (C - 1) * 2 * kLcRows * 8);
+        else dsmem_bulk_copy(tc::cluster_addr_of(mine, (uint32_t)warp), mine, 2 * kLcRows * 8, tc::cluster_addr_of(stats_full, (uint32_t)warp));
+      };
+      // (F32 behind the last layer: the final LayerNorm's rows go to memory, for the output head.)
+      const bool next = step != 2 || p.pre;
+      if (next || F32) {
         if (step != 3 && warp_lives) {                     // mean and sum of squared deviations of the thread's 32 columns
           float s0 = 0.f, s1 = 0.f, s2 = 0.f, s3 = 0.f;
 #pragma unroll
@@ -624,12 +636,6 @@ layer_chain_kernel(const __grid_constant__ LayerChainMaps maps, const __grid_con
           }
           if (lives) stats[(rank * 2 + half) * kLcRows + row] = make_float2(mean, (s0 + s1) + (s2 + s3));
         }
-        // a warp per destination: copies that eight lanes of one warp send are issued one after the other
-        auto send_stats = [&]() {
-          const float2* mine = stats + rank * 2 * kLcRows;
-          if (warp == rank) tc::mbar_expect_tx(stats_full, (C - 1) * 2 * kLcRows * 8);
-          else dsmem_bulk_copy(tc::cluster_addr_of(mine, (uint32_t)warp), mine, 2 * kLcRows * 8, tc::cluster_addr_of(stats_full, (uint32_t)warp));
-        };
         if constexpr (F32) {
           if (step != 3) {
             tc::fence_proxy_async_smem();
@@ -643,6 +649,8 @@ layer_chain_kernel(const __grid_constant__ LayerChainMaps maps, const __grid_con
               w[i >> 1] = pack_bf16x2((x[i] - nm.x) * nm.y * g[i] + g[64 + i], (x[i + 1] - nm.x) * nm.y * g[i + 1] + g[65 + i]);
           }
         }
+      }
+      if (next) {
         if (use > 0) tc::mbar_wait_cluster(a_free, (use - 1) & 1, abort_flag);
         ++use;
         if (lives) {
@@ -660,6 +668,10 @@ layer_chain_kernel(const __grid_constant__ LayerChainMaps maps, const __grid_con
           if (!F32 && step != 3) send_stats();
         }
         __syncwarp();
+      } else if (F32 && valid) {
+        uint4* dst = reinterpret_cast<uint4*>(p.h_final + mm * p.D + col0);
+#pragma unroll
+        for (int j = 0; j < 4; ++j) dst[j] = make_uint4(w[4 * j], w[4 * j + 1], w[4 * j + 2], w[4 * j + 3]);
       }
       if (step == 4 || (step == 2 && !p.pre)) {            // the stream as the next kernel finds it
         if (valid) {
@@ -706,7 +718,7 @@ bool layer_chain_takes(const grace_decoder_t* d, int t) {
       if (!grace_aligned16(q)) return false;
     return true;
   };
-  if (!aligned({d->x, d->x_bf16, d->attn, d->qkv, d->embed, d->pos})) return false;
+  if (!aligned({d->x, d->x_bf16, d->attn, d->qkv, d->h, d->embed, d->pos})) return false;
   for (int l = 0; l < d->n_layers; ++l) {
     const grace_layer_t& w = d->layers[l];
     if (w.qkv_slabs == nullptr || !aligned({w.qkv_slabs, w.w_qkv, w.w_o, w.w_qc, w.w_oc, w.w_1, w.w_2})) return false;
@@ -739,7 +751,7 @@ static grace_status_t launch_chain(const LayerChainMaps& maps, const LayerChainP
 }
 
 // The part of layer `post` behind its cross-attention (post < 0: none; then the rows are embedded first) and the part of
-// layer post + 1 in front of its own (where there is one).
+// layer post + 1 in front of its own; behind the last layer, with an fp32 stream, the final LayerNorm into d->h.
 grace_status_t layer_chain(const grace_decoder_t* d, int t, int post, void* stream) {
   const int D = d->d_model, C = D / 64, R = d->B * d->beam_sizes[t], pre = post + 1;
   LayerChainMaps maps;
@@ -772,6 +784,8 @@ grace_status_t layer_chain(const grace_decoder_t* d, int t, int post, void* stre
     p.cb_qkv = w.cb_qkv; p.cs_qkv = w.cs_qkv; p.cb_qc = w.cb_qc; p.cs_qc = w.cs_qc;
     p.ln1_g = w.ln1_g; p.ln1_b = w.ln1_b; p.ln2_g = w.ln2_g; p.ln2_b = w.ln2_b;
     p.slabs = w.qkv_slabs;
+  } else {
+    p.ln1_g = d->lnf_g; p.ln1_b = d->lnf_b; p.h_final = d->h;
   }
   if (!ok) return GRACE_CUDA_ERROR;
   cudaStream_t s = (cudaStream_t)stream;
