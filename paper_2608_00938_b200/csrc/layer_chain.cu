@@ -718,10 +718,14 @@ bool layer_chain_takes(const grace_decoder_t* d, int t) {
       if (!grace_aligned16(q)) return false;
     return true;
   };
-  if (!aligned({d->x, d->x_bf16, d->attn, d->qkv, d->h, d->embed, d->pos})) return false;
+  // (what the launches refuse for its alignment is left to them)
+  if (!aligned({d->x, d->x_bf16, d->attn, d->qkv, d->h, d->embed, d->pos, d->lnf_g, d->lnf_b})) return false;
   for (int l = 0; l < d->n_layers; ++l) {
     const grace_layer_t& w = d->layers[l];
-    if (w.qkv_slabs == nullptr || !aligned({w.qkv_slabs, w.w_qkv, w.w_o, w.w_qc, w.w_oc, w.w_1, w.w_2})) return false;
+    if (w.qkv_slabs == nullptr || !aligned({w.qkv_slabs, w.w_qkv, w.w_o, w.w_qc, w.w_oc, w.w_1, w.w_2, w.ln1_g, w.ln1_b, w.ln2_g,
+                                             w.ln2_b, w.ln3_g, w.ln3_b}))
+      return false;
+    if (d->x == nullptr && !aligned({w.cb_qkv, w.cs_qkv, w.cb_qc, w.cs_qc, w.cb_1, w.cs_1})) return false;
   }
   const int64_t R = (int64_t)d->B * d->beam_sizes[t];
   return t <= 3 && R <= (int64_t)layer_chain_clusters(C) * kLcRows;
