@@ -401,7 +401,8 @@ layer_chain_kernel(const __grid_constant__ LayerChainMaps maps, const __grid_con
       if (step & 1) {
         float2 ar = make_float2(1.f, 0.f);                 // folded: y = rstd acc + (-rstd mean) col_sum + col_bias
         uint32_t qw[16];
-        if (step == 3 && lives) {
+        auto fetch_prefix = [&]() {
+          if (step != 3 || !lives) return;
 #pragma unroll 1
           for (int j = 0; j < p.t; ++j) {
             const int64_t a = j == 0 ? anc[0] : j == 1 ? anc[1] : anc[2];
@@ -412,11 +413,17 @@ layer_chain_kernel(const __grid_constant__ LayerChainMaps maps, const __grid_con
               asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(tc::smem_addr(prefix_at(j, 1, i))), "l"(src + p.D + 8 * i) : "memory");
             }
           }
-        }
+        };
+        // The prefix overwrites the CTA's hidden k-blocks, the source of the copies to the pair's other CTA.  That they have
+        // arrived there is known from what the other CTA does behind its second product: its arrival after the partial sums
+        // (C >= 4), or its statistics of step 2, which an fp32 stream has waited for and a bf16 one waits for here.
+        constexpr bool kPrefixFirst = F32 || C >= 4;
+        if (kPrefixFirst) fetch_prefix();
         if constexpr (!F32) {
           const float2 nm = row_norm();
           ar = make_float2(nm.y, -nm.y * nm.x);
         }
+        if (!kPrefixFirst) fetch_prefix();
         const int chunks = step == 1 ? n_h : step == 3 ? 3 : 1;
 #pragma unroll 1
         for (int c = 0; c < chunks; ++c) {

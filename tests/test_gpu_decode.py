@@ -303,3 +303,24 @@ def test_layers_in_one_kernel_equal_the_layers_as_launches(B, schedule, residual
             assert differ(one.qkv_slabs[li][t][:R, 1], many.k_cache[li][t][:R]) <= bound, f"step {t}: K of layer {li}"
             assert differ(one.qkv_slabs[li][t][:R, 2], many.v_cache[li][t][:R]) <= bound, f"step {t}: V of layer {li}"
     assert api.grace_wait_timeouts() == 0
+
+
+@pytest.mark.parametrize("B,schedule,residual_bf16,shape", [
+    (74, (1, 64, 64, 64), True, (2, 128, 4, 32, 512, 128)),            # the prefix comes in where the hidden columns were
+])
+def test_layers_in_one_kernel_repeat_their_bits(B, schedule, residual_bf16, shape):
+    """Shared memory that a copy to another CTA reads is written again only once the copy has arrived: steps of as many
+    rows as one launch takes, again and again, leave the same residual stream, K, V and scores."""
+    dec, api = _make_gpu_decoder(_config1(B=B, matcher_kind="node", schedule=schedule, final_k=16, n_sids=4000, shape=shape,
+                                          ln_affine=True, T_ctx=40), residual_bf16=residual_bf16)
+    dec.reset()
+    for t in range(dec.L):
+        R, K = B * schedule[t], dec.beam_sizes[t + 1]
+        seen = []
+        for _ in range(12):
+            dec.step(t)
+            seen.append([dec.x[:R].clone(), dec.score[(t + 1) & 1][:B * K].clone()] + [s[t][:R].clone() for s in dec.qkv_slabs])
+        torch.cuda.synchronize()
+        for again in seen[1:]:
+            assert all(torch.equal(a, b) for a, b in zip(seen[0], again)), f"step {t}"
+    assert api.grace_wait_timeouts() == 0
