@@ -269,8 +269,9 @@ layer_chain_kernel(const __grid_constant__ LayerChainMaps maps, const __grid_con
         __syncwarp();
         if (++slot == kLcStages) { slot = 0; lap ^= 1; }
       }
-      // the last product on this tile: the cluster may fill it again
-      const bool last = g == 0 || g == n_pass || g == n_post + 1 || g == n_post + 2;
+      // the last product on this tile: the cluster may fill it again.  (Said only where every CTA waits for it before it leaves:
+      // with two CTAs and no layer behind, nothing comes after the hidden columns.)
+      const bool last = g == 0 || (g == n_pass && (C >= 4 || p.pre)) || g == n_post + 1 || g == n_post + 2;
       if (tc::elect_one()) {
         if (last) mma_commit_cluster(a_free, kAll);
         tc::mma_commit(acc_full + (ev & 1));
