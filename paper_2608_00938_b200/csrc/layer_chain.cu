@@ -630,37 +630,47 @@ layer_chain_kernel(const __grid_constant__ LayerChainMaps maps, const __grid_con
       };
       // (F32 behind the last layer: the final LayerNorm's rows go to memory, for the output head.)
       const bool next = step != 2 || p.pre;
-      if (next || F32) {
-        if (step != 3 && warp_lives) {                     // mean and sum of squared deviations of the thread's 32 columns
-          float s0 = 0.f, s1 = 0.f, s2 = 0.f, s3 = 0.f;
-#pragma unroll
-          for (int i = 0; i < 32; i += 4) { s0 += x[i]; s1 += x[i + 1]; s2 += x[i + 2]; s3 += x[i + 3]; }
-          const float mean = ((s0 + s1) + (s2 + s3)) * (1.f / 32.f);
-          s0 = s1 = s2 = s3 = 0.f;
-#pragma unroll
-          for (int i = 0; i < 32; i += 4) {
-            const float a = x[i] - mean, b = x[i + 1] - mean, c = x[i + 2] - mean, d = x[i + 3] - mean;
-            s0 = fmaf(a, a, s0); s1 = fmaf(b, b, s1); s2 = fmaf(c, c, s2); s3 = fmaf(d, d, s3);
-          }
-          if (lives) stats[(rank * 2 + half) * kLcRows + row] = make_float2(mean, (s0 + s1) + (s2 + s3));
-        }
-        if constexpr (F32) {
-          if (step != 3) {
-            tc::fence_proxy_async_smem();
-            tc::named_bar_sync(1, 256);
-            if (warp < C && tc::elect_one()) send_stats();
-            __syncwarp();
-            const float2 nm = row_norm();
-            const float* g = vec + (step == 0 ? 256 : step == 2 ? 0 : 128) + half * 32;
-#pragma unroll
-            for (int i = 0; i < 32; i += 2)
-              w[i >> 1] = pack_bf16x2((x[i] - nm.x) * nm.y * g[i] + g[64 + i], (x[i + 1] - nm.x) * nm.y * g[i + 1] + g[65 + i]);
-          }
-        }
-      }
-      if (next) {
+      auto tile_free = [&]() {                             // every CTA is done with its operand tile
         if (use > 0) tc::mbar_wait_cluster(a_free, (use - 1) & 1, abort_flag);
         ++use;
+      };
+      float2 mine32 = make_float2(0.f, 0.f);
+      if ((next || F32) && step != 3 && warp_lives) {      // mean and sum of squared deviations of the thread's 32 columns
+        float s0 = 0.f, s1 = 0.f, s2 = 0.f, s3 = 0.f;
+#pragma unroll
+        for (int i = 0; i < 32; i += 4) { s0 += x[i]; s1 += x[i + 1]; s2 += x[i + 2]; s3 += x[i + 3]; }
+        const float mean = ((s0 + s1) + (s2 + s3)) * (1.f / 32.f);
+        s0 = s1 = s2 = s3 = 0.f;
+#pragma unroll
+        for (int i = 0; i < 32; i += 4) {
+          const float a = x[i] - mean, b = x[i + 1] - mean, c = x[i + 2] - mean, d = x[i + 3] - mean;
+          s0 = fmaf(a, a, s0); s1 = fmaf(b, b, s1); s2 = fmaf(c, c, s2); s3 = fmaf(d, d, s3);
+        }
+        mine32 = make_float2(mean, (s0 + s1) + (s2 + s3));
+        if (F32 && lives) stats[(rank * 2 + half) * kLcRows + row] = mine32;
+      }
+      // The statistics before these were the source of copies.  That they have arrived: an fp32 stream's last tiles came
+      // behind every CTA's wait for them; for a bf16 stream, whose tiles travel beside them, a free tile says it (step 2: all
+      // CTAs have added their partial sums or, with two, the other one's hidden columns have come; step 4: all are through
+      // the self-attention).
+      if constexpr (!F32) {
+        if (next) {
+          tile_free();
+          if (step != 3 && lives) stats[(rank * 2 + half) * kLcRows + row] = mine32;
+        }
+      } else if (step != 3) {
+        tc::fence_proxy_async_smem();
+        tc::named_bar_sync(1, 256);
+        if (warp < C && tc::elect_one()) send_stats();
+        __syncwarp();
+        const float2 nm = row_norm();
+        const float* g = vec + (step == 0 ? 256 : step == 2 ? 0 : 128) + half * 32;
+#pragma unroll
+        for (int i = 0; i < 32; i += 2)
+          w[i >> 1] = pack_bf16x2((x[i] - nm.x) * nm.y * g[i] + g[64 + i], (x[i + 1] - nm.x) * nm.y * g[i + 1] + g[65 + i]);
+      }
+      if (next) {
+        if (F32) tile_free();
         if (lives) {
           uint8_t* tile = tile_a + rank * kLcTile + row * 128;
 #pragma unroll

@@ -309,6 +309,8 @@ def test_layers_in_one_kernel_equal_the_layers_as_launches(B, schedule, residual
     (74, (1, 64, 64, 64), True, (2, 128, 4, 32, 512, 128)),            # the prefix comes in where the hidden columns were
     (74, (1, 64, 64, 64), True, (1, 128, 4, 32, 512, 128)),            # two CTAs, nothing after the hidden columns of a launch
     (74, (1, 64, 64, 64), False, (1, 128, 4, 32, 512, 128)),
+    (15, (1, 64, 64, 64), True, (2, 512, 8, 64, 2048, 512)),           # statistics beside the tiles, of eight and of four CTAs
+    (33, (1, 64, 64, 64), "uncentred", (2, 256, 4, 64, 1024, 256)),
 ])
 def test_layers_in_one_kernel_repeat_their_bits(B, schedule, residual_bf16, shape):
     """Shared memory that a copy to another CTA reads is written again only once the copy has arrived: steps of as many
