@@ -729,7 +729,7 @@ bool layer_chain_takes(const grace_decoder_t* d, int t) {
   const int D = d->d_model;
   if ((D != 128 && D != 256 && D != 512) || d->H * d->d_h != D || (d->d_h != 32 && d->d_h != 64)) return false;
   const int C = D / 64;
-  if (d->d_ffn % (64 * C) != 0 || d->d_ffn / (64 * C) > kLcMaxHidden) return false;
+  if (d->d_ffn <= 0 || d->d_ffn % (64 * C) != 0 || d->d_ffn / (64 * C) > kLcMaxHidden) return false;
   if (d->x == nullptr && d->row_affine == nullptr) return false;       // bf16 stream with LayerNorm kernels of its own
   auto aligned = [](std::initializer_list<const void*> ps) {
     for (const void* q : ps)

@@ -328,3 +328,15 @@ def test_layers_in_one_kernel_repeat_their_bits(B, schedule, residual_bf16, shap
         for again in seen[1:]:
             assert all(torch.equal(a, b) for a, b in zip(seen[0], again)), f"step {t}"
     assert api.grace_wait_timeouts() == 0
+
+
+@pytest.mark.parametrize("residual_bf16", [True, False])
+@pytest.mark.parametrize("d_ffn", [0, -512])
+def test_step_without_hidden_columns_is_refused(residual_bf16, d_ffn):
+    dec, api = _make_gpu_decoder(_config1(), residual_bf16=residual_bf16)
+    dec.reset()
+    dec.struct.d_ffn = d_ffn
+    with pytest.raises(api.GraceError) as refused:
+        dec.step(0)
+    assert refused.value.code == api.GRACE_INVALID_ARG
+    torch.cuda.synchronize()
