@@ -338,5 +338,5 @@ def test_step_without_hidden_columns_is_refused(residual_bf16, d_ffn):
     dec.struct.d_ffn = d_ffn
     with pytest.raises(api.GraceError) as refused:
         dec.step(0)
-    assert refused.value.code == api.GRACE_INVALID_ARG
+    assert refused.value.code == 1                           # GRACE_INVALID_ARG
     torch.cuda.synchronize()
