@@ -56,6 +56,7 @@ constexpr int kMsSoftmaxWarps = 16;
 constexpr int kMsThreads = (kMsSoftmaxWarps + 4) * 32;   // + one MMA issuer / TMA producer warp per stream
 constexpr int kMsBarBytes = 1024;
 constexpr int kMsSmemBytes = 1024 + 8 * kMsQBytes + 2 * kMsStages * 2 * kMsKVBytes + kMsBarBytes;
+static_assert(kMsSmemBytes >= tc::kTmemAllSmem, "");
 
 struct CrossMsParams {
   float* lse;

@@ -44,7 +44,9 @@ template <int DH, int SPLIT> struct CaCfg {
   static constexpr int kQBufs = SPLIT > 1 ? 1 : 2;
   static constexpr int kSlice = DH / SPLIT;                      // output columns a CTA finishes
   static constexpr int kXBytes = SPLIT > 1 ? (SPLIT - 1) * 128 * kSlice * 4 + SPLIT * 128 * 8 : 0;
-  static constexpr int kSmemBytes = kTileBytes * (kQBufs + 2 * kCaStages) + 1024 + kCaBarBytes + 2 * 2 * 128 * 4 + 2 * 2 * 128 * 4 + kXBytes;
+  static constexpr int kUsedBytes = kTileBytes * (kQBufs + 2 * kCaStages) + 1024 + kCaBarBytes + 2 * 2 * 128 * 4 + 2 * 2 * 128 * 4 + kXBytes;
+  // (at head size 64 less than the SM has twice, and a CTA takes all of TMEM)
+  static constexpr int kSmemBytes = kUsedBytes > tc::kTmemAllSmem ? kUsedBytes : tc::kTmemAllSmem;
   static_assert(kSmemBytes <= 227 * 1024, "");
   static constexpr uint32_t kTmemCols = 512;                     // S: 0..127, O: 2 x DH (by item parity), P: 2 x 64 (by block parity)
 };

@@ -75,7 +75,7 @@ struct LayerChainSmem {
   static constexpr int kScores = kVec + 1024 * 4;                           // [2][64] float4
   static constexpr int kBars = kScores + 2 * kLcRows * 16;
   static constexpr int kTotal = kBars + 512;
-  static_assert(kTotal <= 227 * 1024, "");
+  static_assert(kTotal <= 227 * 1024 && kTotal >= tc::kTmemAllSmem, "");
 };
 
 __device__ __forceinline__ void dsmem_bulk_copy(uint32_t dst, const void* src, uint32_t bytes, uint32_t bar) {

@@ -434,6 +434,7 @@ constexpr int kQAffBytes = 256 * 2 * 4;                   // the tile's 256 (col
 // no slack for rounding the base up: the dynamic shared memory is declared 1024-byte aligned and the kernel
 // checks it (six stages, the staging buffers and the column vectors leave less than 1 KB of the 227 KB)
 constexpr int kQSmem = kQStages * kQStageBytes + 2 * kPStagingBytes + 256 + kQAffBytes;
+static_assert(kQSmem >= tc::kTmemAllSmem, "");
 
 // STATS: the rows' LayerNorm statistics are not read from memory (aff_row is only a non-null marker then) but
 // formed inside the kernel: four more warps per CTA read every A tile out of the ring while the tensor cores

@@ -238,6 +238,12 @@ __device__ __forceinline__ void mma_commit_pair(uint64_t* bar, uint16_t cta_mask
 }
 
 // ---- TMEM ----------------------------------------------------------------------------------
+// A CTA that finds too few free columns waits in tmem_alloc until others on its SM have given theirs back.  So that these
+// others never wait for it in turn, kernels that take all 512 columns ask for kTmemAllSmem bytes of shared memory or more,
+// too much for two such CTAs on an SM: the CTAs of two clusters, say, each of which waits for its own other CTA.
+constexpr int kSmSmem = 228 * 1024, kCtaSmemReserved = 1024;
+constexpr int kTmemAllSmem = 114 * 1024;
+static_assert(2 * (kTmemAllSmem + kCtaSmemReserved) > kSmSmem, "");
 // Whole warp.  `ncols` a power of two in [32, 512].  The base address lands in *slot (shared).
 __device__ __forceinline__ void tmem_alloc(uint32_t* slot, uint32_t ncols) {
   asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_addr(slot)), "r"(ncols) : "memory");
