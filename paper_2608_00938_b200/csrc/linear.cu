@@ -80,8 +80,9 @@ linear_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_constant__
   // the wait on that kernel, so their trip from HBM overlaps its tail.  (The step's first kernel has waited for everything
   // in front of the step.)  Otherwise, and for whatever else an earlier kernel may have written (activations, row
   // statistics, the residual), every thread waits before its first access.
-  pdl_trigger();
   using S = GemmCfg<BN, STAGES, SPLIT>;
+  constexpr bool kTriggerLate = S::kTotal <= tc::kMostSmemBesideTmemAll;
+  if (!kTriggerLate) pdl_trigger();
   constexpr int kSlice = S::kSlice;
   extern __shared__ uint8_t smem_raw[];
   uint8_t* tiles = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
@@ -121,6 +122,7 @@ linear_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_constant__
   tc::tc_fence_before();
   __syncthreads();
   tc::tc_fence_after();
+  if (kTriggerLate) pdl_trigger();                         // see tc::kMostSmemBesideTmemAll
   const uint32_t tmem_base = *tmem_slot;
 
   bool ok = true;

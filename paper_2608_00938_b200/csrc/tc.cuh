@@ -244,6 +244,9 @@ __device__ __forceinline__ void mma_commit_pair(uint64_t* bar, uint16_t cta_mask
 constexpr int kSmSmem = 228 * 1024, kCtaSmemReserved = 1024;
 constexpr int kTmemAllSmem = 114 * 1024;
 static_assert(2 * (kTmemAllSmem + kCtaSmemReserved) > kSmSmem, "");
+// For the same reason a kernel that takes fewer columns lets the next kernel start only behind its allocation if a CTA of it
+// can share an SM with one of those: the next kernel's CTA would hold all columns and wait for this kernel to complete.
+constexpr int kMostSmemBesideTmemAll = kSmSmem - kTmemAllSmem - 2 * kCtaSmemReserved;
 // Whole warp.  `ncols` a power of two in [32, 512].  The base address lands in *slot (shared).
 __device__ __forceinline__ void tmem_alloc(uint32_t* slot, uint32_t ncols) {
   asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_addr(slot)), "r"(ncols) : "memory");
