@@ -244,25 +244,26 @@ def test_decode_without_materialised_candidates_equals_the_materialised_path(kin
     assert torch.equal(outs[0][3], outs[1][3])
 
 
-@pytest.mark.parametrize("B,schedule,residual_bf16,shape", [
-    (1, (1, 1, 16, 16), True, (2, 128, 4, 32, 512, 128)),              # one row, one tile with few live rows
-    (1, (1, 63, 64, 65), True, (2, 512, 8, 64, 2048, 512)),            # around a tile of 64 rows; all eight CTAs
-    (3, (1, 64, 43, 65), "uncentred", (2, 512, 8, 64, 2048, 512)),     # requests across tiles, column sums
-    (3, (1, 64, 43, 65), False, (2, 512, 8, 64, 2048, 512)),
-    (2, (1, 33, 100, 64), True, (3, 256, 4, 64, 1024, 256)),           # four CTAs
-    (2, (1, 33, 100, 64), False, (1, 256, 8, 32, 512, 256)),           # a layer on its own, two heads a CTA, 128 hidden columns each
-    (2, (1, 33, 100, 64), True, (2, 512, 16, 32, 1536, 512)),          # 192 hidden columns a CTA: a pass of 128, one of 64
-    (2, (1, 33, 60, 64), False, (2, 128, 2, 64, 128, 128)),            # 64 hidden columns a CTA
-])
-def test_layers_in_one_kernel_equal_the_layers_as_launches(B, schedule, residual_bf16, shape):
+# d_model / 64 CTAs to a cluster -> clusters that a B200 holds at once, 64 rows each at most
+_CLUSTERS = {2: 74, 4: 33, 8: 15}
+
+
+def _tile_rows(R, shape):
+    """Rows of a cluster's tile in a step of R rows: as few as spread them over the clusters, in eights; None: as launches."""
+    rows = -(-R // _CLUSTERS[shape[1] // 64])
+    return None if rows > 64 else (rows + 7) // 8 * 8
+
+
+def _layers_in_one_kernel_and_as_launches(B, schedule, residual_bf16, shape, n_sids=4000):
     """Steps of few rows run what lies between two cross-attentions as one kernel where the cache is kept in place; with a
     cache of its own (kv_in_place=False) every stage is a launch.  Same inputs, step by step: residual stream, K and V.
     Both round the same values to bf16 (three additions into the stream per layer, or three LayerNorms and as many
     products in front of the fp32 stream), and a sum in another order moves a rounding by at most 2^-8 of the value:
-    relative difference <= 2^-8 sqrt(3 layers)."""
+    relative difference <= 2^-8 sqrt(3 layers).  Logits: the final LayerNorm's rows are rounded once more, and so are the
+    differences they start from: <= 2^-8 (sqrt(3 layers) + 1)."""
     from paper_2608_00938_b200 import api
     from paper_2608_00938_b200.decoder import Decoder
-    cfg = _config1(B=B, matcher_kind="node", schedule=schedule, final_k=16, n_sids=4000, shape=shape, ln_affine=True, T_ctx=40)
+    cfg = _config1(B=B, matcher_kind="node", schedule=schedule, final_k=16, n_sids=n_sids, shape=shape, ln_affine=True, T_ctx=40)
     made = []
     dec, _ = _make_gpu_decoder(cfg, residual_bf16=residual_bf16)
     made.append(dec)
@@ -297,12 +298,52 @@ def test_layers_in_one_kernel_equal_the_layers_as_launches(B, schedule, residual
             torch.cuda.synchronize()
             assert d.d_status.item() & ~api.DEV_TOPK_EXACT_PATH == 0
             launches.append(api.grace_kernel_launch_count() - n)
-        assert launches[0] < launches[1]
+        assert launches[0] < launches[1] if _tile_rows(R, shape) else launches[0] == launches[1]
         assert differ(one.x[:R], many.x[:R]) <= bound, f"step {t}: residual stream"
+        assert differ(one.logp[:R], many.logp[:R]) <= bound + 2.0 ** -8, f"step {t}: logits"
         for li in range(shp.n_layers):
             assert differ(one.qkv_slabs[li][t][:R, 1], many.k_cache[li][t][:R]) <= bound, f"step {t}: K of layer {li}"
             assert differ(one.qkv_slabs[li][t][:R, 2], many.v_cache[li][t][:R]) <= bound, f"step {t}: V of layer {li}"
     assert api.grace_wait_timeouts() == 0
+
+
+# tiles of 8 rows, of 16 with three requests at d_model 512
+@pytest.mark.parametrize("B,schedule,residual_bf16,shape", [
+    (1, (1, 1, 16, 16), True, (2, 128, 4, 32, 512, 128)),              # one row, two tiles
+    (1, (1, 63, 64, 65), True, (2, 512, 8, 64, 2048, 512)),            # a last tile of 7, 8 and 1 rows; all eight CTAs
+    (3, (1, 64, 43, 65), "uncentred", (2, 512, 8, 64, 2048, 512)),     # requests across tiles, column sums
+    (3, (1, 64, 43, 65), False, (2, 512, 8, 64, 2048, 512)),
+    (2, (1, 33, 100, 64), True, (3, 256, 4, 64, 1024, 256)),           # four CTAs
+    (2, (1, 33, 100, 64), False, (1, 256, 8, 32, 512, 256)),           # a layer on its own, two heads a CTA, 128 hidden columns each
+    (2, (1, 33, 100, 64), True, (2, 512, 16, 32, 1536, 512)),          # 192 hidden columns a CTA: a pass of 128, one of 64
+    (2, (1, 33, 60, 64), False, (2, 128, 2, 64, 128, 128)),            # 64 hidden columns a CTA
+])
+def test_layers_in_one_kernel_equal_the_layers_as_launches(B, schedule, residual_bf16, shape):
+    _layers_in_one_kernel_and_as_launches(B, schedule, residual_bf16, shape)
+
+
+# Tiles of up to 64 rows, the last one with a few or all of them; the most rows that are taken, and one more.
+@pytest.mark.parametrize("residual_bf16", [True, False])
+@pytest.mark.parametrize("B,schedule,shape,tile", [
+    (4, (1, 64, 63, 64), (2, 512, 8, 64, 2048, 512), 24),              # 256 and 252 rows
+    (8, (1, 64, 63, 64), (2, 512, 8, 64, 2048, 512), 40),              # 512, 504
+    (1, (1, 64, 953, 950), (2, 512, 8, 64, 2048, 512), 64),            # last tiles of 57 and 54 rows
+    (15, (1, 64, 64, 64), (2, 512, 16, 32, 1536, 512), 64),            # 960
+    (1, (1, 64, 961, 961), (1, 512, 8, 64, 2048, 512), None),
+    (11, (1, 62, 60, 60), (2, 256, 4, 64, 1024, 256), 24),             # 682, 660
+    (20, (1, 62, 60, 60), (2, 256, 8, 32, 1024, 256), 40),             # 1240, 1200
+    (5, (1, 64, 421, 420), (2, 256, 4, 64, 1024, 256), 64),            # 2105, 2100
+    (33, (1, 64, 64, 64), (2, 256, 4, 64, 512, 256), 64),              # 2112
+    (1, (1, 64, 2113, 2113), (1, 256, 4, 64, 1024, 256), None),
+    (24, (1, 62, 62, 61), (2, 128, 4, 32, 512, 128), 24),              # 1488, 1464
+    (37, (1, 64, 72, 72), (2, 128, 2, 64, 512, 128), 40),              # 2368 (tiles of 32), 2664
+    (29, (1, 64, 163, 162), (2, 128, 4, 32, 512, 128), 64),            # 4727, 4698
+    (74, (1, 64, 64, 64), (2, 128, 2, 64, 128, 128), 64),              # 4736
+    (3, (1, 64, 1579, 1579), (1, 128, 4, 32, 512, 128), None),         # 4737
+])
+def test_layers_in_one_kernel_with_whole_tiles(B, schedule, shape, tile, residual_bf16):
+    assert all(_tile_rows(B * m, shape) == tile for m in schedule[2:])
+    _layers_in_one_kernel_and_as_launches(B, schedule, residual_bf16, shape, n_sids=20000)
 
 
 @pytest.mark.parametrize("B,schedule,residual_bf16,shape", [
