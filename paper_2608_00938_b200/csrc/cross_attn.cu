@@ -42,7 +42,7 @@ template <int DH, int WARPS, int PAIRS>
 __global__ void __launch_bounds__(WARPS * PAIRS * 32)
 cross_attn_row_kernel(const CrossRowParams p) {
   pdl_wait();
-  pdl_trigger();
+  pdl_trigger();                              // not before the wait: layer_chain_kernel reads weights before its own
   constexpr int G = DH / 8;                   // lanes per encoder position
   constexpr int RP = 32 / G;                  // positions per warp pass
   constexpr bool kAhead = WARPS <= 8;

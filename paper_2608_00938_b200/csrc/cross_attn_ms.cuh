@@ -138,7 +138,7 @@ cross_attn_ms_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_con
   tc::tc_fence_after();
   const uint32_t tmem_base = *tmem_slot;
   pdl_wait();                                  // barrier set-up and TMEM allocation overlapped the previous kernel's tail
-  pdl_trigger();
+  pdl_trigger();                               // not before the wait: layer_chain_kernel reads weights before its own
   // Half `hf` of CTA c works on the items c + (2 k + hf) gridDim, k = 0, 1, ...: neighbouring CTAs run
   // neighbouring items, which share K/V in L2, and with fewer items than halves every SM gets one before any
   // gets two.

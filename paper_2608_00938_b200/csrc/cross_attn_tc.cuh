@@ -186,7 +186,7 @@ cross_attn_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_con
   tc::tc_fence_after();
   const uint32_t tmem_base = *tmem_slot;
   pdl_wait();                                  // barrier set-up and TMEM allocation overlapped the previous kernel's tail
-  pdl_trigger();
+  pdl_trigger();                               // not before the wait: layer_chain_kernel reads weights before its own
   const uint32_t tmem_s = tmem_base;           // S fp32, 128 columns
   // O of an item lives in one of two accumulators (item parity) and P of a block in one of two column sets (block
   // parity), so the softmax threads hand P(g) over and go straight on to block g + 1 (whose S is already there)
@@ -260,8 +260,8 @@ cross_attn_tc_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_con
     // ---------------- MMA issuer ----------------
     // (An elected lane, not a branch on the lane number: the compiler then knows that one thread is left and takes operands
     // straight to the registers that tcgen05.mma and TMA read.  What the issuing warps save, the softmax warps of their
-    // schedulers gain: 16 x 1000 x 16 x 128 x 50..200 67.2 -> 62.5 us, 4 x 700 x 16 x 128 x 256..1024 35.2 -> 30.9,
-    // 40 x 6 x 16 x 128 x 100..600 44.8 -> 37.1, 1 x 300 x 16 x 128 x 1024 11.25 -> 10.7, 1 x 512 x 8 x 64 x 1024 7.35 -> 7.1.)
+    // schedulers gain: 16 x 1000 x 16 x 128 x 50..200 62.5 -> 59.5 us, 4 x 700 x 16 x 128 x 256..1024 42.4 -> 35.7,
+    // 40 x 6 x 16 x 128 x 100..600 42.6 -> 35.9, 1 x 300 x 16 x 128 x 1024 11.05 -> 10.45, 1 x 512 x 8 x 64 x 1024 7.1 -> 6.85.)
     if (tc::elect_one()) {
       constexpr uint32_t idesc_s = tc::idesc_bf16(kCaBM, kCaBN, 0);     // Q K^T : B K-major
       constexpr uint32_t idesc_o = tc::idesc_bf16(kCaBM, DH, 1);        // P V   : B MN-major, all output columns at once

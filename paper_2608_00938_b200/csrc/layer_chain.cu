@@ -19,18 +19,28 @@
 // added there in a fixed order.
 //
 // Every role runs its stages through one loop body: written out one by one they take a launch through far more code, of which
-// it executes every line once (a step of 2 layers of 128: 55 us, of 4 layers of 512 at 512 rows: 187; so 47 and 167).  Shared
-// memories exchange about 18 bytes per clock and CTA (8 KB to and from each of seven CTAs: 3200 clocks, 1 KB: 620), so a tile
+// it executes every line once (a step of 2 layers of 128: 55 us, of 4 layers of 512 at 512 rows: 187; so 47 and 167).  A tile
 // has no more rows than it takes to spread them over the clusters that fit, and only rows in use are sent.  What bounds a
-// layer now is the latency of its stages, about 26 us in all at d_model 512 where the launches took 37: a quarter of it the
-// exchanges, a third the products (an MMA of 128 columns takes 64 clocks), the rest what a warp does to 32 columns of a row.
+// layer is the latency of its stages, one behind the other.  4 x 512, third step, a launch between two cross-attentions, by
+// the clock of its first CTA (us; 16 rows in tiles of 8 / 512 in tiles of 40 / 960 in tiles of 64): the rows and their
+// parents 1.4 / 1.4 / 1.8; Wo_cross and the first exchange 1.7 / 1.6 / 1.6; hidden columns 4.9 / 6.1 / 6.5; their product, the
+// partial sums and the next exchange 5.3 / 5.3 / 6.5; QKV and self-attention 5.5 / 6.8 / 8.9 (16 rows of the first step, without a
+// prefix: 4.6); Wo 2.1 / 2.9 / 3.8; the queries 2.0 / 2.8 / 2.9; leaving, up to the next kernel's start 2.3 / 3.5 / 4.0.  No unit is
+// busy (512 rows: tensor pipe in 23 % of the cycles of the SMs that have a CTA, L1 22 %).
 // Measured and left out: sixteen epilogue warps of 16 columns (167 -> 204 us), a deeper ring (165), all columns of a k-block in
-// one MMA (164, d_model 128: 47 -> 50).
+// one MMA (164, d_model 128: 47 -> 50), four chains instead of two for a score (no change), tiles of at least 16 or 32 rows
+// (4 x 512, 16 rows 131 -> 132.5 us a step, 32 rows 133 -> 133.5 and 142).
 //
 // With an fp32 stream the final LayerNorm comes out of the last launch as well (2 x 128, three steps of up to 16 rows: 174 -> 168
 // us a search); the bf16 stream's is folded into the output head.
 //
 // Row statistics travel with the tiles as (mean, sum of squared deviations) per 32 columns and are merged by the reader.
+//
+// Shared memory that a bulk copy reads may be written again only once the copy is known to have arrived, and that shows at its
+// destination alone.  What says so here, for each source: a k-block of the operand tile, a_free, which every CTA gives behind
+// the products that read the copy; the hidden k-blocks, over which the cache's prefix comes in, and the row statistics, see
+// there.  Every copy, and every arrival on another CTA's barrier, is waited for by its destination in front of the final
+// cluster barrier.
 #include "common.cuh"
 #include "tc.cuh"
 #include <initializer_list>
@@ -145,7 +155,11 @@ layer_chain_kernel(const __grid_constant__ LayerChainMaps maps, const __grid_con
   if (warp == 8) tc::tmem_alloc(tmem_slot, 512);
   tc::tc_fence_before();
   __syncthreads();
-  pdl_trigger();                                           // (behind the allocation: no kernel behind this one can take TMEM first)
+  // Behind the allocation: no kernel behind this one can take TMEM first.  In front of the wait: the ring fills with weights,
+  // and in a later launch of a step the vectors are read, before the kernel in front has completed.  Whoever wrote them has: the
+  // step's first launch waits before it reads either, and between two launches lies a cross-attention, which lets the second one
+  // start only behind its own wait for the first.
+  pdl_trigger();
   tc::cluster_sync_all();                                  // every CTA's barriers exist before the first copy into it
   tc::tc_fence_after();
   const uint32_t tmem = *tmem_slot;
@@ -720,11 +734,16 @@ int layer_chain_timeouts() { return tc::tc_timeouts_read_and_clear(); }
 static int layer_chain_clusters(int C) { return C == 2 ? kSmsInTwos / 2 : C == 4 ? kSmsInFours / 4 : kSmsInEights / 8; }
 
 // Whether grace_decode_step runs the layers of step t through the kernel above: where its clusters take all rows at once (a
-// second wave costs as much again).  A step of 2 x 128, 3 tokens, selection included, launches / so (us): 16 rows 56 / 47,
-// 4096 rows 128 / 109, 8192 rows 184 / 207 (two waves); fp32 stream 63 / 49, 137 / 113.  2 x 256: 16 rows 65 / 66, 256 rows
-// 92 / 81, 2048 rows 113 / 100, 4096 rows 132 / 168.  4 x 512: 1 row 116 / 121, 64 rows 137 / 140, 256 rows 182 / 165, 960 rows
-// 212 / 190, 1024 rows 218 / 324; fp32 stream 145 / 124, 157 / 142, 195 / 170, 234 / 198.  (One to 64 rows of the bf16 stream are
-// no faster on the GPU; the host, which has 13 launches to make instead of 36, is.)
+// second wave costs as much again).  A step replayed from a graph, 3 tokens, selection included, launches / so (us).  2 x 128: 16
+// rows 56 / 48, 256 rows 76 / 65, 4096 rows 139 / 119, 4736 rows 138 / 114 (8192 rows, two waves, 184 / 207); fp32 stream 64 / 50,
+// 84 / 66, 147 / 118, 146 / 114.  2 x 256: 1 row 59 / 55, 16 rows 65 / 65, 256 rows 92 / 82, 2112 rows 112 / 98; fp32 67 / 57, 74 / 68,
+// 98 / 84, 123 / 99.  4 x 512: 1 row 116 / 116, 16 rows 127 / 132, 32 rows 130 / 133, 64 rows 136 / 137, 128 rows 155 / 145, 512 rows
+// 193 / 175, 960 rows 221 / 200; fp32 137 / 122, 151 / 137, 151 / 138, 157 / 143, 174 / 151, 213 / 183, 245 / 207.
+// So 16 to 64 rows of 4 x 512 with a bf16 stream take the GPU up to 4 % longer.  They are taken all the same, for what the host
+// has to launch (2 kernels a layer instead of 8): a search of one request, projection included, 4 x 512 bf16, beam 16, 64, 512: as
+// calls 626 -> 596, 688 -> 651, 859 -> 818 us, each waited for 680 -> 650, 741 -> 705, 914 -> 874, and from a graph 571 -> 574,
+// 630 -> 626, 801 -> 791; 2 x 256, beam 16: 307 -> 296, 353 -> 340, 278 -> 282.  One row per request, a search's first step, costs
+// nothing (1 request 115 / 115, 32 requests 121 / 121).
 bool layer_chain_takes(const grace_decoder_t* d, int t) {
   const int D = d->d_model;
   if ((D != 128 && D != 256 && D != 512) || d->H * d->d_h != D || (d->d_h != 32 && d->d_h != 64)) return false;
