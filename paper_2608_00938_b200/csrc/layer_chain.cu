@@ -739,11 +739,13 @@ static int layer_chain_clusters(int C) { return C == 2 ? kSmsInTwos / 2 : C == 4
 // 84 / 66, 147 / 118, 146 / 114.  2 x 256: 1 row 59 / 55, 16 rows 65 / 65, 256 rows 92 / 82, 2112 rows 112 / 98; fp32 67 / 57, 74 / 68,
 // 98 / 84, 123 / 99.  4 x 512: 1 row 116 / 116, 16 rows 127 / 132, 32 rows 130 / 133, 64 rows 136 / 137, 128 rows 155 / 145, 512 rows
 // 193 / 175, 960 rows 221 / 200; fp32 137 / 122, 151 / 137, 151 / 138, 157 / 143, 174 / 151, 213 / 183, 245 / 207.
-// So 16 to 64 rows of 4 x 512 with a bf16 stream take the GPU up to 4 % longer.  They are taken all the same, for what the host
-// has to launch (2 kernels a layer instead of 8): a search of one request, projection included, 4 x 512 bf16, beam 16, 64, 512: as
-// calls 626 -> 596, 688 -> 651, 859 -> 818 us, each waited for 680 -> 650, 741 -> 705, 914 -> 874, and from a graph 571 -> 574,
-// 630 -> 626, 801 -> 791; 2 x 256, beam 16: 307 -> 296, 353 -> 340, 278 -> 282.  One row per request, a search's first step, costs
-// nothing (1 request 115 / 115, 32 requests 121 / 121).
+// So up to 64 rows of a bf16 stream with 4 d_model hidden columns can take the GPU longer, by what the prefix costs inside the
+// kernel: 4 x 512, steps 1 and 3, 1 row 113 / 116 and 113 / 120, 8 rows 117 / 117 and 119 / 121, 64 rows 135 / 136 and 137 / 140; 2 x 256, 16
+// rows 63.5 / 65 and 64 / 67; a search's first step loses nothing (1 request 115 / 115, 32 requests 121 / 121).  They are taken all
+// the same, for what the host has to launch (2 kernels a layer instead of 8).  A search of one request, projection included, 4 x 512
+// bf16, beam 1, 4, 16, 64, 512: as calls 587 -> 555 us, 596 -> 557, 627 -> 594, 689 -> 649, 859 -> 818, each waited for 641 -> 606,
+// 650 -> 610, 680 -> 649, 742 -> 702, 914 -> 874, and from a graph 529 -> 533, 543 -> 539, 570 -> 569, 628 -> 623, 801 -> 791; 2 x 256, beam 16:
+// 305 -> 288, 349 -> 331, 275 -> 272.
 bool layer_chain_takes(const grace_decoder_t* d, int t) {
   const int D = d->d_model;
   if ((D != 128 && D != 256 && D != 512) || d->H * d->d_h != D || (d->d_h != 32 && d->d_h != 64)) return false;
